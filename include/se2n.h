@@ -73,13 +73,20 @@ typedef enum se2n_status {
 #define SE2N_DIFFUSE_SPLIT_DIAG 2  /* keep a_r^2/beta apart from the angular second difference
                                       (always on when beta * T > 8, see se2n_diffuse) */
 #define SE2N_DIFFUSE_FULL_CORRECTION 4  /* apply the corner correction on every angle (no truncation) */
-/* Integrate by the S-step propagator: for every class of frequencies that
- * share it (rows s, H/2 - s as they are and rows H/2 + s, H - s with the
- * angles reversed, times columns l and (W/2 - l) mod W) the matrix
- * (B-^{-1} B+)^S - I is built once in FP32 by the powering program of
- * se2n_prop_chain, in increment form, and applied as one N x N product per frequency (Section 4: the
- * integration over an interval is one linear map). The same result as S
- * Crank-Nicolson steps up to rounding. The plan keeps the matrices
+/* Integrate by the S-step propagator: the S steps of an interval are one
+ * linear map (B-^{-1} B+)^S a frequency (Section 4: the integration over an
+ * interval is one linear map), the same result as S Crank-Nicolson steps up to
+ * rounding. Outside the column pass (below) the map is applied as a polynomial of the
+ * operator, the truncated Chebyshev series of ((1 + dt x / 2) / (1 - dt x / 2))^S
+ * on the operator's spectrum (cut off below FP32 resolution: about 12
+ * multiplications by the three-point operator for T (2 + 4 beta) / 2 = 3, about
+ * 50 for 75), whose coefficients the host makes when beta, T or steps change;
+ * where more than 64 coefficients would be needed, and in the column pass, as a matrix:
+ * for every class of frequencies that share it (rows s, H/2 - s as they are
+ * and rows H/2 + s, H - s with the angles reversed, times columns l and
+ * (W/2 - l) mod W) (B-^{-1} B+)^S - I is built once in FP32 by the powering
+ * program of se2n_prop_chain, in increment form, and applied as one N x N
+ * product per frequency. The plan keeps the matrices
  * (symmetric; by cyclic diagonals, 4 N (N/2 + 1) bytes a class, or as rows,
  * 4 N^2 bytes a class, for the column pass below and for N = 64 on the
  * Hermitian half, where they are applied 16 classes of one row slot at a
@@ -252,6 +259,10 @@ SE2N_API se2n_status se2n_inverse(se2n_plan *plan, void *vol);
  * with the fused coefficient 2 + a_r^2/beta, whose FP32 rounding perturbs
  * decay rates by ~1.2e-7 beta per unit time; it costs one FMA more per angle
  * and is selected automatically when beta * T > 8.
+ * With flags = 0 and dt (2 + 4 beta) <= 2, an interval whose polynomial (see
+ * SE2N_DIFFUSE_PROPAGATOR) takes fewer operations than its steps is applied as
+ * that polynomial, the same map of S steps to FP32 rounding; any flag keeps
+ * the steps.
  * When beta*dt <= ~0.067 (no FP64 flag), a packed fast path runs: the corner
  * correction vector decays by a factor <= 1e-9 within 6 angles of the tear,
  * so it is applied on those angles only (below FP32 resolution elsewhere);
@@ -362,7 +373,9 @@ SE2N_API se2n_status se2n_plan_diffuse_info(se2n_plan *plan, int *regs_per_threa
 #define SE2N_STAGE_MIX 4
 #define SE2N_STAGE_PROJECT 5
 #define SE2N_STAGE_DR 6       /* growth steps of dynamic restoration */
-#define SE2N_STAGE_PROPAGATOR 7  /* building S-step propagators (applying them counts as diffusion) */
+#define SE2N_STAGE_PROPAGATOR 7  /* building S-step propagators (applying them counts as diffusion); the
+                                    coefficients of an interval polynomial count as one build that takes
+                                    no device time */
 #define SE2N_NUM_STAGES 8
 
 typedef struct se2n_profile {
@@ -388,7 +401,8 @@ SE2N_API se2n_status se2n_plan_profile_read(se2n_plan *plan, se2n_profile *out, 
  * method (orientation, lift, DFT, diffusion, restoration, inverse DFT,
  * projection) for every image, captured on the batch's stream. Each warp of
  * the persistent kernel claims (image, frequency-tile) items from an atomic
- * counter; the tile size, block size and threads per frequency are taken
+ * counter, integrated as se2n_diffuse would (the interval polynomial or the
+ * steps); the tile size, block size and threads per frequency are taken
  * from the built-in table or, with SE2N_BATCH_AUTOTUNE, chosen by timing
  * the candidates on this batch. se2n_batch_run replays the graph.
  * ------------------------------------------------------------------------- */
@@ -432,7 +446,7 @@ typedef struct se2n_batch_info {
  * in p->diffuse_flags, the images of each distinct (H, W, N) are integrated
  * by that shape's S-step propagators (built once a run, shared by the images)
  * when that is estimated to cost less than stepping them, the others by the
- * persistent step-by-step kernel; se2n_batch_get_info reports how many.
+ * persistent kernel; se2n_batch_get_info reports how many.
  * When every image takes propagators (on the Hermitian half), the graph runs
  * the shapes side by side: each shape's images in turn, as se2n_inpaint
  * runs one image, on a branch of their own. */

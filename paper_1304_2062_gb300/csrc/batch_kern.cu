@@ -12,6 +12,7 @@
 // The counter only grows and every claim is bounded by the item count: no
 // warp waits on another, and the kernel cannot hang.
 #include "diffuse_x2.cuh"
+#include "poly.cuh"
 #include "se2n_batch.h"
 
 namespace se2n {
@@ -58,6 +59,48 @@ __global__ void __launch_bounds__(FAST ? kDiffuseMaxBlock : 256, 1) k_diffuse_ba
     }
 }
 
+// The interval polynomial on the same items (poly_group), so that a batched
+// result is again bitwise the image's own.
+template <int N, bool REINSCH>
+__device__ __forceinline__ void poly_item(const PolyTable &t, const float *sc, const float *tables,
+                                          const BatchImage &im, const BatchItem &item, int lane) {
+    constexpr int P = poly_lanes<N>(), PER = 32 / P;
+    const float *cs = tables + im.table;
+    for (int base = 0; base < item.count; base += PER) {
+        const int o = base + lane / P;
+        const bool active = o < item.count;
+        poly_group<N, REINSCH>(t, sc, cs, cs + N, im.vol, im.H, im.W, im.Wc, im.HW, item.first + (active ? o : 0),
+                               active, 0);
+    }
+}
+
+template <bool REINSCH>
+__global__ void __launch_bounds__(256) k_poly_batch(const __grid_constant__ PolyTable t,
+                                                    const float *__restrict__ tables,
+                                                    const BatchImage *__restrict__ imgs,
+                                                    const BatchItem *__restrict__ items, int n_items,
+                                                    unsigned int *counter) {
+    __shared__ float sc[kPolyBuckets * kPolyMax];
+    poly_stage(sc, t, threadIdx.x, blockDim.x);
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    for (;;) {
+        unsigned int it = 0;
+        if (lane == 0) it = atomicAdd(counter, 1u);
+        it = __shfl_sync(0xffffffffu, it, 0);
+        if (it >= (unsigned int)n_items) return;
+        const BatchItem item = items[it];
+        const BatchImage im = imgs[item.image];
+        if (im.N == 64) {
+            poly_item<64, REINSCH>(t, sc, tables, im, item, lane);
+        } else if (im.N == 32) {
+            poly_item<32, REINSCH>(t, sc, tables, im, item, lane);
+        } else {
+            poly_item<16, REINSCH>(t, sc, tables, im, item, lane);
+        }
+    }
+}
+
 }  // namespace se2n
 
 // Launch configurations the autotuner chooses among: threads per frequency
@@ -96,4 +139,19 @@ cudaError_t se2n_launch_diffuse_batch(int config, bool fast, bool split, const S
     void *args[] = {(void *)&sp, (void *)&tables, (void *)&imgs, (void *)&items, (void *)&n_items,
                     (void *)&counter};
     return cudaLaunchKernel(batch_kernel(config, fast, split), dim3(blocks), dim3(block), args, 0, s);
+}
+
+static const void *poly_batch_kernel(bool reinsch) {
+    return reinsch ? (const void *)&se2n::k_poly_batch<true> : (const void *)&se2n::k_poly_batch<false>;
+}
+
+cudaError_t se2n_poly_batch_occupancy(bool reinsch, int block, int *blocks_per_sm) {
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, poly_batch_kernel(reinsch), block, 0);
+}
+
+cudaError_t se2n_launch_poly_batch(const PolyTable &t, const float *tables, const BatchImage *imgs,
+                                   const BatchItem *items, int n_items, unsigned int *counter, int block, int blocks,
+                                   cudaStream_t s) {
+    void *args[] = {(void *)&t, (void *)&tables, (void *)&imgs, (void *)&items, (void *)&n_items, (void *)&counter};
+    return cudaLaunchKernel(poly_batch_kernel(t.reinsch != 0), dim3(blocks), dim3(block), args, 0, s);
 }

@@ -246,6 +246,33 @@ se2n_status propagate_impl(se2n_plan *plan, float2 *vol, double beta, double bdt
     return cuda_status(plan, se2n_launch_prop_apply(plan->N, a, plan->num_sms, plan->stream));
 }
 
+// The interval polynomial of (beta, T, steps), made on the host when they
+// change; null where the form does not apply.
+const PolyTable *poly_get(se2n_plan *plan, double beta, double T, int steps) {
+    if (!plan->poly_made || plan->poly_beta != beta || plan->poly_T != T || plan->poly_steps != steps) {
+        plan->poly_ok = se2n_poly_make(beta, T, steps, plan->poly);
+        plan->poly_made = true;
+        plan->poly_built = false;
+        plan->poly_beta = beta;
+        plan->poly_T = T;
+        plan->poly_steps = steps;
+    }
+    return plan->poly_ok ? &plan->poly : nullptr;
+}
+
+// The polynomial in place of the steps: its packed instructions an angle
+// against five a step and the set-up of the step kernel's factors (N = 32,
+// 1024 x 1024, T = 2: 136 us against 120 us + 15 us a step).
+bool poly_beats_steps(const PolyTable &t, int steps) { return se2n_poly_cost(t) < 5.0 * steps + 36.0; }
+
+// The polynomial stands for the propagators: one build a change of beta, T or
+// steps, as for the matrices (it is made on the host, the stage times nothing).
+void poly_count_build(se2n_plan *plan) {
+    if (plan->poly_built) return;
+    StageTimer timer(plan, SE2N_STAGE_PROPAGATOR);
+    plan->poly_built = true;
+}
+
 // Row and column passes of the Hermitian half (rowfft.cu, colprop.cu): the
 // row-transformed volume [Wc][H][N] complex and the twiddle tables.
 bool col_path(const se2n_plan *plan, const se2n_params *p) {
@@ -360,6 +387,23 @@ se2n_status col_diffuse(se2n_plan *plan, double beta, double T, int steps) {
     return cuda_status(plan, se2n_launch_col_prop(plan->N, a, plan->stream));
 }
 
+// One interval's polynomial applied to the spectrum vol (half, k0 and rows as
+// for diffuse_impl).
+se2n_status poly_impl(se2n_plan *plan, float2 *vol, const PolyTable &t, bool half, int k0, int rows) {
+    PolyArgs a;
+    a.vol = vol;
+    a.Wc = half ? plan->Wc : plan->W;
+    a.HW = (long long)(rows >= 0 ? rows : plan->H) * a.Wc;
+    a.k0 = rows >= 0 ? k0 : 0;
+    a.H = plan->H;
+    a.W = plan->W;
+    angle_table(plan->N, plan->angle_conv, a.cs, a.sn, SE2N_MAX_N);
+    a.t = t;
+    StageTimer timer(plan, SE2N_STAGE_DIFFUSE);
+    plan->kernels += 1;
+    return cuda_status(plan, se2n_launch_poly(plan->N, a, plan->stream));
+}
+
 // half: vol holds the Hermitian half [N][H][W/2 + 1] of the spectrum.
 // rows >= 0: vol holds only spectrum rows k0 .. k0 + rows - 1 of every plane
 // ([N][rows][W], a row shard of the full spectrum).
@@ -375,8 +419,17 @@ se2n_status diffuse_impl(se2n_plan *plan, float2 *vol, double beta, double T, in
     if (!(bdt >= 1e-30 && bdt <= 1e3)) return SE2N_ENUMERIC;
     if (flags & SE2N_DIFFUSE_PROPAGATOR) {
         if (!se2n_prop_supported(plan->N) || rows >= 0) return SE2N_EUNSUPPORTED;
-        if (prop_admissible(beta, dt)) return propagate_impl(plan, vol, beta, bdt, steps, half);
+        if (prop_admissible(beta, dt)) {
+            const PolyTable *t = poly_get(plan, beta, T, steps);
+            if (!t) return propagate_impl(plan, vol, beta, bdt, steps, half);
+            poly_count_build(plan);
+            return poly_impl(plan, vol, *t, half, k0, rows);
+        }
         flags &= ~SE2N_DIFFUSE_PROPAGATOR;  // stiff: the step kernel keeps the accuracy
+    }
+    if (flags == 0) {
+        const PolyTable *t = poly_get(plan, beta, T, steps);
+        if (t && poly_beats_steps(*t, steps)) return poly_impl(plan, vol, *t, half, k0, rows);
     }
     const bool fp64 = (flags & SE2N_DIFFUSE_SM_FP64) != 0;
     // The fused diagonal 2 + a^2/beta perturbs decay rates by ~1.2e-7 beta per
@@ -995,6 +1048,7 @@ se2n_status se2n_inpaint_host(se2n_plan *plan, const float *f_host, const uint8_
 se2n_status se2n_plan_drop_propagators(se2n_plan *plan, int free_memory) {
     SE2N_TRY(check_plan(plan));
     plan->prop_valid = false;
+    plan->poly_built = false;
     if (free_memory && plan->prop_D) {
         prop_join(plan);  // a build still running on the side stream
         SE2N_TRY(cuda_status(plan, cudaStreamSynchronize(plan->stream)));
@@ -1102,6 +1156,8 @@ struct se2n_batch {
     unsigned int *d_counter = nullptr;
     int n_items = 0, config = 0, passes = 8, block = 256, blocks = 0;
     bool fast = false, split = false;
+    bool poly_on = false;  // the persistent kernel applies the interval polynomial
+    PolyTable poly{};
     int candidates = 0;
     double best_ms = 0.0, worst_ms = 0.0, updates = 0.0;
     cudaGraph_t graph = nullptr;
@@ -1160,7 +1216,10 @@ se2n_status batch_diffuse(se2n_batch *b, int steps, double T) {
     const double dt = T / steps;
     const StepParams sp = step_params(b->p.beta, b->p.beta * dt, steps);
     cudaError_t e = cudaMemsetAsync(b->d_counter, 0, sizeof(unsigned int), b->stream);
-    if (e == cudaSuccess)
+    if (e == cudaSuccess && b->poly_on)
+        e = se2n_launch_poly_batch(b->poly, b->d_tables, b->d_imgs, b->d_items, b->n_items, b->d_counter, b->block,
+                                   b->blocks, b->stream);
+    else if (e == cudaSuccess)
         e = se2n_launch_diffuse_batch(b->config, b->fast, b->split, sp, b->d_tables, b->d_imgs, b->d_items,
                                       b->n_items, b->d_counter, b->block, b->blocks, b->stream);
     return e == cudaSuccess ? SE2N_OK : SE2N_ECUDA;
@@ -1236,7 +1295,9 @@ void choose_propagators(se2n_batch *b) {
 
 se2n_status set_shape(se2n_batch *b, int config, int passes, int block) {
     int per_sm = 0;
-    if (se2n_batch_occupancy(config, b->fast, b->split, block, &per_sm) != cudaSuccess) return SE2N_ECUDA;
+    if ((b->poly_on ? se2n_poly_batch_occupancy(b->poly.reinsch != 0, block, &per_sm)
+                    : se2n_batch_occupancy(config, b->fast, b->split, block, &per_sm)) != cudaSuccess)
+        return SE2N_ECUDA;
     b->config = config;
     b->passes = passes;
     b->block = block;
@@ -1525,6 +1586,8 @@ se2n_status create_batch(se2n_batch *b, const se2n_image_desc *imgs) {
     const double bdt = b->p.beta * Tr / b->p.steps;
     b->split = (b->p.diffuse_flags & SE2N_DIFFUSE_SPLIT_DIAG) || b->p.beta * Tr > 8.0;
     b->fast = !(b->p.diffuse_flags & SE2N_DIFFUSE_FULL_CORRECTION) && se2n_diffuse_truncation_ok(bdt);
+    b->poly_on = (b->p.diffuse_flags & ~SE2N_DIFFUSE_PROPAGATOR) == 0 && b->p.T > 0.0 &&
+                 se2n_poly_make(b->p.beta, Tr, b->p.steps, b->poly) && poly_beats_steps(b->poly, b->p.steps);
     if (cudaMemsetAsync(b->arena, 0, b->vol_bytes, b->stream) != cudaSuccess) return SE2N_ECUDA;
     // transforms of the Hermitian-half path are planned before the capture
     if (!b->p.full_spectrum)
@@ -1659,7 +1722,7 @@ se2n_status se2n_batch_run(se2n_batch *b) {
 se2n_status se2n_batch_run_per_image(se2n_batch *b) {
     if (!b) return SE2N_EINVAL;
     // the same work as the graph: every shape's propagators built again
-    for (se2n_plan *pl : b->plans) pl->prop_valid = false;
+    for (se2n_plan *pl : b->plans) pl->prop_valid = pl->poly_built = false;
     for (int i = 0; i < b->count; ++i) {
         se2n_params q = b->p;
         q.N = b->imgs[i].N;

@@ -24,3 +24,8 @@ cudaError_t se2n_batch_occupancy(int config, bool fast, bool split, int block, i
 cudaError_t se2n_launch_diffuse_batch(int config, bool fast, bool split, const StepParams &sp, const float *tables,
                                       const BatchImage *imgs, const BatchItem *items, int n_items,
                                       unsigned int *counter, int block, int blocks, cudaStream_t s);
+// The same launch with the interval polynomial in place of the steps.
+cudaError_t se2n_poly_batch_occupancy(bool reinsch, int block, int *blocks_per_sm);
+cudaError_t se2n_launch_poly_batch(const PolyTable &t, const float *tables, const BatchImage *imgs,
+                                   const BatchItem *items, int n_items, unsigned int *counter, int block, int blocks,
+                                   cudaStream_t s);

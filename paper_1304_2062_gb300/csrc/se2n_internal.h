@@ -7,6 +7,7 @@
 
 #include <vector>
 
+#include "poly.h"
 #include "se2n.h"
 
 struct DrState {
@@ -55,6 +56,14 @@ struct se2n_plan {
     int chain_steps;
     unsigned char chain[SE2N_PROP_CHAIN_MAX];
     int chain_len, chain_in_r;
+    // the interval polynomial (poly.cuh) of (poly_beta, poly_T, poly_steps):
+    // poly_made once tried for them, poly_ok when the form applies;
+    // poly_built while it stands for the propagators asked for by
+    // SE2N_DIFFUSE_PROPAGATOR
+    bool poly_made, poly_ok, poly_built;
+    double poly_beta, poly_T;
+    int poly_steps;
+    PolyTable poly;
     // side stream for a build that overlaps the start of an inpaint, and the
     // events that order it after the plan's stream and the plan's stream
     // after it (join_pending until the plan's stream waits on ev_join)
@@ -103,6 +112,18 @@ struct DiffuseArgs {
     float cs[SE2N_MAX_N];
     float sn[SE2N_MAX_N];
 };
+
+// Parameters of one launch of the interval polynomial on an angle-major
+// spectrum (poly.cu).
+struct PolyArgs {
+    float2 *vol;
+    long long HW;
+    int H, W, Wc, k0;  // as in DiffuseArgs
+    float cs[SE2N_MAX_N];
+    float sn[SE2N_MAX_N];
+    PolyTable t;
+};
+cudaError_t se2n_launch_poly(int N, const PolyArgs &a, cudaStream_t s);
 
 // Parameters of the propagator kernels (propagator.cu): build D_S for every
 // class of frequencies with equal coefficients, or apply it to the volume.

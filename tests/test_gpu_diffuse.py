@@ -242,3 +242,25 @@ def test_fast_path_equals_general_path_and_oracle(N, P, beta, T, S):
     print(f"N={N} P={P} beta*dt={beta * T / S:.4f}: fast {ef:.2e} general {eg:.2e}")
     assert ef <= REL_L2 and eg <= REL_L2
     assert rel_l2(fast, full) <= 2e-6
+
+
+@pytest.mark.parametrize("N,H,W,beta,T,S,flags", [
+    (32, 24, 20, 0.25, 2.0, 3, 0),       # dt (2 + 4 beta) = 2, the largest admitted step
+    (32, 24, 20, 0.5, 0.5, 1, 0),        # one step: near the line where stepping costs as little
+    (32, 24, 20, 0.25, 11.0, 300, 0),    # the widest increment form
+    (32, 24, 20, 0.25, 13.0, 300, 0),    # Reinsch's recurrence from here on
+    (64, 18, 22, 0.25, 60.0, 900, 0), (64, 18, 22, 0.25, 120.0, 900, 0),   # near and past 64 coefficients
+    (32, 18, 22, 0.25, 120.0, 900, 8), (16, 18, 22, 0.25, 120.0, 900, 8),  # past them: matrices
+    (16, 2, 2, 0.004, 9.0, 60, 0),       # a small beta: coefficients out of range for powers of A / beta
+    (4, 10, 6, 2.0, 0.4, 30, 0), (8, 6, 34, 0.25, 30.0, 200, 0), (12, 14, 10, 0.3, 3.0, 50, 0),
+    (24, 26, 18, 0.3, 1.5, 60, 0), (30, 22, 26, 0.2, 6.0, 80, 8), (48, 12, 20, 0.1, 20.0, 100, 0)])
+@pytest.mark.parametrize("conv", [0, 1])
+def test_interval_polynomial_matches_oracle(N, H, W, beta, T, S, flags, conv):
+    """Both forms of the interval polynomial over their range, on both sides
+    of every line of the rule that picks them, against the oracle's steps."""
+    vol = synth.random_volume(N, H, W, seed=N + S + H).astype(np.complex64)
+    ref = oracle.diffuse(vol.astype(np.complex128), beta, T, S, angle_conv=conv)
+    got = _run(vol, N, beta, T, S, conv=conv, flags=flags)
+    err = rel_l2(got, ref)
+    print(f"N={N} {H}x{W} beta={beta} T={T} S={S} flags={flags} conv={conv}: rel-L2 {err:.2e}")
+    assert err <= REL_L2
