@@ -76,12 +76,13 @@ typedef enum se2n_status {
 /* Integrate by the S-step propagator: the S steps of an interval are one
  * linear map (B-^{-1} B+)^S a frequency (Section 4: the integration over an
  * interval is one linear map), the same result as S Crank-Nicolson steps up to
- * rounding. Outside the column pass (below) the map is applied as a polynomial of the
- * operator, the truncated Chebyshev series of ((1 + dt x / 2) / (1 - dt x / 2))^S
+ * rounding. The map is applied as a polynomial of the operator, the truncated Chebyshev series of ((1 + dt x / 2) / (1 - dt x / 2))^S
  * on the operator's spectrum (cut off below FP32 resolution: about 12
  * multiplications by the three-point operator for T (2 + 4 beta) / 2 = 3, about
  * 50 for 75), whose coefficients the host makes when beta, T or steps change;
- * where more than 64 coefficients would be needed, and in the column pass, as a matrix:
+ * where more than 64 coefficients would be needed, and in the column pass (below)
+ * with N = 16 or where applying kept matrices is faster (T (2 + 4 beta) / 2 above
+ * about 3), as a matrix:
  * for every class of frequencies that share it (rows s, H/2 - s as they are
  * and rows H/2 + s, H - s with the angles reversed, times columns l and
  * (W/2 - l) mod W) (B-^{-1} B+)^S - I is built once in FP32 by the powering
@@ -97,12 +98,15 @@ typedef enum se2n_status {
  * 32 x 32 matrices whose last two rows and columns are zero (the bytes of
  * N = 32). The other flags do not apply.
  * In se2n_inpaint on the Hermitian half with N = 16, 30 or 32 and H, W each one
- * of 64, 128, 256, 384, 512, 768, 1024, this flag alone selects the row and column passes: the
- * volume stays row-transformed between intervals in a plan buffer of
- * 8 (W/2 + 1) H N bytes, each interval is one kernel a column (DFT along y,
- * propagators, inverse DFT) and one kernel a row (real DFTs along x around
- * the restoration), and no cuFFT call is made. The first such call
- * allocates that buffer and a second stream of the plan, on which each
+ * of 64, 128, 256, 384, 512, 768, 1024, this flag alone selects the row and column passes (as
+ * does flags = 0 where the polynomial takes the place of the steps and has at
+ * most 32 coefficients): the
+ * volume stays row-transformed between intervals in the caller's volume
+ * buffer, each interval is one kernel a column (DFT along y,
+ * the interval's map, inverse DFT) and one kernel a row (real DFTs along x around
+ * the restoration), and no cuFFT call is made between intervals. The first
+ * such call allocates two tables of 8 H and 8 W bytes and, where matrices are
+ * built, a second stream of the plan, on which each
  * build runs beside the orientation and the lift (ordered after the work
  * already on the plan's stream, joined before the first column pass);
  * call once before capturing se2n_inpaint into a graph.

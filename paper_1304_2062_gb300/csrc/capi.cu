@@ -273,12 +273,31 @@ void poly_count_build(se2n_plan *plan) {
     plan->poly_built = true;
 }
 
+// The polynomial the column pass takes for one interval with these flags (0 or
+// SE2N_DIFFUSE_PROPAGATOR); null where it takes matrices, or with flags = 0
+// where there is no column pass. Asked for propagators, N = 30 and 32 take the
+// polynomial while it is no slower than applying matrices the plan has kept
+// from an earlier call (512 x 512, T = 2, 42 instructions an angle: 45.5 us a
+// column pass either way, and no build), and N = 16 matrices, which are small
+// (768 x 1024: 65 us against 72).
+const PolyTable *col_poly(se2n_plan *plan, double beta, double T, int steps, int flags) {
+    if (flags != 0 && plan->N < 30) return nullptr;
+    const PolyTable *t = poly_get(plan, beta, T, steps);
+    if (!t || !se2n_col_has_poly(*t)) return nullptr;
+    if (flags == 0) return poly_beats_steps(*t, steps) ? t : nullptr;
+    return se2n_poly_cost(*t) <= 45 ? t : nullptr;
+}
+
 // Row and column passes of the Hermitian half (rowfft.cu, colprop.cu): the
-// row-transformed volume [Wc][H][N] complex and the twiddle tables.
-bool col_path(const se2n_plan *plan, const se2n_params *p) {
-    return !p->full_spectrum && p->diffuse_flags == SE2N_DIFFUSE_PROPAGATOR &&
-           prop_admissible(p->beta, p->T / p->rounds / p->steps) && se2n_col_supported(plan->N, plan->H) &&
-           se2n_row_supported(plan->N, plan->W);
+// row-transformed volume [Wc][H][N] complex and the twiddle tables. Taken with
+// propagators, and with no flag where the interval's polynomial takes the
+// place of the steps.
+bool col_path(se2n_plan *plan, const se2n_params *p) {
+    if (p->full_spectrum || (p->diffuse_flags & ~SE2N_DIFFUSE_PROPAGATOR) || !(p->T > 0.0)) return false;
+    const double Tr = p->T / p->rounds;
+    if (!prop_admissible(p->beta, Tr / p->steps)) return false;
+    if (!se2n_col_supported(plan->N, plan->H) || !se2n_row_supported(plan->N, plan->W)) return false;
+    return p->diffuse_flags != 0 || col_poly(plan, p->beta, Tr, p->steps, 0) != nullptr;
 }
 
 // exp(-2 pi i m / n), m < n, from the exact fraction m / n
@@ -301,16 +320,6 @@ se2n_status upload_twiddles(float2 **dst, int n) {
 
 se2n_status col_ensure(se2n_plan *plan) {
     if (plan->col_ready) return SE2N_OK;
-    if (!plan->colbuf) {
-        // N = 30 is held in 32 slots
-        cudaError_t e =
-            cudaMalloc(&plan->colbuf, (size_t)plan->Wc * se2n_prop_dim(plan->N) * plan->H * sizeof(float2));
-        if (e != cudaSuccess) {
-            plan->colbuf = nullptr;
-            (void)cudaGetLastError();
-            return e == cudaErrorMemoryAllocation ? SE2N_ENOMEM : SE2N_ECUDA;
-        }
-    }
     if (!plan->col_tw) SE2N_TRY(upload_twiddles(&plan->col_tw, plan->H));
     if (!plan->row_tw) SE2N_TRY(upload_twiddles(&plan->row_tw, plan->W));
     if (cuda_status(plan, se2n_col_prepare(plan->N, plan->H)) != SE2N_OK ||
@@ -320,22 +329,22 @@ se2n_status col_ensure(se2n_plan *plan) {
     return SE2N_OK;
 }
 
-// The row and column passes' buffers, and the propagators: they depend on
-// beta dt and S only, so they are built on the side stream while the
+// The row and column passes' buffers, and the propagators' matrices where they
+// are taken: they depend on beta dt and S only, so they are built on the side stream while the
 // orientation, the lift (and the host copies of se2n_inpaint_host) run.
 se2n_status col_start(se2n_plan *plan, const se2n_params *p) {
     SE2N_TRY(col_ensure(plan));
-    const double bdt = p->beta * (p->T / p->rounds) / p->steps;
-    if (p->T > 0.0 && bdt >= 1e-30 && bdt <= 1e3)
+    const double Tr = p->T / p->rounds, bdt = p->beta * Tr / p->steps;
+    if (p->T > 0.0 && bdt >= 1e-30 && bdt <= 1e3 && !col_poly(plan, p->beta, Tr, p->steps, p->diffuse_flags))
         SE2N_TRY(prop_ensure(plan, p->beta, bdt, p->steps, true, PROP_CHUNKS, true));
     return SE2N_OK;
 }
 
-RowArgs row_args(se2n_plan *plan, const float *f, const uint8_t *mask, const uint8_t *bins, float scale, float eps,
-                 float guard) {
+RowArgs row_args(se2n_plan *plan, float2 *spec, const float *f, const uint8_t *mask, const uint8_t *bins, float scale,
+                 float eps, float guard) {
     RowArgs r;
-    r.spec_in = plan->colbuf;
-    r.spec_out = plan->colbuf;
+    r.spec_in = spec;
+    r.spec_out = spec;
     r.real_in = nullptr;
     r.real_out = nullptr;
     r.proj_out = nullptr;
@@ -366,15 +375,23 @@ se2n_status row_pass(se2n_plan *plan, const RowArgs &r) {
     return cuda_status(plan, se2n_launch_row(plan->N, plan->W, r, plan->stream));
 }
 
-se2n_status col_diffuse(se2n_plan *plan, double beta, double T, int steps) {
+se2n_status col_diffuse(se2n_plan *plan, float2 *spec, double beta, double T, int steps, int flags) {
     if (!(beta > 0.0) || !(T >= 0.0) || steps < 1 || !isfinite(beta) || !isfinite(T)) return SE2N_EINVAL;
     if (T == 0.0) return SE2N_OK;
     const double bdt = beta * (T / steps);
     if (!(bdt >= 1e-30 && bdt <= 1e3)) return SE2N_ENUMERIC;
-    SE2N_TRY(prop_ensure(plan, beta, bdt, steps, true, PROP_CHUNKS));
-    prop_join(plan);
     ColArgs a;
-    a.col = plan->colbuf;
+    if (const PolyTable *t = col_poly(plan, beta, T, steps, flags)) {
+        if (flags & SE2N_DIFFUSE_PROPAGATOR) poly_count_build(plan);
+        a.use_poly = 1;
+        a.t = *t;
+        angle_table(plan->N, plan->angle_conv, a.cs, a.sn, 32);
+    } else {
+        SE2N_TRY(prop_ensure(plan, beta, bdt, steps, true, PROP_CHUNKS));
+        prop_join(plan);
+        a.use_poly = 0;
+    }
+    a.col = spec;
     a.D = plan->prop_D;
     a.tw = plan->col_tw;
     a.H = plan->H;
@@ -679,17 +696,17 @@ se2n_status inpaint_impl(se2n_plan *plan, const float *f, const uint8_t *mask, c
         // real-to-complex transforms, and let the inverse transform rebuild
         // the rest.
         if (col) {
-            // With propagators on a supported shape the volume stays
+            // On a supported shape the volume stays, in vol,
             // row-transformed between intervals: a row pass (lift, or
             // inverse DFT along x, restoration and forward DFT along x) and
-            // a column pass (DFT along y, propagators, inverse DFT along y)
+            // a column pass (DFT along y, the interval, inverse DFT along y)
             // an interval, the projection fused into the last row pass.
             // Dynamic restoration adds a row pass that gives the image
             // value and its argmax angle before each growth step.
-            RowArgs r = row_args(plan, f, mask, bins, inv_hw, eps, guard);
+            RowArgs r = row_args(plan, vol, f, mask, bins, inv_hw, eps, guard);
             r.in_mode = SE2N_ROW_IN_LIFT;
             SE2N_TRY(row_pass(plan, r));
-            SE2N_TRY(col_diffuse(plan, p->beta, Tr, p->steps));
+            SE2N_TRY(col_diffuse(plan, vol, p->beta, Tr, p->steps, p->diffuse_flags));
             for (int i = 1; i <= p->rounds; ++i) {
                 const bool last = i == p->rounds;
                 const float *rf = f;
@@ -698,7 +715,7 @@ se2n_status inpaint_impl(se2n_plan *plan, const float *f, const uint8_t *mask, c
                     // a growth step: the image value h and its argmax angle
                     // from one row pass, then the set grows; the restoration
                     // below pulls the grown set to its references
-                    r = row_args(plan, f, mask, bins, inv_hw, eps, guard);
+                    r = row_args(plan, vol, f, mask, bins, inv_hw, eps, guard);
                     r.out_mode = SE2N_ROW_OUT_H;
                     r.h_out = dr->h;
                     r.amax_out = dr->amax;
@@ -708,7 +725,7 @@ se2n_status inpaint_impl(se2n_plan *plan, const float *f, const uint8_t *mask, c
                     rmask = dr->mask[dr->cur];
                     rbins = dr->bins;
                 }
-                r = row_args(plan, rf, rmask, rbins, inv_hw, eps, guard);
+                r = row_args(plan, vol, rf, rmask, rbins, inv_hw, eps, guard);
                 r.rf = f;     // reinjection keeps the given known pixels
                 r.rmask = mask;
                 if (last) {
@@ -722,7 +739,7 @@ se2n_status inpaint_impl(se2n_plan *plan, const float *f, const uint8_t *mask, c
                 }
                 r.mix = 1;
                 SE2N_TRY(row_pass(plan, r));
-                SE2N_TRY(col_diffuse(plan, p->beta, Tr, p->steps));
+                SE2N_TRY(col_diffuse(plan, vol, p->beta, Tr, p->steps, p->diffuse_flags));
             }
         } else {
             SE2N_TRY(ensure_half(plan));
@@ -776,7 +793,6 @@ void free_plan(se2n_plan *plan) {
         cudaEventDestroy(plan->ev_fork);
         cudaEventDestroy(plan->ev_join);
     }
-    cudaFree(plan->colbuf);
     cudaFree(plan->col_tw);
     cudaFree(plan->row_tw);
     cudaFree(plan->spec);
@@ -1238,7 +1254,8 @@ se2n_status batch_interval(se2n_batch *b, double Tr, bool half) {
     return SE2N_OK;
 }
 
-// With SE2N_DIFFUSE_PROPAGATOR, the images of one shape are integrated by
+// With SE2N_DIFFUSE_PROPAGATOR, where the interval polynomial does not apply,
+// the images of one shape are integrated by
 // that shape's propagators when building them once and applying them to every
 // image and interval is estimated to cost less than the step-by-step kernel on
 // those images. The estimate uses this library's measured rates on a GB300:
@@ -1257,6 +1274,27 @@ void choose_propagators(se2n_batch *b) {
     if (!(p.diffuse_flags & SE2N_DIFFUSE_PROPAGATOR)) return;
     if (!prop_admissible(p.beta, p.T / p.rounds / p.steps)) return;
     const bool half = !p.full_spectrum;
+    if (b->poly_on) {
+        // The interval polynomial runs the same arithmetic either way. Shapes
+        // on the row and column passes, and planes with enough angles to give
+        // a launch of their own work for the whole device, run apart from the
+        // others (which the graph can then do side by side); the small ones
+        // share the persistent launch. 2^17 angles are 8192 threads, two
+        // warps an SM.
+        for (se2n_plan *pl : b->plans) {
+            const bool fused = col_path(pl, &p);
+            const long long freqs = (long long)pl->H * (half ? pl->Wc : pl->W);
+            if (!fused && freqs * pl->N < (1LL << 17)) continue;
+            for (int i = 0; i < b->count; ++i)
+                if (b->plan_of[i] == pl) {
+                    b->img_prop[i] = 1;
+                    b->prop_images += 1;
+                    b->img_fused[i] = fused;
+                    b->fused_images += fused;
+                }
+        }
+        return;
+    }
     const int S = p.steps;
     unsigned char ops[SE2N_PROP_CHAIN_MAX];
     int len = 0, in_r = 0, products = 0;
@@ -1604,9 +1642,10 @@ se2n_status create_batch(se2n_batch *b, const se2n_image_desc *imgs) {
             // everything the whole inpaints allocate or create, before the capture
             SE2N_TRY(col_ensure(pl));
             SE2N_TRY(side_ensure(pl));
-            SE2N_TRY(prop_reserve(pl, true, PROP_CHUNKS));
+            if (!col_poly(pl, b->p.beta, Tr, b->p.steps, b->p.diffuse_flags))
+                SE2N_TRY(prop_reserve(pl, true, PROP_CHUNKS));
             if (b->p.dynamic) SE2N_TRY(dr_alloc(pl->dr, pl->HW));
-        } else {
+        } else if (!b->poly_on) {
             SE2N_TRY(prop_reserve(pl, !b->p.full_spectrum, se2n_prop_apply_fmt(pl->N, !b->p.full_spectrum)));
         }
         if (se2n_prop_prepare(pl->N) != cudaSuccess) return SE2N_ECUDA;

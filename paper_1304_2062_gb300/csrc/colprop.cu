@@ -5,11 +5,11 @@
 // contiguous and a frequency's N angles are adjacent. For every column l:
 //   1. the DFT along y (index k) of every angle plane (unnormalised), which
 //      completes the two-dimensional DFT of the lifted volume;
-//   2. x <- x + D_S x for the N-vector of every frequency (k, l), D_S the
-//      S-step propagator of its class, stored by 16-byte chunks of its rows,
-//      chunk-major (eq. (4.2), Theorem 2, integrated by S Crank-Nicolson
-//      steps; see propagator.cu), with the angles reversed for rows H/2 + s
-//      and H - s;
+//   2. the interval of eq. (4.2) (Theorem 2, S Crank-Nicolson steps) for the
+//      N-vector of every frequency (k, l): as the polynomial of its operator
+//      (poly.cuh), or x <- x + D_S x with D_S the S-step propagator of the
+//      frequency's class, stored by 16-byte chunks of its rows, chunk-major
+//      (propagator.cu), with the angles reversed for rows H/2 + s and H - s;
 //   3. the inverse DFT along k,
 // in shared memory, so the spectrum of the interval never goes through
 // device memory.
@@ -29,6 +29,7 @@
 // halves one after the other, v and then the even half's result y_e held in
 // the rows of the column's own block in device memory.
 #include "diffuse_x2.cuh"
+#include "poly.cuh"
 #include "prop_classes.cuh"
 #include "se2n_internal.h"
 #include "smem_fft.cuh"
@@ -131,6 +132,40 @@ __device__ __forceinline__ void col_apply(float2 *X, const float *D, int scol, i
     }
 }
 
+// Coefficients and angles of the interval polynomial, in shared memory. The
+// increment form has at most 32 coefficients (poly.cu).
+constexpr int kColPolyLen = 32;
+struct ColPoly {
+    float c[kPolyBuckets * kColPolyLen];
+    float cs[32], sn[32];
+};
+__device__ __forceinline__ void col_poly_stage(ColPoly &q, const ColArgs &a, int tid, int threads) {
+    poly_stage(q.c, a.t, tid, threads);
+    for (int i = tid; i < 32; i += threads) {
+        q.cs[i] = a.cs[i];
+        q.sn[i] = a.sn[i];
+    }
+}
+
+// x <- x + g(A) A x for frequency k of a column with wx = sin(2 pi l / W): the
+// K angles r0 .. r0 + K - 1 of one of the NE / K lanes of the frequency. get(v)
+// fills v from shared memory, add(v) adds v to it (x is read a second time
+// there: keeping it would cost 2 K registers). wy = sin(2 pi k / H).
+template <int NE, int K, typename Get, typename Add>
+__device__ __forceinline__ void col_poly(const ColPoly &q, const PolyTable &t, float wx, float wy, int r0, Get get,
+                                         Add add) {
+    f32x2 v[K];
+    get(v);
+    float e[K];
+#pragma unroll
+    for (int j = 0; j < K; ++j) {
+        const float ar = fmaf(wx, q.cs[r0 + j], wy * q.sn[r0 + j]);
+        e[j] = ar * ar * t.inv_beta;
+    }
+    poly_increment<K, NE / K>(v, e, poly_lane(q.c, t, wx, wy));
+    add(v);
+}
+
 template <int N, int H>
 struct ColCfg {
     static constexpr int L = H / 2;                      // half a column
@@ -141,6 +176,36 @@ struct ColCfg {
     static constexpr int NP = N * L / 2 / T;
     static_assert(NP * 2 * T == N * L, "whole half blocks");
 };
+
+// The polynomial on one half of a column in angle planes: frequency
+// k = parity + 2 i at index i of every plane, two lanes a frequency.
+template <int N, int H, int NE>
+__device__ __forceinline__ void col_poly_planes(float2 *X, const ColPoly &q, const PolyTable &t, float wx,
+                                                const float2 *tws, int parity, int tid) {
+    constexpr int L = H / 2, P = 2, K = NE / P, T = col_threads<H>();
+    static_assert((L * P) % 32 == 0, "whole warps");
+#pragma unroll 1
+    for (int u = tid; u < L * P; u += T) {
+        const int i = u / P, r0 = (u % P) * K;
+        const float wy = -tws[parity + 2 * i].y;
+        col_poly<NE, K>(
+            q, t, wx, wy, r0,
+            [&](f32x2(&v)[K]) {
+#pragma unroll
+                for (int j = 0; j < K; ++j) {
+                    const float2 x = X[xsm<L>(slot_of_angle<N, NE>(r0 + j) * L + i)];
+                    v[j] = pk2(x.x, x.y);
+                }
+            },
+            [&](const f32x2(&v)[K]) {
+#pragma unroll
+                for (int j = 0; j < K; ++j) {
+                    float2 &x = X[xsm<L>(slot_of_angle<N, NE>(r0 + j) * L + i)];
+                    x = make_float2(x.x + lo2(v[j]), x.y + hi2(v[j]));
+                }
+            });
+    }
+}
 
 // a float4 of two angles n, n + 1 of frequency (half row) k, from / into the
 // half-column transforms [n][k]
@@ -153,9 +218,10 @@ __device__ __forceinline__ void put2(float2 *X, int k, int n, float2 a, float2 b
 
 // Block b takes column b / 2 (b even) or W/2 - b / 2 (b odd), so the two
 // columns of a class run side by side and share its propagators in L2.
-template <int N, int H>
+template <int N, int H, int POLY>
 __global__ void __launch_bounds__(col_threads<H>(), H >= 768 ? 1 : 2) k_col_prop(const __grid_constant__ ColArgs a) {
     using C = ColCfg<N, H>;
+    __shared__ ColPoly cp;
     constexpr int L = C::L, T = C::T, HALF4 = N * L / 2;  // float4s in half a block
     extern __shared__ __align__(16) float2 csm[];
     float2 *X = csm;
@@ -168,6 +234,13 @@ __global__ void __launch_bounds__(col_threads<H>(), H >= 768 ? 1 : 2) k_col_prop
     float4 *g = reinterpret_cast<float4 *>(a.col + (long long)l * (N * H));
     for (int m = tid; m < H; m += T) tws[m] = a.tw[m];
     fft_twiddles<T, L, 2>(twp, a.tw, tid);  // from the table in device memory
+    if constexpr (POLY > 0) col_poly_stage(cp, a, tid, T);
+    auto apply = [&](int parity) {
+        if constexpr (POLY == 0)
+            col_apply<N, H>(X, a.D, scol, a.col_slots, parity, tid);
+        else
+            col_poly_planes<N, H, POLY>(X, cp, a.t, sin_2pi_frac(l, a.W), tws, parity, tid);
+    };
     __syncthreads();
     // 1. u = x_k + x_{k+L} into shared memory, v = (x_k - x_{k+L}) w^k into
     //    the upper rows of the block (each thread later reads back only what
@@ -186,7 +259,7 @@ __global__ void __launch_bounds__(col_threads<H>(), H >= 768 ? 1 : 2) k_col_prop
     // 2. the even frequencies, into y_e in the lower rows of the block
     fft_smem<T, N, L, -1>(X, twp, tid);
     __syncthreads();
-    col_apply<N, H>(X, a.D, scol, a.col_slots, 0, tid);
+    apply(0);
     __syncthreads();
     fft_smem<T, N, L, 1>(X, twp, tid);
     __syncthreads();
@@ -208,7 +281,7 @@ __global__ void __launch_bounds__(col_threads<H>(), H >= 768 ? 1 : 2) k_col_prop
     __syncthreads();
     fft_smem<T, N, L, -1>(X, twp, tid);
     __syncthreads();
-    col_apply<N, H>(X, a.D, scol, a.col_slots, 1, tid);
+    apply(1);
     __syncthreads();
     fft_smem<T, N, L, 1>(X, twp, tid);
     __syncthreads();
@@ -400,6 +473,61 @@ __device__ __forceinline__ void col_apply_rows(float2 *XA, float2 *XB, const flo
     }
 }
 
+// The polynomial on a whole column in rows (angles in the order of rd_swz): row
+// p of a half holds frequency 2 rd_index(p) + half. Lane q of a row takes angles
+// q NE / P ..; with NE = 30 they start at slots 0 and 16, slot 17 is skipped.
+// Slots a lane takes. 16: the fewest exchanges, but 128 registers a thread do
+// not quite hold them (about 150 bytes spilled once a column); 8 spill nothing. Measured
+// a column pass: 512 x 512, N = 32 45.5 us with 16 and 48.6 with 8, 768 x 1024,
+// N = 16 75.7 and 71.6.
+template <int NE>
+__host__ __device__ constexpr int col_poly_slots() {
+    return NE == 16 ? 8 : 16;
+}
+template <int T, int N, int H, int NE>
+__device__ __forceinline__ void col_poly_rows(float2 *XA, const ColPoly &q, const PolyTable &t, float wx,
+                                              const float2 *tws, int tid) {
+    constexpr int L = H / 2, KL = col_poly_slots<NE>(), P = N / KL, K = NE / P;
+    static_assert((H * P) % 32 == 0, "whole warps");
+#pragma unroll 1
+    for (int u = tid; u < H * P; u += T) {
+        const int row = u / P, q0 = u % P, half = row / L;
+        const int k = 2 * rd_index<L>(row - half * L) + half;
+        const int s = rd_swz_key<N, KL>(row, q0);
+        float4 *X4 = reinterpret_cast<float4 *>(XA + row * N + q0 * KL);
+        // 16 slots a lane, 2 i and 2 i + 1 in unit i. 15 angles in them: the first
+        // lane's last slot is empty, and the second lane's second one
+        const bool skip = NE < N && q0;
+        col_poly<NE, K>(
+            q, t, wx, -tws[k].y, q0 * K,
+            [&](f32x2(&v)[K]) {
+                f32x2 w[KL];
+#pragma unroll
+                for (int i = 0; i < KL / 2; ++i) {
+                    const float4 x = X4[i ^ s];
+                    w[2 * i] = pk2(x.x, x.y);
+                    w[2 * i + 1] = pk2(x.z, x.w);
+                }
+#pragma unroll
+                for (int j = 0; j < K; ++j) v[j] = NE < N && j > 0 && skip ? w[(j + 1) % KL] : w[j];
+            },
+            [&](const f32x2(&v)[K]) {
+                auto slot = [&](int w) -> f32x2 {  // the increment of slot w
+                    if constexpr (NE == N) return v[w];
+                    if (w == 0) return v[0];
+                    const f32x2 none = pk2(0.0f, 0.0f);
+                    return skip ? (w == 1 ? none : v[w - 1]) : (w == 15 ? none : v[w == 15 ? 0 : w]);
+                };
+#pragma unroll
+                for (int i = 0; i < KL / 2; ++i) {
+                    float4 x = X4[i ^ s];
+                    const f32x2 d0 = slot(2 * i), d1 = slot(2 * i + 1);
+                    X4[i ^ s] = make_float4(x.x + lo2(d0), x.y + hi2(d0), x.z + lo2(d1), x.w + hi2(d1));
+                }
+            });
+    }
+}
+
 template <int N, int H>
 struct ColTmaCfg {
     static constexpr int L = H / 2;
@@ -430,9 +558,11 @@ __device__ __forceinline__ int col_of_unit(int c, int W) { return (c & 1) ? W / 
 // to spare.) Every wait for a copy-in is bounded; one that runs out sets
 // g_col_fault and returns once the copies in flight have landed (again
 // bounded), leaving the unit's column as it was.
-template <int N, int H>
+// POLY: angles of the interval polynomial, 0 for matrices.
+template <int N, int H, int POLY>
 __global__ void __launch_bounds__(ColTmaCfg<N, H>::T, ColTmaCfg<N, H>::MINB)
     k_col_tma(const __grid_constant__ ColArgs a) {
+    __shared__ ColPoly cp;
     using C = ColTmaCfg<N, H>;
     constexpr int L = C::L, T = C::T, HB = C::HB, HF = L * N;  // HF: complex a half
     extern __shared__ __align__(128) float2 ctm[];
@@ -456,6 +586,9 @@ __global__ void __launch_bounds__(ColTmaCfg<N, H>::T, ColTmaCfg<N, H>::MINB)
     };
     if (tid == 0) copy_in(c);
     for (int m = tid; m < H; m += T) tws[m] = a.tw[m];
+    if constexpr (POLY > 0) col_poly_stage(cp, a, tid, T);  // read after the first barrier below
+    constexpr int KL = col_poly_slots<POLY>();
+    constexpr int OUT = POLY > 0 ? RD_SWZ_OUT : RD_PLAIN, IN = POLY > 0 ? RD_SWZ_IN : RD_PLAIN;
     for (uint32_t ph = 0; c < a.Wc; c += gridDim.x, ph ^= 1u) {
         const int l = col_of_unit(c, a.W);
         const bool ok = bulk::bar_wait(bar, ph) && bulk::bar_wait(bar + 8, ph);
@@ -468,11 +601,14 @@ __global__ void __launch_bounds__(ColTmaCfg<N, H>::T, ColTmaCfg<N, H>::MINB)
             }
             return;
         }
-        rd_dif<T, N, L, -1, RD_SPLIT, RD_TWO>(XA, XB, tws, tid);
+        rd_dif<T, N, L, -1, RD_SPLIT, RD_TWO, OUT, KL>(XA, XB, tws, tid);
         __syncthreads();
-        col_apply_rows<T, N, H>(XA, XB, a.D, half_col_slot(l, a.W), a.col_slots, tid);
+        if constexpr (POLY > 0)
+            col_poly_rows<T, N, H, POLY>(XA, cp, a.t, sin_2pi_frac(l, a.W), tws, tid);
+        else
+            col_apply_rows<T, N, H>(XA, XB, a.D, half_col_slot(l, a.W), a.col_slots, tid);
         __syncthreads();
-        rd_dit<T, N, L, 1, RD_TWO, RD_MERGE>(XA, XB, tws, tid);
+        rd_dit<T, N, L, 1, RD_TWO, RD_MERGE, IN, KL>(XA, XB, tws, tid);
         bulk::fence_to_async();
         __syncthreads();
         if (tid == 0) {
@@ -490,11 +626,11 @@ __global__ void __launch_bounds__(ColTmaCfg<N, H>::T, ColTmaCfg<N, H>::MINB)
 }
 
 // persistent grid: the columns, at most the blocks resident at once
-template <int N, int H>
+template <int N, int H, int POLY>
 int col_grid(const ColArgs &a) {
     static int per_sm = 0;  // per instantiation, the same on every GB300
-    if (per_sm <= 0 && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_col_tma<N, H>, ColTmaCfg<N, H>::T,
-                                                                      ColTmaCfg<N, H>::SMEM) != cudaSuccess)
+    if (per_sm <= 0 && cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                           &per_sm, k_col_tma<N, H, POLY>, ColTmaCfg<N, H>::T, ColTmaCfg<N, H>::SMEM) != cudaSuccess)
         per_sm = 0;
     const long long cap = (long long)(a.num_sms > 0 ? a.num_sms : 1) * (per_sm > 0 ? per_sm : 1);
     return (int)(a.Wc < cap ? a.Wc : cap);
@@ -502,39 +638,51 @@ int col_grid(const ColArgs &a) {
 
 // the whole-column kernel where the column fits in shared memory, else the
 // kernel of half columns
-template <int N, int H>
+template <int N, int H, int POLY>
 cudaError_t col_attr() {
     if constexpr (col_tma_fits<N, H>())
-        return cudaFuncSetAttribute(k_col_tma<N, H>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        return cudaFuncSetAttribute(k_col_tma<N, H, POLY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     ColTmaCfg<N, H>::SMEM);
     else
-        return cudaFuncSetAttribute(k_col_prop<N, H>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        return cudaFuncSetAttribute(k_col_prop<N, H, POLY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     ColCfg<N, H>::SMEM);
 }
 
-template <int N, int H>
+template <int N, int H, int POLY>
 cudaError_t col_launch(const ColArgs &a, cudaStream_t s) {
-    cudaError_t e = col_attr<N, H>();
+    cudaError_t e = col_attr<N, H, POLY>();
     if (e != cudaSuccess) return e;
     if constexpr (col_tma_fits<N, H>())
-        k_col_tma<N, H><<<col_grid<N, H>(a), ColTmaCfg<N, H>::T, ColTmaCfg<N, H>::SMEM, s>>>(a);
+        k_col_tma<N, H, POLY><<<col_grid<N, H, POLY>(a), ColTmaCfg<N, H>::T, ColTmaCfg<N, H>::SMEM, s>>>(a);
     else
-        k_col_prop<N, H><<<a.Wc, ColCfg<N, H>::T, ColCfg<N, H>::SMEM, s>>>(a);
+        k_col_prop<N, H, POLY><<<a.Wc, ColCfg<N, H>::T, ColCfg<N, H>::SMEM, s>>>(a);
     return cudaGetLastError();
 }
 
-template <int N>
+template <int N, int POLY>
 cudaError_t col_dispatch(int H, const ColArgs *a, cudaStream_t s) {
     switch (H) {
-        case 64: return a ? col_launch<N, 64>(*a, s) : col_attr<N, 64>();
-        case 128: return a ? col_launch<N, 128>(*a, s) : col_attr<N, 128>();
-        case 256: return a ? col_launch<N, 256>(*a, s) : col_attr<N, 256>();
-        case 512: return a ? col_launch<N, 512>(*a, s) : col_attr<N, 512>();
-        case 1024: return a ? col_launch<N, 1024>(*a, s) : col_attr<N, 1024>();
-        case 384: return a ? col_launch<N, 384>(*a, s) : col_attr<N, 384>();
-        case 768: return a ? col_launch<N, 768>(*a, s) : col_attr<N, 768>();
+        case 64: return a ? col_launch<N, 64, POLY>(*a, s) : col_attr<N, 64, POLY>();
+        case 128: return a ? col_launch<N, 128, POLY>(*a, s) : col_attr<N, 128, POLY>();
+        case 256: return a ? col_launch<N, 256, POLY>(*a, s) : col_attr<N, 256, POLY>();
+        case 512: return a ? col_launch<N, 512, POLY>(*a, s) : col_attr<N, 512, POLY>();
+        case 1024: return a ? col_launch<N, 1024, POLY>(*a, s) : col_attr<N, 1024, POLY>();
+        case 384: return a ? col_launch<N, 384, POLY>(*a, s) : col_attr<N, 384, POLY>();
+        case 768: return a ? col_launch<N, 768, POLY>(*a, s) : col_attr<N, 768, POLY>();
         default: return cudaErrorInvalidValue;
     }
+}
+
+// a = nullptr: set the kernels' attributes, of both forms
+cudaError_t col_any(int N, int H, const ColArgs *a, cudaStream_t s) {
+    cudaError_t e = cudaSuccess;
+    if (!a || a->use_poly)
+        e = N == 16   ? col_dispatch<16, 16>(H, a, s)
+            : N == 30 ? col_dispatch<32, 30>(H, a, s)
+                      : col_dispatch<32, 32>(H, a, s);
+    if (e == cudaSuccess && (!a || !a->use_poly))
+        e = N == 16 ? col_dispatch<16, 0>(H, a, s) : col_dispatch<32, 0>(H, a, s);
+    return e;
 }
 
 }  // namespace
@@ -547,14 +695,16 @@ bool se2n_col_supported(int N, int H) {
            (H == 64 || H == 128 || H == 256 || H == 512 || H == 1024 || H == 384 || H == 768);
 }
 
+bool se2n_col_has_poly(const PolyTable &t) { return !t.reinsch && t.len <= se2n::kColPolyLen; }
+
 cudaError_t se2n_col_prepare(int N, int H) {
     if (!se2n_col_supported(N, H)) return cudaErrorInvalidValue;
-    return N == 16 ? se2n::col_dispatch<16>(H, nullptr, nullptr) : se2n::col_dispatch<32>(H, nullptr, nullptr);
+    return se2n::col_any(N, H, nullptr, nullptr);
 }
 
 cudaError_t se2n_launch_col_prop(int N, const ColArgs &a, cudaStream_t s) {
     if (!se2n_col_supported(N, a.H)) return cudaErrorInvalidValue;
-    return N == 16 ? se2n::col_dispatch<16>(a.H, &a, s) : se2n::col_dispatch<32>(a.H, &a, s);
+    return se2n::col_any(N, a.H, &a, s);
 }
 
 cudaError_t se2n_col_fault(int *host_flag, bool reset) {

@@ -49,7 +49,10 @@ int cheb(double w, double T, double dt, int S, bool inc, int n, double *c) {
 }
 
 int cheb_auto(double w, double T, double dt, int S, bool inc, double *c) {
-    for (int n = 32; n <= kNodesMax; n *= 2) {
+    // the degree grows as the square root of T w: start near enough nodes
+    int n = 32;
+    while (n < kNodesMax && n * n < 160.0 * T * w) n *= 2;
+    for (; n <= kNodesMax; n *= 2) {
         const int m = cheb(w, T, dt, S, inc, n, c);
         if (m > 0) return m;
     }
@@ -71,7 +74,7 @@ bool se2n_poly_make(double beta, double T, int steps, PolyTable &t) {
     // 24 ulp (1.4e-6 of the fastest modes, far less of the slow ones) allowed.
     // Its coefficients in M must also stay clear of the ends of FP32's range.
     bool horner = true;
-    for (int b = 0; b < kPolyBuckets && horner; ++b) {
+    for (int b = kPolyBuckets - 1; b >= 0 && horner; --b) {  // the widest first: it decides
         const double w = width(b), h = 0.5 * w / beta;
         const int m = cheb_auto(w, T, dt, steps, true, c);
         if (m < 0 || m > 32) {
@@ -126,15 +129,17 @@ namespace se2n {
 // loaded before the first use; the volume is read and written once. Measured
 // (events, full spectrum, 1024 x 1024, one GB300) against the step kernel it
 // replaces there:
-//   N = 32, T = 2 in 100 steps     136 us (3.9 TB/s), steps 1391 us
-//   N = 64, T = 50 in 1000 steps   985 us, steps 29.1 ms
+//   N = 32, T = 2 in 100 steps     122 us (4.4 TB/s), steps 1391 us
+//   N = 64, T = 50 in 1000 steps   949 us, steps 29.1 ms
 // At T = 2 the loads and the arithmetic of a warp (77 us of packed FP32 at its
-// measured rate, 79 us of copies) follow one another at 12 warps an SM; large T
-// is bound by the packed FP32 pipe.
+// measured rate, 79 us of copies) follow one another, so the increment form is
+// held to 128 registers, 16 warps an SM (N = 16, 32, 64: 65, 122, 261 us; 71, 140,
+// 302 with 12 warps). Large T is bound by the packed FP32 pipe and Reinsch's form
+// runs fastest unconstrained (949 us; 1003 with 16 warps).
 constexpr int kPolyBlock = 128;
 
 template <int N, bool REINSCH>
-__global__ void __launch_bounds__(kPolyBlock) k_poly(const __grid_constant__ PolyArgs a) {
+__global__ void __launch_bounds__(kPolyBlock, REINSCH ? 3 : 4) k_poly(const __grid_constant__ PolyArgs a) {
     __shared__ float sc[kPolyBuckets * kPolyMax];
     constexpr int P = poly_lanes<N>();
     poly_stage(sc, a.t, threadIdx.x, kPolyBlock);

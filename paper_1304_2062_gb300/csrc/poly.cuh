@@ -110,33 +110,45 @@ __device__ __forceinline__ void poly_steps(f32x2 (&b)[K], const float *c, int st
     }
 }
 
-// One frequency group: x <- f(A) x for the K angles of each of the P lanes
-// (e[j] = a_r^2 / beta of the lane's angles). Every lane of the warp calls it
-// together.
+// The increment form of one frequency group: v <- g(A) A v for the K angles of
+// each of the P lanes (e[j] = a_r^2 / beta of the lane's angles). Every lane of
+// the warp calls it together, as the functions below.
+template <int K, int P>
+__device__ __forceinline__ void poly_increment(f32x2 (&v)[K], const float (&e)[K], const PolyLane &p) {
+    const int top = (int)__reduce_max_sync(0xffffffffu, (unsigned)p.m) - 1;  // highest coefficient in the warp
+    f32x2 lo, hi, b[K], nd[K];
+    poly_edges<P>(v[0], v[K - 1], lo, hi);
+    const f32x2 ct = dup2(p.c[top]), m2 = dup2(-2.0f);
+    f32x2 prev = lo;
+#pragma unroll
+    for (int j = 0; j < K; ++j) {
+        const f32x2 cur = v[j], next = j == K - 1 ? hi : v[j + 1];
+        v[j] = fma2(dup2(-e[j]), cur, fma2(m2, cur, add2(prev, next)));
+        nd[j] = dup2((p.h - 2.0f) - e[j]);
+        b[j] = mul2(ct, v[j]);
+        prev = cur;
+    }
+    poly_steps<K, P>(b, p.c, top, [&](f32x2 l, f32x2 o, f32x2 r, int j, f32x2 ck) {
+        return fma2(ck, v[j], fma2(nd[j], o, add2(l, r)));
+    });
+#pragma unroll
+    for (int j = 0; j < K; ++j) v[j] = b[j];
+}
+
+// x <- f(A) x in either form.
 template <int K, int P, bool REINSCH>
 __device__ __forceinline__ void poly_apply(f32x2 (&x)[K], const float (&e)[K], const PolyLane &p) {
-    const int top = (int)__reduce_max_sync(0xffffffffu, (unsigned)p.m) - 1;  // highest coefficient in the warp
-    f32x2 lo, hi, b[K];
-    const f32x2 ct = dup2(p.c[top]);
     if constexpr (!REINSCH) {
-        f32x2 y[K], nd[K];
-        const f32x2 m2 = dup2(-2.0f);
-        poly_edges<P>(x[0], x[K - 1], lo, hi);
+        f32x2 v[K];
 #pragma unroll
-        for (int j = 0; j < K; ++j) {
-            const f32x2 L = j == 0 ? lo : x[j - 1], R = j == K - 1 ? hi : x[j + 1];
-            y[j] = fma2(dup2(-e[j]), x[j], fma2(m2, x[j], add2(L, R)));
-            nd[j] = dup2((p.h - 2.0f) - e[j]);
-            b[j] = mul2(ct, y[j]);
-        }
-        poly_steps<K, P>(b, p.c, top, [&](f32x2 l, f32x2 o, f32x2 r, int j, f32x2 ck) {
-            return fma2(ck, y[j], fma2(nd[j], o, add2(l, r)));
-        });
+        for (int j = 0; j < K; ++j) v[j] = x[j];
+        poly_increment<K, P>(v, e, p);
 #pragma unroll
-        for (int j = 0; j < K; ++j) x[j] = add2(x[j], b[j]);
+        for (int j = 0; j < K; ++j) x[j] = add2(x[j], v[j]);
     } else {
-        f32x2 ne[K], d[K];
-        const f32x2 ih = dup2(1.0f / p.h), kap = dup2(2.0f / p.h);
+        const int top = (int)__reduce_max_sync(0xffffffffu, (unsigned)p.m) - 1;
+        f32x2 lo, hi, b[K], ne[K], d[K];
+        const f32x2 ct = dup2(p.c[top]), ih = dup2(1.0f / p.h), kap = dup2(2.0f / p.h);
 #pragma unroll
         for (int j = 0; j < K; ++j) {
             ne[j] = dup2(-2.0f - e[j]);

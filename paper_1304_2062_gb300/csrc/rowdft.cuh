@@ -51,6 +51,24 @@ __device__ __forceinline__ int rd_index(int p) {
 // inverse pass).
 enum { RD_ONE = 0, RD_TWO = 1, RD_SPLIT = 2, RD_MERGE = 3 };
 
+// The order of a row's angles while the polynomial is applied to it
+// (colprop.cu): a lane then holds KL = 8 or 16 consecutive angles, KL / 2 units
+// of 16 bytes, so in plain order the lanes of a quarter-warp, which read the same unit
+// of theirs at a time, would meet in one or two of the eight bank groups. Unit i
+// of lane p of row r sits at unit i ^ s of the lane's, s chosen so that the
+// eight lanes read eight different groups.
+template <int N, int KL>
+__host__ __device__ __forceinline__ constexpr int rd_swz_key(int r, int p) {
+    return KL == 16 ? (N == 32 ? (2 * r + p) & 7 : r & 7) : (N == 32 ? (2 * r + (p >> 1)) & 3 : r & 3);
+}
+template <int N, int KL>
+__host__ __device__ __forceinline__ constexpr int rd_swz(int r, int n) {
+    return n ^ (rd_swz_key<N, KL>(r, n / KL) << 1);
+}
+// RD_PLAIN: rows in angle order; RD_SWZ_OUT, RD_SWZ_IN: the pass writes, reads
+// them in the order of rd_swz.
+enum { RD_PLAIN = 0, RD_SWZ_OUT = 1, RD_SWZ_IN = 2 };
+
 // One in-place radix-R pass over blocks of LS rows (S = LS / R): butterfly
 // (block c, j < S) of angle n on rows c LS + j + m S, m < R. Decimation in
 // frequency (DIF): the R-point DFT with exp(DIR 2 pi i / R), output r times
@@ -58,13 +76,18 @@ enum { RD_ONE = 0, RD_TWO = 1, RD_SPLIT = 2, RD_MERGE = 3 };
 // input r times w^{j r}, then the R-point DFT. tws[e] = exp(-2 pi i e / 2L),
 // so w^{j r} is tws[j r 2L / LS] or its conjugate. Each butterfly reads and
 // writes the same rows: no barrier inside a pass.
-template <int T, int N, int L, int R, int LS, int DIR, bool DIF, int MODE>
+// The lanes of a row (or of two rows, N = 16) are in one warp, so a pass
+// that changes the order within rows only has to keep a warp's reads ahead
+// of its writes.
+template <int T, int N, int L, int R, int LS, int DIR, bool DIF, int MODE, int ORDER = RD_PLAIN, int KL = 16>
 __device__ __forceinline__ void rd_pass(float2 *XA, float2 *XB, const float2 *tws, int tid) {
     constexpr int S = LS / R, BLK = L / LS, TW = 2 * L / LS;
     constexpr int BF = BLK * S;  // butterflies of one block and angle
     constexpr bool PAIR = MODE == RD_SPLIT || MODE == RD_MERGE;
     constexpr int TASKS = (MODE == RD_TWO ? 2 : 1) * BF * N;
     static_assert(T % N == 0, "one angle a thread");
+    static_assert(ORDER == RD_PLAIN || (S == 1 && LS % 8 == 0 && !PAIR && (N == 16 || N == 32) && TASKS % 32 == 0),
+                  "the order changes in the pass of single rows");
     static_assert(MODE != RD_SPLIT || (DIF && DIR < 0), "the split is the first forward pass");
     static_assert(MODE != RD_MERGE || (!DIF && DIR > 0), "the recombination is the last inverse pass");
     const int n = tid % N;
@@ -87,10 +110,11 @@ __device__ __forceinline__ void rd_pass(float2 *XA, float2 *XB, const float2 *tw
         } else {
 #pragma unroll
             for (int m = 0; m < R; ++m) {
-                p[m] = Xa[m * S * N];
+                p[m] = ORDER == RD_SWZ_IN ? Xa[m * N + rd_swz<N, KL>(m, n) - n] : Xa[m * S * N];
                 if constexpr (MODE == RD_MERGE) q[m] = Xb[m * S * N];
             }
         }
+        if constexpr (ORDER != RD_PLAIN) __syncwarp();
         if constexpr (!DIF) {
 #pragma unroll
             for (int r = 1; r < R; ++r) {
@@ -119,7 +143,10 @@ __device__ __forceinline__ void rd_pass(float2 *XA, float2 *XB, const float2 *tw
         } else {
 #pragma unroll
             for (int m = 0; m < R; ++m) {
-                Xa[m * S * N] = p[m];
+                if constexpr (ORDER == RD_SWZ_OUT)
+                    Xa[m * N + rd_swz<N, KL>(m, n) - n] = p[m];
+                else
+                    Xa[m * S * N] = p[m];
                 if constexpr (MODE == RD_SPLIT) Xb[m * S * N] = q[m];
             }
         }
@@ -127,29 +154,30 @@ __device__ __forceinline__ void rd_pass(float2 *XA, float2 *XB, const float2 *tw
 }
 
 // decimation in frequency, natural order in, digit-reversed out (FIRST: the
-// first pass's mode, REST: the others'); the caller synchronises before and after
-template <int T, int N, int L, int DIR, int FIRST, int REST>
+// first pass's mode, REST: the others'; ORDER: the last pass's order of the
+// angles); the caller synchronises before and after
+template <int T, int N, int L, int DIR, int FIRST, int REST, int ORDER = RD_PLAIN, int KL = 16>
 __device__ __forceinline__ void rd_dif(float2 *XA, float2 *XB, const float2 *tws, int tid) {
     using P = RdPlan<L>;
     rd_pass<T, N, L, P::R1, L, DIR, true, FIRST>(XA, XB, tws, tid);
     __syncthreads();
-    rd_pass<T, N, L, P::R2, L / P::R1, DIR, true, REST>(XA, XB, tws, tid);
+    rd_pass<T, N, L, P::R2, L / P::R1, DIR, true, REST, P::R3 == 1 ? ORDER : RD_PLAIN, KL>(XA, XB, tws, tid);
     if constexpr (P::R3 > 1) {
         __syncthreads();
-        rd_pass<T, N, L, P::R3, P::R3, DIR, true, REST>(XA, XB, tws, tid);
+        rd_pass<T, N, L, P::R3, P::R3, DIR, true, REST, ORDER, KL>(XA, XB, tws, tid);
     }
 }
 
 // decimation in time, digit-reversed in, natural order out (LAST: the last
-// pass's mode, REST: the others')
-template <int T, int N, int L, int DIR, int REST, int LAST>
+// pass's mode, REST: the others'; ORDER: the first pass's order of the angles)
+template <int T, int N, int L, int DIR, int REST, int LAST, int ORDER = RD_PLAIN, int KL = 16>
 __device__ __forceinline__ void rd_dit(float2 *XA, float2 *XB, const float2 *tws, int tid) {
     using P = RdPlan<L>;
     if constexpr (P::R3 > 1) {
-        rd_pass<T, N, L, P::R3, P::R3, DIR, false, REST>(XA, XB, tws, tid);
+        rd_pass<T, N, L, P::R3, P::R3, DIR, false, REST, ORDER, KL>(XA, XB, tws, tid);
         __syncthreads();
     }
-    rd_pass<T, N, L, P::R2, L / P::R1, DIR, false, REST>(XA, XB, tws, tid);
+    rd_pass<T, N, L, P::R2, L / P::R1, DIR, false, REST, P::R3 == 1 ? ORDER : RD_PLAIN, KL>(XA, XB, tws, tid);
     __syncthreads();
     rd_pass<T, N, L, P::R1, L, DIR, false, LAST>(XA, XB, tws, tid);
 }

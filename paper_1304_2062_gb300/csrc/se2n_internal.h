@@ -70,9 +70,7 @@ struct se2n_plan {
     cudaStream_t side;
     cudaEvent_t ev_fork, ev_join;
     bool join_pending;
-    // row and column passes of the Hermitian half (se2n_inpaint with
-    // propagators): the row-transformed volume [Wc][H][N] complex
-    float2 *colbuf;
+    // row and column passes of the Hermitian half (se2n_inpaint): the twiddles
     float2 *col_tw;        // exp(-2 pi i m / H), m < H
     float2 *row_tw;        // exp(-2 pi i m / W), m < W
     bool col_ready;
@@ -191,9 +189,15 @@ struct ColArgs {
     const float2 *tw;   // exp(-2 pi i m / H), m < H
     int H, W, Wc, col_slots;
     int num_sms;        // the device's SMs (the persistent grid's size)
+    // use_poly: the interval polynomial (increment form) in place of D
+    int use_poly;
+    PolyTable t;
+    float cs[32], sn[32];  // cos, sin of the angles (poly)
 };
 bool se2n_col_supported(int N, int H);
 cudaError_t se2n_col_prepare(int N, int H);
+// Whether the column pass has a kernel for the polynomial t.
+bool se2n_col_has_poly(const PolyTable &t);
 cudaError_t se2n_launch_col_prop(int N, const ColArgs &a, cudaStream_t s);
 // 1 in *host_flag when a column pass gave up waiting for its copy-in (reset clears it)
 cudaError_t se2n_col_fault(int *host_flag, bool reset);
