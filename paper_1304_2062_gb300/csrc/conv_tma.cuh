@@ -506,44 +506,55 @@ __global__ void __launch_bounds__(192, 1)
 
 // ---------------------------------------------------------------------------
 // Weight gradient: dW[co][tap * C + ci] += sum over pixels p of
-// In[p shifted by tap][ci] * gz[p][co], as D[m][n] with m = tap * C + ci
-// (rows, M = 128 per tile), n = co (N = Cout), K = pixels. Both operands come
-// from NHWC tensors, so they are MN-major in shared memory: a TMA box of MG
-// channels x BKX pixels of one image row lands as BKX rows (one per pixel,
-// the K index) of MG contiguous channels, the MN-major swizzled layout
-// (MG = 64: 128-byte rows and swizzle; MG = 32: 64-byte). The tap shift
-// moves the pixel coordinates, never the innermost (channel) one; rows of
-// the M tile past 9 C are zero-filled by a box that starts out of range.
-// A unit of work is (M tile, a range of pixel blocks); its partial D is
-// added to dW with FP32 atomics by the epilogue, which overlaps the next
-// unit's MMAs (two accumulators).
+// In[p shifted by tap][ci] * gz[p][co], as D[m][n] = sum over k of A(m, k) B(n, k)
+// with k the pixels. Both operands come from NHWC tensors, so they are MN-major
+// in shared memory: a TMA box of 64 channels x BKX pixels x some image rows lands
+// as one 128-byte swizzled row a pixel.
+//
+// What bounds a weight gradient with few channels is the rate at which the TMA
+// unit writes box rows (about 8 cycles a row, whether of 64 or of 128 bytes), so
+// the kernel loads few and full ones:
+//  * A box of In holds the R + 3 image rows y0 - 1 .. y0 + R + 1 for one
+//    horizontal offset dx. The vertical offsets read it one image row further
+//    on, a whole number of swizzle atoms, and two neighbouring offsets are the
+//    two 64-row groups of one M = 128 operand (leading byte offset = one image
+//    row): accumulators (dy -1, 0) and (dy 1, none). 3 (R + 3) / R + 1 box rows a pixel
+//    feed all nine taps of 64 input and 64 output channels (5.1 with R = 8; one
+//    box a tap and operand, as before, takes 15).
+//  * Layers whose channels are not whole groups of 64 (C = 32, 96) are read as
+//    pairs of pixels, tensors of 2 C channels and W / 2 columns: D of a pair
+//    offset s then holds, for each parity px of In's pixel and pg of gz's, the
+//    tap dx = 2 s + px - pg; s = -1, 0, 1 give every combination that is a tap,
+//    the others are left out by the epilogue (or not loaded, where a group of 64
+//    holds one parity only). Half the box rows again.
+// A unit of work is (64 channels of In, 64 of gz, a range of pixel blocks); every
+// CTA takes one, accumulates it in tensor memory (up to 3 offsets x 2 tiles x 64
+// columns) and adds it to dW with FP32 atomics at the end.
+// Measured (batch 32, 256 x 256): 32 -> 32 channels 145 us (1008 with a box a
+// tap), 96 -> 32 420, all 13 layers 1713 us (4832).
 // ---------------------------------------------------------------------------
 
+constexpr int kWgR = 8;                    // image rows of a pixel block
+constexpr int kWgXSlots = 3, kWgGSlots = 2;  // ring slots of In and of gz
+
 struct WgradGeo {
-    int B, H, W, C, Cout;
-    int bkx;            // pixels per K block (one image row segment), 16 / 32 / 64
-    int xblocks;        // W / bkx
-    int kblocks;        // B * H * xblocks
-    int mtiles;         // ceil(9 C / 128)
-    int ksplit;         // pixel ranges per M tile
-    int units;          // mtiles * ksplit
+    int B, H, W;        // of the tensors as read (W / 2 columns for pairs)
+    int C, Cout;        // channels of the layer
+    int pair;           // 1: read as pairs of pixels
+    int bkx;            // columns of a pixel block, 16 or 32
+    int xblocks, yblocks, kblocks;
+    int cgroups, ngroups;  // 64-channel groups of In and gz as read
+    int ksplit;         // pixel ranges a (channel group, channel group)
 };
 
-template <int MG, int NG>
-struct WgCfg {
-    static_assert((MG == 32 || MG == 64) && (NG == 32 || NG == 64), "32- or 64-channel groups");
-    static constexpr uint64_t LAYOUT_A = MG == 64 ? 2 : 4, LAYOUT_B = NG == 64 ? 2 : 4;
-    static constexpr uint32_t SBO_A = 8 * MG * 2, SBO_B = 8 * NG * 2;
-};
-
-// MN-major matrix descriptor: leading byte offset = stride between MN groups,
-// stride byte offset = stride between 8-row groups along K.
-__device__ __forceinline__ uint64_t sdesc_mn(uint32_t saddr, uint32_t lbo, uint32_t sbo, uint64_t layout) {
+// MN-major matrix descriptor, 128-byte swizzle: leading byte offset = stride
+// between 64-row groups, stride byte offset = stride between 8-pixel groups.
+__device__ __forceinline__ uint64_t sdesc_mn(uint32_t saddr, uint32_t lbo) {
     uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
     d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
-    d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
+    d |= (uint64_t)(1024u >> 4) << 32;
     d |= (uint64_t)1 << 46;
-    d |= layout << 61;
+    d |= (uint64_t)2 << 61;
     return d;
 }
 
@@ -554,43 +565,57 @@ __device__ __forceinline__ constexpr uint32_t idesc_bf16_mn() {
            ((uint32_t)(128 >> 4) << 24);
 }
 
-template <int BN, int MG, int NG>
 __global__ void __launch_bounds__(192, 1)
     k_wgrad_tma(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapG, const WgradGeo g,
-                float *dw, int S, int *err) {
-    using Cf = WgCfg<MG, NG>;
-    constexpr int ACC = BN <= 32 ? 32 : BN <= 64 ? 64 : BN <= 128 ? 128 : 256;
-    constexpr int TMEM_COLS = 2 * ACC;
+                float *dw, int *err) {
+    constexpr int R = kWgR, XS = kWgXSlots, GS = kWgGSlots, TMEM_COLS = 512;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     const int bkx = g.bkx;
-    const uint32_t A_BYTES = 128u * bkx * 2, B_BYTES = (uint32_t)BN * bkx * 2, STAGE = A_BYTES + B_BYTES;
-    const uint32_t bar_full = base + S * STAGE;
-    const uint32_t bar_empty = bar_full + 8 * S;
-    const uint32_t bar_afull = bar_empty + 8 * S;
-    const uint32_t bar_aempty = bar_afull + 16;
-    const uint32_t tmem_slot = bar_aempty + 16;
+    const uint32_t ROW = (uint32_t)bkx * 128u;            // one image row of a box
+    const uint32_t X_BYTES = (R + 3) * ROW, G_BYTES = R * ROW;
+    const uint32_t gbase = base + XS * X_BYTES;
+    const uint32_t bar_xfull = gbase + GS * G_BYTES;
+    const uint32_t bar_xempty = bar_xfull + 8 * XS;
+    const uint32_t bar_gfull = bar_xempty + 8 * XS;
+    const uint32_t bar_gempty = bar_gfull + 8 * GS;
+    const uint32_t bar_done = bar_gempty + 8 * GS;
+    const uint32_t tmem_slot = bar_done + 8;
     volatile int *abort = (volatile int *)(smem_raw + (tmem_slot + 4 - raw));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m_total = 9 * g.C;
+
+    // the unit: channel groups cg (of In) and ng (of gz), pixel blocks [kb0, kb1)
+    const int ks = blockIdx.x % g.ksplit, gr = blockIdx.x / g.ksplit;
+    const int c0 = (gr % g.cgroups) * 64, n0 = (gr / g.cgroups) * 64;
+    const int per = (g.kblocks + g.ksplit - 1) / g.ksplit;
+    const int kb0 = ks * per, kb1 = min(g.kblocks, kb0 + per);
+    // offsets s0 .. s1 (pixels, or pairs: -1 needs In's second pixel and gz's
+    // first, 1 the reverse)
+    int s0 = -1, s1 = 1;
+    if (g.pair) {
+        const bool x1 = (c0 + 63) / g.C > 0, x0 = c0 / g.C == 0, g1 = (n0 + 63) / g.Cout > 0, g0 = n0 / g.Cout == 0;
+        s0 = x1 && g0 ? -1 : 0;
+        s1 = x0 && g1 ? 1 : 0;
+    }
 
     if (threadIdx.x == 0) {
         *abort = *(volatile int *)err;
-        for (int s = 0; s < S; ++s) {
-            tc::mbar_init(bar_full + 8 * s, 1);
-            tc::mbar_init(bar_empty + 8 * s, 1);
+        for (int s = 0; s < XS; ++s) {
+            tc::mbar_init(bar_xfull + 8 * s, 1);
+            tc::mbar_init(bar_xempty + 8 * s, 1);
         }
-        for (int a = 0; a < 2; ++a) {
-            tc::mbar_init(bar_afull + 8 * a, 1);
-            tc::mbar_init(bar_aempty + 8 * a, 4);
+        for (int s = 0; s < GS; ++s) {
+            tc::mbar_init(bar_gfull + 8 * s, 1);
+            tc::mbar_init(bar_gempty + 8 * s, 1);
         }
+        tc::mbar_init(bar_done, 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         asm volatile("prefetch.tensormap [%0];\n" ::"l"((uint64_t)&mapX) : "memory");
         asm volatile("prefetch.tensormap [%0];\n" ::"l"((uint64_t)&mapG) : "memory");
     }
     __syncthreads();
-    if (*abort) return;
+    if (*abort || kb0 >= kb1) return;
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(tmem_slot),
                      "r"((uint32_t)TMEM_COLS));
@@ -602,58 +627,48 @@ __global__ void __launch_bounds__(192, 1)
     uint32_t tmem_base;
     asm volatile("ld.shared.u32 %0, [%1];\n" : "=r"(tmem_base) : "r"(tmem_slot));
 
-    // unit u = mt * ksplit + ks covers pixel blocks [kb0, kb1) of M tile mt
-    auto unit_range = [&](int u, int &mt, int &kb0, int &kb1) {
-        mt = u / g.ksplit;
-        const int ks = u - mt * g.ksplit;
-        const int per = (g.kblocks + g.ksplit - 1) / g.ksplit;
-        kb0 = ks * per;
-        kb1 = min(g.kblocks, kb0 + per);
+    // origin of pixel block kb
+    auto block = [&](int kb, int &b, int &y0, int &x0) {
+        const int xb = kb % g.xblocks, r = kb / g.xblocks;
+        b = r / g.yblocks;
+        y0 = (r - b * g.yblocks) * R;
+        x0 = xb * bkx;
     };
 
     if (warp == 0) {
         if (lane == 0) {
             // ---------------- TMA producer ----------------
-            int s = 0;
-            uint32_t ph = 0;
+            int xs = 0, gs = 0;
+            uint32_t xph = 0, gph = 0;
             bool ok = true;
-            for (int u = blockIdx.x; u < g.units && ok; u += gridDim.x) {
-                int mt, kb0, kb1;
-                unit_range(u, mt, kb0, kb1);
-                for (int kb = kb0; kb < kb1; ++kb) {
-                    const int xb = kb % g.xblocks;
-                    const int r = kb / g.xblocks;
-                    const int y = r % g.H, b = r / g.H;
-                    const int x0 = xb * bkx;
-                    if (!tc::mbar_wait(bar_empty + 8 * s, ph ^ 1u, abort)) {
+            for (int kb = kb0; kb < kb1 && ok; ++kb) {
+                int b, y0, x0;
+                block(kb, b, y0, x0);
+                if (!tc::mbar_wait(bar_gempty + 8 * gs, gph ^ 1u, abort)) {
+                    ok = false;
+                    break;
+                }
+                arrive_expect_tx(bar_gfull + 8 * gs, G_BYTES);
+                tma_load_4d(gbase + gs * G_BYTES, &mapG, n0, x0, y0, b, bar_gfull + 8 * gs);
+                if (++gs == GS) {
+                    gs = 0;
+                    gph ^= 1u;
+                }
+                for (int s = s0; s <= s1; ++s) {
+                    if (!tc::mbar_wait(bar_xempty + 8 * xs, xph ^ 1u, abort)) {
                         ok = false;
                         break;
                     }
-                    const uint32_t sa = base + s * STAGE, sb = sa + A_BYTES;
-                    arrive_expect_tx(bar_full + 8 * s, STAGE);
-#pragma unroll
-                    for (int gi = 0; gi < 128 / MG; ++gi) {
-                        const int m0 = mt * 128 + gi * MG;
-                        int c0 = g.C, dy = 0, dx = 0;  // past the last row: a box entirely out of range (zeros)
-                        if (m0 < m_total) {
-                            const int tap = m0 / g.C;
-                            c0 = m0 - tap * g.C;
-                            dy = tap / 3 - 1;
-                            dx = tap % 3 - 1;
-                        }
-                        tma_load_4d(sa + gi * (uint32_t)(bkx * MG * 2), &mapX, c0, x0 + dx, y + dy, b,
-                                    bar_full + 8 * s);
-                    }
-#pragma unroll
-                    for (int gi = 0; gi < BN / NG; ++gi)
-                        tma_load_4d(sb + gi * (uint32_t)(bkx * NG * 2), &mapG, gi * NG, x0, y, b, bar_full + 8 * s);
-                    if (++s == S) {
-                        s = 0;
-                        ph ^= 1u;
+                    arrive_expect_tx(bar_xfull + 8 * xs, X_BYTES);
+                    tma_load_4d(base + xs * X_BYTES, &mapX, c0, x0 + s, y0 - 1, b, bar_xfull + 8 * xs);
+                    if (++xs == XS) {
+                        xs = 0;
+                        xph ^= 1u;
                     }
                 }
             }
             if (!ok) {
+                // loads already issued finish on their own within microseconds
                 const long long t0 = clock64();
                 while (clock64() - t0 < 200000LL) {
                 }
@@ -662,81 +677,86 @@ __global__ void __launch_bounds__(192, 1)
     } else if (warp == 1) {
         if (lane == 0) {
             // ---------------- MMA issuer ----------------
-            constexpr uint32_t IDESC = idesc_bf16_mn<BN>();
-            const uint32_t lbo_a = (uint32_t)(bkx * MG * 2), lbo_b = (uint32_t)(bkx * NG * 2);
-            int s = 0, acc = 0;
-            uint32_t ph = 0, aph = 0;
+            constexpr uint32_t IDESC = idesc_bf16_mn<64>();
+            int xs = 0, gs = 0;
+            uint32_t xph = 0, gph = 0;
             bool ok = true;
             uint32_t last_bar = 0, last_par = 0;
-            for (int u = blockIdx.x; u < g.units && ok; u += gridDim.x) {
-                int mt, kb0, kb1;
-                unit_range(u, mt, kb0, kb1);
-                if (!tc::mbar_wait(bar_aempty + 8 * acc, aph ^ 1u, abort)) {
+            for (int kb = kb0; kb < kb1 && ok; ++kb) {
+                int b, y0, x0;
+                block(kb, b, y0, x0);
+                const int rows = min(R, g.H - y0);
+                if (!tc::mbar_wait(bar_gfull + 8 * gs, gph, abort)) {
                     ok = false;
                     break;
                 }
-                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                const uint32_t d = tmem_base + (uint32_t)(acc * ACC);
-                bool first = true;
-                for (int kb = kb0; kb < kb1; ++kb) {
-                    if (!tc::mbar_wait(bar_full + 8 * s, ph, abort)) {
+                const uint32_t sg = gbase + gs * G_BYTES;
+                for (int s = s0; s <= s1; ++s) {
+                    if (!tc::mbar_wait(bar_xfull + 8 * xs, xph, abort)) {
                         ok = false;
                         break;
                     }
                     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                    const uint32_t sa = base + s * STAGE, sb = sa + A_BYTES;
-                    for (int kk = 0; kk < bkx / 16; ++kk) {
-                        // 16 pixels = two 8-row groups along K
-                        tc::mma_f16(d, sdesc_mn(sa + kk * 2 * Cf::SBO_A, lbo_a, Cf::SBO_A, Cf::LAYOUT_A),
-                                    sdesc_mn(sb + kk * 2 * Cf::SBO_B, lbo_b, Cf::SBO_B, Cf::LAYOUT_B), IDESC,
-                                    first ? 0u : 1u);
-                        first = false;
-                    }
-                    tc::mma_commit(bar_empty + 8 * s);
-                    last_bar = bar_empty + 8 * s;
-                    last_par = ph;
-                    if (++s == S) {
-                        s = 0;
-                        ph ^= 1u;
+                    const uint32_t sx = base + xs * X_BYTES;
+                    const uint32_t d = tmem_base + (uint32_t)((s - s0) * 128);
+                    for (int j = 0; j < rows; ++j)
+                        for (int kk = 0; kk < bkx / 16; ++kk) {
+                            // 16 pixels = 2048 bytes; image row j of gz against rows j, j + 1 and
+                            // j + 2, j + 3 of the box
+                            const uint32_t off = (uint32_t)j * ROW + (uint32_t)kk * 2048u;
+                            const uint64_t db = sdesc_mn(sg + off, ROW);
+                            const uint32_t add = kb > kb0 || j > 0 || kk > 0 ? 1u : 0u;
+                            tc::mma_f16(d, sdesc_mn(sx + off, ROW), db, IDESC, add);
+                            tc::mma_f16(d + 64u, sdesc_mn(sx + off + 2 * ROW, ROW), db, IDESC, add);
+                        }
+                    tc::mma_commit(bar_xempty + 8 * xs);
+                    last_bar = bar_xempty + 8 * xs;
+                    last_par = xph;
+                    if (++xs == XS) {
+                        xs = 0;
+                        xph ^= 1u;
                     }
                 }
                 if (!ok) break;
-                tc::mma_commit(bar_afull + 8 * acc);
-                if (++acc == 2) {
-                    acc = 0;
-                    aph ^= 1u;
+                tc::mma_commit(bar_gempty + 8 * gs);
+                if (++gs == GS) {
+                    gs = 0;
+                    gph ^= 1u;
                 }
             }
-            if (!ok && last_bar) tc::mbar_wait(last_bar, last_par, nullptr);
+            if (ok)
+                tc::mma_commit(bar_done);
+            else if (last_bar)
+                tc::mbar_wait(last_bar, last_par, nullptr);  // tensor core idle before release
         }
     } else {
         // ---------------- epilogue (warps 2..5): atomic adds into dW ----------------
         const int q = warp & 3;
-        int acc = 0;
-        uint32_t aph = 0;
-        for (int u = blockIdx.x; u < g.units; u += gridDim.x) {
-            int mt, kb0, kb1;
-            unit_range(u, mt, kb0, kb1);
-            if (!tc::mbar_wait(bar_afull + 8 * acc, aph, abort)) break;
+        if (tc::mbar_wait(bar_done, 0, abort)) {
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-            const int m = mt * 128 + q * 32 + lane;
-            const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * ACC);
+            const int i = (q & 1) * 32 + lane;   // channel of In in the group
+            const int e = c0 + i;
+            const int px = g.pair && e >= g.C, ci = px ? e - g.C : e;
+            for (int s = s0; s <= s1; ++s)
+                for (int t = 0; t < 2; ++t) {
+                    const int dy = 2 * t + (q >> 1) - 1;
+                    if (dy > 1) continue;  // the second group of the second tile is no tap (warp-uniform)
+                    const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)((s - s0) * 128 + t * 64);
 #pragma unroll 1
-            for (int j0 = 0; j0 < BN; j0 += 16) {
-                uint32_t v[16];
-                tc::tmem_ld16(taddr + (uint32_t)j0, v);
-                if (m < m_total && kb1 > kb0) {
+                    for (int j0 = 0; j0 < 64; j0 += 16) {
+                        uint32_t v[16];
+                        tc::tmem_ld16(taddr + (uint32_t)j0, v);
+                        const int f = n0 + j0;  // 16 columns of one parity: Cout is a multiple of 32
+                        const int pg = g.pair && f >= g.Cout, co = pg ? f - g.Cout : f;
+                        const int dx = g.pair ? 2 * s + px - pg : s;
+                        if (dx >= -1 && dx <= 1) {
+                            float *p = dw + ((long long)co * 9 + (dy + 1) * 3 + (dx + 1)) * g.C + ci;
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) atomicAdd(dw + (long long)(j0 + i) * m_total + m, __uint_as_float(v[i]));
+                            for (int c = 0; c < 16; ++c) atomicAdd(p + (long long)c * 9 * g.C, __uint_as_float(v[c]));
+                        }
+                    }
                 }
-            }
             asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-            __syncwarp();
-            if (lane == 0) arrive(bar_aempty + 8 * acc);
-            if (++acc == 2) {
-                acc = 0;
-                aph ^= 1u;
-            }
         }
     }
     __syncthreads();
