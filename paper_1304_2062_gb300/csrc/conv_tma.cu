@@ -213,9 +213,9 @@ cudaError_t launch_halo(const __nv_bfloat16 *A, int B, int H, int W, int C, cons
     if (W % tma::HBW || H % tma::HBH || C % CK || N % BN) return cudaErrorNotSupported;
     const int nblk = 9 * (C / CK);
     const int wbytes = nblk * Cf::BBLK;
-    int S = (Cf::SMEM_BUDGET - wbytes) / Cf::A_BYTES;
-    if (S > 8) S = 8;
-    if (S < 3) return cudaErrorNotSupported;
+    int S = (Cf::SMEM_BUDGET - wbytes) / Cf::STAGE;
+    if (S > 4) S = 4;
+    if (S < 2) return cudaErrorNotSupported;
     auto enc = encoder();
     const int nsm = sm_count();
     int *err = fault_ptr();
@@ -256,7 +256,7 @@ cudaError_t launch_halo(const __nv_bfloat16 *A, int B, int H, int W, int C, cons
     g.nchunk = C / CK;
     g.KB = 3 * g.nchunk;
     g.flip = flip;
-    const int smem = 1024 + wbytes + S * Cf::A_BYTES + 256;
+    const int smem = 1024 + wbytes + S * Cf::STAGE + 256;
     auto *fn = &tma::k_conv_halo<BN, CK, EPI>;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
@@ -272,8 +272,8 @@ cudaError_t launch_halo(const __nv_bfloat16 *A, int B, int H, int W, int C, cons
 // [Cout][9 C] FP32 (accumulated).
 cudaError_t launch_wgrad(const __nv_bfloat16 *x, int B, int H, int W, int C, const __nv_bfloat16 *gz, int Cout,
                          float *dw, cudaStream_t s) {
-    const int pair = C % 64 != 0 || Cout % 64 != 0;
-    if (C % 32 || Cout % 32 || (pair && W % 2)) return cudaErrorNotSupported;
+    const int F = C % 64 == 0 && Cout % 64 == 0 ? 1 : C % 32 == 0 ? 2 : 8;
+    if ((F * C) % 64 || Cout % 32 || W % F) return cudaErrorNotSupported;
     auto enc = encoder();
     const int nsm = sm_count();
     int *err = fault_ptr();
@@ -281,15 +281,15 @@ cudaError_t launch_wgrad(const __nv_bfloat16 *x, int B, int H, int W, int C, con
     tma::WgradGeo g;
     g.B = B;
     g.H = H;
-    g.W = pair ? W / 2 : W;
+    g.W = W / F;
     g.C = C;
     g.Cout = Cout;
-    g.pair = pair;
-    g.bkx = g.W > 16 ? 32 : 16;
-    g.xblocks = (g.W + g.bkx - 1) / g.bkx;
+    g.F = F;
+    const int bkx = g.W > 16 ? 32 : 16;  // columns of a pixel block
+    g.xblocks = (g.W + bkx - 1) / bkx;
     g.yblocks = (H + tma::kWgR - 1) / tma::kWgR;
     g.kblocks = B * g.xblocks * g.yblocks;
-    const int cv = C << pair, nv = Cout << pair;
+    const int cv = F * C, nv = F * Cout;
     g.cgroups = cv / 64;
     g.ngroups = nv / 64;
     // one unit a CTA and one CTA an SM: as many pixel ranges as fill the device once
@@ -300,7 +300,7 @@ cudaError_t launch_wgrad(const __nv_bfloat16 *x, int B, int H, int W, int C, con
     auto map = [&](CUtensorMap *m, const __nv_bfloat16 *p, int ch, int rows) {
         const cuuint64_t dims[4] = {(cuuint64_t)ch, (cuuint64_t)g.W, (cuuint64_t)H, (cuuint64_t)B};
         const cuuint64_t strides[3] = {(cuuint64_t)ch * 2, (cuuint64_t)g.W * ch * 2, (cuuint64_t)H * g.W * ch * 2};
-        const cuuint32_t box[4] = {64, (cuuint32_t)g.bkx, (cuuint32_t)rows, 1};
+        const cuuint32_t box[4] = {64, (cuuint32_t)bkx, (cuuint32_t)rows, 1};
         const cuuint32_t es[4] = {1, 1, 1, 1};
         return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void *)p, dims, strides, box, es,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -308,11 +308,12 @@ cudaError_t launch_wgrad(const __nv_bfloat16 *x, int B, int H, int W, int C, con
     };
     CUtensorMap mx, mg;
     if (!map(&mx, x, cv, tma::kWgR + 3) || !map(&mg, gz, nv, tma::kWgR)) return cudaErrorInvalidValue;
-    const int row = g.bkx * 128;
+    const int row = bkx * 128;
     const int smem = 1024 + tma::kWgXSlots * (tma::kWgR + 3) * row + tma::kWgGSlots * tma::kWgR * row + 256;
-    cudaError_t e = cudaFuncSetAttribute(tma::k_wgrad_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    auto *fn = bkx == 32 ? &tma::k_wgrad_tma<32> : &tma::k_wgrad_tma<16>;
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    tma::k_wgrad_tma<<<groups * g.ksplit, 192, smem, s>>>(mx, mg, g, dw, err);
+    fn<<<groups * g.ksplit, 192, smem, s>>>(mx, mg, g, dw, err);
     return cudaGetLastError();
 }
 

@@ -306,6 +306,7 @@ template <int BN, int CK>
 struct HaloCfg {
     static_assert(BN % 16 == 0 && BN >= 16 && BN <= 128, "narrow layers");
     static constexpr int A_BYTES = HROWS * CK * 2;
+    static constexpr int STAGE = 3 * A_BYTES;  // the boxes of the three horizontal offsets
     static constexpr int BBLK = BN * CK * 2;   // one (tap, channel block) of weights
     static constexpr int ACC_COLS = BN <= 32 ? 32 : BN <= 64 ? 64 : 128;
     static constexpr int TMEM_COLS = 2 * ACC_COLS;
@@ -322,8 +323,8 @@ __global__ void __launch_bounds__(192, 1)
     const uint32_t base = (raw + 1023u) & ~1023u;
     const int nblk = 9 * g.nchunk;                       // resident weight blocks
     const uint32_t wres = base;                          // nblk x BBLK
-    const uint32_t stages = wres + nblk * Cf::BBLK;      // S x A_BYTES
-    const uint32_t bar_w = stages + S * Cf::A_BYTES;
+    const uint32_t stages = wres + nblk * Cf::BBLK;      // S x STAGE
+    const uint32_t bar_w = stages + S * Cf::STAGE;
     const uint32_t bar_full = bar_w + 8;
     const uint32_t bar_empty = bar_full + 8 * S;
     const uint32_t bar_afull = bar_empty + 8 * S;
@@ -380,20 +381,21 @@ __global__ void __launch_bounds__(192, 1)
             for (int t = first_tile; t < end_tile && ok; t += tile_step) {
                 int b, x0, y0, nt;
                 tile_origin(g, t, b, x0, y0, nt);
-                for (int ch = 0; ch < g.nchunk && ok; ++ch)
-                    for (int sxi = 0; sxi < 3; ++sxi) {
-                        if (!tc::mbar_wait(bar_empty + 8 * s, ph ^ 1u, abort)) {
-                            ok = false;
-                            break;
-                        }
-                        arrive_expect_tx(bar_full + 8 * s, Cf::A_BYTES);
-                        tma_load_4d(stages + s * Cf::A_BYTES, &mapA, ch * CK, x0 + sxi - 1, y0 - 1, b,
-                                    bar_full + 8 * s);
-                        if (++s == S) {
-                            s = 0;
-                            ph ^= 1u;
-                        }
+                for (int ch = 0; ch < g.nchunk; ++ch) {
+                    if (!tc::mbar_wait(bar_empty + 8 * s, ph ^ 1u, abort)) {
+                        ok = false;
+                        break;
                     }
+                    arrive_expect_tx(bar_full + 8 * s, Cf::STAGE);
+#pragma unroll
+                    for (int sxi = 0; sxi < 3; ++sxi)
+                        tma_load_4d(stages + s * Cf::STAGE + sxi * Cf::A_BYTES, &mapA, ch * CK, x0 + sxi - 1, y0 - 1, b,
+                                    bar_full + 8 * s);
+                    if (++s == S) {
+                        s = 0;
+                        ph ^= 1u;
+                    }
+                }
             }
             if (!ok) {
                 const long long t0 = clock64();
@@ -406,6 +408,7 @@ __global__ void __launch_bounds__(192, 1)
             // ---------------- MMA issuer ----------------
             constexpr uint32_t IDESC = tc::idesc_bf16_f32<BN>();
             const uint64_t a_desc0 = sdesc<BN, CK>(stages), w_desc0 = sdesc<BN, CK>(wres);
+            const int wstep = (g.nchunk * Cf::BBLK) >> 4;  // weights of the next tap, in 16-byte units
             int s = 0, acc = 0;
             uint32_t ph = 0, aph = 0;
             bool ok = tc::mbar_wait(bar_w, 0, abort);
@@ -417,37 +420,36 @@ __global__ void __launch_bounds__(192, 1)
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 const uint32_t d = tmem_base + (uint32_t)(acc * Cf::ACC_COLS);
-                bool first = true;
-                for (int ch = 0; ch < g.nchunk && ok; ++ch)
-                    for (int sxi = 0; sxi < 3; ++sxi) {
-                        if (!tc::mbar_wait(bar_full + 8 * s, ph, abort)) {
-                            ok = false;
-                            break;
-                        }
-                        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                        const uint32_t sa = stages + s * Cf::A_BYTES;
-#pragma unroll
-                        for (int syi = 0; syi < 3; ++syi) {
-                            // source offset (sy, sx) = (syi - 1, sxi - 1); the weight tap reads it
-                            const int tap = g.flip ? (2 - syi) * 3 + (2 - sxi) : syi * 3 + sxi;
-                            // descriptors = the base descriptors plus the offset in 16-byte units
-                            const uint64_t da = a_desc0 + ((sa - stages + syi * HBW * CK * 2) >> 4);
-                            const uint64_t dw = w_desc0 + (((tap * g.nchunk + ch) * Cf::BBLK) >> 4);
-#pragma unroll
-                            for (int kk = 0; kk < CK / 16; ++kk) {
-                                tc::mma_f16(d, da + (uint64_t)(kk * 2), dw + (uint64_t)(kk * 2), IDESC,
-                                            first ? 0u : 1u);
-                                first = false;
-                            }
-                        }
-                        tc::mma_commit(bar_empty + 8 * s);
-                        last_bar = bar_empty + 8 * s;
-                        last_par = ph;
-                        if (++s == S) {
-                            s = 0;
-                            ph ^= 1u;
-                        }
+                for (int ch = 0; ch < g.nchunk; ++ch) {
+                    if (!tc::mbar_wait(bar_full + 8 * s, ph, abort)) {
+                        ok = false;
+                        break;
                     }
+                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                    const uint64_t da = a_desc0 + (uint64_t)((uint32_t)(s * Cf::STAGE) >> 4);
+                    uint64_t dw = w_desc0 + (uint64_t)((uint32_t)(ch * Cf::BBLK) >> 4);
+                    // source offset (sy, sx) = (syi - 1, sxi - 1) of tap syi * 3 + sxi (mirrored: 8 - that)
+                    if (g.flip) dw += (uint64_t)(8 * wstep);
+                    const uint64_t step = (uint64_t)(int64_t)(g.flip ? -wstep : wstep);
+#pragma unroll
+                    for (int syi = 0; syi < 3; ++syi)
+#pragma unroll
+                        for (int sxi = 0; sxi < 3; ++sxi) {
+#pragma unroll
+                            for (int kk = 0; kk < CK / 16; ++kk)
+                                tc::mma_f16(d, da + (uint64_t)((sxi * Cf::A_BYTES + syi * HBW * CK * 2) / 16 + kk * 2),
+                                            dw + (uint64_t)(kk * 2), IDESC,
+                                            syi + sxi + kk > 0 || ch > 0 ? 1u : 0u);
+                            dw += step;
+                        }
+                    tc::mma_commit(bar_empty + 8 * s);
+                    last_bar = bar_empty + 8 * s;
+                    last_par = ph;
+                    if (++s == S) {
+                        s = 0;
+                        ph ^= 1u;
+                    }
+                }
                 if (!ok) break;
                 tc::mma_commit(bar_afull + 8 * acc);
                 if (++acc == 2) {
@@ -521,12 +523,13 @@ __global__ void __launch_bounds__(192, 1)
 //    row): accumulators (dy -1, 0) and (dy 1, none). 3 (R + 3) / R + 1 box rows a pixel
 //    feed all nine taps of 64 input and 64 output channels (5.1 with R = 8; one
 //    box a tap and operand, as before, takes 15).
-//  * Layers whose channels are not whole groups of 64 (C = 32, 96) are read as
-//    pairs of pixels, tensors of 2 C channels and W / 2 columns: D of a pair
-//    offset s then holds, for each parity px of In's pixel and pg of gz's, the
-//    tap dx = 2 s + px - pg; s = -1, 0, 1 give every combination that is a tap,
-//    the others are left out by the epilogue (or not loaded, where a group of 64
-//    holds one parity only). Half the box rows again.
+//  * Layers whose channels are not whole groups of 64 (C = 32, 96, and 8, the
+//    first layer's) are read with F = 2 or 8 neighbouring pixels as one column,
+//    tensors of F C channels and W / F columns: D of a column offset s then
+//    holds, for pixel px of In's column and pg of gz's, the tap
+//    dx = F s + px - pg; s = -1, 0, 1 give every combination that is a tap, the
+//    others are left out by the epilogue (or not loaded, where a group of 64
+//    channels holds no such pixels). 1 / F of the box rows.
 // A unit of work is (64 channels of In, 64 of gz, a range of pixel blocks); every
 // CTA takes one, accumulates it in tensor memory (up to 3 offsets x 2 tiles x 64
 // columns) and adds it to dW with FP32 atomics at the end.
@@ -538,10 +541,9 @@ constexpr int kWgR = 8;                    // image rows of a pixel block
 constexpr int kWgXSlots = 3, kWgGSlots = 2;  // ring slots of In and of gz
 
 struct WgradGeo {
-    int B, H, W;        // of the tensors as read (W / 2 columns for pairs)
+    int B, H, W;        // of the tensors as read (W columns of F pixels)
     int C, Cout;        // channels of the layer
-    int pair;           // 1: read as pairs of pixels
-    int bkx;            // columns of a pixel block, 16 or 32
+    int F;              // pixels a column
     int xblocks, yblocks, kblocks;
     int cgroups, ngroups;  // 64-channel groups of In and gz as read
     int ksplit;         // pixel ranges a (channel group, channel group)
@@ -565,6 +567,7 @@ __device__ __forceinline__ constexpr uint32_t idesc_bf16_mn() {
            ((uint32_t)(128 >> 4) << 24);
 }
 
+template <int BKX>
 __global__ void __launch_bounds__(192, 1)
     k_wgrad_tma(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapG, const WgradGeo g,
                 float *dw, int *err) {
@@ -572,9 +575,8 @@ __global__ void __launch_bounds__(192, 1)
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
-    const int bkx = g.bkx;
-    const uint32_t ROW = (uint32_t)bkx * 128u;            // one image row of a box
-    const uint32_t X_BYTES = (R + 3) * ROW, G_BYTES = R * ROW;
+    constexpr uint32_t ROW = (uint32_t)BKX * 128u;        // one image row of a box
+    constexpr uint32_t X_BYTES = (R + 3) * ROW, G_BYTES = R * ROW;
     const uint32_t gbase = base + XS * X_BYTES;
     const uint32_t bar_xfull = gbase + GS * G_BYTES;
     const uint32_t bar_xempty = bar_xfull + 8 * XS;
@@ -590,14 +592,10 @@ __global__ void __launch_bounds__(192, 1)
     const int c0 = (gr % g.cgroups) * 64, n0 = (gr / g.cgroups) * 64;
     const int per = (g.kblocks + g.ksplit - 1) / g.ksplit;
     const int kb0 = ks * per, kb1 = min(g.kblocks, kb0 + per);
-    // offsets s0 .. s1 (pixels, or pairs: -1 needs In's second pixel and gz's
-    // first, 1 the reverse)
-    int s0 = -1, s1 = 1;
-    if (g.pair) {
-        const bool x1 = (c0 + 63) / g.C > 0, x0 = c0 / g.C == 0, g1 = (n0 + 63) / g.Cout > 0, g0 = n0 / g.Cout == 0;
-        s0 = x1 && g0 ? -1 : 0;
-        s1 = x0 && g1 ? 1 : 0;
-    }
+    // column offsets s0 .. s1: -1 needs In's last pixel and gz's first one, 1 the
+    // reverse (c0 / C is 0 and every group holds all there is when F = 1)
+    const int s0 = (c0 + 63) / g.C >= g.F - 1 && n0 / g.Cout == 0 || g.F == 1 ? -1 : 0;
+    const int s1 = c0 / g.C == 0 && (n0 + 63) / g.Cout >= g.F - 1 || g.F == 1 ? 1 : 0;
 
     if (threadIdx.x == 0) {
         *abort = *(volatile int *)err;
@@ -632,7 +630,7 @@ __global__ void __launch_bounds__(192, 1)
         const int xb = kb % g.xblocks, r = kb / g.xblocks;
         b = r / g.yblocks;
         y0 = (r - b * g.yblocks) * R;
-        x0 = xb * bkx;
+        x0 = xb * BKX;
     };
 
     if (warp == 0) {
@@ -678,6 +676,7 @@ __global__ void __launch_bounds__(192, 1)
         if (lane == 0) {
             // ---------------- MMA issuer ----------------
             constexpr uint32_t IDESC = idesc_bf16_mn<64>();
+            const uint64_t x_desc0 = sdesc_mn(base, ROW), g_desc0 = sdesc_mn(gbase, ROW);
             int xs = 0, gs = 0;
             uint32_t xph = 0, gph = 0;
             bool ok = true;
@@ -690,25 +689,28 @@ __global__ void __launch_bounds__(192, 1)
                     ok = false;
                     break;
                 }
-                const uint32_t sg = gbase + gs * G_BYTES;
                 for (int s = s0; s <= s1; ++s) {
                     if (!tc::mbar_wait(bar_xfull + 8 * xs, xph, abort)) {
                         ok = false;
                         break;
                     }
                     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                    const uint32_t sx = base + xs * X_BYTES;
                     const uint32_t d = tmem_base + (uint32_t)((s - s0) * 128);
-                    for (int j = 0; j < rows; ++j)
-                        for (int kk = 0; kk < bkx / 16; ++kk) {
-                            // 16 pixels = 2048 bytes; image row j of gz against rows j, j + 1 and
-                            // j + 2, j + 3 of the box
-                            const uint32_t off = (uint32_t)j * ROW + (uint32_t)kk * 2048u;
-                            const uint64_t db = sdesc_mn(sg + off, ROW);
-                            const uint32_t add = kb > kb0 || j > 0 || kk > 0 ? 1u : 0u;
-                            tc::mma_f16(d, sdesc_mn(sx + off, ROW), db, IDESC, add);
-                            tc::mma_f16(d + 64u, sdesc_mn(sx + off + 2 * ROW, ROW), db, IDESC, add);
+                    // 16 pixels = 2048 bytes; image row j of gz against rows j, j + 1 and j + 2, j + 3 of the
+                    // box. Descriptors = the first ones plus constants (in 16-byte units)
+                    const uint64_t dx = x_desc0 + (uint64_t)((uint32_t)xs * (X_BYTES / 16));
+                    const uint64_t dg = g_desc0 + (uint64_t)((uint32_t)gs * (G_BYTES / 16));
+#pragma unroll
+                    for (int j = 0; j < R; ++j) {
+                        if (j >= rows) break;
+#pragma unroll
+                        for (int kk = 0; kk < BKX / 16; ++kk) {
+                            const uint64_t off = (j * ROW + kk * 2048u) / 16;
+                            const uint32_t add = j + kk > 0 || kb > kb0 ? 1u : 0u;
+                            tc::mma_f16(d, dx + off, dg + off, IDESC, add);
+                            tc::mma_f16(d + 64u, dx + off + 2 * ROW / 16, dg + off, IDESC, add);
                         }
+                    }
                     tc::mma_commit(bar_xempty + 8 * xs);
                     last_bar = bar_xempty + 8 * xs;
                     last_par = xph;
@@ -736,7 +738,7 @@ __global__ void __launch_bounds__(192, 1)
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
             const int i = (q & 1) * 32 + lane;   // channel of In in the group
             const int e = c0 + i;
-            const int px = g.pair && e >= g.C, ci = px ? e - g.C : e;
+            const int px = g.F > 1 ? e / g.C : 0, ci = e - px * g.C;
             for (int s = s0; s <= s1; ++s)
                 for (int t = 0; t < 2; ++t) {
                     const int dy = 2 * t + (q >> 1) - 1;
@@ -746,9 +748,9 @@ __global__ void __launch_bounds__(192, 1)
                     for (int j0 = 0; j0 < 64; j0 += 16) {
                         uint32_t v[16];
                         tc::tmem_ld16(taddr + (uint32_t)j0, v);
-                        const int f = n0 + j0;  // 16 columns of one parity: Cout is a multiple of 32
-                        const int pg = g.pair && f >= g.Cout, co = pg ? f - g.Cout : f;
-                        const int dx = g.pair ? 2 * s + px - pg : s;
+                        const int f = n0 + j0;  // 16 channels of one pixel: Cout is a multiple of 32
+                        const int pg = g.F > 1 ? f / g.Cout : 0, co = f - pg * g.Cout;
+                        const int dx = g.F * s + px - pg;
                         if (dx >= -1 && dx <= 1) {
                             float *p = dw + ((long long)co * 9 + (dy + 1) * 3 + (dx + 1)) * g.C + ci;
 #pragma unroll
