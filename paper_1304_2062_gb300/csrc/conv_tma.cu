@@ -43,7 +43,11 @@ struct FwdEpi {
     __device__ __forceinline__ void prepare(float *sm, int i, int n) const {
         for (int k = i; k < nb; k += n) sm[k] = bias[k];
     }
-    __device__ __forceinline__ void store(int m, int n, const float (&v)[16], float &, const float *sm) const {
+    struct Pre {};
+    struct PrePix {};
+    __device__ __forceinline__ Pre prefetch(int, int) const { return {}; }
+    __device__ __forceinline__ PrePix prefetch_pixel(int) const { return {}; }
+    __device__ __forceinline__ void store(int m, int n, const float (&v)[16], float &, const float *sm, Pre) const {
         float w[16];
 #pragma unroll
         for (int q = 0; q < 16; ++q) {
@@ -52,7 +56,7 @@ struct FwdEpi {
         }
         store16(out + (long long)m * N + n, w);
     }
-    __device__ __forceinline__ void finish(int, float, const float *) const {}
+    __device__ __forceinline__ void finish(int, float, const float *, PrePix) const {}
 };
 
 // The last convolution (32 channels, ReLU) with the 1x1 head and the input
@@ -69,7 +73,14 @@ struct HeadEpi {
     __device__ __forceinline__ void prepare(float *sm, int i, int n) const {
         for (int k = i; k < 65; k += n) sm[k] = k < 32 ? bias[k] : k < 64 ? hw[k - 32] : hb[0];
     }
-    __device__ __forceinline__ void store(int m, int n, const float (&v)[16], float &st, const float *sm) const {
+    struct Pre {};
+    struct PrePix {
+        float f;
+        uint8_t mask;
+    };
+    __device__ __forceinline__ Pre prefetch(int, int) const { return {}; }
+    __device__ __forceinline__ PrePix prefetch_pixel(int m) const { return {f[m], mask[m]}; }
+    __device__ __forceinline__ void store(int m, int n, const float (&v)[16], float &st, const float *sm, Pre) const {
         float w[16];
         if (n == 0) st = sm[64];
 #pragma unroll
@@ -80,8 +91,8 @@ struct HeadEpi {
         }
         if (out) store16(out + (long long)m * 32 + n, w);
     }
-    __device__ __forceinline__ void finish(int m, float st, const float *) const {
-        y[m] = (mask[m] ? f[m] : 0.0f) + st;
+    __device__ __forceinline__ void finish(int m, float st, const float *, PrePix p) const {
+        y[m] = (p.mask ? p.f : 0.0f) + st;
     }
 };
 
@@ -93,15 +104,27 @@ struct DgradEpi {
     int split, N;
     static constexpr int SMEM_FLOATS = 1;
     __device__ __forceinline__ void prepare(float *, int, int) const {}
-    __device__ __forceinline__ void store(int m, int n, const float (&v)[16], float &, const float *) const {
+    struct Pre {
+        uint4 a0, a1;  // the 16 activations (bf16)
+    };
+    struct PrePix {};
+    __device__ __forceinline__ Pre prefetch(int m, int n) const {
+        Pre p{};
+        if (act && n < split) {
+            const uint4 *a4 = (const uint4 *)(act + (long long)m * split + n);
+            p.a0 = a4[0];
+            p.a1 = a4[1];
+        }
+        return p;
+    }
+    __device__ __forceinline__ PrePix prefetch_pixel(int) const { return {}; }
+    __device__ __forceinline__ void store(int m, int n, const float (&v)[16], float &, const float *, const Pre &p) const {
         float w[16];
 #pragma unroll
         for (int q = 0; q < 16; ++q) w[q] = v[q];
         if (n < split) {
             if (act) {
-                const uint4 *a4 = (const uint4 *)(act + (long long)m * split + n);
-                const uint4 a0 = a4[0], a1 = a4[1];
-                const uint32_t aw[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+                const uint32_t aw[8] = {p.a0.x, p.a0.y, p.a0.z, p.a0.w, p.a1.x, p.a1.y, p.a1.z, p.a1.w};
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
                     const __nv_bfloat162 h = *(const __nv_bfloat162 *)&aw[q];
@@ -114,7 +137,7 @@ struct DgradEpi {
             store16(din2 + (long long)m * (N - split) + (n - split), w);
         }
     }
-    __device__ __forceinline__ void finish(int, float, const float *) const {}
+    __device__ __forceinline__ void finish(int, float, const float *, PrePix) const {}
 };
 
 PFN_cuTensorMapEncodeTiled_v12000 encoder() {
@@ -264,7 +287,7 @@ cudaError_t launch_halo(const __nv_bfloat16 *A, int B, int H, int W, int C, cons
     const int per = nsm / g.ntiles;
     if (per < 1) return cudaErrorNotSupported;
     const int grid = (g.mtiles < per ? g.mtiles : per) * g.ntiles;
-    fn<<<grid, 192, smem, s>>>(ma, mb, g, epi, S, err);
+    fn<<<grid, tma::kHaloThreads, smem, s>>>(ma, mb, g, epi, S, err);
     return cudaGetLastError();
 }
 

@@ -113,8 +113,11 @@ __device__ __forceinline__ void tile_origin(const ConvGeo &g, int t, int &b, int
 // EPI provides
 //   SMEM_FLOATS, prepare(sm, i, n)    constants copied to shared memory by the
 //                                      epilogue threads i = 0..n-1 once per CTA
-//   store(m, n, v[16], float &state, sm)  the 16 outputs of pixel m, columns n..n+15
-//   finish(m, float state, sm)        after the last column group of pixel m
+//   Pre, prefetch(m, n)               what store(m, n) reads from device memory (may be loaded
+//                                      before the accumulator is complete)
+//   PrePix, prefetch_pixel(m)         the same for finish(m)
+//   store(m, n, v[16], float &state, sm, pre)  the 16 outputs of pixel m, columns n..n+15
+//   finish(m, float state, sm, pre)   after the last column group of pixel m
 template <int BN, int CK, class EPI>
 __global__ void __launch_bounds__(192, 1)
     k_conv_tma(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, const ConvGeo g,
@@ -265,9 +268,9 @@ __global__ void __launch_bounds__(192, 1)
                 float f[16];
 #pragma unroll
                 for (int i = 0; i < 16; ++i) f[i] = __uint_as_float(v[i]);
-                epi.store(m, nt * BN + j0, f, state, epi_const);
+                epi.store(m, nt * BN + j0, f, state, epi_const, epi.prefetch(m, nt * BN + j0));
             }
-            epi.finish(m, state, epi_const);
+            epi.finish(m, state, epi_const, epi.prefetch_pixel(m));
             asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
             __syncwarp();
             if (lane == 0) arrive(bar_aempty + 8 * acc);
@@ -301,6 +304,7 @@ __global__ void __launch_bounds__(192, 1)
 
 constexpr int HBW = 16, HBH = 8;             // tile 16 x 8 pixels
 constexpr int HROWS = HBW * (HBH + 2);        // 160 box rows
+constexpr int kHaloThreads = 320;             // producer, MMA issuer and eight epilogue warps
 
 template <int BN, int CK>
 struct HaloCfg {
@@ -309,12 +313,13 @@ struct HaloCfg {
     static constexpr int STAGE = 3 * A_BYTES;  // the boxes of the three horizontal offsets
     static constexpr int BBLK = BN * CK * 2;   // one (tap, channel block) of weights
     static constexpr int ACC_COLS = BN <= 32 ? 32 : BN <= 64 ? 64 : 128;
-    static constexpr int TMEM_COLS = 2 * ACC_COLS;
+    static constexpr int NACC = 4;             // accumulators
+    static constexpr int TMEM_COLS = NACC * ACC_COLS;
     static constexpr int SMEM_BUDGET = 196608;
 };
 
 template <int BN, int CK, class EPI>
-__global__ void __launch_bounds__(192, 1)
+__global__ void __launch_bounds__(kHaloThreads, 1)
     k_conv_halo(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, const ConvGeo g,
                 const EPI epi, int S, int *err) {
     using Cf = HaloCfg<BN, CK>;
@@ -328,8 +333,8 @@ __global__ void __launch_bounds__(192, 1)
     const uint32_t bar_full = bar_w + 8;
     const uint32_t bar_empty = bar_full + 8 * S;
     const uint32_t bar_afull = bar_empty + 8 * S;
-    const uint32_t bar_aempty = bar_afull + 16;
-    const uint32_t tmem_slot = bar_aempty + 16;
+    const uint32_t bar_aempty = bar_afull + 8 * Cf::NACC;
+    const uint32_t tmem_slot = bar_aempty + 8 * Cf::NACC;
     volatile int *abort = (volatile int *)(smem_raw + (tmem_slot + 4 - raw));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // tiles t = nt * mtiles + mt; CTA c takes n tile c % ntiles and every
@@ -345,7 +350,7 @@ __global__ void __launch_bounds__(192, 1)
             tc::mbar_init(bar_full + 8 * s, 1);
             tc::mbar_init(bar_empty + 8 * s, 1);
         }
-        for (int a = 0; a < 2; ++a) {
+        for (int a = 0; a < Cf::NACC; ++a) {
             tc::mbar_init(bar_afull + 8 * a, 1);
             tc::mbar_init(bar_aempty + 8 * a, 4);
         }
@@ -452,7 +457,7 @@ __global__ void __launch_bounds__(192, 1)
                 }
                 if (!ok) break;
                 tc::mma_commit(bar_afull + 8 * acc);
-                if (++acc == 2) {
+                if (++acc == Cf::NACC) {
                     acc = 0;
                     aph ^= 1u;
                 }
@@ -460,38 +465,46 @@ __global__ void __launch_bounds__(192, 1)
             if (!ok && last_bar) tc::mbar_wait(last_bar, last_par, nullptr);
         }
     } else {
-        // ---------------- epilogue (warps 2..5) ----------------
+        // ---------------- epilogue (two groups of four warps) ----------------
+        // The groups take the CTA's tiles in turn, so each has two tiles' time
+        // for one; what a tile's outputs need from device memory is loaded
+        // before its accumulator is waited for.
         __shared__ float epi_const[EPI::SMEM_FLOATS];
-        epi.prepare(epi_const, threadIdx.x - 64, 128);
-        asm volatile("bar.sync 1, 128;\n" ::: "memory");  // the four epilogue warps only
-        const int q = warp & 3;
-        int acc = 0;
+        epi.prepare(epi_const, threadIdx.x - 64, 256);
+        asm volatile("bar.sync 1, 256;\n" ::: "memory");  // the epilogue warps only
+        const int q = warp & 3, group = (warp - 2) >> 2;
+        int acc = group;
         uint32_t aph = 0;
-        for (int t = first_tile; t < end_tile; t += tile_step) {
-            if (!tc::mbar_wait(bar_afull + 8 * acc, aph, abort)) break;
-            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+        for (int t = first_tile + group * tile_step; t < end_tile; t += 2 * tile_step) {
             int b, x0, y0, nt;
             tile_origin(g, t, b, x0, y0, nt);
             const int r = q * 32 + lane;
             const int y = y0 + r / HBW, x = x0 + r % HBW;
             const int m = (b * g.H + y) * g.W + x;
+            typename EPI::Pre pre[BN / 16];
+#pragma unroll
+            for (int j = 0; j < BN / 16; ++j) pre[j] = epi.prefetch(m, nt * BN + 16 * j);
+            const typename EPI::PrePix pp = epi.prefetch_pixel(m);
+            if (!tc::mbar_wait(bar_afull + 8 * acc, aph, abort)) break;
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
             const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * Cf::ACC_COLS);
             float state = 0.0f;
-#pragma unroll 1
-            for (int j0 = 0; j0 < BN; j0 += 16) {
+#pragma unroll
+            for (int j = 0; j < BN / 16; ++j) {
                 uint32_t v[16];
-                tc::tmem_ld16(taddr + (uint32_t)j0, v);
+                tc::tmem_ld16(taddr + (uint32_t)(16 * j), v);
                 float f[16];
 #pragma unroll
                 for (int i = 0; i < 16; ++i) f[i] = __uint_as_float(v[i]);
-                epi.store(m, nt * BN + j0, f, state, epi_const);
+                epi.store(m, nt * BN + 16 * j, f, state, epi_const, pre[j]);
             }
-            epi.finish(m, state, epi_const);
             asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
             __syncwarp();
             if (lane == 0) arrive(bar_aempty + 8 * acc);
-            if (++acc == 2) {
-                acc = 0;
+            epi.finish(m, state, epi_const, pp);
+            acc += 2;
+            if (acc >= Cf::NACC) {
+                acc = group;
                 aph ^= 1u;
             }
         }
