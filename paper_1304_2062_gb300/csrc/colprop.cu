@@ -28,6 +28,7 @@
 // H = 1024) keeps half a column in angle planes [n][k] (smem_fft.cuh), the
 // halves one after the other, v and then the even half's result y_e held in
 // the rows of the column's own block in device memory.
+#include "dependent.cuh"
 #include "diffuse_x2.cuh"
 #include "poly.cuh"
 #include "prop_classes.cuh"
@@ -232,9 +233,11 @@ __global__ void __launch_bounds__(col_threads<H>(), H >= 768 ? 1 : 2) k_col_prop
     const int l = (b & 1) ? a.W / 2 - h : h;
     const int scol = half_col_slot(l, a.W);
     float4 *g = reinterpret_cast<float4 *>(a.col + (long long)l * (N * H));
+    dependent_launch();
     for (int m = tid; m < H; m += T) tws[m] = a.tw[m];
     fft_twiddles<T, L, 2>(twp, a.tw, tid);  // from the table in device memory
     if constexpr (POLY > 0) col_poly_stage(cp, a, tid, T);
+    dependent_wait();
     auto apply = [&](int parity) {
         if constexpr (POLY == 0)
             col_apply<N, H>(X, a.D, scol, a.col_slots, parity, tid);
@@ -571,6 +574,7 @@ __global__ void __launch_bounds__(ColTmaCfg<N, H>::T, ColTmaCfg<N, H>::MINB)
     const uint32_t bar = bulk::saddr(tws + H), sa = bulk::saddr(XA), sb = bulk::saddr(XB);  // barriers at bar, bar + 8
     const int tid = threadIdx.x;
     int c = blockIdx.x;
+    dependent_launch();
     if (c >= a.Wc) return;
     if (tid == 0) {
         bulk::bar_init(bar, 1);
@@ -584,9 +588,10 @@ __global__ void __launch_bounds__(ColTmaCfg<N, H>::T, ColTmaCfg<N, H>::MINB)
         bulk::bar_expect(bar + 8, HB);
         bulk::load(sb, g + HF, HB, bar + 8);
     };
-    if (tid == 0) copy_in(c);
     for (int m = tid; m < H; m += T) tws[m] = a.tw[m];
     if constexpr (POLY > 0) col_poly_stage(cp, a, tid, T);  // read after the first barrier below
+    dependent_wait();
+    if (tid == 0) copy_in(c);
     constexpr int KL = col_poly_slots<POLY>();
     constexpr int OUT = POLY > 0 ? RD_SWZ_OUT : RD_PLAIN, IN = POLY > 0 ? RD_SWZ_IN : RD_PLAIN;
     for (uint32_t ph = 0; c < a.Wc; c += gridDim.x, ph ^= 1u) {
@@ -653,10 +658,10 @@ cudaError_t col_launch(const ColArgs &a, cudaStream_t s) {
     cudaError_t e = col_attr<N, H, POLY>();
     if (e != cudaSuccess) return e;
     if constexpr (col_tma_fits<N, H>())
-        k_col_tma<N, H, POLY><<<col_grid<N, H, POLY>(a), ColTmaCfg<N, H>::T, ColTmaCfg<N, H>::SMEM, s>>>(a);
+        return launch_dependent(k_col_tma<N, H, POLY>, col_grid<N, H, POLY>(a), ColTmaCfg<N, H>::T,
+                                ColTmaCfg<N, H>::SMEM, s, a);
     else
-        k_col_prop<N, H, POLY><<<a.Wc, ColCfg<N, H>::T, ColCfg<N, H>::SMEM, s>>>(a);
-    return cudaGetLastError();
+        return launch_dependent(k_col_prop<N, H, POLY>, a.Wc, ColCfg<N, H>::T, ColCfg<N, H>::SMEM, s, a);
 }
 
 template <int N, int POLY>

@@ -1,0 +1,33 @@
+// Programmatic dependent launches between the passes of one stream: a kernel
+// lets the next one start (dependent_launch) while its last blocks still run,
+// and the next one sets up (tables, barriers: nothing the previous kernels write)
+// before it waits for them (dependent_wait: every earlier kernel of the stream
+// has completed and its writes are visible). Blocks that return without waiting
+// are harmless: the kernel as a whole is not complete before its waiting blocks.
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace se2n {
+
+__device__ __forceinline__ void dependent_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void dependent_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Launch fn so that it may start before the previous kernel of the stream has
+// ended; fn must call dependent_wait before it touches what that one writes or reads.
+template <typename Args>
+cudaError_t launch_dependent(void (*fn)(Args), int grid, int block, size_t smem, cudaStream_t s, const Args &a) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, fn, a);
+}
+
+}  // namespace se2n

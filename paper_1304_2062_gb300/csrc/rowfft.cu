@@ -23,6 +23,7 @@
 // imaginary parts of X_0 and X_{W/2} ignored): Z_l = P + i Q and
 // Z_{W/2-l} = conj P + i conj Q with P = X_l + conj X_{W/2-l} and
 // Q = conj(w^l) (X_l - conj X_{W/2-l}), then z = inverse DFT of Z.
+#include "dependent.cuh"
 #include "prop_classes.cuh"
 #include "restore.cuh"
 #include "se2n_internal.h"
@@ -56,8 +57,10 @@ __global__ void __launch_bounds__(row_threads<W>()) k_row(const __grid_constant_
     const int tid = threadIdx.x, y = blockIdx.x;
     const long long H = a.H;
     const long long row = (long long)y * W;  // first pixel of the row
+    dependent_launch();
     for (int m = tid; m < W; m += T) tws[m] = a.tw[m];
     fft_twiddles<T, WH, 2>(twp, a.tw, tid);  // from the table in device memory
+    dependent_wait();
     // 1. the row
     if (a.in_mode == SE2N_ROW_IN_LIFT) {
         for (int m = tid; m < WH; m += T) {
@@ -243,8 +246,7 @@ cudaError_t row_launch(const RowArgs &a, cudaStream_t s) {
     if (NE != N && (a.in_mode == SE2N_ROW_IN_REAL || a.out_mode == SE2N_ROW_OUT_REAL)) return cudaErrorInvalidValue;
     cudaError_t e = row_attr<N, W, NE>();
     if (e != cudaSuccess) return e;
-    k_row<N, W, NE><<<a.H, row_threads<W>(), RowCfg<N, W>::SMEM, s>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(k_row<N, W, NE>, a.H, row_threads<W>(), RowCfg<N, W>::SMEM, s, a);
 }
 
 template <int N, int NE = N>
