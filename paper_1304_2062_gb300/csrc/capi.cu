@@ -515,11 +515,10 @@ se2n_status orient_impl(se2n_plan *plan, const float *f, const uint8_t *mask, do
     float2 *spec = plan->spec;
     StageTimer timer(plan, SE2N_STAGE_ORIENT);
     plan->kernels += 4;
-    SE2N_TRY(cuda_status(plan, se2n_launch_orient_prep(f, mask, spec, HW, plan->stream)));
+    SE2N_TRY(cuda_status(plan, se2n_launch_orient_prep(f, mask, spec, HW, plan->gmax, plan->stream)));
     SE2N_TRY(fft(plan, plan->fft_one, spec, CUFFT_FORWARD));
     SE2N_TRY(cuda_status(plan, se2n_launch_grad_spec(spec, plan->H, plan->W, (float)sigma, plan->stream)));
     SE2N_TRY(fft(plan, plan->fft_two, spec + HW, CUFFT_INVERSE));
-    SE2N_TRY(cuda_status(plan, cudaMemsetAsync(plan->gmax, 0, sizeof(unsigned int), plan->stream)));
     SE2N_TRY(cuda_status(plan, se2n_launch_grad_max(spec + HW, spec + 2 * HW, HW, plan->gmax, plan->stream)));
     const float tol2 = (float)(flat_tol * flat_tol);
     return cuda_status(plan, se2n_launch_bins(spec + HW, spec + 2 * HW, HW, plan->gmax, tol2, plan->N,

@@ -4,6 +4,8 @@
 // before it waits for them (dependent_wait: every earlier kernel of the stream
 // has completed and its writes are visible). Blocks that return without waiting
 // are harmless: the kernel as a whole is not complete before its waiting blocks.
+// After a library kernel, which never lets its successor start, such a launch
+// is an ordinary one.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -15,8 +17,8 @@ __device__ __forceinline__ void dependent_wait() { asm volatile("griddepcontrol.
 
 // Launch fn so that it may start before the previous kernel of the stream has
 // ended; fn must call dependent_wait before it touches what that one writes or reads.
-template <typename Args>
-cudaError_t launch_dependent(void (*fn)(Args), int grid, int block, size_t smem, cudaStream_t s, const Args &a) {
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*fn)(P...), int grid, int block, size_t smem, cudaStream_t s, A... a) {
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
@@ -27,7 +29,7 @@ cudaError_t launch_dependent(void (*fn)(Args), int grid, int block, size_t smem,
     cfg.stream = s;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, fn, a);
+    return cudaLaunchKernelEx(&cfg, fn, static_cast<P>(a)...);
 }
 
 }  // namespace se2n

@@ -4,10 +4,15 @@
 // plane is a coalesced 16-byte (two complex) or 8-byte (two float) access.
 // H and W are even, so a pixel pair never straddles a plane and every plane
 // starts 16-byte aligned.
+#include "dependent.cuh"
 #include "restore.cuh"
 #include "se2n_internal.h"
 
 namespace {
+
+using se2n::dependent_launch;
+using se2n::dependent_wait;
+using se2n::launch_dependent;
 
 constexpr int kBlock = 256;
 
@@ -17,9 +22,13 @@ inline int grid_for(long long n, int per_block = kBlock) {
     return (int)(g < 1 ? 1 : g);
 }
 
-// spec = f * (mask != 0) as complex, two pixels per thread.
+// spec = f * (mask != 0) as complex, two pixels per thread; the gradient's
+// maximum starts at zero.
 __global__ void k_orient_prep(const float2 *__restrict__ f, const uchar2 *__restrict__ mask,
-                              float4 *__restrict__ spec, long long npairs) {
+                              float4 *__restrict__ spec, long long npairs, unsigned int *__restrict__ gmax) {
+    dependent_launch();
+    dependent_wait();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *gmax = 0;  // for k_grad_max
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < npairs;
          i += (long long)gridDim.x * blockDim.x) {
         const float2 v = f[i];
@@ -34,6 +43,8 @@ __global__ void k_orient_prep(const float2 *__restrict__ f, const uchar2 *__rest
 // frequencies and the Nyquist derivative term set to zero.
 __global__ void k_grad_spec(const float2 *__restrict__ F, float2 *__restrict__ gx, float2 *__restrict__ gy,
                             int H, int W, float sigma) {
+    dependent_launch();
+    dependent_wait();
     const long long HW = (long long)H * W;
     const float two_pi = 6.28318530717958647692f;
     const float c = -2.0f * 9.86960440108935861883f * sigma * sigma;  // -2 pi^2 sigma^2
@@ -56,6 +67,8 @@ __global__ void k_grad_spec(const float2 *__restrict__ F, float2 *__restrict__ g
 // scale of the unnormalised inverse cancels in every later use.
 __global__ void k_grad_max(const float2 *__restrict__ gx, const float2 *__restrict__ gy, long long HW,
                            unsigned int *__restrict__ gmax) {
+    dependent_launch();
+    dependent_wait();
     float m = 0.0f;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < HW;
          i += (long long)gridDim.x * blockDim.x) {
@@ -79,6 +92,8 @@ __global__ void k_grad_max(const float2 *__restrict__ gx, const float2 *__restri
 __global__ void k_bins(const float2 *__restrict__ gx, const float2 *__restrict__ gy, long long HW,
                        const unsigned int *__restrict__ gmax, float flat_tol2, int N, float inv_dth,
                        uint8_t *__restrict__ bins) {
+    dependent_launch();
+    dependent_wait();
     const float pi = 3.14159265358979323846f;
     const float thresh = flat_tol2 * __uint_as_float(*gmax);
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < HW;
@@ -207,6 +222,8 @@ __device__ __forceinline__ long long real_off(long long i, int W, int Wp) {
 __global__ void k_lift_r(const float2 *__restrict__ f, const uchar2 *__restrict__ mask,
                          const uchar2 *__restrict__ bins, float *__restrict__ vol, long long npairs, int W, int Wp,
                          long long plane, int N) {
+    dependent_launch();
+    dependent_wait();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < npairs;
          i += (long long)gridDim.x * blockDim.x) {
         const float2 v = f[i];
@@ -225,6 +242,8 @@ __global__ void k_lift_r(const float2 *__restrict__ f, const uchar2 *__restrict_
 __global__ void k_mix_r(float *__restrict__ vol, const float2 *__restrict__ f, const uchar2 *__restrict__ mask,
                         const uchar2 *__restrict__ bins, long long npairs, int W, int Wp, long long plane, int N,
                         float scale, float eps, float guard) {
+    dependent_launch();
+    dependent_wait();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < npairs;
          i += (long long)gridDim.x * blockDim.x) {
         float2 *col = (float2 *)(vol + real_off(i, W, Wp));
@@ -254,6 +273,8 @@ __global__ void k_mix_r(float *__restrict__ vol, const float2 *__restrict__ f, c
 __global__ void k_project_r(const float *__restrict__ vol, long long npairs, int W, int Wp, long long plane, int N,
                             float scale, int proj, const float2 *__restrict__ f, const uchar2 *__restrict__ mask,
                             float2 *__restrict__ out) {
+    dependent_launch();
+    dependent_wait();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < npairs;
          i += (long long)gridDim.x * blockDim.x) {
         const float2 *col = (const float2 *)(vol + real_off(i, W, Wp));
@@ -392,31 +413,27 @@ __global__ void k_scale(float4 *__restrict__ v, long long n4, float s) {
 }  // namespace
 
 cudaError_t se2n_launch_orient_prep(const float *f, const uint8_t *mask, float2 *spec, long long HW,
-                                    cudaStream_t s) {
+                                    unsigned int *gmax, cudaStream_t s) {
     const long long n = HW / 2;
-    k_orient_prep<<<grid_for(n), kBlock, 0, s>>>((const float2 *)f, (const uchar2 *)mask, (float4 *)spec, n);
-    return cudaGetLastError();
+    return launch_dependent(k_orient_prep, grid_for(n), kBlock, 0, s, (const float2 *)f, (const uchar2 *)mask, (float4 *)spec, n, gmax);
 }
 
 cudaError_t se2n_launch_grad_spec(float2 *spec, int H, int W, float sigma, cudaStream_t s) {
     const long long HW = (long long)H * W;
-    k_grad_spec<<<grid_for(HW), kBlock, 0, s>>>(spec, spec + HW, spec + 2 * HW, H, W, sigma);
-    return cudaGetLastError();
+    return launch_dependent(k_grad_spec, grid_for(HW), kBlock, 0, s, spec, spec + HW, spec + 2 * HW, H, W, sigma);
 }
 
 cudaError_t se2n_launch_grad_max(const float2 *gx, const float2 *gy, long long HW, unsigned int *gmax,
                                  cudaStream_t s) {
     int g = grid_for(HW);
     if (g > 4096) g = 4096;
-    k_grad_max<<<g, kBlock, 0, s>>>(gx, gy, HW, gmax);
-    return cudaGetLastError();
+    return launch_dependent(k_grad_max, g, kBlock, 0, s, gx, gy, HW, gmax);
 }
 
 cudaError_t se2n_launch_bins(const float2 *gx, const float2 *gy, long long HW, const unsigned int *gmax,
                              float flat_tol2, int N, int angle_conv, uint8_t *bins, cudaStream_t s) {
     const float dth = (angle_conv ? 2.0f : 1.0f) * 3.14159265358979323846f / (float)N;
-    k_bins<<<grid_for(HW), kBlock, 0, s>>>(gx, gy, HW, gmax, flat_tol2, N, 1.0f / dth, bins);
-    return cudaGetLastError();
+    return launch_dependent(k_bins, grid_for(HW), kBlock, 0, s, gx, gy, HW, gmax, flat_tol2, N, 1.0f / dth, bins);
 }
 
 cudaError_t se2n_launch_lift(const float *f, const uint8_t *mask, const uint8_t *bins, float2 *vol,
@@ -455,27 +472,21 @@ cudaError_t se2n_launch_lift_r(const float *f, const uint8_t *mask, const uint8_
                                int N, cudaStream_t s) {
     const long long n = (long long)H * W / 2;
     const int Wp = W + 2;
-    k_lift_r<<<grid_for(n), kBlock, 0, s>>>((const float2 *)f, (const uchar2 *)mask, (const uchar2 *)bins, vol, n, W,
-                                            Wp, (long long)H * Wp, N);
-    return cudaGetLastError();
+    return launch_dependent(k_lift_r, grid_for(n), kBlock, 0, s, (const float2 *)f, (const uchar2 *)mask, (const uchar2 *)bins, vol, n, W, Wp, (long long)H * Wp, N);
 }
 
 cudaError_t se2n_launch_mix_r(float *vol, const float *f, const uint8_t *mask, const uint8_t *bins, int H, int W,
                               int N, float scale, float eps, float guard, cudaStream_t s) {
     const long long n = (long long)H * W / 2;
     const int Wp = W + 2;
-    k_mix_r<<<grid_for(n), kBlock, 0, s>>>(vol, (const float2 *)f, (const uchar2 *)mask, (const uchar2 *)bins, n, W, Wp,
-                                           (long long)H * Wp, N, scale, eps, guard);
-    return cudaGetLastError();
+    return launch_dependent(k_mix_r, grid_for(n), kBlock, 0, s, vol, (const float2 *)f, (const uchar2 *)mask, (const uchar2 *)bins, n, W, Wp, (long long)H * Wp, N, scale, eps, guard);
 }
 
 cudaError_t se2n_launch_project_r(const float *vol, int H, int W, int N, float scale, int proj, const float *f,
                                   const uint8_t *mask, float *out, cudaStream_t s) {
     const long long n = (long long)H * W / 2;
     const int Wp = W + 2;
-    k_project_r<<<grid_for(n), kBlock, 0, s>>>(vol, n, W, Wp, (long long)H * Wp, N, scale, proj, (const float2 *)f,
-                                               (const uchar2 *)mask, (float2 *)out);
-    return cudaGetLastError();
+    return launch_dependent(k_project_r, grid_for(n), kBlock, 0, s, vol, n, W, Wp, (long long)H * Wp, N, scale, proj, (const float2 *)f, (const uchar2 *)mask, (float2 *)out);
 }
 
 cudaError_t se2n_launch_dr_max(const float2 *vol, long long HW, int N, float scale, float *h, uint8_t *amax,

@@ -1,5 +1,6 @@
 // Coefficient tables of the interval polynomials (host) and the kernel that
 // applies them to an angle-major spectrum (poly.cuh has the method).
+#include "dependent.cuh"
 #include "poly.cuh"
 
 #include <math.h>
@@ -142,8 +143,10 @@ template <int N, bool REINSCH>
 __global__ void __launch_bounds__(kPolyBlock, REINSCH ? 3 : 4) k_poly(const __grid_constant__ PolyArgs a) {
     __shared__ float sc[kPolyBuckets * kPolyMax];
     constexpr int P = poly_lanes<N>();
+    dependent_launch();
     poly_stage(sc, a.t, threadIdx.x, kPolyBlock);
     __syncthreads();
+    dependent_wait();
     const long long f = ((long long)blockIdx.x * kPolyBlock + threadIdx.x) / P;
     const bool active = f < a.HW;
     poly_group<N, REINSCH>(a.t, sc, a.cs, a.sn, a.vol, a.H, a.W, a.Wc, a.HW, active ? f : a.HW - 1, active, a.k0);
@@ -155,11 +158,7 @@ template <int N>
 cudaError_t launch(const PolyArgs &a, cudaStream_t s) {
     const long long blocks = (a.HW * poly_lanes<N>() + kPolyBlock - 1) / kPolyBlock;
     if (blocks > INT_MAX) return cudaErrorInvalidValue;
-    if (a.t.reinsch)
-        k_poly<N, true><<<(int)blocks, kPolyBlock, 0, s>>>(a);
-    else
-        k_poly<N, false><<<(int)blocks, kPolyBlock, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(a.t.reinsch ? k_poly<N, true> : k_poly<N, false>, (int)blocks, kPolyBlock, 0, s, a);
 }
 
 }  // namespace

@@ -262,7 +262,7 @@ int se2n_diffuse_default_P(int N);
 
 // Pixel kernels (pixel.cu).
 cudaError_t se2n_launch_orient_prep(const float *f, const uint8_t *mask, float2 *spec, long long HW,
-                                    cudaStream_t s);
+                                    unsigned int *gmax, cudaStream_t s);
 cudaError_t se2n_launch_grad_spec(float2 *spec, int H, int W, float sigma, cudaStream_t s);
 cudaError_t se2n_launch_grad_max(const float2 *gx, const float2 *gy, long long HW, unsigned int *gmax,
                                  cudaStream_t s);
