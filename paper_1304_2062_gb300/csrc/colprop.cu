@@ -138,13 +138,18 @@ __device__ __forceinline__ void col_apply(float2 *X, const float *D, int scol, i
 constexpr int kColPolyLen = 32;
 struct ColPoly {
     float c[kPolyBuckets * kColPolyLen];
-    float cs[32], sn[32];
+    float4 t[2][9];  // cos, sin of the angles, four at a time (a lane may start at 15: one row more)
 };
-__device__ __forceinline__ void col_poly_stage(ColPoly &q, const ColArgs &a, int tid, int threads) {
+__device__ __forceinline__ void col_poly_stage(ColPoly &q, const ColArgs &a, bool split, int tid, int threads) {
     poly_stage(q.c, a.t, tid, threads);
+    // lane p of a frequency starts at angle 16 p, or at 15 where 30 angles take two
+    // lanes: its angles then start at entry 16 all the same
     for (int i = tid; i < 32; i += threads) {
-        q.cs[i] = a.cs[i];
-        q.sn[i] = a.sn[i];
+        const int e = split && i >= 15 ? i + 1 : i;
+        if (e < 36) {
+            reinterpret_cast<float *>(q.t[0])[e] = a.cs[i];
+            reinterpret_cast<float *>(q.t[1])[e] = a.sn[i];
+        }
     }
 }
 
@@ -158,10 +163,20 @@ __device__ __forceinline__ void col_poly(const ColPoly &q, const PolyTable &t, f
     f32x2 v[K];
     get(v);
     float e[K];
+    const float root = sqrtf(t.inv_beta), ux = wx * root, uy = wy * root;  // e = a_r^2 / beta
+    const int t0 = (K == 15 ? (r0 ? 16 : 0) : r0) / 4;
 #pragma unroll
-    for (int j = 0; j < K; ++j) {
-        const float ar = fmaf(wx, q.cs[r0 + j], wy * q.sn[r0 + j]);
-        e[j] = ar * ar * t.inv_beta;
+    for (int i = 0; i < (K + 3) / 4; ++i) {
+        const float4 c = q.t[0][t0 + i], s = q.t[1][t0 + i];
+        const float cc[4] = {c.x, c.y, c.z, c.w}, ss[4] = {s.x, s.y, s.z, s.w};
+#pragma unroll
+        for (int z = 0; z < 4; ++z) {
+            const int j = 4 * i + z;
+            if (j < K) {
+                const float ar = fmaf(ux, cc[z], uy * ss[z]);
+                e[j] = ar * ar;
+            }
+        }
     }
     poly_increment<K, NE / K>(v, e, poly_lane(q.c, t, wx, wy));
     add(v);
@@ -199,9 +214,11 @@ __device__ __forceinline__ void col_poly_planes(float2 *X, const ColPoly &q, con
                 }
             },
             [&](const f32x2(&v)[K]) {
+                int i2 = i, r2 = r0;  // form the addresses again (see col_poly_rows)
+                asm volatile("" : "+r"(i2), "+r"(r2));
 #pragma unroll
                 for (int j = 0; j < K; ++j) {
-                    float2 &x = X[xsm<L>(slot_of_angle<N, NE>(r0 + j) * L + i)];
+                    float2 &x = X[xsm<L>(slot_of_angle<N, NE>(r2 + j) * L + i2)];
                     x = make_float2(x.x + lo2(v[j]), x.y + hi2(v[j]));
                 }
             });
@@ -236,7 +253,7 @@ __global__ void __launch_bounds__(col_threads<H>(), H >= 768 ? 1 : 2) k_col_prop
     dependent_launch();
     for (int m = tid; m < H; m += T) tws[m] = a.tw[m];
     fft_twiddles<T, L, 2>(twp, a.tw, tid);  // from the table in device memory
-    if constexpr (POLY > 0) col_poly_stage(cp, a, tid, T);
+    if constexpr (POLY > 0) col_poly_stage(cp, a, POLY == 30, tid, T);
     dependent_wait();
     auto apply = [&](int parity) {
         if constexpr (POLY == 0)
@@ -476,13 +493,15 @@ __device__ __forceinline__ void col_apply_rows(float2 *XA, float2 *XB, const flo
     }
 }
 
-// The polynomial on a whole column in rows (angles in the order of rd_swz): row
-// p of a half holds frequency 2 rd_index(p) + half. Lane q of a row takes angles
+// The polynomial on a whole column in rows (angles in the order of rd_swz):
+// frequency 2 f + half is at row rd_pos(f) of its half. A warp takes consecutive
+// frequencies, so that their polynomials have about the same degree, and a warp
+// with two rounds takes the second a quarter of the column on, where wy^2 is
+// large if it was small and the reverse. Lane q of a frequency takes angles
 // q NE / P ..; with NE = 30 they start at slots 0 and 16, slot 17 is skipped.
-// Slots a lane takes. 16: the fewest exchanges, but 128 registers a thread do
-// not quite hold them (about 150 bytes spilled once a column); 8 spill nothing. Measured
-// a column pass: 512 x 512, N = 32 45.5 us with 16 and 48.6 with 8, 768 x 1024,
-// N = 16 75.7 and 71.6.
+// Slots a lane takes: 16 for the fewest exchanges, and 8 for N = 16, whose eight
+// rows of a quarter-warp would need eight frequencies of one butterfly. Measured
+// a column pass: 512 x 512, N = 32 45.5 us with 16 and 48.6 with 8.
 template <int NE>
 __host__ __device__ constexpr int col_poly_slots() {
     return NE == 16 ? 8 : 16;
@@ -494,9 +513,13 @@ __device__ __forceinline__ void col_poly_rows(float2 *XA, const ColPoly &q, cons
     static_assert((H * P) % 32 == 0, "whole warps");
 #pragma unroll 1
     for (int u = tid; u < H * P; u += T) {
-        const int row = u / P, q0 = u % P, half = row / L;
-        const int k = 2 * rd_index<L>(row - half * L) + half;
-        const int s = rd_swz_key<N, KL>(row, q0);
+        const int q0 = u % P;
+        int f = u / P;  // of both halves: half f / L
+        const int half = f / L;
+        f -= half * L;
+        if (half) f = f + L / 4 < L ? f + L / 4 : f + L / 4 - L;
+        const int k = 2 * f + half, row = half * L + rd_pos<L>(f);
+        const int s = rd_swz_key<N, KL>(f, q0);
         float4 *X4 = reinterpret_cast<float4 *>(XA + row * N + q0 * KL);
         // 16 slots a lane, 2 i and 2 i + 1 in unit i. 15 angles in them: the first
         // lane's last slot is empty, and the second lane's second one
@@ -521,11 +544,16 @@ __device__ __forceinline__ void col_poly_rows(float2 *XA, const ColPoly &q, cons
                     const f32x2 none = pk2(0.0f, 0.0f);
                     return skip ? (w == 1 ? none : v[w - 1]) : (w == 15 ? none : v[w == 15 ? 0 : w]);
                 };
+                // form the addresses again: kept across the polynomial, they would
+                // push 200 bytes a thread out of the registers
+                int s2 = s;
+                float4 *X5 = X4;
+                asm volatile("" : "+r"(s2), "+l"(X5));
 #pragma unroll
                 for (int i = 0; i < KL / 2; ++i) {
-                    float4 x = X4[i ^ s];
-                    const f32x2 d0 = slot(2 * i), d1 = slot(2 * i + 1);
-                    X4[i ^ s] = make_float4(x.x + lo2(d0), x.y + hi2(d0), x.z + lo2(d1), x.w + hi2(d1));
+                    const float4 x = X5[i ^ s2];
+                    const f32x2 y0 = add2(pk2(x.x, x.y), slot(2 * i)), y1 = add2(pk2(x.z, x.w), slot(2 * i + 1));
+                    X5[i ^ s2] = make_float4(lo2(y0), hi2(y0), lo2(y1), hi2(y1));
                 }
             });
     }
@@ -589,7 +617,7 @@ __global__ void __launch_bounds__(ColTmaCfg<N, H>::T, ColTmaCfg<N, H>::MINB)
         bulk::load(sb, g + HF, HB, bar + 8);
     };
     for (int m = tid; m < H; m += T) tws[m] = a.tw[m];
-    if constexpr (POLY > 0) col_poly_stage(cp, a, tid, T);  // read after the first barrier below
+    if constexpr (POLY > 0) col_poly_stage(cp, a, POLY == 30, tid, T);  // read after the first barrier below
     dependent_wait();
     if (tid == 0) copy_in(c);
     constexpr int KL = col_poly_slots<POLY>();
