@@ -277,15 +277,17 @@ void poly_count_build(se2n_plan *plan) {
 // SE2N_DIFFUSE_PROPAGATOR); null where it takes matrices, or with flags = 0
 // where there is no column pass. Asked for propagators, N = 30 and 32 take the
 // polynomial while it is no slower than applying matrices the plan has kept
-// from an earlier call (512 x 512, T = 2, 42 instructions an angle: 45.5 us a
-// column pass either way, and no build), and N = 16 matrices, which are small
-// (768 x 1024: 65 us against 72).
+// from an earlier call (512 x 512, T = 2, 42 instructions an angle: 43.2 us a
+// column pass against 45.3; about 1 us more every 3 instructions), and N = 16
+// matrices, which are small (768 x 1024: 65 us against 68, 512 x 512: 21 against 23). A batch builds its
+// matrices again in every run and takes the polynomial wherever it applies (a
+// build is 60 .. 300 us).
 const PolyTable *col_poly(se2n_plan *plan, double beta, double T, int steps, int flags) {
-    if (flags != 0 && plan->N < 30) return nullptr;
+    if (flags != 0 && !plan->rebuilds && plan->N < 30) return nullptr;
     const PolyTable *t = poly_get(plan, beta, T, steps);
     if (!t || !se2n_col_has_poly(*t)) return nullptr;
     if (flags == 0) return poly_beats_steps(*t, steps) ? t : nullptr;
-    return se2n_poly_cost(*t) <= 45 ? t : nullptr;
+    return plan->rebuilds || se2n_poly_cost(*t) <= 48 ? t : nullptr;
 }
 
 // Row and column passes of the Hermitian half (rowfft.cu, colprop.cu): the
@@ -1554,6 +1556,7 @@ se2n_status create_batch(se2n_batch *b, const se2n_image_desc *imgs) {
             if (pl->H == d.H && pl->W == d.W && pl->N == d.N) found = pl;
         if (!found) {
             SE2N_TRY(se2n_plan_create(&found, d.H, d.W, d.N, b->angle_conv, (void *)b->stream));
+            found->rebuilds = true;
             b->plans.push_back(found);
         }
         b->plan_of[i] = found;

@@ -499,17 +499,17 @@ __device__ __forceinline__ void col_apply_rows(float2 *XA, float2 *XB, const flo
 // with two rounds takes the second a quarter of the column on, where wy^2 is
 // large if it was small and the reverse. Lane q of a frequency takes angles
 // q NE / P ..; with NE = 30 they start at slots 0 and 16, slot 17 is skipped.
-// Slots a lane takes: 16 for the fewest exchanges, and 8 for N = 16, whose eight
-// rows of a quarter-warp would need eight frequencies of one butterfly. Measured
-// a column pass: 512 x 512, N = 32 45.5 us with 16 and 48.6 with 8.
-template <int NE>
+// Slots a lane takes: 16 for the fewest exchanges (512 x 512, N = 32: 45.5 us a
+// column pass, 48.6 with 8); 8 for N = 16, H = 64, whose last pass has no eight
+// frequencies of one butterfly for the eight rows of a quarter-warp.
+template <int NE, int H>
 __host__ __device__ constexpr int col_poly_slots() {
-    return NE == 16 ? 8 : 16;
+    return NE == 16 && H < 128 ? 8 : 16;
 }
 template <int T, int N, int H, int NE>
 __device__ __forceinline__ void col_poly_rows(float2 *XA, const ColPoly &q, const PolyTable &t, float wx,
                                               const float2 *tws, int tid) {
-    constexpr int L = H / 2, KL = col_poly_slots<NE>(), P = N / KL, K = NE / P;
+    constexpr int L = H / 2, KL = col_poly_slots<NE, H>(), P = N / KL, K = NE / P;
     static_assert((H * P) % 32 == 0, "whole warps");
 #pragma unroll 1
     for (int u = tid; u < H * P; u += T) {
@@ -620,7 +620,7 @@ __global__ void __launch_bounds__(ColTmaCfg<N, H>::T, ColTmaCfg<N, H>::MINB)
     if constexpr (POLY > 0) col_poly_stage(cp, a, POLY == 30, tid, T);  // read after the first barrier below
     dependent_wait();
     if (tid == 0) copy_in(c);
-    constexpr int KL = col_poly_slots<POLY>();
+    constexpr int KL = col_poly_slots<POLY, H>();
     constexpr int OUT = POLY > 0 ? RD_SWZ_OUT : RD_PLAIN, IN = POLY > 0 ? RD_SWZ_IN : RD_PLAIN;
     for (uint32_t ph = 0; c < a.Wc; c += gridDim.x, ph ^= 1u) {
         const int l = col_of_unit(c, a.W);

@@ -131,12 +131,13 @@ namespace se2n {
 // (events, full spectrum, 1024 x 1024, one GB300) against the step kernel it
 // replaces there:
 //   N = 32, T = 2 in 100 steps     122 us (4.4 TB/s), steps 1391 us
-//   N = 64, T = 50 in 1000 steps   949 us, steps 29.1 ms
+//   N = 64, T = 50 in 1000 steps   925 us, steps 29.1 ms
 // At T = 2 the loads and the arithmetic of a warp (77 us of packed FP32 at its
 // measured rate, 79 us of copies) follow one another, so the increment form is
 // held to 128 registers, 16 warps an SM (N = 16, 32, 64: 65, 122, 261 us; 71, 140,
 // 302 with 12 warps). Large T is bound by the packed FP32 pipe and Reinsch's form
-// runs fastest unconstrained (949 us; 1003 with 16 warps).
+// runs fastest unconstrained (949 us; 1003 with 16 warps; 925 since the addresses
+// are formed again for the stores instead of kept).
 constexpr int kPolyBlock = 128;
 
 template <int N, bool REINSCH>

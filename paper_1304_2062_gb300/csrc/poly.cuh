@@ -206,6 +206,8 @@ __device__ __forceinline__ void poly_group(const PolyTable &t, const float *sc, 
         e[j] = ar * ar * t.inv_beta;
     }
     poly_apply<K, P, REINSCH>(x, e, poly_lane(sc, t, wx, wy));
+    // form the addresses again: kept across the polynomial they take 2 K registers
+    asm volatile("" : "+l"(col), "+l"(HW));
     if (active) {
 #pragma unroll
         for (int j = 0; j < K; ++j) col[j * HW] = make_float2(lo2(x[j]), hi2(x[j]));

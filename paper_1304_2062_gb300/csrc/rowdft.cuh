@@ -53,14 +53,14 @@ enum { RD_ONE = 0, RD_TWO = 1, RD_SPLIT = 2, RD_MERGE = 3 };
 
 // The order of a row's angles while the polynomial is applied to it
 // (colprop.cu): a lane then holds KL = 8 or 16 consecutive angles, KL / 2 units
-// of 16 bytes, and a quarter-warp four consecutive frequencies f, whose rows lie
+// of 16 bytes, and a quarter-warp two to eight consecutive frequencies f, whose rows lie
 // whole multiples of 128 bytes apart, so that in plain order its lanes, which
 // read the same unit of theirs at a time, would meet in one or two of the eight
 // bank groups. Unit i of lane p of frequency f sits at unit i ^ rd_swz_key(f, p)
 // of the lane's, which sends the eight lanes to eight different groups.
 template <int N, int KL>
 __host__ __device__ __forceinline__ constexpr int rd_swz_key(int f, int p) {
-    return KL == 16 ? (2 * f + p) & 7 : N == 32 ? (2 * f + (p >> 1)) & 3 : f & 3;
+    return N == 16 ? (KL == 16 ? f & 7 : f & 3) : KL == 16 ? (2 * f + p) & 7 : (2 * f + (p >> 1)) & 3;
 }
 template <int N, int KL>
 __host__ __device__ __forceinline__ constexpr int rd_swz(int f, int n) {
@@ -88,8 +88,8 @@ __device__ __forceinline__ void rd_pass(float2 *XA, float2 *XB, const float2 *tw
     constexpr int TASKS = (MODE == RD_TWO ? 2 : 1) * BF * N;
     static_assert(T % N == 0, "one angle a thread");
     static_assert(ORDER == RD_PLAIN || (S == 1 && !PAIR && (N == 16 || N == 32) && TASKS % 32 == 0 &&
-                                        (RdPlan<L>::R1 * (RdPlan<L>::R3 > 1 ? RdPlan<L>::R2 : 1)) % 4 == 0),
-                  "the order changes in the pass of single rows, whose butterflies are of one f mod 4");
+                                        (RdPlan<L>::R1 * (RdPlan<L>::R3 > 1 ? RdPlan<L>::R2 : 1)) % (N == 16 && KL == 16 ? 8 : 4) == 0),
+                  "the order changes in the pass of single rows, whose butterflies are of one f mod 4 (8)");
     static_assert(MODE != RD_SPLIT || (DIF && DIR < 0), "the split is the first forward pass");
     static_assert(MODE != RD_MERGE || (!DIF && DIR > 0), "the recombination is the last inverse pass");
     const int n = tid % N;
@@ -101,7 +101,7 @@ __device__ __forceinline__ void rd_pass(float2 *XA, float2 *XB, const float2 *tw
         const int c = rest / S, j = rest - c * S;
         float2 *Xa = (half ? XB : XA) + (c * LS + j) * N + n;  // row m of the butterfly: Xa[m S N]
         float2 *Xb = XB + (c * LS + j) * N + n;                // the same row of the odd half
-        // the butterfly of the pass of single rows holds frequencies f1 + R1 f2 + 4 (..), c = f1 R2 + f2
+        // the butterfly of the pass of single rows holds frequencies f1 + R1 f2 + 4 (..) (8 (..)), c = f1 R2 + f2
         const int f4 = RdPlan<L>::R3 > 1 ? c / RdPlan<L>::R2 + RdPlan<L>::R1 * (c % RdPlan<L>::R2) : c;
         const int sw = ORDER == RD_PLAIN ? 0 : rd_swz<N, KL>(f4, n) - n;
         float2 p[R], q[PAIR ? R : 1];
