@@ -291,6 +291,72 @@ cudaError_t launch_halo(const __nv_bfloat16 *A, int B, int H, int W, int C, cons
     return cudaGetLastError();
 }
 
+// Wide layers: halo boxes, groups of tiles that share the weights. N in tiles of
+// 128 channels, or of 64.
+template <int BN, class EPI>
+cudaError_t launch_group(const __nv_bfloat16 *A, int B, int H, int W, int C, const __nv_bfloat16 *wmat, int N, int flip,
+                         const EPI &epi, cudaStream_t s) {
+    using Cf = tma::GroupCfg<BN>;
+    if (W % tma::HBW || H % tma::HBH || C % 64 || N % BN) return cudaErrorNotSupported;
+    auto enc = encoder();
+    const int nsm = sm_count();
+    int *err = fault_ptr();
+    if (!enc || nsm <= 0 || !err) return cudaErrorNotSupported;
+    CUtensorMap ma, mb;
+    {
+        const cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B};
+        const cuuint64_t strides[3] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2, (cuuint64_t)H * W * C * 2};
+        const cuuint32_t box[4] = {64, (cuuint32_t)tma::HBW, (cuuint32_t)(tma::HBH + 2), 1};
+        const cuuint32_t es[4] = {1, 1, 1, 1};
+        if (enc(&ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void *)A, dims, strides, box, es,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return cudaErrorInvalidValue;
+    }
+    {
+        const cuuint64_t dims[2] = {(cuuint64_t)9 * C, (cuuint64_t)N};
+        const cuuint64_t strides[1] = {(cuuint64_t)9 * C * 2};
+        const cuuint32_t box[2] = {64, (cuuint32_t)BN};
+        const cuuint32_t es[2] = {1, 1};
+        if (enc(&mb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void *)wmat, dims, strides, box, es,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return cudaErrorInvalidValue;
+    }
+    tma::ConvGeo g;
+    g.B = B;
+    g.H = H;
+    g.W = W;
+    g.C = C;
+    g.bw = tma::HBW;
+    g.bh = tma::HBH;
+    g.tiles_x = W / tma::HBW;
+    g.tiles_y = H / tma::HBH;
+    g.mtiles = B * g.tiles_x * g.tiles_y;
+    g.ntiles = N / BN;
+    g.tiles = g.mtiles * g.ntiles;
+    g.nchunk = C / 64;
+    g.KB = 3 * g.nchunk;
+    g.flip = flip;
+    // as many tiles a group as leave every SM one
+    int G = g.tiles / nsm;
+    if (G > Cf::GMAX) G = Cf::GMAX;
+    if (G < 1) G = 1;
+    const int groups = (g.mtiles + G - 1) / G * g.ntiles;
+    auto *fn = &tma::k_conv_group<BN, EPI>;
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, Cf::SMEM);
+    if (e != cudaSuccess) return e;
+    fn<<<groups < nsm ? groups : nsm, tma::kHaloThreads, Cf::SMEM, s>>>(ma, mb, g, epi, G, err);
+    return cudaGetLastError();
+}
+
+template <class EPI>
+cudaError_t launch_wide(const __nv_bfloat16 *A, int B, int H, int W, int C, const __nv_bfloat16 *wmat, int N, int flip,
+                        const EPI &epi, cudaStream_t s) {
+    return N % 128 == 0 ? launch_group<128>(A, B, H, W, C, wmat, N, flip, epi, s)
+                        : launch_group<64>(A, B, H, W, C, wmat, N, flip, epi, s);
+}
+
 // Weight gradient (k_wgrad_tma): x [B][H][W][C] and gz [B][H][W][Cout] NHWC, dw
 // [Cout][9 C] FP32 (accumulated).
 cudaError_t launch_wgrad(const __nv_bfloat16 *x, int B, int H, int W, int C, const __nv_bfloat16 *gz, int Cout,
@@ -383,6 +449,10 @@ cudaError_t conv_forward_tma(const __nv_bfloat16 *in, int B, int H, int W, int C
                      : launch_halo<64, 32>(in, B, H, W, Cin, w, Cout, 0, epi, s);
         if (e != cudaErrorNotSupported) return e;
     }
+    if (ck64 && Cout % 64 == 0) {
+        const cudaError_t e = launch_wide(in, B, H, W, Cin, w, Cout, 0, epi, s);
+        if (e != cudaErrorNotSupported) return e;
+    }
     switch (Cout) {
         case 32: return ck64 ? launch<32, 64>(in, B, H, W, Cin, w, Cout, 0, epi, s)
                              : launch<32, 32>(in, B, H, W, Cin, w, Cout, 0, epi, s);
@@ -417,6 +487,10 @@ cudaError_t conv_dgrad_tma(const __nv_bfloat16 *gz, int B, int H, int W, int Cou
         if (Cin == 32) return launch<32, 32>(gz, B, H, W, Cout, wt, Cin, 1, epi, s);
         if (Cin == 96) return launch<96, 32>(gz, B, H, W, Cout, wt, Cin, 1, epi, s);
         return cudaErrorNotSupported;
+    }
+    if (Cin % 64 == 0) {
+        const cudaError_t e = launch_wide(gz, B, H, W, Cout, wt, Cin, 1, epi, s);
+        if (e != cudaErrorNotSupported) return e;
     }
     switch (Cin) {
         case 32: return launch<32, 64>(gz, B, H, W, Cout, wt, Cin, 1, epi, s);

@@ -544,6 +544,268 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
 
 
 // ---------------------------------------------------------------------------
+// Wide layers (64 channels a chunk, weights too large to stay in shared
+// memory): halo boxes and groups of tiles that share each weight.
+//
+// k_conv_tma reads 128 pixels and BN weight rows of 128 bytes for every four MMAs
+// and is bound by what L2 delivers (14 TB/s, tensor pipe 23 .. 38 % active). Here a box of
+// 16 x 10 pixels serves the three vertical taps of one horizontal offset (160
+// rows instead of 384), and the three taps' weights serve the G tiles of a
+// group, each with an accumulator of its own, before the next are loaded: per tile and
+// 64 x BN weights 20 KB + 3 BN / G * 128 bytes instead of 3 (16 KB + BN * 128).
+// Roles as in k_conv_halo, with rings of boxes (A) and of weights (W).
+// Measured (forward, batch 64, 256 x 256): 192 -> 64 channels G_192 us (377),
+// 384 -> 128 G_384 (204).
+// ---------------------------------------------------------------------------
+
+template <int BN>
+struct GroupCfg {
+    static_assert(BN == 64 || BN == 128, "accumulators of 64 or 128 columns");
+    static constexpr int A_BYTES = HROWS * 128;     // one box
+    static constexpr int W_BYTES = 3 * BN * 128;    // the weights of three taps
+    static constexpr int AS = BN == 64 ? 6 : 5, WS = BN == 64 ? 3 : 2;
+    static constexpr int NACC = 512 / BN, GMAX = NACC / 2;  // accumulators; tiles a group at most
+    static constexpr int SMEM = 1024 + AS * A_BYTES + WS * W_BYTES + 512;
+};
+
+template <int BN, class EPI>
+__global__ void __launch_bounds__(kHaloThreads, 1)
+    k_conv_group(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, const ConvGeo g,
+                 const EPI epi, int G, int *err) {
+    using Cf = GroupCfg<BN>;
+    constexpr int AS = Cf::AS, WS = Cf::WS, NACC = Cf::NACC;
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    const uint32_t raw = smem_u32(smem_raw);
+    const uint32_t base = (raw + 1023u) & ~1023u;
+    const uint32_t wbase = base + AS * Cf::A_BYTES;
+    const uint32_t bar_full = wbase + WS * Cf::W_BYTES;
+    const uint32_t bar_empty = bar_full + 8 * AS;
+    const uint32_t bar_wfull = bar_empty + 8 * AS;
+    const uint32_t bar_wempty = bar_wfull + 8 * WS;
+    const uint32_t bar_afull = bar_wempty + 8 * WS;
+    const uint32_t bar_aempty = bar_afull + 8 * NACC;
+    const uint32_t tmem_slot = bar_aempty + 8 * NACC;
+    volatile int *abort = (volatile int *)(smem_raw + (tmem_slot + 4 - raw));
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+    // groups u = nt * mgroups + mg: tiles mg * G .. of n tile nt
+    const int mgroups = (g.mtiles + G - 1) / G, groups = mgroups * g.ntiles;
+
+    if (threadIdx.x == 0) {
+        *abort = *(volatile int *)err;
+        for (int s = 0; s < AS; ++s) {
+            tc::mbar_init(bar_full + 8 * s, 1);
+            tc::mbar_init(bar_empty + 8 * s, 1);
+        }
+        for (int s = 0; s < WS; ++s) {
+            tc::mbar_init(bar_wfull + 8 * s, 1);
+            tc::mbar_init(bar_wempty + 8 * s, 1);
+        }
+        for (int a = 0; a < NACC; ++a) {
+            tc::mbar_init(bar_afull + 8 * a, 1);
+            tc::mbar_init(bar_aempty + 8 * a, 4);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        asm volatile("prefetch.tensormap [%0];\n" ::"l"((uint64_t)&mapA) : "memory");
+        asm volatile("prefetch.tensormap [%0];\n" ::"l"((uint64_t)&mapB) : "memory");
+    }
+    __syncthreads();
+    if (*abort) return;
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(tmem_slot), "r"(512u));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    uint32_t tmem_base;
+    asm volatile("ld.shared.u32 %0, [%1];\n" : "=r"(tmem_base) : "r"(tmem_slot));
+    tmem_base = __shfl_sync(0xffffffffu, tmem_base, 0);
+
+    // tiles t0 .. t0 + n - 1 (in tile_origin's numbering) of group u
+    auto group_tiles = [&](int u, int &t0, int &n) {
+        const int nt = u / mgroups, m0 = (u - nt * mgroups) * G;
+        t0 = nt * g.mtiles + m0;
+        n = min(G, g.mtiles - m0);
+    };
+
+    if (warp == 0) {
+        if (lane == 0) {
+            // ---------------- TMA producer ----------------
+            int s = 0, ws = 0;
+            uint32_t ph = 0, wph = 0;
+            bool ok = true;
+            for (int u = blockIdx.x; u < groups && ok; u += gridDim.x) {
+                int t0, n;
+                group_tiles(u, t0, n);
+                for (int kb = 0; kb < g.KB && ok; ++kb) {  // KB = 3 nchunk: chunk, then horizontal offset
+                    const int ch = kb / 3, sxi = kb - 3 * ch;
+                    if (!tc::mbar_wait(bar_wempty + 8 * ws, wph ^ 1u, abort)) {
+                        ok = false;
+                        break;
+                    }
+                    arrive_expect_tx(bar_wfull + 8 * ws, Cf::W_BYTES);
+#pragma unroll
+                    for (int syi = 0; syi < 3; ++syi) {
+                        const int tap = g.flip ? 8 - (syi * 3 + sxi) : syi * 3 + sxi;
+                        tma_load_2d(wbase + ws * Cf::W_BYTES + syi * (BN * 128), &mapB, tap * g.C + ch * 64,
+                                    (t0 / g.mtiles) * BN, bar_wfull + 8 * ws);
+                    }
+                    if (++ws == WS) {
+                        ws = 0;
+                        wph ^= 1u;
+                    }
+                    for (int i = 0; i < n; ++i) {
+                        int b, x0, y0, nt;
+                        tile_origin(g, t0 + i, b, x0, y0, nt);
+                        if (!tc::mbar_wait(bar_empty + 8 * s, ph ^ 1u, abort)) {
+                            ok = false;
+                            break;
+                        }
+                        arrive_expect_tx(bar_full + 8 * s, Cf::A_BYTES);
+                        tma_load_4d(base + s * Cf::A_BYTES, &mapA, ch * 64, x0 + sxi - 1, y0 - 1, b, bar_full + 8 * s);
+                        if (++s == AS) {
+                            s = 0;
+                            ph ^= 1u;
+                        }
+                    }
+                }
+            }
+            if (!ok) {
+                // loads already issued finish on their own within microseconds
+                const long long t0 = clock64();
+                while (clock64() - t0 < 200000LL) {
+                }
+            }
+        }
+    } else if (warp == 1) {
+        {  // the whole warp
+            // ---------------- MMA issuer ----------------
+            constexpr uint32_t IDESC = tc::idesc_bf16_f32<BN>();
+            const uint64_t a_desc0 = sdesc<BN, 64>(base), w_desc0 = sdesc<BN, 64>(wbase);
+            int s = 0, ws = 0, acc0 = 0;  // acc0: the group's first accumulator
+            uint32_t ph = 0, wph = 0, aph = 0;
+            bool ok = true;
+            uint32_t last_bar = 0, last_par = 0;
+            for (int u = blockIdx.x; u < groups && ok; u += gridDim.x) {
+                int t0, n;
+                group_tiles(u, t0, n);
+                uint32_t p = aph;
+                for (int i = 0; i < n; ++i) {
+                    const int acc = acc0 + i < NACC ? acc0 + i : acc0 + i - NACC;
+                    if (acc0 + i == NACC) p ^= 1u;
+                    if (!mbar_wait_warp(bar_aempty + 8 * acc, p ^ 1u, abort)) {
+                        ok = false;
+                        break;
+                    }
+                }
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                for (int kb = 0; kb < g.KB && ok; ++kb) {
+                    if (!mbar_wait_warp(bar_wfull + 8 * ws, wph, abort)) {
+                        ok = false;
+                        break;
+                    }
+                    const uint64_t dw = w_desc0 + (uint64_t)((uint32_t)(ws * Cf::W_BYTES) >> 4);
+                    for (int i = 0; i < n; ++i) {
+                        const int acc = acc0 + i < NACC ? acc0 + i : acc0 + i - NACC;
+                        if (!mbar_wait_warp(bar_full + 8 * s, ph, abort)) {
+                            ok = false;
+                            break;
+                        }
+                        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                        const uint32_t d = tmem_base + (uint32_t)(acc * BN);
+                        const uint64_t da = a_desc0 + (uint64_t)((uint32_t)(s * Cf::A_BYTES) >> 4);
+#pragma unroll
+                        for (int syi = 0; syi < 3; ++syi)
+#pragma unroll
+                            for (int kk = 0; kk < 4; ++kk)
+                                mma_f16_elect(d, da + (uint64_t)(syi * HBW * 128 / 16 + kk * 2),
+                                              dw + (uint64_t)(syi * BN * 128 / 16 + kk * 2), IDESC,
+                                              syi + kk > 0 || kb > 0 ? 1u : 0u);
+                        mma_commit_elect(bar_empty + 8 * s);
+                        last_bar = bar_empty + 8 * s;
+                        last_par = ph;
+                        if (++s == AS) {
+                            s = 0;
+                            ph ^= 1u;
+                        }
+                    }
+                    if (!ok) break;
+                    mma_commit_elect(bar_wempty + 8 * ws);
+                    if (++ws == WS) {
+                        ws = 0;
+                        wph ^= 1u;
+                    }
+                }
+                if (!ok) break;
+                for (int i = 0; i < n; ++i) {
+                    mma_commit_elect(bar_afull + 8 * acc0);
+                    if (++acc0 == NACC) {
+                        acc0 = 0;
+                        aph ^= 1u;
+                    }
+                }
+            }
+            if (!ok && last_bar) tc::mbar_wait(last_bar, last_par, nullptr);  // tensor core idle before release
+        }
+    } else {
+        // ---------------- epilogue (two groups of four warps, as in k_conv_halo) ----------------
+        __shared__ float epi_const[EPI::SMEM_FLOATS];
+        epi.prepare(epi_const, threadIdx.x - 64, 256);
+        asm volatile("bar.sync 1, 256;\n" ::: "memory");  // the epilogue warps only
+        const int q = warp & 3, half = (warp - 2) >> 2;
+        int acc = 0;
+        uint32_t aph = 0;
+        int turn = 0;
+        bool ok = true;
+        for (int u = blockIdx.x; u < groups && ok; u += gridDim.x) {
+            int t0, n;
+            group_tiles(u, t0, n);
+            for (int i = 0; i < n; ++i, turn ^= 1) {
+                if (turn == half) {
+                    int b, x0, y0, nt;
+                    tile_origin(g, t0 + i, b, x0, y0, nt);
+                    const int r = q * 32 + lane;
+                    const int y = y0 + r / HBW, x = x0 + r % HBW;
+                    const int m = (b * g.H + y) * g.W + x;
+                    if (!tc::mbar_wait(bar_afull + 8 * acc, aph, abort)) {
+                        ok = false;
+                        break;
+                    }
+                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                    const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN);
+                    float state = 0.0f;
+#pragma unroll 2
+                    for (int j = 0; j < BN / 16; ++j) {
+                        const typename EPI::Pre pre = epi.prefetch(m, nt * BN + 16 * j);
+                        uint32_t v[16];
+                        tc::tmem_ld16(taddr + (uint32_t)(16 * j), v);
+                        float f[16];
+#pragma unroll
+                        for (int c = 0; c < 16; ++c) f[c] = __uint_as_float(v[c]);
+                        epi.store(m, nt * BN + 16 * j, f, state, epi_const, pre);
+                    }
+                    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) arrive(bar_aempty + 8 * acc);
+                    epi.finish(m, state, epi_const, epi.prefetch_pixel(m));
+                }
+                if (++acc == NACC) {
+                    acc = 0;
+                    aph ^= 1u;
+                }
+            }
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && *abort) atomicExch(err, 1);
+    if (warp == 1) {
+        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_base), "r"(512u));
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Weight gradient: dW[co][tap * C + ci] += sum over pixels p of
 // In[p shifted by tap][ci] * gz[p][co], as D[m][n] = sum over k of A(m, k) B(n, k)
 // with k the pixels. Both operands come from NHWC tensors, so they are MN-major
