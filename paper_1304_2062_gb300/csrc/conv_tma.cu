@@ -35,10 +35,18 @@ __device__ __forceinline__ void store16(__nv_bfloat16 *dst, const float (&w)[16]
 
 // out[m][n..n+15] = relu?(v + bias) as bf16; pixel m's channels at out + m * N;
 // nb bias values (the output channels).
+// pool: also the 2x2 averages of the bf16 outputs (sums in the order of k_pool); a
+// warp has to hold 16 x 2 pixels then (k_conv_halo, k_conv_group). It saves the
+// kernel that read the output again: 120 us for the three poolings at 64 images of
+// 256 x 256, for about 40 of a longer epilogue. The upsampling in the same way (four
+// stores for one) took as long here as in its own kernel, which is bound by
+// writing.
 struct FwdEpi {
     const float *bias;
     __nv_bfloat16 *out;
     int N, relu, nb;
+    __nv_bfloat16 *pool = nullptr;
+    int W = 1;
     static constexpr int SMEM_FLOATS = 256;
     __device__ __forceinline__ void prepare(float *sm, int i, int n) const {
         for (int k = i; k < nb; k += n) sm[k] = bias[k];
@@ -48,13 +56,49 @@ struct FwdEpi {
     __device__ __forceinline__ Pre prefetch(int, int) const { return {}; }
     __device__ __forceinline__ PrePix prefetch_pixel(int) const { return {}; }
     __device__ __forceinline__ void store(int m, int n, const float (&v)[16], float &, const float *sm, Pre) const {
-        float w[16];
+        uint32_t p[8];
 #pragma unroll
-        for (int q = 0; q < 16; ++q) {
-            w[q] = v[q] + sm[n + q];
-            if (relu) w[q] = fmaxf(w[q], 0.0f);
+        for (int q = 0; q < 8; ++q) {
+            float a = v[2 * q] + sm[n + 2 * q], b = v[2 * q + 1] + sm[n + 2 * q + 1];
+            if (relu) {
+                a = fmaxf(a, 0.0f);
+                b = fmaxf(b, 0.0f);
+            }
+            p[q] = pack2(a, b);
         }
-        store16(out + (long long)m * N + n, w);
+        uint4 *d4 = (uint4 *)(out + (long long)m * N + n);
+        d4[0] = make_uint4(p[0], p[1], p[2], p[3]);
+        d4[1] = make_uint4(p[4], p[5], p[6], p[7]);
+        if (pool) {
+            // the 2 x 2 pixels are lanes l, l ^ 1, l ^ 16, l ^ 17: each gets four of the 16
+            // channels of all of them, in two exchanges
+            const int lane = threadIdx.x & 31;
+            const bool odd = lane & 1, hi = lane >> 4;
+            uint32_t pa[4], pb[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const uint32_t mine = odd ? p[4 + k] : p[k];
+                const uint32_t oth = __shfl_xor_sync(0xffffffffu, odd ? p[k] : p[4 + k], 1);
+                pa[k] = odd ? oth : mine;
+                pb[k] = odd ? mine : oth;
+            }
+            uint32_t o[2];
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const uint32_t ma = hi ? pa[2 + k] : pa[k], mb = hi ? pb[2 + k] : pb[k];
+                const uint32_t oa = __shfl_xor_sync(0xffffffffu, hi ? pa[k] : pa[2 + k], 16);
+                const uint32_t ob = __shfl_xor_sync(0xffffffffu, hi ? pb[k] : pb[2 + k], 16);
+                const uint32_t a = hi ? oa : ma, b = hi ? ob : mb, c = hi ? ma : oa, d = hi ? mb : ob;
+                const float s0 = __uint_as_float(a << 16) + __uint_as_float(b << 16) + __uint_as_float(c << 16) +
+                                 __uint_as_float(d << 16);
+                const float s1 = __uint_as_float(a & 0xffff0000u) + __uint_as_float(b & 0xffff0000u) +
+                                 __uint_as_float(c & 0xffff0000u) + __uint_as_float(d & 0xffff0000u);
+                o[k] = pack2(0.25f * s0, 0.25f * s1);
+            }
+            const int row = m / W;
+            const long long px = (long long)(row >> 1) * (W >> 1) + ((m - row * W) >> 1);
+            *(uint2 *)(pool + px * nb + n + (odd ? 8 : 0) + (hi ? 4 : 0)) = make_uint2(o[0], o[1]);
+        }
     }
     __device__ __forceinline__ void finish(int, float, const float *, PrePix) const {}
 };
@@ -427,7 +471,7 @@ cudaError_t tma_fault(int *host_flag, bool reset) {
 
 cudaError_t conv_forward_tma(const __nv_bfloat16 *in, int B, int H, int W, int Cin, const __nv_bfloat16 *w,
                              const float *bias, int Cout, int relu, __nv_bfloat16 *out, int ldo, const HeadArgs *head,
-                             cudaStream_t s) {
+                             cudaStream_t s, __nv_bfloat16 *pool, bool *pooled) {
     const bool ck64 = Cin % 64 == 0;
     if (head) {
         if (Cout != 32 || !relu || ldo != 32) return cudaErrorNotSupported;
@@ -438,21 +482,24 @@ cudaError_t conv_forward_tma(const __nv_bfloat16 *in, int B, int H, int W, int C
         return ck64 ? launch<32, 64>(in, B, H, W, Cin, w, Cout, 0, epi, s)
                     : launch<32, 32>(in, B, H, W, Cin, w, Cout, 0, epi, s);
     }
+    // the kernels with 16 x 8 tiles write the averages too
+    FwdEpi fepi{bias, out, ldo, relu, Cout};
+    fepi.pool = pool;
+    fepi.W = W;
+    cudaError_t e = cudaErrorNotSupported;
+    if (Cout == 32)
+        e = ck64 ? launch_halo<32, 64>(in, B, H, W, Cin, w, Cout, 0, fepi, s)
+                 : launch_halo<32, 32>(in, B, H, W, Cin, w, Cout, 0, fepi, s);
+    else if (Cout == 64)
+        e = ck64 ? launch_halo<64, 64>(in, B, H, W, Cin, w, Cout, 0, fepi, s)
+                 : launch_halo<64, 32>(in, B, H, W, Cin, w, Cout, 0, fepi, s);
+    if (e == cudaErrorNotSupported && ck64 && Cout % 64 == 0)
+        e = launch_wide(in, B, H, W, Cin, w, Cout, 0, fepi, s);
+    if (e != cudaErrorNotSupported) {
+        if (pooled) *pooled = pool != nullptr;
+        return e;
+    }
     const FwdEpi epi{bias, out, ldo, relu, Cout};
-    if (Cout == 32 || Cout == 64) {
-        cudaError_t e;
-        if (Cout == 32)
-            e = ck64 ? launch_halo<32, 64>(in, B, H, W, Cin, w, Cout, 0, epi, s)
-                     : launch_halo<32, 32>(in, B, H, W, Cin, w, Cout, 0, epi, s);
-        else
-            e = ck64 ? launch_halo<64, 64>(in, B, H, W, Cin, w, Cout, 0, epi, s)
-                     : launch_halo<64, 32>(in, B, H, W, Cin, w, Cout, 0, epi, s);
-        if (e != cudaErrorNotSupported) return e;
-    }
-    if (ck64 && Cout % 64 == 0) {
-        const cudaError_t e = launch_wide(in, B, H, W, Cin, w, Cout, 0, epi, s);
-        if (e != cudaErrorNotSupported) return e;
-    }
     switch (Cout) {
         case 32: return ck64 ? launch<32, 64>(in, B, H, W, Cin, w, Cout, 0, epi, s)
                              : launch<32, 32>(in, B, H, W, Cin, w, Cout, 0, epi, s);

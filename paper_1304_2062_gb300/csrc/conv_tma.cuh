@@ -554,8 +554,8 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
 // group, each with an accumulator of its own, before the next are loaded: per tile and
 // 64 x BN weights 20 KB + 3 BN / G * 128 bytes instead of 3 (16 KB + BN * 128).
 // Roles as in k_conv_halo, with rings of boxes (A) and of weights (W).
-// Measured (forward, batch 64, 256 x 256): 192 -> 64 channels G_192 us (377),
-// 384 -> 128 G_384 (204).
+// Measured (forward, batch 64, 256 x 256): 192 -> 64 channels 202 us (377),
+// 384 -> 128 147 (204).
 // ---------------------------------------------------------------------------
 
 template <int BN>

@@ -34,25 +34,6 @@ struct WeightNLoader {
     }
 };
 
-// A operand of backward weight: dOut[pix][co], M(=co)-major.
-struct GradOutMLoader {
-    const __nv_bfloat16 *g;
-    int Cout, P;  // P = number of pixels (the GEMM's K)
-    __device__ __forceinline__ const void *chunk(int k, int m) const {
-        return (k < P && m < Cout) ? (const void *)(g + (long long)k * Cout + m) : nullptr;
-    }
-};
-
-// B operand of backward weight: B(k = pixel, n = tap*Cin + ci) = In[shift(pixel, tap)][ci].
-struct InNLoader {
-    ConvInLoader in;  // flip = 0; chunk(m = pixel, k = n) gives the gathered input
-    int P;
-    __device__ __forceinline__ const void *chunk(int k, int n) const {
-        if (k >= P) return nullptr;
-        return in.chunk(k, n);
-    }
-};
-
 template <int BM, int BN, bool AK, bool BK_, class LA, class LB>
 __device__ __forceinline__ void run_tile(const LA &la, const LB &lb, int m0, int n0, int kt0, int kt1,
                                          float (&acc)[BM / 32][BN / 16][4]) {
@@ -120,30 +101,6 @@ __global__ void __launch_bounds__(128) k_conv_dgrad(ConvInLoader la, WeightNLoad
                     const int c2 = Cin - split;
                     *(__nv_bfloat162 *)(din2 + (long long)m * c2 + (n - split)) = __floats2bfloat162_rn(v0, v1);
                 }
-            }
-}
-
-// Backward weight (split K over pixels): dW[co][tap*Cin+ci] += sum dZ * In.
-template <int BM, int BN>
-__global__ void __launch_bounds__(128) k_conv_wgrad(GradOutMLoader la, InNLoader lb, float *dw, int N, int ktiles_per) {
-    float acc[BM / 32][BN / 16][4];
-    const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
-    const int kt_total = (lb.P + kBK - 1) / kBK;
-    const int kt0 = blockIdx.z * ktiles_per;
-    const int kt1 = min(kt_total, kt0 + ktiles_per);
-    run_tile<BM, BN, false, false>(la, lb, m0, n0, kt0, kt1, acc);
-    if (kt1 <= kt0) return;
-#pragma unroll
-    for (int i = 0; i < BM / 32; ++i)
-#pragma unroll
-        for (int j = 0; j < BN / 16; ++j)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                int m, n;
-                acc_pos<BM, BN>(i, j, q, m, n);
-                m += m0;
-                n += n0;
-                if (m < la.Cout && n < N) atomicAdd(dw + (long long)m * N + n, acc[i][j][q]);
             }
 }
 
@@ -322,24 +279,38 @@ __global__ void k_upsample_into(const __nv_bfloat16 *lo, int C1, __nv_bfloat16 *
 
 // First convolution straight from the image: the input channels are
 // bf16(f m) and m (the other six are zero), so each of the 32 outputs is a
-// sum over 9 taps x 2 channels, done in FP32 on the CUDA cores. A block
-// takes 32 x 8 pixel tiles; the tile and its 1-pixel halo of (bf16(f m), m)
-// are staged in shared memory with coalesced loads, and the weights sit
-// there as [tap][channel][4 outputs] float4 (one 16-byte load per 4 FMAs).
-constexpr int C0_TW = 32, C0_TH = 8;
+// sum over 9 taps x 2 channels. What should bound it is writing the outputs, 64
+// bytes a pixel; 576 multiply-adds a pixel on the CUDA cores took four times as
+// long (202 us for 64 images of 256 x 256; 168 packed and two pixels a thread; 75 now),
+// mostly for the weights' way out of shared memory and for stores of 16 bytes per
+// 64. As matrix products of 16 pixels by 18 (padded to 32) by 32 the weights stay in
+// registers and 8 MMAs do a warp's 16 pixels; a contraction this short gains nothing
+// from tensor memory, so they are warp-level ones (BF16 in, FP32 sums).
+// A block takes 32 x 16 pixel tiles; the tile and its 1-pixel halo of (bf16(f m), m)
+// pairs are staged in shared memory with coalesced loads. K = 2 tap + channel, so a
+// pair is what a lane's A registers hold two of k of: register k pair t (+ 4) of
+// pixel g is tap t (+ 4). Column 2 t + e of n tile j is output 8 t + 2 j + e: a lane
+// ends up with 8 neighbouring outputs of two pixels, and a warp's store is 512
+// contiguous bytes.
+constexpr int C0_TW = 32, C0_TH = 16;
 __global__ void __launch_bounds__(256) k_conv0(const float *f, const uint8_t *mask, const __nv_bfloat16 *w,
                                                const float *bias, __nv_bfloat16 *out, int B, int H, int W) {
-    __shared__ float4 sw[9][2][8];
-    __shared__ float sb[32];
-    __shared__ float2 tile[C0_TH + 2][C0_TW + 2];
-    for (int i = threadIdx.x; i < 9 * 2 * 8; i += blockDim.x) {
-        const int tap = i / 16, ci = (i / 8) % 2, q = i % 8;
-        const __nv_bfloat16 *wq = w + tap * 8 + ci;  // w[co][tap][ci], 72 per output channel
-        sw[tap][ci][q] = make_float4(__bfloat162float(wq[(4 * q + 0) * 72]), __bfloat162float(wq[(4 * q + 1) * 72]),
-                                     __bfloat162float(wq[(4 * q + 2) * 72]), __bfloat162float(wq[(4 * q + 3) * 72]));
+    __shared__ uint32_t tile[C0_TH + 2][C0_TW + 2];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int g = lane >> 2, t4 = lane & 3;
+    // B(k, n): column n = g of n tile j is output 8 (g / 2) + 2 j + g % 2; w[co][tap][ci], 8
+    // channels a tap
+    uint32_t bw[4][3];
+    float bs[8];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const uint32_t *wq = (const uint32_t *)(w + (8 * (g >> 1) + 2 * j + (g & 1)) * 72);
+        bw[j][0] = wq[t4 * 4];
+        bw[j][1] = wq[(t4 + 4) * 4];
+        bw[j][2] = t4 == 0 ? wq[8 * 4] : 0u;
     }
-    if (threadIdx.x < 32) sb[threadIdx.x] = bias[threadIdx.x];
-    const int tx = threadIdx.x % C0_TW, ty = threadIdx.x / C0_TW;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) bs[c] = bias[8 * t4 + c];
     const int ntx = (W + C0_TW - 1) / C0_TW, nty = (H + C0_TH - 1) / C0_TH;
     const long long ntiles = (long long)B * ntx * nty;
     for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
@@ -348,42 +319,52 @@ __global__ void __launch_bounds__(256) k_conv0(const float *f, const uint8_t *ma
         const int by = (int)(r % nty);
         const long long b = r / nty;
         const int x0 = bx * C0_TW, y0 = by * C0_TH;
-        __syncthreads();  // the previous tile is consumed (and the tables are ready)
+        __syncthreads();  // the previous tile is consumed
         for (int i = threadIdx.x; i < (C0_TH + 2) * (C0_TW + 2); i += blockDim.x) {
             const int ly = i / (C0_TW + 2), lx = i % (C0_TW + 2);
             const int yy = y0 + ly - 1, xx = x0 + lx - 1;
-            float2 v = make_float2(0.0f, 0.0f);
+            uint32_t v = 0;
             if (yy >= 0 && yy < H && xx >= 0 && xx < W) {
                 const long long q = (b * H + yy) * W + xx;
                 const float m = mask[q] ? 1.0f : 0.0f;
-                v = make_float2(__bfloat162float(__float2bfloat16_rn(f[q] * m)), m);
+                const __nv_bfloat162 h = __floats2bfloat162_rn(f[q] * m, m);
+                v = *(const uint32_t *)&h;
             }
             tile[ly][lx] = v;
         }
         __syncthreads();
-        const int x = x0 + tx, y = y0 + ty;
-        if (x >= W || y >= H) continue;
-        float acc[32];
 #pragma unroll
-        for (int co = 0; co < 32; ++co) acc[co] = 0.0f;
+        for (int i = 0; i < 4; ++i) {
+            const int ly = warp * 2 + (i >> 1), lx = (i & 1) * 16 + g;
+            const int y = y0 + ly;
+            // taps t4, t4 + 4 (and 8) of pixels lx and lx + 8
+            const uint32_t *p0 = &tile[ly + t4 / 3][lx + t4 % 3];
+            const uint32_t *p1 = &tile[ly + (t4 + 4) / 3][lx + (t4 + 4) % 3];
+            const uint32_t a0[4] = {p0[0], p0[8], p1[0], p1[8]};
+            const uint32_t *p2 = &tile[ly + 2][lx + 2];
+            const uint32_t a1[4] = {t4 == 0 ? p2[0] : 0u, t4 == 0 ? p2[8] : 0u, 0u, 0u};
+            float d[4][4];
 #pragma unroll
-        for (int tap = 0; tap < 9; ++tap) {
-            const float2 v = tile[ty + tap / 3][tx + tap % 3];
+            for (int j = 0; j < 4; ++j) {
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const float4 a = sw[tap][0][q], c = sw[tap][1][q];
-                acc[4 * q + 0] = fmaf(c.x, v.y, fmaf(a.x, v.x, acc[4 * q + 0]));
-                acc[4 * q + 1] = fmaf(c.y, v.y, fmaf(a.y, v.x, acc[4 * q + 1]));
-                acc[4 * q + 2] = fmaf(c.z, v.y, fmaf(a.z, v.x, acc[4 * q + 2]));
-                acc[4 * q + 3] = fmaf(c.w, v.y, fmaf(a.w, v.x, acc[4 * q + 3]));
+                for (int k = 0; k < 4; ++k) d[j][k] = 0.0f;
+                mma_bf16(d[j], a0, bw[j][0], bw[j][1]);
+                mma_bf16(d[j], a1, bw[j][2], 0u);
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int x = x0 + lx + 8 * h;
+                if (x >= W || y >= H) continue;
+                uint32_t o[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const __nv_bfloat162 v = __floats2bfloat162_rn(fmaxf(d[j][2 * h] + bs[2 * j], 0.0f),
+                                                                   fmaxf(d[j][2 * h + 1] + bs[2 * j + 1], 0.0f));
+                    o[j] = *(const uint32_t *)&v;
+                }
+                *(uint4 *)(out + ((b * H + y) * W + x) * 32 + 8 * t4) = make_uint4(o[0], o[1], o[2], o[3]);
             }
         }
-        __align__(16) __nv_bfloat16 o[32];
-#pragma unroll
-        for (int co = 0; co < 32; ++co) o[co] = __float2bfloat16_rn(fmaxf(acc[co] + sb[co], 0.0f));
-        uint4 *dst = (uint4 *)(out + ((b * H + y) * W + x) * 32);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) dst[k] = ((const uint4 *)o)[k];
     }
 }
 
@@ -604,18 +585,6 @@ cudaError_t launch_dgrad(const ConvInLoader &la, const WeightNLoader &lb, const 
     return cudaGetLastError();
 }
 
-template <int BM, int BN>
-cudaError_t launch_wgrad(const GradOutMLoader &la, const InNLoader &lb, float *dw, int N, int splits, cudaStream_t s) {
-    using S = Smem<BM, BN, false, false>;
-    auto *fn = &k_conv_wgrad<BM, BN>;
-    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, S::BYTES);
-    const int kt_total = (lb.P + kBK - 1) / kBK;
-    const int per = (kt_total + splits - 1) / splits;
-    dim3 grid((la.Cout + BM - 1) / BM, (N + BN - 1) / BN, (kt_total + per - 1) / per);
-    fn<<<grid, 128, S::BYTES, s>>>(la, lb, dw, N, per);
-    return cudaGetLastError();
-}
-
 template <int BN, int STAGES, int LAG>
 cudaError_t launch_fwd_tc(const ConvInLoader &la, const WeightKLoader &lb, const FwdEpi &epi, cudaStream_t s) {
     constexpr int bytes = tc::smem_bytes<BN, STAGES>();
@@ -655,9 +624,11 @@ cudaError_t tc_fault(int *host_flag, bool reset) {
 
 cudaError_t conv_forward(const __nv_bfloat16 *in, const __nv_bfloat16 *lo, int C1, int B, int H, int W, int Cin,
                          const __nv_bfloat16 *w, const float *bias, int Cout, int relu, __nv_bfloat16 *out, int ldo,
-                         cudaStream_t s) {
+                         cudaStream_t s, __nv_bfloat16 *pool, bool *pooled) {
+    if (pooled) *pooled = false;
     if (!lo) {
-        const cudaError_t e = conv_forward_tma(in, B, H, W, Cin, w, bias, Cout, relu, out, ldo, nullptr, s);
+        const cudaError_t e =
+            conv_forward_tma(in, B, H, W, Cin, w, bias, Cout, relu, out, ldo, nullptr, s, pool, pooled);
         if (e != cudaErrorNotSupported) return e;
     }
     ConvInLoader la{{B, H, W}, in, lo, Cin, C1, B * H * W, 9 * Cin, 0};
@@ -702,27 +673,6 @@ cudaError_t conv_backward_data(const __nv_bfloat16 *gz, int B, int H, int W, int
     if (Cin <= 32) return launch_dgrad<128, 32>(la, lb, act, din, din2, split, s);
     if (Cin <= 64) return launch_dgrad<128, 64>(la, lb, act, din, din2, split, s);
     return launch_dgrad<128, 128>(la, lb, act, din, din2, split, s);
-}
-
-cudaError_t conv_backward_weight(const __nv_bfloat16 *gz, int B, int H, int W, int Cout, const __nv_bfloat16 *in,
-                                 const __nv_bfloat16 *lo, int C1, int Cin, float *dw, cudaStream_t s) {
-    if (!lo) {
-        const cudaError_t e = conv_wgrad_tma(in, B, H, W, Cin, gz, Cout, dw, s);
-        if (e != cudaErrorNotSupported) return e;
-    }
-    const int P = B * H * W;
-    GradOutMLoader la{gz, Cout, P};
-    InNLoader lb{{{B, H, W}, in, lo, Cin, C1, P, 9 * Cin, 0}, P};
-    const int N = 9 * Cin;
-    const int kt_total = (P + kBK - 1) / kBK;
-    // enough CTAs to fill the GPU, each reducing a slab of pixels
-    const int tiles = ((Cout + 63) / 64) * ((N + 63) / 64);
-    int splits = (4 * 152 + tiles - 1) / tiles;
-    if (splits > kt_total) splits = kt_total;
-    if (splits < 1) splits = 1;
-    if (Cout <= 32) return launch_wgrad<32, 64>(la, lb, dw, N, splits, s);
-    if (Cout <= 64) return launch_wgrad<64, 64>(la, lb, dw, N, splits, s);
-    return launch_wgrad<128, 64>(la, lb, dw, N, splits, s);
 }
 
 cudaError_t colsum(const __nv_bfloat16 *g, long long P, int C, float *db, cudaStream_t s) {

@@ -12,9 +12,11 @@ namespace nn {
 // or, when lo != null, the channel concatenation [nearest-upsample(lo) (C1
 // channels, half resolution), in (Cin - C1 channels)]. out = relu?(conv + bias),
 // pixel p's Cout channels at out + p * ldo (ldo >= Cout, a multiple of 8).
+// pool: also the 2x2 averages of the output, dense, where the kernel that takes the
+// shape can; *pooled says whether.
 cudaError_t conv_forward(const __nv_bfloat16 *in, const __nv_bfloat16 *lo, int C1, int B, int H, int W, int Cin,
                          const __nv_bfloat16 *w, const float *bias, int Cout, int relu, __nv_bfloat16 *out, int ldo,
-                         cudaStream_t s);
+                         cudaStream_t s, __nv_bfloat16 *pool = nullptr, bool *pooled = nullptr);
 // Gradient w.r.t. the input from the pre-activation gradient gz [P][Cout];
 // channels < split go to din (multiplied by act > 0 when act != null),
 // channels >= split to din2. wt_scratch (Cout*9*Cin elements) receives the
@@ -38,7 +40,7 @@ struct HeadArgs {
 // multiples of 32), and the caller uses the general kernels.
 cudaError_t conv_forward_tma(const __nv_bfloat16 *in, int B, int H, int W, int Cin, const __nv_bfloat16 *w,
                              const float *bias, int Cout, int relu, __nv_bfloat16 *out, int ldo, const HeadArgs *head,
-                             cudaStream_t s);
+                             cudaStream_t s, __nv_bfloat16 *pool = nullptr, bool *pooled = nullptr);
 cudaError_t conv_dgrad_tma(const __nv_bfloat16 *gz, int B, int H, int W, int Cout, const __nv_bfloat16 *wt, int Cin,
                            const __nv_bfloat16 *act, __nv_bfloat16 *din, __nv_bfloat16 *din2, int split,
                            cudaStream_t s);
@@ -55,9 +57,6 @@ cudaError_t upsample_into(const __nv_bfloat16 *lo, int C1, __nv_bfloat16 *out, i
 // with w the layer's bf16 weights [32][9][8] (input channels 0 and 1 used).
 cudaError_t conv0_direct(const float *f, const uint8_t *mask, const __nv_bfloat16 *w, const float *bias,
                          __nv_bfloat16 *out, int B, int H, int W, cudaStream_t s);
-// dw[Cout][9*Cin] += weight gradient (FP32, atomically accumulated).
-cudaError_t conv_backward_weight(const __nv_bfloat16 *gz, int B, int H, int W, int Cout, const __nv_bfloat16 *in,
-                                 const __nv_bfloat16 *lo, int C1, int Cin, float *dw, cudaStream_t s);
 cudaError_t colsum(const __nv_bfloat16 *g, long long P, int C, float *db, cudaStream_t s);
 cudaError_t pack_input(const float *f, const uint8_t *mask, __nv_bfloat16 *x, long long P, cudaStream_t s);
 // in: C channels per pixel at in + p * ldi; out dense (C per pixel).

@@ -83,10 +83,6 @@ se2n_status check_tc() {
     return f ? SE2N_ECUDA : SE2N_OK;
 }
 
-long long level_pixels(const se2n_unet *u, int count, int level) {
-    return (long long)count * (u->H >> level) * (u->W >> level);
-}
-
 bool dev_ptr(const void *p, size_t align) {
     if (!p || ((uintptr_t)p % align) != 0) return false;
     cudaPointerAttributes attr;
@@ -105,6 +101,7 @@ se2n_status forward(se2n_unet *u, const float *f, const uint8_t *mask, int n, bo
     const int H = u->H, W = u->W;
     auto Wt = [&](int l) { return u->pb + u->w_off[l]; };
     auto Bi = [&](int l) { return u->p + u->b_off[l]; };
+    bool pooled = false;  // the last convolution has written its output's 2x2 averages as well
     for (int l = 0; l < 4; ++l) {
         const int Hl = H >> l, Wl = W >> l;
         const LayerSpec &A = kLayers[2 * l], &Bb = kLayers[2 * l + 1];
@@ -112,13 +109,15 @@ se2n_status forward(se2n_unet *u, const float *f, const uint8_t *mask, int n, bo
             // the first layer reads the image and mask directly (2 meaningful input channels)
             TRYC(conv0_direct(f, mask, Wt(0), Bi(0), u->a[0], n, H, W, s));
         } else {
-            TRYC(pool(u->e[l - 1], u->e_ld[l - 1], u->pl[l], n, H >> (l - 1), W >> (l - 1), kLayers[2 * l - 1].cout, s));
+            if (!pooled)
+                TRYC(pool(u->e[l - 1], u->e_ld[l - 1], u->pl[l], n, H >> (l - 1), W >> (l - 1), kLayers[2 * l - 1].cout,
+                          s));
             TRYC(conv_forward(u->pl[l], nullptr, 0, n, Hl, Wl, A.cin, Wt(2 * l), Bi(2 * l), A.cout, 1, u->a[l], A.cout,
                               s));
         }
         // e[l] (l < 3) is written straight into the skip channels of decoder level l's input
         TRYC(conv_forward(u->a[l], nullptr, 0, n, Hl, Wl, Bb.cin, Wt(2 * l + 1), Bi(2 * l + 1), Bb.cout, 1, u->e[l],
-                          u->e_ld[l], s));
+                          u->e_ld[l], s, l < 3 ? u->pl[l + 1] : nullptr, &pooled));
     }
     // decoder levels 2, 1, 0 (layer indices 8..13)
     const __nv_bfloat16 *below = u->e[3];
@@ -166,13 +165,13 @@ se2n_status backward(se2n_unet *u, const float *f, const uint8_t *mask, int n) {
         const int la = 8 + 2 * k, lb = 9 + 2 * k;
         const LayerSpec &A = kLayers[la], &Bb = kLayers[lb];
         const int Hl = H >> level, Wl = W >> level;
-        const long long P = level_pixels(u, n, level);
+        const long long P = (long long)n * Hl * Wl;
         // second conv: c[k] -> d[k]
-        TRYC(conv_backward_weight(u->gd[k], n, Hl, Wl, Bb.cout, u->c[k], nullptr, 0, Bb.cin, dW(lb), s));
+        TRYC(conv_wgrad_tma(u->c[k], n, Hl, Wl, Bb.cin, u->gd[k], Bb.cout, dW(lb), s));
         TRYC(colsum(u->gd[k], P, Bb.cout, dB(lb), s));
         TRYC(conv_backward_data(u->gd[k], n, Hl, Wl, Bb.cout, Wt(lb), Bb.cin, u->c[k], u->gc[k], nullptr, Bb.cin, u->wt, s));
         // first conv: [up(below), e[level]] -> c[k]
-        TRYC(conv_backward_weight(u->gc[k], n, Hl, Wl, A.cout, u->cat[k], nullptr, 0, A.cin, dW(la), s));
+        TRYC(conv_wgrad_tma(u->cat[k], n, Hl, Wl, A.cin, u->gc[k], A.cout, dW(la), s));
         TRYC(colsum(u->gc[k], P, A.cout, dB(la), s));
         TRYC(conv_backward_data(u->gc[k], n, Hl, Wl, A.cout, Wt(la), A.cin, nullptr, u->gup[k], u->gskip[k],
                                 A.lo_ch, u->wt, s));
@@ -186,7 +185,7 @@ se2n_status backward(se2n_unet *u, const float *f, const uint8_t *mask, int n) {
     // encoder, from the bottleneck down: gradient into e[l] is ge[l]
     for (int l = 3; l >= 0; --l) {
         const int Hl = H >> l, Wl = W >> l;
-        const long long P = level_pixels(u, n, l);
+        const long long P = (long long)n * Hl * Wl;
         const LayerSpec &A = kLayers[2 * l], &Bb = kLayers[2 * l + 1];
         if (l < 3) {
             // e[l] feeds the pool of level l+1 (gradient gp[l+1]) and the skip of decoder level l
@@ -194,11 +193,11 @@ se2n_status backward(se2n_unet *u, const float *f, const uint8_t *mask, int n) {
                                         Bb.cout, s));
         }
         const __nv_bfloat16 *in = (l == 0) ? u->x0 : u->pl[l];
-        TRYC(conv_backward_weight(u->ge[l], n, Hl, Wl, Bb.cout, u->a[l], nullptr, 0, Bb.cin, dW(2 * l + 1), s));
+        TRYC(conv_wgrad_tma(u->a[l], n, Hl, Wl, Bb.cin, u->ge[l], Bb.cout, dW(2 * l + 1), s));
         TRYC(colsum(u->ge[l], P, Bb.cout, dB(2 * l + 1), s));
         TRYC(conv_backward_data(u->ge[l], n, Hl, Wl, Bb.cout, Wt(2 * l + 1), Bb.cin, u->a[l], u->ga[l], nullptr,
                                 Bb.cin, u->wt, s));
-        TRYC(conv_backward_weight(u->ga[l], n, Hl, Wl, A.cout, in, nullptr, 0, A.cin, dW(2 * l), s));
+        TRYC(conv_wgrad_tma(in, n, Hl, Wl, A.cin, u->ga[l], A.cout, dW(2 * l), s));
         TRYC(colsum(u->ga[l], P, A.cout, dB(2 * l), s));
         if (l > 0) {
             TRYC(conv_backward_data(u->ga[l], n, Hl, Wl, A.cout, Wt(2 * l), A.cin, nullptr, u->gp[l], nullptr, A.cin, u->wt, s));
