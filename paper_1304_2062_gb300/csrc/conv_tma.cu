@@ -36,7 +36,7 @@ __device__ __forceinline__ void store16(__nv_bfloat16 *dst, const float (&w)[16]
 // out[m][n..n+15] = relu?(v + bias) as bf16; pixel m's channels at out + m * N;
 // nb bias values (the output channels).
 // pool: also the 2x2 averages of the bf16 outputs (sums in the order of k_pool); a
-// warp has to hold 16 x 2 pixels then (k_conv_halo, k_conv_group). It saves the
+// warp has to hold 8 x 4 pixels then (k_conv_halo, k_conv_group). It saves the
 // kernel that read the output again: 120 us for the three poolings at 64 images of
 // 256 x 256, for about 40 of a longer epilogue. The upsampling in the same way (four
 // stores for one) took as long here as in its own kernel, which is bound by
@@ -55,8 +55,9 @@ struct FwdEpi {
     struct PrePix {};
     __device__ __forceinline__ Pre prefetch(int, int) const { return {}; }
     __device__ __forceinline__ PrePix prefetch_pixel(int) const { return {}; }
-    __device__ __forceinline__ void store(int m, int n, const float (&v)[16], float &, const float *sm, Pre) const {
-        uint32_t p[8];
+    // the 16 outputs as bf16, stored
+    __device__ __forceinline__ void pack(int m, int n, const float (&v)[16], const float *sm, bool valid,
+                                         uint32_t (&p)[8]) const {
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
             float a = v[2 * q] + sm[n + 2 * q], b = v[2 * q + 1] + sm[n + 2 * q + 1];
@@ -66,39 +67,68 @@ struct FwdEpi {
             }
             p[q] = pack2(a, b);
         }
-        uint4 *d4 = (uint4 *)(out + (long long)m * N + n);
-        d4[0] = make_uint4(p[0], p[1], p[2], p[3]);
-        d4[1] = make_uint4(p[4], p[5], p[6], p[7]);
-        if (pool) {
-            // the 2 x 2 pixels are lanes l, l ^ 1, l ^ 16, l ^ 17: each gets four of the 16
-            // channels of all of them, in two exchanges
-            const int lane = threadIdx.x & 31;
-            const bool odd = lane & 1, hi = lane >> 4;
-            uint32_t pa[4], pb[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const uint32_t mine = odd ? p[4 + k] : p[k];
-                const uint32_t oth = __shfl_xor_sync(0xffffffffu, odd ? p[k] : p[4 + k], 1);
-                pa[k] = odd ? oth : mine;
-                pb[k] = odd ? mine : oth;
-            }
-            uint32_t o[2];
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                const uint32_t ma = hi ? pa[2 + k] : pa[k], mb = hi ? pb[2 + k] : pb[k];
-                const uint32_t oa = __shfl_xor_sync(0xffffffffu, hi ? pa[k] : pa[2 + k], 16);
-                const uint32_t ob = __shfl_xor_sync(0xffffffffu, hi ? pb[k] : pb[2 + k], 16);
-                const uint32_t a = hi ? oa : ma, b = hi ? ob : mb, c = hi ? ma : oa, d = hi ? mb : ob;
-                const float s0 = __uint_as_float(a << 16) + __uint_as_float(b << 16) + __uint_as_float(c << 16) +
-                                 __uint_as_float(d << 16);
-                const float s1 = __uint_as_float(a & 0xffff0000u) + __uint_as_float(b & 0xffff0000u) +
-                                 __uint_as_float(c & 0xffff0000u) + __uint_as_float(d & 0xffff0000u);
-                o[k] = pack2(0.25f * s0, 0.25f * s1);
-            }
-            const int row = m / W;
-            const long long px = (long long)(row >> 1) * (W >> 1) + ((m - row * W) >> 1);
-            *(uint2 *)(pool + px * nb + n + (odd ? 8 : 0) + (hi ? 4 : 0)) = make_uint2(o[0], o[1]);
+        if (valid) {
+            uint4 *d4 = (uint4 *)(out + (long long)m * N + n);
+            d4[0] = make_uint4(p[0], p[1], p[2], p[3]);
+            d4[1] = make_uint4(p[4], p[5], p[6], p[7]);
         }
+    }
+    // average of two channels of four pixels
+    static __device__ __forceinline__ uint32_t mean(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+        const float s0 = __uint_as_float(a << 16) + __uint_as_float(b << 16) + __uint_as_float(c << 16) +
+                         __uint_as_float(d << 16);
+        const float s1 = __uint_as_float(a & 0xffff0000u) + __uint_as_float(b & 0xffff0000u) +
+                         __uint_as_float(c & 0xffff0000u) + __uint_as_float(d & 0xffff0000u);
+        return pack2(0.25f * s0, 0.25f * s1);
+    }
+    __device__ __forceinline__ __nv_bfloat16 *pool_at(int m) const {
+        const int row = m / W;
+        return pool + ((long long)(row >> 1) * (W >> 1) + ((m - row * W) >> 1)) * nb;
+    }
+    __device__ __forceinline__ void store(int m, int n, const float (&v)[16], float &, const float *sm, Pre,
+                                          bool valid) const {
+        uint32_t p[8];
+        pack(m, n, v, sm, valid, p);
+        if (!pool) return;
+        // the 2 x 2 pixels are lanes l, l ^ 1, l ^ 8, l ^ 9: each gets four of the 16
+        // channels of all of them, in two exchanges
+        const int lane = threadIdx.x & 31;
+        const bool odd = lane & 1, hi = lane & 8;
+        uint32_t pa[4], pb[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t mine = odd ? p[4 + k] : p[k];
+            const uint32_t oth = __shfl_xor_sync(0xffffffffu, odd ? p[k] : p[4 + k], 1);
+            pa[k] = odd ? oth : mine;
+            pb[k] = odd ? mine : oth;
+        }
+        uint32_t o[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const uint32_t ma = hi ? pa[2 + k] : pa[k], mb = hi ? pb[2 + k] : pb[k];
+            const uint32_t oa = __shfl_xor_sync(0xffffffffu, hi ? pa[k] : pa[2 + k], 8);
+            const uint32_t ob = __shfl_xor_sync(0xffffffffu, hi ? pb[k] : pb[2 + k], 8);
+            o[k] = mean(hi ? oa : ma, hi ? ob : mb, hi ? ma : oa, hi ? mb : ob);
+        }
+        if (valid) *(uint2 *)(pool_at(m) + n + (odd ? 8 : 0) + (hi ? 4 : 0)) = make_uint2(o[0], o[1]);
+    }
+    __device__ __forceinline__ void store_pair(int m, int n, const float (&v)[2][16], float (&)[2], const float *sm, Pre,
+                                               Pre, bool valid) const {
+        uint32_t p[8], r[8];
+        pack(m, n, v[0], sm, valid, p);
+        pack(m + 1, n, v[1], sm, valid, r);
+        if (!pool) return;
+        // the other two pixels are lane l ^ 8's: each lane gets half of the channels
+        const bool hi = threadIdx.x & 8;
+        uint32_t o[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t ma = hi ? p[4 + k] : p[k], mb = hi ? r[4 + k] : r[k];
+            const uint32_t oa = __shfl_xor_sync(0xffffffffu, hi ? p[k] : p[4 + k], 8);
+            const uint32_t ob = __shfl_xor_sync(0xffffffffu, hi ? r[k] : r[4 + k], 8);
+            o[k] = mean(hi ? oa : ma, hi ? ob : mb, hi ? ma : oa, hi ? mb : ob);
+        }
+        if (valid) *(uint4 *)(pool_at(m) + n + (hi ? 8 : 0)) = make_uint4(o[0], o[1], o[2], o[3]);
     }
     __device__ __forceinline__ void finish(int, float, const float *, PrePix) const {}
 };
@@ -124,7 +154,7 @@ struct HeadEpi {
     };
     __device__ __forceinline__ Pre prefetch(int, int) const { return {}; }
     __device__ __forceinline__ PrePix prefetch_pixel(int m) const { return {f[m], mask[m]}; }
-    __device__ __forceinline__ void store(int m, int n, const float (&v)[16], float &st, const float *sm, Pre) const {
+    __device__ __forceinline__ void store(int m, int n, const float (&v)[16], float &st, const float *sm, Pre, bool valid) const {
         float w[16];
         if (n == 0) st = sm[64];
 #pragma unroll
@@ -133,7 +163,12 @@ struct HeadEpi {
             w[q] = __bfloat162float(__float2bfloat16_rn(w[q]));
             st = fmaf(sm[32 + n + q], w[q], st);
         }
-        if (out) store16(out + (long long)m * 32 + n, w);
+        if (out && valid) store16(out + (long long)m * 32 + n, w);
+    }
+    __device__ __forceinline__ void store_pair(int m, int n, const float (&v)[2][16], float (&st)[2], const float *sm,
+                                               const Pre &p, const Pre &p1, bool valid) const {
+        store(m, n, v[0], st[0], sm, p, valid);
+        store(m + 1, n, v[1], st[1], sm, p1, valid);
     }
     __device__ __forceinline__ void finish(int m, float st, const float *, PrePix p) const {
         y[m] = (p.mask ? p.f : 0.0f) + st;
@@ -162,7 +197,8 @@ struct DgradEpi {
         return p;
     }
     __device__ __forceinline__ PrePix prefetch_pixel(int) const { return {}; }
-    __device__ __forceinline__ void store(int m, int n, const float (&v)[16], float &, const float *, const Pre &p) const {
+    __device__ __forceinline__ void store(int m, int n, const float (&v)[16], float &, const float *, const Pre &p,
+                                          bool valid) const {
         float w[16];
 #pragma unroll
         for (int q = 0; q < 16; ++q) w[q] = v[q];
@@ -176,10 +212,15 @@ struct DgradEpi {
                     if (!(__bfloat162float(h.y) > 0.0f)) w[2 * q + 1] = 0.0f;
                 }
             }
-            store16(din + (long long)m * split + n, w);
-        } else {
+            if (valid) store16(din + (long long)m * split + n, w);
+        } else if (valid) {
             store16(din2 + (long long)m * (N - split) + (n - split), w);
         }
+    }
+    __device__ __forceinline__ void store_pair(int m, int n, const float (&v)[2][16], float (&st)[2], const float *sm,
+                                               const Pre &p, const Pre &p1, bool valid) const {
+        store(m, n, v[0], st[0], sm, p, valid);
+        store(m + 1, n, v[1], st[1], sm, p1, valid);
     }
     __device__ __forceinline__ void finish(int, float, const float *, PrePix) const {}
 };
@@ -272,16 +313,23 @@ cudaError_t launch(const __nv_bfloat16 *A, int B, int H, int W, int C, const __n
     return cudaGetLastError();
 }
 
-// Narrow layers: 16 x 8 tiles, halo boxes, weights resident in shared memory.
+// Whether the kernels with 8 x 16 tiles take an image: at most half of the tiles'
+// pixels outside it.
+bool box_shape(int H, int W) {
+    const long long px = (long long)((W + tma::HBW - 1) / tma::HBW * tma::HBW) * ((H + tma::HBH - 1) / tma::HBH * tma::HBH);
+    return px <= 2LL * W * H;
+}
+
+// Narrow layers: 8 x 16 tiles, halo boxes, weights resident in shared memory.
 template <int BN, int CK, class EPI>
 cudaError_t launch_halo(const __nv_bfloat16 *A, int B, int H, int W, int C, const __nv_bfloat16 *wmat, int N, int flip,
                         const EPI &epi, cudaStream_t s) {
     using Cf = tma::HaloCfg<BN, CK>;
-    if (W % tma::HBW || H % tma::HBH || C % CK || N % BN) return cudaErrorNotSupported;
+    if (!box_shape(H, W) || C % CK || N % BN) return cudaErrorNotSupported;
     const int nblk = 9 * (C / CK);
     const int wbytes = nblk * Cf::BBLK;
     int S = (Cf::SMEM_BUDGET - wbytes) / Cf::STAGE;
-    if (S > 4) S = 4;
+    if (S > 8) S = 8;
     if (S < 2) return cudaErrorNotSupported;
     auto enc = encoder();
     const int nsm = sm_count();
@@ -291,7 +339,7 @@ cudaError_t launch_halo(const __nv_bfloat16 *A, int B, int H, int W, int C, cons
     {
         const cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B};
         const cuuint64_t strides[3] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2, (cuuint64_t)H * W * C * 2};
-        const cuuint32_t box[4] = {(cuuint32_t)CK, (cuuint32_t)tma::HBW, (cuuint32_t)(tma::HBH + 2), 1};
+        const cuuint32_t box[4] = {(cuuint32_t)CK, (cuuint32_t)tma::HPITCH, (cuuint32_t)(tma::HBH + 2), 1};
         const cuuint32_t es[4] = {1, 1, 1, 1};
         if (enc(&ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void *)A, dims, strides, box, es,
                 CU_TENSOR_MAP_INTERLEAVE_NONE, CK == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
@@ -315,8 +363,8 @@ cudaError_t launch_halo(const __nv_bfloat16 *A, int B, int H, int W, int C, cons
     g.C = C;
     g.bw = tma::HBW;
     g.bh = tma::HBH;
-    g.tiles_x = W / tma::HBW;
-    g.tiles_y = H / tma::HBH;
+    g.tiles_x = (W + tma::HBW - 1) / tma::HBW;
+    g.tiles_y = (H + tma::HBH - 1) / tma::HBH;
     g.mtiles = B * g.tiles_x * g.tiles_y;
     g.ntiles = N / BN;
     g.tiles = g.mtiles * g.ntiles;
@@ -335,13 +383,72 @@ cudaError_t launch_halo(const __nv_bfloat16 *A, int B, int H, int W, int C, cons
     return cudaGetLastError();
 }
 
+// 32 output channels: pairs of pixels (W even), halo boxes, weights resident in shared memory.
+template <class EPI>
+cudaError_t launch_pair(const __nv_bfloat16 *A, int B, int H, int W, int C, const __nv_bfloat16 *wmat, int flip,
+                        const EPI &epi, cudaStream_t s) {
+    using Cf = tma::PairCfg;
+    if (W % 2 || !box_shape(H, W / 2) || C % 32) return cudaErrorNotSupported;
+    const int nblk = 9 * (C / 32);
+    const int wbytes = nblk * Cf::BBLK;
+    int S = (Cf::SMEM_BUDGET - wbytes) / Cf::STAGE;
+    if (S > 8) S = 8;
+    if (S < 2) return cudaErrorNotSupported;
+    auto enc = encoder();
+    const int nsm = sm_count();
+    int *err = fault_ptr();
+    if (!enc || nsm <= 0 || !err) return cudaErrorNotSupported;
+    tma::ConvGeo g;
+    g.B = B;
+    g.H = H;
+    g.W = W / 2;  // columns of two pixels
+    g.C = C;
+    g.bw = tma::HBW;
+    g.bh = tma::HBH;
+    g.tiles_x = (g.W + tma::HBW - 1) / tma::HBW;
+    g.tiles_y = (H + tma::HBH - 1) / tma::HBH;
+    g.mtiles = B * g.tiles_x * g.tiles_y;
+    g.ntiles = 1;
+    g.tiles = g.mtiles;
+    g.nchunk = C / 32;
+    g.KB = g.nchunk;
+    g.flip = flip;
+    CUtensorMap ma, mb;
+    {
+        const cuuint64_t dims[4] = {(cuuint64_t)2 * C, (cuuint64_t)g.W, (cuuint64_t)H, (cuuint64_t)B};
+        const cuuint64_t strides[3] = {(cuuint64_t)C * 4, (cuuint64_t)W * C * 2, (cuuint64_t)H * W * C * 2};
+        const cuuint32_t box[4] = {32, (cuuint32_t)tma::HPITCH, (cuuint32_t)(tma::HBH + 2), 1};
+        const cuuint32_t es[4] = {1, 1, 1, 1};
+        if (enc(&ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void *)A, dims, strides, box, es,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return cudaErrorInvalidValue;
+    }
+    {
+        const cuuint64_t dims[2] = {(cuuint64_t)9 * C, 32};
+        const cuuint64_t strides[1] = {(cuuint64_t)9 * C * 2};
+        const cuuint32_t box[2] = {32, 32};
+        const cuuint32_t es[2] = {1, 1};
+        if (enc(&mb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void *)wmat, dims, strides, box, es,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return cudaErrorInvalidValue;
+    }
+    const int smem = 1024 + wbytes + S * Cf::STAGE + 256;
+    auto *fn = &tma::k_conv_pair<EPI>;
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    fn<<<g.mtiles < nsm ? g.mtiles : nsm, tma::kHaloThreads, smem, s>>>(ma, mb, g, epi, S, err);
+    return cudaGetLastError();
+}
+
 // Wide layers: halo boxes, groups of tiles that share the weights. N in tiles of
 // 128 channels, or of 64.
 template <int BN, class EPI>
 cudaError_t launch_group(const __nv_bfloat16 *A, int B, int H, int W, int C, const __nv_bfloat16 *wmat, int N, int flip,
                          const EPI &epi, cudaStream_t s) {
     using Cf = tma::GroupCfg<BN>;
-    if (W % tma::HBW || H % tma::HBH || C % 64 || N % BN) return cudaErrorNotSupported;
+    if (!box_shape(H, W) || C % 64 || N % BN) return cudaErrorNotSupported;
     auto enc = encoder();
     const int nsm = sm_count();
     int *err = fault_ptr();
@@ -350,7 +457,7 @@ cudaError_t launch_group(const __nv_bfloat16 *A, int B, int H, int W, int C, con
     {
         const cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B};
         const cuuint64_t strides[3] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2, (cuuint64_t)H * W * C * 2};
-        const cuuint32_t box[4] = {64, (cuuint32_t)tma::HBW, (cuuint32_t)(tma::HBH + 2), 1};
+        const cuuint32_t box[4] = {64, (cuuint32_t)tma::HPITCH, (cuuint32_t)(tma::HBH + 2), 1};
         const cuuint32_t es[4] = {1, 1, 1, 1};
         if (enc(&ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void *)A, dims, strides, box, es,
                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -374,8 +481,8 @@ cudaError_t launch_group(const __nv_bfloat16 *A, int B, int H, int W, int C, con
     g.C = C;
     g.bw = tma::HBW;
     g.bh = tma::HBH;
-    g.tiles_x = W / tma::HBW;
-    g.tiles_y = H / tma::HBH;
+    g.tiles_x = (W + tma::HBW - 1) / tma::HBW;
+    g.tiles_y = (H + tma::HBH - 1) / tma::HBH;
     g.mtiles = B * g.tiles_x * g.tiles_y;
     g.ntiles = N / BN;
     g.tiles = g.mtiles * g.ntiles;
@@ -476,20 +583,18 @@ cudaError_t conv_forward_tma(const __nv_bfloat16 *in, int B, int H, int W, int C
     if (head) {
         if (Cout != 32 || !relu || ldo != 32) return cudaErrorNotSupported;
         const HeadEpi epi{bias, out, head->hw, head->hb, head->f, head->mask, head->y};
-        cudaError_t e = ck64 ? launch_halo<32, 64>(in, B, H, W, Cin, w, Cout, 0, epi, s)
-                             : launch_halo<32, 32>(in, B, H, W, Cin, w, Cout, 0, epi, s);
+        const cudaError_t e = launch_pair(in, B, H, W, Cin, w, 0, epi, s);
         if (e != cudaErrorNotSupported) return e;
         return ck64 ? launch<32, 64>(in, B, H, W, Cin, w, Cout, 0, epi, s)
                     : launch<32, 32>(in, B, H, W, Cin, w, Cout, 0, epi, s);
     }
-    // the kernels with 16 x 8 tiles write the averages too
+    // the kernels with 8 x 16 tiles write the averages too
     FwdEpi fepi{bias, out, ldo, relu, Cout};
     fepi.pool = pool;
     fepi.W = W;
     cudaError_t e = cudaErrorNotSupported;
     if (Cout == 32)
-        e = ck64 ? launch_halo<32, 64>(in, B, H, W, Cin, w, Cout, 0, fepi, s)
-                 : launch_halo<32, 32>(in, B, H, W, Cin, w, Cout, 0, fepi, s);
+        e = launch_pair(in, B, H, W, Cin, w, 0, fepi, s);
     else if (Cout == 64)
         e = ck64 ? launch_halo<64, 64>(in, B, H, W, Cin, w, Cout, 0, fepi, s)
                  : launch_halo<64, 32>(in, B, H, W, Cin, w, Cout, 0, fepi, s);
@@ -521,8 +626,7 @@ cudaError_t conv_dgrad_tma(const __nv_bfloat16 *gz, int B, int H, int W, int Cou
     if (Cin == 32 || Cin == 64 || Cin == 96) {
         cudaError_t e = cudaErrorNotSupported;
         if (Cin == 32)
-            e = ck64 ? launch_halo<32, 64>(gz, B, H, W, Cout, wt, Cin, 1, epi, s)
-                     : launch_halo<32, 32>(gz, B, H, W, Cout, wt, Cin, 1, epi, s);
+            e = launch_pair(gz, B, H, W, Cout, wt, 1, epi, s);
         else if (Cin == 64)
             e = ck64 ? launch_halo<64, 64>(gz, B, H, W, Cout, wt, Cin, 1, epi, s)
                      : launch_halo<64, 32>(gz, B, H, W, Cout, wt, Cin, 1, epi, s);

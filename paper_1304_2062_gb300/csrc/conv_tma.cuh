@@ -138,7 +138,10 @@ __device__ __forceinline__ void tile_origin(const ConvGeo &g, int t, int &b, int
 //   Pre, prefetch(m, n)               what store(m, n) reads from device memory (may be loaded
 //                                      before the accumulator is complete)
 //   PrePix, prefetch_pixel(m)         the same for finish(m)
-//   store(m, n, v[16], float &state, sm, pre)  the 16 outputs of pixel m, columns n..n+15
+//   store(m, n, v[16], float &state, sm, pre, valid)  the 16 outputs of pixel m, columns n..n+15;
+//                                      called by whole warps, of pixel 0 for lanes without one
+//   store_pair(m, n, v[2][16], float (&state)[2], sm, pre, pre1, valid)  the same of pixels m
+//                                      and m + 1 (k_conv_pair)
 //   finish(m, float state, sm, pre)   after the last column group of pixel m
 template <int BN, int CK, class EPI>
 __global__ void __launch_bounds__(192, 1)
@@ -291,7 +294,7 @@ __global__ void __launch_bounds__(192, 1)
                 float f[16];
 #pragma unroll
                 for (int i = 0; i < 16; ++i) f[i] = __uint_as_float(v[i]);
-                epi.store(m, nt * BN + j0, f, state, epi_const, epi.prefetch(m, nt * BN + j0));
+                epi.store(m, nt * BN + j0, f, state, epi_const, epi.prefetch(m, nt * BN + j0), true);
             }
             epi.finish(m, state, epi_const, epi.prefetch_pixel(m));
             asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
@@ -314,32 +317,47 @@ __global__ void __launch_bounds__(192, 1)
 
 
 // ---------------------------------------------------------------------------
-// Narrow layers (BN <= 64): halo boxes and resident weights.
+// Narrow layers (64 or 96 output channels): halo boxes and resident weights.
 //
-// Tiles are 16 x 8 pixels. For each channel block and each horizontal
-// offset sx in {-1, 0, 1} one TMA box brings the 16 x 10 pixels (rows
-// y0 - 1 .. y0 + 8) shifted by sx; the three vertical offsets sy are the
-// same box read from row (sy + 1) * 16, a whole number of swizzle atoms, so
-// one box feeds three taps (160 box rows instead of 3 x 128). All weights of
-// the layer (9 C x BN) are loaded into shared memory once per CTA, so the
-// K loop moves no weight rows at all.
+// Tiles are 8 x 16 pixels. For each channel block one TMA box brings the
+// 10 x 18 pixels around a tile, and each of the nine taps is the same box read from
+// pixel (sy + 1) * 10 + sx + 1 on: the operand's groups of eight rows are image rows,
+// one box row (10 pixels) apart, and the swizzle is a function of the shared-memory
+// address alone, so a group may start anywhere in a swizzle atom. 180 box rows feed
+// the nine taps; the TMA unit writes box rows at 2.7 cycles each, and a box a horizontal
+// offset makes 480 of them, one a tap 1152. (64 -> 64 channels, batch 64, 128 x 128: 76 us,
+// 86 with a box a horizontal offset.) All weights of the layer (9 C x BN) are loaded into shared memory
+// once per CTA, so the K loop moves no weight rows at all. Pixels of a tile outside the
+// image are computed and not stored.
 // ---------------------------------------------------------------------------
 
-constexpr int HBW = 16, HBH = 8;             // tile 16 x 8 pixels
-constexpr int HROWS = HBW * (HBH + 2);        // 160 box rows
+constexpr int HBW = 8, HBH = 16;              // tile 8 x 16 pixels
+constexpr int HPITCH = HBW + 2;               // pixels a box row
+constexpr int HROWS = HPITCH * (HBH + 2);     // 180 pixels a box
 constexpr int kHaloThreads = 320;             // producer, MMA issuer and eight epilogue warps
 
 template <int BN, int CK>
 struct HaloCfg {
     static_assert(BN % 16 == 0 && BN >= 16 && BN <= 128, "narrow layers");
     static constexpr int A_BYTES = HROWS * CK * 2;
-    static constexpr int STAGE = 3 * A_BYTES;  // the boxes of the three horizontal offsets
+    static constexpr int STAGE = (A_BYTES + 1023) / 1024 * 1024;
     static constexpr int BBLK = BN * CK * 2;   // one (tap, channel block) of weights
     static constexpr int ACC_COLS = BN <= 32 ? 32 : BN <= 64 ? 64 : 128;
     static constexpr int NACC = 4;             // accumulators
     static constexpr int TMEM_COLS = NACC * ACC_COLS;
     static constexpr int SMEM_BUDGET = 196608;
 };
+
+// Descriptor of a tile's pixels in a box: image rows HPITCH pixels apart.
+template <int CK>
+__device__ __forceinline__ uint64_t sdesc_box(uint32_t saddr) {
+    uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)(16u >> 4) << 16;
+    d |= (uint64_t)((uint32_t)(HPITCH * CK * 2) >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)(CK == 64 ? 2 : 4) << 61;
+    return d;
+}
 
 template <int BN, int CK, class EPI>
 __global__ void __launch_bounds__(kHaloThreads, 1)
@@ -415,11 +433,8 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
                         ok = false;
                         break;
                     }
-                    arrive_expect_tx(bar_full + 8 * s, Cf::STAGE);
-#pragma unroll
-                    for (int sxi = 0; sxi < 3; ++sxi)
-                        tma_load_4d(stages + s * Cf::STAGE + sxi * Cf::A_BYTES, &mapA, ch * CK, x0 + sxi - 1, y0 - 1, b,
-                                    bar_full + 8 * s);
+                    arrive_expect_tx(bar_full + 8 * s, Cf::A_BYTES);
+                    tma_load_4d(stages + s * Cf::STAGE, &mapA, ch * CK, x0 - 1, y0 - 1, b, bar_full + 8 * s);
                     if (++s == S) {
                         s = 0;
                         ph ^= 1u;
@@ -436,7 +451,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
         {  // the whole warp
             // ---------------- MMA issuer ----------------
             constexpr uint32_t IDESC = tc::idesc_bf16_f32<BN>();
-            const uint64_t a_desc0 = sdesc<BN, CK>(stages), w_desc0 = sdesc<BN, CK>(wres);
+            const uint64_t a_desc0 = sdesc_box<CK>(stages), w_desc0 = sdesc<BN, CK>(wres);
             const int wstep = (g.nchunk * Cf::BBLK) >> 4;  // weights of the next tap, in 16-byte units
             int s = 0, acc = 0;
             uint32_t ph = 0, aph = 0;
@@ -466,7 +481,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
                         for (int sxi = 0; sxi < 3; ++sxi) {
 #pragma unroll
                             for (int kk = 0; kk < CK / 16; ++kk)
-                                mma_f16_elect(d, da + (uint64_t)((sxi * Cf::A_BYTES + syi * HBW * CK * 2) / 16 + kk * 2),
+                                mma_f16_elect(d, da + (uint64_t)((syi * HPITCH + sxi) * CK * 2 / 16 + kk * 2),
                                             dw + (uint64_t)(kk * 2), IDESC,
                                             syi + sxi + kk > 0 || ch > 0 ? 1u : 0u);
                             dw += step;
@@ -504,7 +519,8 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
             tile_origin(g, t, b, x0, y0, nt);
             const int r = q * 32 + lane;
             const int y = y0 + r / HBW, x = x0 + r % HBW;
-            const int m = (b * g.H + y) * g.W + x;
+            const bool valid = x < g.W && y < g.H;
+            const int m = valid ? (b * g.H + y) * g.W + x : 0;
             typename EPI::Pre pre[BN / 16];
 #pragma unroll
             for (int j = 0; j < BN / 16; ++j) pre[j] = epi.prefetch(m, nt * BN + 16 * j);
@@ -520,12 +536,256 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
                 float f[16];
 #pragma unroll
                 for (int i = 0; i < 16; ++i) f[i] = __uint_as_float(v[i]);
-                epi.store(m, nt * BN + 16 * j, f, state, epi_const, pre[j]);
+                epi.store(m, nt * BN + 16 * j, f, state, epi_const, pre[j], valid);
             }
             asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
             __syncwarp();
             if (lane == 0) arrive(bar_aempty + 8 * acc);
-            epi.finish(m, state, epi_const, pp);
+            if (valid) epi.finish(m, state, epi_const, pp);
+            acc += 2;
+            if (acc >= Cf::NACC) {
+                acc = group;
+                aph ^= 1u;
+            }
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && *abort) atomicExch(err, 1);
+    if (warp == 1) {
+        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_base),
+                     "r"((uint32_t)Cf::TMEM_COLS));
+    }
+}
+
+
+// ---------------------------------------------------------------------------
+// Layers with 32 output channels: columns of two pixels.
+//
+// A matrix product of 128 rows, 16 channels and 32 columns takes as long as one of 64
+// columns (about 48 cycles: reading the pixels from shared memory), and that is what
+// bounds k_conv_halo there. So a row of the operand is a pair of pixels, the output
+// 2 x 32 columns. Of the pair itself, the even pixels' channels go into both outputs
+// (horizontal source offsets 0 and -1), so do the odd ones' (1 and 0): 64 columns
+// each, whose weights are neighbours when a row of taps is kept in the order 1, 0, -1.
+// The odd pixel of the pair before belongs to the even output alone, the even pixel of the
+// next to the odd one: 32 columns. 24 products a 32 channels and 256 pixels
+// instead of 36. The pixels of either parity are a box of their own (of the tensor as
+// W / 2 columns of 2 C channels).
+// Measured (forward, batch 64, 256 x 256): 32 -> 32 channels 153 us with the pooling (169),
+// 96 -> 32 224 (317), 32 -> 32 with the head 91 (137).
+// ---------------------------------------------------------------------------
+
+struct PairCfg {
+    static constexpr int A_BYTES = HROWS * 64;  // 32 channels of the pixels of one parity
+    static constexpr int A_SLOT = (A_BYTES + 1023) / 1024 * 1024;
+    static constexpr int STAGE = 2 * A_SLOT;
+    static constexpr int BBLK = 32 * 64;        // one (tap, channel block) of weights
+    static constexpr int ACC_COLS = 64, NACC = 4, TMEM_COLS = NACC * ACC_COLS;
+    static constexpr int SMEM_BUDGET = 196608;
+};
+
+template <class EPI>
+__global__ void __launch_bounds__(kHaloThreads, 1)
+    k_conv_pair(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, const ConvGeo g,
+                const EPI epi, int S, int *err) {
+    using Cf = PairCfg;
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    const uint32_t raw = smem_u32(smem_raw);
+    const uint32_t base = (raw + 1023u) & ~1023u;
+    const int nblk = 9 * g.nchunk;                       // resident weight blocks
+    const uint32_t wres = base;                          // nblk x BBLK
+    const uint32_t stages = wres + nblk * Cf::BBLK;      // S x STAGE
+    const uint32_t bar_w = stages + S * Cf::STAGE;
+    const uint32_t bar_full = bar_w + 8;
+    const uint32_t bar_empty = bar_full + 8 * S;
+    const uint32_t bar_afull = bar_empty + 8 * S;
+    const uint32_t bar_aempty = bar_afull + 8 * Cf::NACC;
+    const uint32_t tmem_slot = bar_aempty + 8 * Cf::NACC;
+    volatile int *abort = (volatile int *)(smem_raw + (tmem_slot + 4 - raw));
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+    const int first_tile = blockIdx.x, end_tile = g.mtiles, tile_step = gridDim.x;
+
+    if (threadIdx.x == 0) {
+        *abort = *(volatile int *)err;
+        tc::mbar_init(bar_w, 1);
+        for (int s = 0; s < S; ++s) {
+            tc::mbar_init(bar_full + 8 * s, 1);
+            tc::mbar_init(bar_empty + 8 * s, 1);
+        }
+        for (int a = 0; a < Cf::NACC; ++a) {
+            tc::mbar_init(bar_afull + 8 * a, 1);
+            tc::mbar_init(bar_aempty + 8 * a, 4);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        asm volatile("prefetch.tensormap [%0];\n" ::"l"((uint64_t)&mapA) : "memory");
+        asm volatile("prefetch.tensormap [%0];\n" ::"l"((uint64_t)&mapB) : "memory");
+    }
+    __syncthreads();
+    if (*abort) return;
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(tmem_slot),
+                     "r"((uint32_t)Cf::TMEM_COLS));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    uint32_t tmem_base;
+    asm volatile("ld.shared.u32 %0, [%1];\n" : "=r"(tmem_base) : "r"(tmem_slot));
+    tmem_base = __shfl_sync(0xffffffffu, tmem_base, 0);
+
+    if (warp == 0) {
+        if (lane == 0) {
+            // ---------------- TMA producer ----------------
+            arrive_expect_tx(bar_w, (uint32_t)(nblk * Cf::BBLK));
+            for (int i = 0; i < nblk; ++i) {
+                // block (syi, ch, j): the tap of source offset (syi - 1, 1 - j), mirrored when flip
+                const int j = i % 3, ch = i / 3 % g.nchunk, syi = i / (3 * g.nchunk);
+                const int tap = g.flip ? 8 - (syi * 3 + 2 - j) : syi * 3 + 2 - j;
+                tma_load_2d(wres + i * Cf::BBLK, &mapB, tap * g.C + ch * 32, 0, bar_w);
+            }
+            int s = 0;
+            uint32_t ph = 0;
+            bool ok = true;
+            for (int t = first_tile; t < end_tile && ok; t += tile_step) {
+                int b, x0, y0, nt;
+                tile_origin(g, t, b, x0, y0, nt);
+                for (int ch = 0; ch < g.nchunk; ++ch) {
+                    if (!tc::mbar_wait(bar_empty + 8 * s, ph ^ 1u, abort)) {
+                        ok = false;
+                        break;
+                    }
+                    arrive_expect_tx(bar_full + 8 * s, 2 * Cf::A_BYTES);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        tma_load_4d(stages + s * Cf::STAGE + h * Cf::A_SLOT, &mapA, h * g.C + ch * 32, x0 - 1, y0 - 1, b,
+                                    bar_full + 8 * s);
+                    if (++s == S) {
+                        s = 0;
+                        ph ^= 1u;
+                    }
+                }
+            }
+            if (!ok) {
+                const long long t0 = clock64();
+                while (clock64() - t0 < 200000LL) {
+                }
+            }
+        }
+    } else if (warp == 1) {
+        {  // the whole warp
+            // ---------------- MMA issuer ----------------
+            constexpr uint32_t IDESC2 = tc::idesc_bf16_f32<64>(), IDESC1 = tc::idesc_bf16_f32<32>();
+            const uint64_t a_desc0 = sdesc_box<32>(stages), w_desc0 = sdesc<32, 32>(wres);
+            const uint64_t wrow = (uint64_t)(uint32_t)((3 * g.nchunk * Cf::BBLK) >> 4);  // the next vertical offset
+            int s = 0, acc = 0;
+            uint32_t ph = 0, aph = 0;
+            bool ok = mbar_wait_warp(bar_w, 0, abort);
+            uint32_t last_bar = 0, last_par = 0;
+            for (int t = first_tile; t < end_tile && ok; t += tile_step) {
+                if (!mbar_wait_warp(bar_aempty + 8 * acc, aph ^ 1u, abort)) {
+                    ok = false;
+                    break;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                const uint32_t d = tmem_base + (uint32_t)(acc * Cf::ACC_COLS);
+                for (int ch = 0; ch < g.nchunk; ++ch) {
+                    if (!mbar_wait_warp(bar_full + 8 * s, ph, abort)) {
+                        ok = false;
+                        break;
+                    }
+                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                    const uint64_t da = a_desc0 + (uint64_t)((uint32_t)(s * Cf::STAGE) >> 4);
+                    uint64_t dw = w_desc0 + (uint64_t)((uint32_t)(3 * ch * Cf::BBLK) >> 4);
+#pragma unroll
+                    for (int syi = 0; syi < 3; ++syi) {
+                        // even pixel: 0 away from an even output, -1 from an odd one; odd pixel: 1 and 0; the
+                        // odd pixel of the pair before: -1 from the even output; the even one of the next: 1
+                        // from the odd output
+                        constexpr uint32_t W1 = Cf::BBLK / 16, ODD = Cf::A_SLOT / 16, PX = 64 / 16;
+                        const uint64_t dr = da + (uint64_t)(syi * HPITCH * PX);
+#pragma unroll
+                        for (int kk = 0; kk < 2; ++kk)
+                            mma_f16_elect(d, dr + (uint64_t)(PX + kk * 2), dw + (uint64_t)(W1 + kk * 2), IDESC2,
+                                          syi + kk > 0 || ch > 0 ? 1u : 0u);
+#pragma unroll
+                        for (int kk = 0; kk < 2; ++kk)
+                            mma_f16_elect(d, dr + (uint64_t)(ODD + PX + kk * 2), dw + (uint64_t)(kk * 2), IDESC2, 1u);
+#pragma unroll
+                        for (int kk = 0; kk < 2; ++kk)
+                            mma_f16_elect(d, dr + (uint64_t)(ODD + kk * 2), dw + (uint64_t)(2 * W1 + kk * 2), IDESC1, 1u);
+#pragma unroll
+                        for (int kk = 0; kk < 2; ++kk)
+                            mma_f16_elect(d + 32u, dr + (uint64_t)(2 * PX + kk * 2), dw + (uint64_t)(kk * 2), IDESC1, 1u);
+                        dw += wrow;
+                    }
+                    mma_commit_elect(bar_empty + 8 * s);
+                    last_bar = bar_empty + 8 * s;
+                    last_par = ph;
+                    if (++s == S) {
+                        s = 0;
+                        ph ^= 1u;
+                    }
+                }
+                if (!ok) break;
+                mma_commit_elect(bar_afull + 8 * acc);
+                if (++acc == Cf::NACC) {
+                    acc = 0;
+                    aph ^= 1u;
+                }
+            }
+            if (!ok && last_bar) tc::mbar_wait(last_bar, last_par, nullptr);
+        }
+    } else {
+        // ---------------- epilogue (two groups of four warps) ----------------
+        // The groups take the CTA's tiles in turn, so each has two tiles' time
+        // for one; what a tile's outputs need from device memory is loaded
+        // before its accumulator is waited for.
+        __shared__ float epi_const[EPI::SMEM_FLOATS];
+        epi.prepare(epi_const, threadIdx.x - 64, 256);
+        asm volatile("bar.sync 1, 256;\n" ::: "memory");  // the epilogue warps only
+        const int q = warp & 3, group = (warp - 2) >> 2;
+        int acc = group;
+        uint32_t aph = 0;
+        for (int t = first_tile + group * tile_step; t < end_tile; t += 2 * tile_step) {
+            int b, x0, y0, nt;
+            tile_origin(g, t, b, x0, y0, nt);
+            const int r = q * 32 + lane;
+            const int y = y0 + r / HBW, x = x0 + r % HBW;
+            const bool valid = x < g.W && y < g.H;
+            const int m = valid ? ((b * g.H + y) * g.W + x) * 2 : 0;  // the even pixel
+            typename EPI::Pre pre[2][2];
+            typename EPI::PrePix pp[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+#pragma unroll
+                for (int j = 0; j < 2; ++j) pre[h][j] = epi.prefetch(m + h, 16 * j);
+                pp[h] = epi.prefetch_pixel(m + h);
+            }
+            if (!tc::mbar_wait(bar_afull + 8 * acc, aph, abort)) break;
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * Cf::ACC_COLS);
+            float state[2] = {0.0f, 0.0f};
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                float f[2][16];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    uint32_t v[16];
+                    tc::tmem_ld16(taddr + (uint32_t)(32 * h + 16 * j), v);
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) f[h][i] = __uint_as_float(v[i]);
+                }
+                epi.store_pair(m, 16 * j, f, state, epi_const, pre[0][j], pre[1][j], valid);
+            }
+            asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+            __syncwarp();
+            if (lane == 0) arrive(bar_aempty + 8 * acc);
+            if (valid) {
+                epi.finish(m, state[0], epi_const, pp[0]);
+                epi.finish(m + 1, state[1], epi_const, pp[1]);
+            }
             acc += 2;
             if (acc >= Cf::NACC) {
                 acc = group;
@@ -549,23 +809,26 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
 //
 // k_conv_tma reads 128 pixels and BN weight rows of 128 bytes for every four MMAs
 // and is bound by what L2 delivers (14 TB/s, tensor pipe 23 .. 38 % active). Here a box of
-// 16 x 10 pixels serves the three vertical taps of one horizontal offset (160
-// rows instead of 384), and the three taps' weights serve the G tiles of a
-// group, each with an accumulator of its own, before the next are loaded: per tile and
-// 64 x BN weights 20 KB + 3 BN / G * 128 bytes instead of 3 (16 KB + BN * 128).
-// Roles as in k_conv_halo, with rings of boxes (A) and of weights (W).
-// Measured (forward, batch 64, 256 x 256): 192 -> 64 channels 202 us (377),
-// 384 -> 128 147 (204).
+// 10 x 18 pixels serves all nine taps (180 rows instead of 1152), and each three taps'
+// weights serve the G tiles of a group, each with an accumulator of its own, before
+// the next are loaded: per tile and 64 channels 23 KB + 9 BN / G * 128 bytes instead of
+// 9 (16 KB + BN * 128). Roles as in k_conv_halo, with rings of boxes (A; a
+// group's boxes stay until its last taps) and of weights (W).
+// Measured (forward, batch 64, 256 x 256): 192 -> 64 channels 189 us (377; 202 with a box a
+// horizontal offset),
+// 384 -> 128 143 (204).
 // ---------------------------------------------------------------------------
 
 template <int BN>
 struct GroupCfg {
     static_assert(BN == 64 || BN == 128, "accumulators of 64 or 128 columns");
     static constexpr int A_BYTES = HROWS * 128;     // one box
+    static constexpr int A_SLOT = (A_BYTES + 1023) / 1024 * 1024;
     static constexpr int W_BYTES = 3 * BN * 128;    // the weights of three taps
-    static constexpr int AS = BN == 64 ? 6 : 5, WS = BN == 64 ? 3 : 2;
+    static constexpr int AS = BN == 64 ? 6 : 5, WS = BN == 64 ? 3 : 2;  // ring slots
     static constexpr int NACC = 512 / BN, GMAX = NACC / 2;  // accumulators; tiles a group at most
-    static constexpr int SMEM = 1024 + AS * A_BYTES + WS * W_BYTES + 512;
+    static_assert(GMAX <= AS, "the boxes of a group");
+    static constexpr int SMEM = 1024 + AS * A_SLOT + WS * W_BYTES + 512;
 };
 
 template <int BN, class EPI>
@@ -577,7 +840,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
-    const uint32_t wbase = base + AS * Cf::A_BYTES;
+    const uint32_t wbase = base + AS * Cf::A_SLOT;
     const uint32_t bar_full = wbase + WS * Cf::W_BYTES;
     const uint32_t bar_empty = bar_full + 8 * AS;
     const uint32_t bar_wfull = bar_empty + 8 * AS;
@@ -637,24 +900,24 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
             for (int u = blockIdx.x; u < groups && ok; u += gridDim.x) {
                 int t0, n;
                 group_tiles(u, t0, n);
-                for (int kb = 0; kb < g.KB && ok; ++kb) {  // KB = 3 nchunk: chunk, then horizontal offset
-                    const int ch = kb / 3, sxi = kb - 3 * ch;
+                for (int kb = 0; kb < g.KB && ok; ++kb) {  // KB = 3 nchunk: chunk, then vertical offset
+                    const int ch = kb / 3, syi = kb - 3 * ch;
                     if (!tc::mbar_wait(bar_wempty + 8 * ws, wph ^ 1u, abort)) {
                         ok = false;
                         break;
                     }
                     arrive_expect_tx(bar_wfull + 8 * ws, Cf::W_BYTES);
 #pragma unroll
-                    for (int syi = 0; syi < 3; ++syi) {
+                    for (int sxi = 0; sxi < 3; ++sxi) {
                         const int tap = g.flip ? 8 - (syi * 3 + sxi) : syi * 3 + sxi;
-                        tma_load_2d(wbase + ws * Cf::W_BYTES + syi * (BN * 128), &mapB, tap * g.C + ch * 64,
+                        tma_load_2d(wbase + ws * Cf::W_BYTES + sxi * (BN * 128), &mapB, tap * g.C + ch * 64,
                                     (t0 / g.mtiles) * BN, bar_wfull + 8 * ws);
                     }
                     if (++ws == WS) {
                         ws = 0;
                         wph ^= 1u;
                     }
-                    for (int i = 0; i < n; ++i) {
+                    for (int i = 0; i < n && syi == 0; ++i) {
                         int b, x0, y0, nt;
                         tile_origin(g, t0 + i, b, x0, y0, nt);
                         if (!tc::mbar_wait(bar_empty + 8 * s, ph ^ 1u, abort)) {
@@ -662,7 +925,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
                             break;
                         }
                         arrive_expect_tx(bar_full + 8 * s, Cf::A_BYTES);
-                        tma_load_4d(base + s * Cf::A_BYTES, &mapA, ch * 64, x0 + sxi - 1, y0 - 1, b, bar_full + 8 * s);
+                        tma_load_4d(base + s * Cf::A_SLOT, &mapA, ch * 64, x0 - 1, y0 - 1, b, bar_full + 8 * s);
                         if (++s == AS) {
                             s = 0;
                             ph ^= 1u;
@@ -681,11 +944,10 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
         {  // the whole warp
             // ---------------- MMA issuer ----------------
             constexpr uint32_t IDESC = tc::idesc_bf16_f32<BN>();
-            const uint64_t a_desc0 = sdesc<BN, 64>(base), w_desc0 = sdesc<BN, 64>(wbase);
+            const uint64_t a_desc0 = sdesc_box<64>(base), w_desc0 = sdesc<BN, 64>(wbase);
             int s = 0, ws = 0, acc0 = 0;  // acc0: the group's first accumulator
             uint32_t ph = 0, wph = 0, aph = 0;
             bool ok = true;
-            uint32_t last_bar = 0, last_par = 0;
             for (int u = blockIdx.x; u < groups && ok; u += gridDim.x) {
                 int t0, n;
                 group_tiles(u, t0, n);
@@ -706,31 +968,37 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
                         break;
                     }
                     const uint64_t dw = w_desc0 + (uint64_t)((uint32_t)(ws * Cf::W_BYTES) >> 4);
+                    const int syi = kb % 3;
+                    // the chunk's boxes are slots s .. s + n - 1 (mod AS), waited for with its first
+                    // taps and released with its last
                     for (int i = 0; i < n; ++i) {
                         const int acc = acc0 + i < NACC ? acc0 + i : acc0 + i - NACC;
-                        if (!mbar_wait_warp(bar_full + 8 * s, ph, abort)) {
+                        const int sl = s + i < AS ? s + i : s + i - AS;
+                        const uint32_t slp = s + i < AS ? ph : ph ^ 1u;
+                        if (syi == 0 && !mbar_wait_warp(bar_full + 8 * sl, slp, abort)) {
                             ok = false;
                             break;
                         }
                         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                         const uint32_t d = tmem_base + (uint32_t)(acc * BN);
-                        const uint64_t da = a_desc0 + (uint64_t)((uint32_t)(s * Cf::A_BYTES) >> 4);
+                        const uint64_t da = a_desc0 + (uint64_t)((uint32_t)(sl * Cf::A_SLOT + syi * HPITCH * 128) >> 4);
 #pragma unroll
-                        for (int syi = 0; syi < 3; ++syi)
+                        for (int sxi = 0; sxi < 3; ++sxi)
 #pragma unroll
                             for (int kk = 0; kk < 4; ++kk)
-                                mma_f16_elect(d, da + (uint64_t)(syi * HBW * 128 / 16 + kk * 2),
-                                              dw + (uint64_t)(syi * BN * 128 / 16 + kk * 2), IDESC,
-                                              syi + kk > 0 || kb > 0 ? 1u : 0u);
-                        mma_commit_elect(bar_empty + 8 * s);
-                        last_bar = bar_empty + 8 * s;
-                        last_par = ph;
-                        if (++s == AS) {
-                            s = 0;
+                                mma_f16_elect(d, da + (uint64_t)(sxi * 128 / 16 + kk * 2),
+                                              dw + (uint64_t)(sxi * BN * 128 / 16 + kk * 2), IDESC,
+                                              sxi + kk > 0 || kb > 0 ? 1u : 0u);
+                        if (syi == 2) mma_commit_elect(bar_empty + 8 * sl);
+                    }
+                    if (!ok) break;
+                    if (syi == 2) {
+                        s += n;
+                        if (s >= AS) {
+                            s -= AS;
                             ph ^= 1u;
                         }
                     }
-                    if (!ok) break;
                     mma_commit_elect(bar_wempty + 8 * ws);
                     if (++ws == WS) {
                         ws = 0;
@@ -746,7 +1014,11 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
                     }
                 }
             }
-            if (!ok && last_bar) tc::mbar_wait(last_bar, last_par, nullptr);  // tensor core idle before release
+            if (!ok) {
+                // tensor core idle before release
+                mma_commit_elect(bar_wempty + 8 * ws);
+                tc::mbar_wait(bar_wempty + 8 * ws, wph, nullptr);
+            }
         }
     } else {
         // ---------------- epilogue (two groups of four warps, as in k_conv_halo) ----------------
@@ -767,7 +1039,8 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
                     tile_origin(g, t0 + i, b, x0, y0, nt);
                     const int r = q * 32 + lane;
                     const int y = y0 + r / HBW, x = x0 + r % HBW;
-                    const int m = (b * g.H + y) * g.W + x;
+                    const bool valid = x < g.W && y < g.H;
+                    const int m = valid ? (b * g.H + y) * g.W + x : 0;
                     if (!tc::mbar_wait(bar_afull + 8 * acc, aph, abort)) {
                         ok = false;
                         break;
@@ -783,12 +1056,12 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
                         float f[16];
 #pragma unroll
                         for (int c = 0; c < 16; ++c) f[c] = __uint_as_float(v[c]);
-                        epi.store(m, nt * BN + 16 * j, f, state, epi_const, pre);
+                        epi.store(m, nt * BN + 16 * j, f, state, epi_const, pre, valid);
                     }
                     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
                     __syncwarp();
                     if (lane == 0) arrive(bar_aempty + 8 * acc);
-                    epi.finish(m, state, epi_const, epi.prefetch_pixel(m));
+                    if (valid) epi.finish(m, state, epi_const, epi.prefetch_pixel(m));
                 }
                 if (++acc == NACC) {
                     acc = 0;
