@@ -271,6 +271,24 @@ void poly_count_build(se2n_plan *plan) {
     if (plan->poly_built) return;
     StageTimer timer(plan, SE2N_STAGE_PROPAGATOR);
     plan->poly_built = true;
+    plan->poly_call = plan->calls;
+}
+
+// Whether one interval asked for with SE2N_DIFFUSE_PROPAGATOR takes matrices from
+// device memory although the polynomial applies: only where that is faster (on the
+// Hermitian half, whose frequencies share matrices, and from a cost of the polynomial
+// on: N = 64, 2048 x 2048, 247 instructions an angle: 1.24 ms against 1.88; N = 32,
+// 1000 x 1000, T = 8 / 50: an inpaint 527 / 642 us with the polynomial, 619 with matrices),
+// and only from the second call for the same beta, T and steps on, since a build (16
+// ms there) costs as much as some ten intervals. A call in a stream capture builds none.
+bool kept_matrices(se2n_plan *plan, const PolyTable &t, double beta, double bdt, int steps, bool half) {
+    if (plan->rebuilds || !half || !t.reinsch || se2n_poly_cost(t) <= (plan->N > 32 ? 160 : 210)) return false;
+    if (plan->prop_valid && plan->prop_beta == beta && plan->prop_bdt == bdt && plan->prop_steps == steps &&
+        plan->prop_half == half && plan->prop_fmt == se2n_prop_apply_fmt(plan->N, half))
+        return true;
+    if (!plan->poly_built || plan->poly_call == plan->calls) return false;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(plan->stream, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone;
 }
 
 // The polynomial the column pass takes for one interval with these flags (0 or
@@ -441,6 +459,10 @@ se2n_status diffuse_impl(se2n_plan *plan, float2 *vol, double beta, double T, in
         if (prop_admissible(beta, dt)) {
             const PolyTable *t = poly_get(plan, beta, T, steps);
             if (!t) return propagate_impl(plan, vol, beta, bdt, steps, half);
+            if (kept_matrices(plan, *t, beta, bdt, steps, half)) {
+                const se2n_status st = propagate_impl(plan, vol, beta, bdt, steps, half);
+                if (st != SE2N_ENOMEM) return st;  // no room for them: the polynomial again
+            }
             poly_count_build(plan);
             return poly_impl(plan, vol, *t, half, k0, rows);
         }
@@ -675,6 +697,7 @@ se2n_status inpaint_impl(se2n_plan *plan, const float *f, const uint8_t *mask, c
     const long long HW = plan->HW;
     const int N = plan->N;
     const uint8_t *bins = bins_in;
+    plan->calls += 1;
     const bool col = allow_col && col_path(plan, p);
     if (col) SE2N_TRY(col_start(plan, p));
     if (!bins) {
