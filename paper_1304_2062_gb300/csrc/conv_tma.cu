@@ -537,19 +537,19 @@ cudaError_t launch_wgrad(const __nv_bfloat16 *x, int B, int H, int W, int C, con
     g.ksplit = nsm / groups;
     if (g.ksplit > g.kblocks) g.ksplit = g.kblocks;
     if (g.ksplit < 1) g.ksplit = 1;
-    auto map = [&](CUtensorMap *m, const __nv_bfloat16 *p, int ch, int rows) {
+    auto map = [&](CUtensorMap *m, const __nv_bfloat16 *p, int ch, int cols, int rows) {
         const cuuint64_t dims[4] = {(cuuint64_t)ch, (cuuint64_t)g.W, (cuuint64_t)H, (cuuint64_t)B};
         const cuuint64_t strides[3] = {(cuuint64_t)ch * 2, (cuuint64_t)g.W * ch * 2, (cuuint64_t)H * g.W * ch * 2};
-        const cuuint32_t box[4] = {64, (cuuint32_t)bkx, (cuuint32_t)rows, 1};
+        const cuuint32_t box[4] = {64, (cuuint32_t)cols, (cuuint32_t)rows, 1};
         const cuuint32_t es[4] = {1, 1, 1, 1};
         return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void *)p, dims, strides, box, es,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     };
     CUtensorMap mx, mg;
-    if (!map(&mx, x, cv, tma::kWgR + 3) || !map(&mg, gz, nv, tma::kWgR)) return cudaErrorInvalidValue;
-    const int row = bkx * 128;
-    const int smem = 1024 + tma::kWgXSlots * (tma::kWgR + 3) * row + tma::kWgGSlots * tma::kWgR * row + 256;
+    if (!map(&mx, x, cv, bkx + 2, tma::kWgR + 2) || !map(&mg, gz, nv, bkx, tma::kWgR)) return cudaErrorInvalidValue;
+    const int smem = 1024 + tma::kWgXSlots * (bkx == 32 ? tma::kWgXSlot<32> : tma::kWgXSlot<16>) +
+                     tma::kWgGSlots * tma::kWgR * bkx * 128 + 256;
     auto *fn = bkx == 32 ? &tma::k_wgrad_tma<32> : &tma::k_wgrad_tma<16>;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;

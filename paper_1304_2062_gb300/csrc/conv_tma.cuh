@@ -1085,16 +1085,18 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
 // in shared memory: a TMA box of 64 channels x BKX pixels x some image rows lands
 // as one 128-byte swizzled row a pixel.
 //
-// What bounds a weight gradient with few channels is the rate at which the TMA
-// unit writes box rows (about 8 cycles a row, whether of 64 or of 128 bytes), so
-// the kernel loads few and full ones:
-//  * A box of In holds the R + 3 image rows y0 - 1 .. y0 + R + 1 for one
-//    horizontal offset dx. The vertical offsets read it one image row further
-//    on, a whole number of swizzle atoms, and two neighbouring offsets are the
-//    two 64-row groups of one M = 128 operand (leading byte offset = one image
-//    row): accumulators (dy -1, 0) and (dy 1, none). 3 (R + 3) / R + 1 box rows a pixel
-//    feed all nine taps of 64 input and 64 output channels (5.1 with R = 8; one
-//    box a tap and operand, as before, takes 15).
+// What bounds it is reading the operands out of shared memory (about 80 cycles a
+// product of 128 x 64 x 16), and with few channels the rate at which the TMA unit writes
+// box rows (2.7 cycles a row, whether of 64 or of 128 bytes), so the kernel loads few and
+// full ones and wastes few products:
+//  * A box of In holds the R + 2 image rows and BKX + 2 columns around a block of
+//    R x BKX pixels of gz. Every tap reads it from another pixel on (the swizzle is a
+//    function of the shared-memory address alone), and two taps are the two 64-row
+//    groups of one M = 128 operand, the leading byte offset their distance:
+//    (dy -1, 0) of each column offset, one image row apart, and dy 1 of two
+//    neighbouring column offsets, one pixel apart. 5 products for 9 taps, and 2.3 box
+//    rows a pixel of gz (6 products and 5.1 rows with a box a column offset, 15 rows
+//    with one a tap and operand).
 //  * Layers whose channels are not whole groups of 64 (C = 32, 96, and 8, the
 //    first layer's) are read with F = 2 or 8 neighbouring pixels as one column,
 //    tensors of F C channels and W / F columns: D of a column offset s then
@@ -1103,14 +1105,19 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
 //    others are left out by the epilogue (or not loaded, where a group of 64
 //    channels holds no such pixels). 1 / F of the box rows.
 // A unit of work is (64 channels of In, 64 of gz, a range of pixel blocks); every
-// CTA takes one, accumulates it in tensor memory (up to 3 offsets x 2 tiles x 64
+// CTA takes one, accumulates it in tensor memory (up to 5 tiles of 64
 // columns) and adds it to dW with FP32 atomics at the end.
-// Measured (batch 32, 256 x 256): 32 -> 32 channels 145 us (1008 with a box a
-// tap), 96 -> 32 420, all 13 layers 1713 us (4832).
+// Measured (batch 32, 256 x 256): 32 -> 32 channels 71 us (1008 with a box a tap and
+// operand), 96 -> 32 193, all 14 layers 886 us (4832; 1071 with a box a column offset).
 // ---------------------------------------------------------------------------
 
 constexpr int kWgR = 8;                    // image rows of a pixel block
 constexpr int kWgXSlots = 3, kWgGSlots = 2;  // ring slots of In and of gz
+// a box of In, and its slot: the last operand's second group may end one pixel behind it
+template <int BKX>
+constexpr int kWgXBytes = (kWgR + 2) * (BKX + 2) * 128;
+template <int BKX>
+constexpr int kWgXSlot = (kWgXBytes<BKX> + 128 + 1023) / 1024 * 1024;
 
 struct WgradGeo {
     int B, H, W;        // of the tensors as read (W columns of F pixels)
@@ -1147,9 +1154,9 @@ __global__ void __launch_bounds__(192, 1)
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
-    constexpr uint32_t ROW = (uint32_t)BKX * 128u;        // one image row of a box
-    constexpr uint32_t X_BYTES = (R + 3) * ROW, G_BYTES = R * ROW;
-    const uint32_t gbase = base + XS * X_BYTES;
+    constexpr uint32_t ROW = (BKX + 2) * 128u, GROW = BKX * 128u;  // one image row of a box of In, of gz
+    constexpr uint32_t X_BYTES = kWgXBytes<BKX>, X_SLOT = kWgXSlot<BKX>, G_BYTES = R * GROW;
+    const uint32_t gbase = base + XS * X_SLOT;
     const uint32_t bar_xfull = gbase + GS * G_BYTES;
     const uint32_t bar_xempty = bar_xfull + 8 * XS;
     const uint32_t bar_gfull = bar_xempty + 8 * XS;
@@ -1225,17 +1232,15 @@ __global__ void __launch_bounds__(192, 1)
                     gs = 0;
                     gph ^= 1u;
                 }
-                for (int s = s0; s <= s1; ++s) {
-                    if (!tc::mbar_wait(bar_xempty + 8 * xs, xph ^ 1u, abort)) {
-                        ok = false;
-                        break;
-                    }
-                    arrive_expect_tx(bar_xfull + 8 * xs, X_BYTES);
-                    tma_load_4d(base + xs * X_BYTES, &mapX, c0, x0 + s, y0 - 1, b, bar_xfull + 8 * xs);
-                    if (++xs == XS) {
-                        xs = 0;
-                        xph ^= 1u;
-                    }
+                if (!tc::mbar_wait(bar_xempty + 8 * xs, xph ^ 1u, abort)) {
+                    ok = false;
+                    break;
+                }
+                arrive_expect_tx(bar_xfull + 8 * xs, X_BYTES);
+                tma_load_4d(base + xs * X_SLOT, &mapX, c0, x0 - 1, y0 - 1, b, bar_xfull + 8 * xs);
+                if (++xs == XS) {
+                    xs = 0;
+                    xph ^= 1u;
                 }
             }
             if (!ok) {
@@ -1249,7 +1254,9 @@ __global__ void __launch_bounds__(192, 1)
         {  // the whole warp
             // ---------------- MMA issuer ----------------
             constexpr uint32_t IDESC = idesc_bf16_mn<64>();
-            const uint64_t x_desc0 = sdesc_mn(base, ROW), g_desc0 = sdesc_mn(gbase, ROW);
+            const uint64_t x_desc0 = sdesc_mn(base, ROW), x_desc1 = sdesc_mn(base, 128u);
+            const uint64_t g_desc0 = sdesc_mn(gbase, GROW);
+            const int ns = s1 - s0 + 1;
             int xs = 0, gs = 0;
             uint32_t xph = 0, gph = 0;
             bool ok = true;
@@ -1262,37 +1269,38 @@ __global__ void __launch_bounds__(192, 1)
                     ok = false;
                     break;
                 }
-                for (int s = s0; s <= s1; ++s) {
-                    if (!mbar_wait_warp(bar_xfull + 8 * xs, xph, abort)) {
-                        ok = false;
-                        break;
-                    }
-                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                    const uint32_t d = tmem_base + (uint32_t)((s - s0) * 128);
-                    // 16 pixels = 2048 bytes; image row j of gz against rows j, j + 1 and j + 2, j + 3 of the
-                    // box. Descriptors = the first ones plus constants (in 16-byte units)
-                    const uint64_t dx = x_desc0 + (uint64_t)((uint32_t)xs * (X_BYTES / 16));
-                    const uint64_t dg = g_desc0 + (uint64_t)((uint32_t)gs * (G_BYTES / 16));
+                if (!mbar_wait_warp(bar_xfull + 8 * xs, xph, abort)) {
+                    ok = false;
+                    break;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                // 16 pixels = 2048 bytes; descriptors = the first ones plus constants (in 16-byte
+                // units); image row j of gz against row j (dy = -1) of the box and the next two
+                const uint64_t dx = (uint64_t)((uint32_t)xs * (X_SLOT / 16) + (uint32_t)(s0 + 1) * 8u);
+                const uint64_t dg = g_desc0 + (uint64_t)((uint32_t)gs * (G_BYTES / 16));
+                const uint64_t d0 = x_desc0 + dx, d1 = x_desc1 + dx + 2 * ROW / 16;
 #pragma unroll
-                    for (int j = 0; j < R; ++j) {
-                        if (j >= rows) break;
+                for (int j = 0; j < R; ++j) {
+                    if (j >= rows) break;
 #pragma unroll
-                        for (int kk = 0; kk < BKX / 16; ++kk) {
-                            const uint64_t off = (j * ROW + kk * 2048u) / 16;
-                            const uint32_t add = j + kk > 0 || kb > kb0 ? 1u : 0u;
-                            mma_f16_elect(d, dx + off, dg + off, IDESC, add);
-                            mma_f16_elect(d + 64u, dx + off + 2 * ROW / 16, dg + off, IDESC, add);
-                        }
-                    }
-                    mma_commit_elect(bar_xempty + 8 * xs);
-                    last_bar = bar_xempty + 8 * xs;
-                    last_par = xph;
-                    if (++xs == XS) {
-                        xs = 0;
-                        xph ^= 1u;
+                    for (int kk = 0; kk < BKX / 16; ++kk) {
+                        const uint64_t off = (j * ROW + kk * 2048u) / 16, goff = (j * GROW + kk * 2048u) / 16;
+                        const uint32_t add = j + kk > 0 || kb > kb0 ? 1u : 0u;
+                        for (int t = 0; t < ns; ++t)
+                            mma_f16_elect(tmem_base + (uint32_t)(t * 64), d0 + off + (uint64_t)(t * 8), dg + goff, IDESC,
+                                          add);
+                        for (int t = 0; t < ns; t += 2)
+                            mma_f16_elect(tmem_base + (uint32_t)(ns * 64 + t * 32), d1 + off + (uint64_t)(t * 8),
+                                          dg + goff, IDESC, add);
                     }
                 }
-                if (!ok) break;
+                mma_commit_elect(bar_xempty + 8 * xs);
+                last_bar = bar_xempty + 8 * xs;
+                last_par = xph;
+                if (++xs == XS) {
+                    xs = 0;
+                    xph ^= 1u;
+                }
                 mma_commit_elect(bar_gempty + 8 * gs);
                 if (++gs == GS) {
                     gs = 0;
@@ -1312,11 +1320,13 @@ __global__ void __launch_bounds__(192, 1)
             const int i = (q & 1) * 32 + lane;   // channel of In in the group
             const int e = c0 + i;
             const int px = g.F > 1 ? e / g.C : 0, ci = e - px * g.C;
-            for (int s = s0; s <= s1; ++s)
-                for (int t = 0; t < 2; ++t) {
-                    const int dy = 2 * t + (q >> 1) - 1;
-                    if (dy > 1) continue;  // the second group of the second tile is no tap (warp-uniform)
-                    const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)((s - s0) * 128 + t * 64);
+            const int ns = s1 - s0 + 1;
+            for (int t = 0; t < ns + (ns + 1) / 2; ++t) {
+                    // tiles (dy -1 | 0) of each s, then (s | s + 1) of dy 1
+                    const int s = t < ns ? s0 + t : s0 + 2 * (t - ns) + (q >> 1);
+                    const int dy = t < ns ? (q >> 1) - 1 : 1;
+                    if (s > s1) continue;  // no tap (warp-uniform)
+                    const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(t * 64);
 #pragma unroll 1
                     for (int j0 = 0; j0 < 64; j0 += 16) {
                         uint32_t v[16];
