@@ -24,10 +24,11 @@ __device__ __forceinline__ uint32_t pack2(float a, float b) {
     return *(const uint32_t *)&h;
 }
 
-__device__ __forceinline__ void store16(__nv_bfloat16 *dst, const float (&w)[16]) {
-    uint32_t p[8];
+__device__ __forceinline__ void pack16(const float (&w)[16], uint32_t (&p)[8]) {
 #pragma unroll
     for (int q = 0; q < 8; ++q) p[q] = pack2(w[2 * q], w[2 * q + 1]);
+}
+__device__ __forceinline__ void store16(__nv_bfloat16 *dst, const uint32_t (&p)[8]) {
     uint4 *d4 = (uint4 *)dst;
     d4[0] = make_uint4(p[0], p[1], p[2], p[3]);
     d4[1] = make_uint4(p[4], p[5], p[6], p[7]);
@@ -55,9 +56,13 @@ struct FwdEpi {
     struct PrePix {};
     __device__ __forceinline__ Pre prefetch(int, int) const { return {}; }
     __device__ __forceinline__ PrePix prefetch_pixel(int) const { return {}; }
-    // the 16 outputs as bf16, stored
-    __device__ __forceinline__ void pack(int m, int n, const float (&v)[16], const float *sm, bool valid,
-                                         uint32_t (&p)[8]) const {
+    __device__ __forceinline__ bool writes() const { return true; }
+    __device__ __forceinline__ bool second(int) const { return false; }
+    __device__ __forceinline__ int column(int n) const { return n; }
+    __device__ __forceinline__ void write(int m, int n, const uint32_t (&p)[8]) const {
+        store16(out + (long long)m * N + n, p);
+    }
+    __device__ __forceinline__ void pack(int n, const float (&v)[16], const float *sm, uint32_t (&p)[8]) const {
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
             float a = v[2 * q] + sm[n + 2 * q], b = v[2 * q + 1] + sm[n + 2 * q + 1];
@@ -66,11 +71,6 @@ struct FwdEpi {
                 b = fmaxf(b, 0.0f);
             }
             p[q] = pack2(a, b);
-        }
-        if (valid) {
-            uint4 *d4 = (uint4 *)(out + (long long)m * N + n);
-            d4[0] = make_uint4(p[0], p[1], p[2], p[3]);
-            d4[1] = make_uint4(p[4], p[5], p[6], p[7]);
         }
     }
     // average of two channels of four pixels
@@ -85,10 +85,9 @@ struct FwdEpi {
         const int row = m / W;
         return pool + ((long long)(row >> 1) * (W >> 1) + ((m - row * W) >> 1)) * nb;
     }
-    __device__ __forceinline__ void store(int m, int n, const float (&v)[16], float &, const float *sm, Pre,
-                                          bool valid) const {
-        uint32_t p[8];
-        pack(m, n, v, sm, valid, p);
+    __device__ __forceinline__ void compute(int m, int n, const float (&v)[16], float &, const float *sm, Pre,
+                                            bool valid, uint32_t (&p)[8]) const {
+        pack(n, v, sm, p);
         if (!pool) return;
         // the 2 x 2 pixels are lanes l, l ^ 1, l ^ 8, l ^ 9: each gets four of the 16
         // channels of all of them, in two exchanges
@@ -112,11 +111,11 @@ struct FwdEpi {
         }
         if (valid) *(uint2 *)(pool_at(m) + n + (odd ? 8 : 0) + (hi ? 4 : 0)) = make_uint2(o[0], o[1]);
     }
-    __device__ __forceinline__ void store_pair(int m, int n, const float (&v)[2][16], float (&)[2], const float *sm, Pre,
-                                               Pre, bool valid) const {
-        uint32_t p[8], r[8];
-        pack(m, n, v[0], sm, valid, p);
-        pack(m + 1, n, v[1], sm, valid, r);
+    __device__ __forceinline__ void compute_pair(int m, int n, const float (&v)[2][16], float (&)[2], const float *sm,
+                                                 Pre, Pre, bool valid, uint32_t (&pr)[2][8]) const {
+        uint32_t(&p)[8] = pr[0], (&r)[8] = pr[1];
+        pack(n, v[0], sm, p);
+        pack(n, v[1], sm, r);
         if (!pool) return;
         // the other two pixels are lane l ^ 8's: each lane gets half of the channels
         const bool hi = threadIdx.x & 8;
@@ -154,7 +153,14 @@ struct HeadEpi {
     };
     __device__ __forceinline__ Pre prefetch(int, int) const { return {}; }
     __device__ __forceinline__ PrePix prefetch_pixel(int m) const { return {f[m], mask[m]}; }
-    __device__ __forceinline__ void store(int m, int n, const float (&v)[16], float &st, const float *sm, Pre, bool valid) const {
+    __device__ __forceinline__ bool writes() const { return out != nullptr; }
+    __device__ __forceinline__ bool second(int) const { return false; }
+    __device__ __forceinline__ int column(int n) const { return n; }
+    __device__ __forceinline__ void write(int m, int n, const uint32_t (&p)[8]) const {
+        store16(out + (long long)m * 32 + n, p);
+    }
+    __device__ __forceinline__ void compute(int, int n, const float (&v)[16], float &st, const float *sm, Pre, bool,
+                                            uint32_t (&p)[8]) const {
         float w[16];
         if (n == 0) st = sm[64];
 #pragma unroll
@@ -163,12 +169,13 @@ struct HeadEpi {
             w[q] = __bfloat162float(__float2bfloat16_rn(w[q]));
             st = fmaf(sm[32 + n + q], w[q], st);
         }
-        if (out && valid) store16(out + (long long)m * 32 + n, w);
+        pack16(w, p);
     }
-    __device__ __forceinline__ void store_pair(int m, int n, const float (&v)[2][16], float (&st)[2], const float *sm,
-                                               const Pre &p, const Pre &p1, bool valid) const {
-        store(m, n, v[0], st[0], sm, p, valid);
-        store(m + 1, n, v[1], st[1], sm, p1, valid);
+    __device__ __forceinline__ void compute_pair(int m, int n, const float (&v)[2][16], float (&st)[2],
+                                                 const float *sm, const Pre &a, const Pre &a1, bool valid,
+                                                 uint32_t (&p)[2][8]) const {
+        compute(m, n, v[0], st[0], sm, a, valid, p[0]);
+        compute(m + 1, n, v[1], st[1], sm, a1, valid, p[1]);
     }
     __device__ __forceinline__ void finish(int m, float st, const float *, PrePix p) const {
         y[m] = (p.mask ? p.f : 0.0f) + st;
@@ -197,30 +204,33 @@ struct DgradEpi {
         return p;
     }
     __device__ __forceinline__ PrePix prefetch_pixel(int) const { return {}; }
-    __device__ __forceinline__ void store(int m, int n, const float (&v)[16], float &, const float *, const Pre &p,
-                                          bool valid) const {
+    __device__ __forceinline__ bool writes() const { return true; }
+    __device__ __forceinline__ bool second(int n) const { return n >= split; }
+    __device__ __forceinline__ int column(int n) const { return n < split ? n : n - split; }
+    __device__ __forceinline__ void write(int m, int n, const uint32_t (&p)[8]) const {
+        store16(n < split ? din + (long long)m * split + n : din2 + (long long)m * (N - split) + (n - split), p);
+    }
+    __device__ __forceinline__ void compute(int, int n, const float (&v)[16], float &, const float *, const Pre &a, bool,
+                                            uint32_t (&p)[8]) const {
         float w[16];
 #pragma unroll
         for (int q = 0; q < 16; ++q) w[q] = v[q];
-        if (n < split) {
-            if (act) {
-                const uint32_t aw[8] = {p.a0.x, p.a0.y, p.a0.z, p.a0.w, p.a1.x, p.a1.y, p.a1.z, p.a1.w};
+        if (act && n < split) {
+            const uint32_t aw[8] = {a.a0.x, a.a0.y, a.a0.z, a.a0.w, a.a1.x, a.a1.y, a.a1.z, a.a1.w};
 #pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const __nv_bfloat162 h = *(const __nv_bfloat162 *)&aw[q];
-                    if (!(__bfloat162float(h.x) > 0.0f)) w[2 * q] = 0.0f;
-                    if (!(__bfloat162float(h.y) > 0.0f)) w[2 * q + 1] = 0.0f;
-                }
+            for (int q = 0; q < 8; ++q) {
+                const __nv_bfloat162 h = *(const __nv_bfloat162 *)&aw[q];
+                if (!(__bfloat162float(h.x) > 0.0f)) w[2 * q] = 0.0f;
+                if (!(__bfloat162float(h.y) > 0.0f)) w[2 * q + 1] = 0.0f;
             }
-            if (valid) store16(din + (long long)m * split + n, w);
-        } else if (valid) {
-            store16(din2 + (long long)m * (N - split) + (n - split), w);
         }
+        pack16(w, p);
     }
-    __device__ __forceinline__ void store_pair(int m, int n, const float (&v)[2][16], float (&st)[2], const float *sm,
-                                               const Pre &p, const Pre &p1, bool valid) const {
-        store(m, n, v[0], st[0], sm, p, valid);
-        store(m + 1, n, v[1], st[1], sm, p1, valid);
+    __device__ __forceinline__ void compute_pair(int m, int n, const float (&v)[2][16], float (&st)[2],
+                                                 const float *sm, const Pre &a, const Pre &a1, bool valid,
+                                                 uint32_t (&p)[2][8]) const {
+        compute(m, n, v[0], st[0], sm, a, valid, p[0]);
+        compute(m + 1, n, v[1], st[1], sm, a1, valid, p[1]);
     }
     __device__ __forceinline__ void finish(int, float, const float *, PrePix) const {}
 };
@@ -320,10 +330,38 @@ bool box_shape(int H, int W) {
     return px <= 2LL * W * H;
 }
 
+// The tensors a kernel's output boxes go to (second: the columns from the first's
+// last on; no tensor: p null), and their maps: 8 or 16 pixels of 4 image rows, ob channels.
+struct OutTensor {
+    __nv_bfloat16 *p;
+    int channels, ld;
+};
+struct OutTensors {
+    OutTensor t[2];
+};
+bool out_maps(PFN_cuTensorMapEncodeTiled_v12000 enc, const OutTensors &o, int B, int H, int W, int ob, int px,
+              CUtensorMap (&m)[2]) {
+    for (int k = 0; k < 2; ++k) {
+        const OutTensor &t = o.t[k].p ? o.t[k] : o.t[0];
+        if (!t.p) continue;  // no output is wanted: the maps are not used
+        if (t.channels % ob) return false;
+        const cuuint64_t dims[4] = {(cuuint64_t)t.channels, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B};
+        const cuuint64_t ld = (cuuint64_t)t.ld * 2;
+        const cuuint64_t strides[3] = {ld, ld * W, ld * W * H};
+        const cuuint32_t box[4] = {(cuuint32_t)ob, (cuuint32_t)px, 4, 1};
+        const cuuint32_t es[4] = {1, 1, 1, 1};
+        if (enc(&m[k], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void *)t.p, dims, strides, box, es,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, ob == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+                CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return false;
+    }
+    return true;
+}
+
 // Narrow layers: 8 x 16 tiles, halo boxes, weights resident in shared memory.
 template <int BN, int CK, class EPI>
 cudaError_t launch_halo(const __nv_bfloat16 *A, int B, int H, int W, int C, const __nv_bfloat16 *wmat, int N, int flip,
-                        const EPI &epi, cudaStream_t s) {
+                        const EPI &epi, const OutTensors &o, cudaStream_t s) {
     using Cf = tma::HaloCfg<BN, CK>;
     if (!box_shape(H, W) || C % CK || N % BN) return cudaErrorNotSupported;
     const int nblk = 9 * (C / CK);
@@ -335,7 +373,8 @@ cudaError_t launch_halo(const __nv_bfloat16 *A, int B, int H, int W, int C, cons
     const int nsm = sm_count();
     int *err = fault_ptr();
     if (!enc || nsm <= 0 || !err) return cudaErrorNotSupported;
-    CUtensorMap ma, mb;
+    CUtensorMap ma, mb, mo[2] = {};
+    if (!out_maps(enc, o, B, H, W, Cf::OB, tma::HBW, mo)) return cudaErrorNotSupported;
     {
         const cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B};
         const cuuint64_t strides[3] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2, (cuuint64_t)H * W * C * 2};
@@ -371,7 +410,7 @@ cudaError_t launch_halo(const __nv_bfloat16 *A, int B, int H, int W, int C, cons
     g.nchunk = C / CK;
     g.KB = 3 * g.nchunk;
     g.flip = flip;
-    const int smem = 1024 + wbytes + S * Cf::STAGE + 256;
+    const int smem = 1024 + wbytes + S * Cf::STAGE + 8 * tma::kOutBytes + 256;
     auto *fn = &tma::k_conv_halo<BN, CK, EPI>;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
@@ -379,14 +418,14 @@ cudaError_t launch_halo(const __nv_bfloat16 *A, int B, int H, int W, int C, cons
     const int per = nsm / g.ntiles;
     if (per < 1) return cudaErrorNotSupported;
     const int grid = (g.mtiles < per ? g.mtiles : per) * g.ntiles;
-    fn<<<grid, tma::kHaloThreads, smem, s>>>(ma, mb, g, epi, S, err);
+    fn<<<grid, tma::kHaloThreads, smem, s>>>(ma, mb, mo[0], mo[1], g, epi, S, err);
     return cudaGetLastError();
 }
 
 // 32 output channels: pairs of pixels (W even), halo boxes, weights resident in shared memory.
 template <class EPI>
 cudaError_t launch_pair(const __nv_bfloat16 *A, int B, int H, int W, int C, const __nv_bfloat16 *wmat, int flip,
-                        const EPI &epi, cudaStream_t s) {
+                        const EPI &epi, const OutTensors &o, cudaStream_t s) {
     using Cf = tma::PairCfg;
     if (W % 2 || !box_shape(H, W / 2) || C % 32) return cudaErrorNotSupported;
     const int nblk = 9 * (C / 32);
@@ -413,7 +452,8 @@ cudaError_t launch_pair(const __nv_bfloat16 *A, int B, int H, int W, int C, cons
     g.nchunk = C / 32;
     g.KB = g.nchunk;
     g.flip = flip;
-    CUtensorMap ma, mb;
+    CUtensorMap ma, mb, mo[2] = {};
+    if (!out_maps(enc, o, B, H, W, 32, 2 * tma::HBW, mo)) return cudaErrorNotSupported;
     {
         const cuuint64_t dims[4] = {(cuuint64_t)2 * C, (cuuint64_t)g.W, (cuuint64_t)H, (cuuint64_t)B};
         const cuuint64_t strides[3] = {(cuuint64_t)C * 4, (cuuint64_t)W * C * 2, (cuuint64_t)H * W * C * 2};
@@ -434,11 +474,11 @@ cudaError_t launch_pair(const __nv_bfloat16 *A, int B, int H, int W, int C, cons
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cudaErrorInvalidValue;
     }
-    const int smem = 1024 + wbytes + S * Cf::STAGE + 256;
+    const int smem = 1024 + wbytes + S * Cf::STAGE + 8 * tma::kOutBytes + 256;
     auto *fn = &tma::k_conv_pair<EPI>;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    fn<<<g.mtiles < nsm ? g.mtiles : nsm, tma::kHaloThreads, smem, s>>>(ma, mb, g, epi, S, err);
+    fn<<<g.mtiles < nsm ? g.mtiles : nsm, tma::kHaloThreads, smem, s>>>(ma, mb, mo[0], mo[1], g, epi, S, err);
     return cudaGetLastError();
 }
 
@@ -446,14 +486,15 @@ cudaError_t launch_pair(const __nv_bfloat16 *A, int B, int H, int W, int C, cons
 // 128 channels, or of 64.
 template <int BN, class EPI>
 cudaError_t launch_group(const __nv_bfloat16 *A, int B, int H, int W, int C, const __nv_bfloat16 *wmat, int N, int flip,
-                         const EPI &epi, cudaStream_t s) {
+                         const EPI &epi, const OutTensors &o, cudaStream_t s) {
     using Cf = tma::GroupCfg<BN>;
     if (!box_shape(H, W) || C % 64 || N % BN) return cudaErrorNotSupported;
     auto enc = encoder();
     const int nsm = sm_count();
     int *err = fault_ptr();
     if (!enc || nsm <= 0 || !err) return cudaErrorNotSupported;
-    CUtensorMap ma, mb;
+    CUtensorMap ma, mb, mo[2] = {};
+    if (!out_maps(enc, o, B, H, W, 64, tma::HBW, mo)) return cudaErrorNotSupported;
     {
         const cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B};
         const cuuint64_t strides[3] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2, (cuuint64_t)H * W * C * 2};
@@ -497,15 +538,15 @@ cudaError_t launch_group(const __nv_bfloat16 *A, int B, int H, int W, int C, con
     auto *fn = &tma::k_conv_group<BN, EPI>;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, Cf::SMEM);
     if (e != cudaSuccess) return e;
-    fn<<<groups < nsm ? groups : nsm, tma::kHaloThreads, Cf::SMEM, s>>>(ma, mb, g, epi, G, err);
+    fn<<<groups < nsm ? groups : nsm, tma::kHaloThreads, Cf::SMEM, s>>>(ma, mb, mo[0], mo[1], g, epi, G, err);
     return cudaGetLastError();
 }
 
 template <class EPI>
 cudaError_t launch_wide(const __nv_bfloat16 *A, int B, int H, int W, int C, const __nv_bfloat16 *wmat, int N, int flip,
-                        const EPI &epi, cudaStream_t s) {
-    return N % 128 == 0 ? launch_group<128>(A, B, H, W, C, wmat, N, flip, epi, s)
-                        : launch_group<64>(A, B, H, W, C, wmat, N, flip, epi, s);
+                        const EPI &epi, const OutTensors &o, cudaStream_t s) {
+    return N % 128 == 0 ? launch_group<128>(A, B, H, W, C, wmat, N, flip, epi, o, s)
+                        : launch_group<64>(A, B, H, W, C, wmat, N, flip, epi, o, s);
 }
 
 // Weight gradient (k_wgrad_tma): x [B][H][W][C] and gz [B][H][W][Cout] NHWC, dw
@@ -582,24 +623,26 @@ cudaError_t conv_forward_tma(const __nv_bfloat16 *in, int B, int H, int W, int C
     const bool ck64 = Cin % 64 == 0;
     if (head) {
         if (Cout != 32 || !relu || ldo != 32) return cudaErrorNotSupported;
+        const OutTensors o{{{out, 32, 32}, {nullptr, 0, 0}}};
         const HeadEpi epi{bias, out, head->hw, head->hb, head->f, head->mask, head->y};
-        const cudaError_t e = launch_pair(in, B, H, W, Cin, w, 0, epi, s);
+        const cudaError_t e = launch_pair(in, B, H, W, Cin, w, 0, epi, o, s);
         if (e != cudaErrorNotSupported) return e;
         return ck64 ? launch<32, 64>(in, B, H, W, Cin, w, Cout, 0, epi, s)
                     : launch<32, 32>(in, B, H, W, Cin, w, Cout, 0, epi, s);
     }
     // the kernels with 8 x 16 tiles write the averages too
+    const OutTensors o{{{out, Cout, ldo}, {nullptr, 0, 0}}};
     FwdEpi fepi{bias, out, ldo, relu, Cout};
     fepi.pool = pool;
     fepi.W = W;
     cudaError_t e = cudaErrorNotSupported;
     if (Cout == 32)
-        e = launch_pair(in, B, H, W, Cin, w, 0, fepi, s);
+        e = launch_pair(in, B, H, W, Cin, w, 0, fepi, o, s);
     else if (Cout == 64)
-        e = ck64 ? launch_halo<64, 64>(in, B, H, W, Cin, w, Cout, 0, fepi, s)
-                 : launch_halo<64, 32>(in, B, H, W, Cin, w, Cout, 0, fepi, s);
+        e = ck64 ? launch_halo<64, 64>(in, B, H, W, Cin, w, Cout, 0, fepi, o, s)
+                 : launch_halo<64, 32>(in, B, H, W, Cin, w, Cout, 0, fepi, o, s);
     if (e == cudaErrorNotSupported && ck64 && Cout % 64 == 0)
-        e = launch_wide(in, B, H, W, Cin, w, Cout, 0, fepi, s);
+        e = launch_wide(in, B, H, W, Cin, w, Cout, 0, fepi, o, s);
     if (e != cudaErrorNotSupported) {
         if (pooled) *pooled = pool != nullptr;
         return e;
@@ -622,16 +665,17 @@ cudaError_t conv_dgrad_tma(const __nv_bfloat16 *gz, int B, int H, int W, int Cou
     if (split % 16) return cudaErrorNotSupported;
     const bool ck64 = Cout % 64 == 0;
     const DgradEpi epi{act, din, din2, split, Cin};
+    const OutTensors o{{{din, split, split}, {split < Cin ? din2 : nullptr, Cin - split, Cin - split}}};
     // A = gz (Cout channels, taps mirrored), B = wt [Cin][9 Cout]
     if (Cin == 32 || Cin == 64 || Cin == 96) {
         cudaError_t e = cudaErrorNotSupported;
         if (Cin == 32)
-            e = launch_pair(gz, B, H, W, Cout, wt, 1, epi, s);
+            e = launch_pair(gz, B, H, W, Cout, wt, 1, epi, o, s);
         else if (Cin == 64)
-            e = ck64 ? launch_halo<64, 64>(gz, B, H, W, Cout, wt, Cin, 1, epi, s)
-                     : launch_halo<64, 32>(gz, B, H, W, Cout, wt, Cin, 1, epi, s);
+            e = ck64 ? launch_halo<64, 64>(gz, B, H, W, Cout, wt, Cin, 1, epi, o, s)
+                     : launch_halo<64, 32>(gz, B, H, W, Cout, wt, Cin, 1, epi, o, s);
         else if (!ck64)
-            e = launch_halo<96, 32>(gz, B, H, W, Cout, wt, Cin, 1, epi, s);
+            e = launch_halo<96, 32>(gz, B, H, W, Cout, wt, Cin, 1, epi, o, s);
         if (e != cudaErrorNotSupported) return e;
     }
     if (!ck64) {
@@ -640,7 +684,7 @@ cudaError_t conv_dgrad_tma(const __nv_bfloat16 *gz, int B, int H, int W, int Cou
         return cudaErrorNotSupported;
     }
     if (Cin % 64 == 0) {
-        const cudaError_t e = launch_wide(gz, B, H, W, Cout, wt, Cin, 1, epi, s);
+        const cudaError_t e = launch_wide(gz, B, H, W, Cout, wt, Cin, 1, epi, o, s);
         if (e != cudaErrorNotSupported) return e;
     }
     switch (Cin) {

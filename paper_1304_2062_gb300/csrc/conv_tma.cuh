@@ -135,13 +135,16 @@ __device__ __forceinline__ void tile_origin(const ConvGeo &g, int t, int &b, int
 // EPI provides
 //   SMEM_FLOATS, prepare(sm, i, n)    constants copied to shared memory by the
 //                                      epilogue threads i = 0..n-1 once per CTA
-//   Pre, prefetch(m, n)               what store(m, n) reads from device memory (may be loaded
+//   Pre, prefetch(m, n)               what compute(m, n) reads from device memory (may be loaded
 //                                      before the accumulator is complete)
 //   PrePix, prefetch_pixel(m)         the same for finish(m)
-//   store(m, n, v[16], float &state, sm, pre, valid)  the 16 outputs of pixel m, columns n..n+15;
-//                                      called by whole warps, of pixel 0 for lanes without one
-//   store_pair(m, n, v[2][16], float (&state)[2], sm, pre, pre1, valid)  the same of pixels m
-//                                      and m + 1 (k_conv_pair)
+//   compute(m, n, v[16], float &state, sm, pre, valid, p[8])  the 16 outputs of pixel m, columns
+//                                      n..n+15, as BF16 pairs; called by whole warps, of pixel 0
+//                                      for lanes without one
+//   compute_pair(m, n, v[2][16], float (&state)[2], sm, pre, pre1, valid, p[2][8])  the same of
+//                                      pixels m and m + 1 (k_conv_pair)
+//   write(m, n, p[8])                 stores them (k_conv_tma; the other kernels write boxes)
+//   writes(), second(n), column(n)    whether they are wanted, in which tensor column n goes and where
 //   finish(m, float state, sm, pre)   after the last column group of pixel m
 template <int BN, int CK, class EPI>
 __global__ void __launch_bounds__(192, 1)
@@ -278,7 +281,7 @@ __global__ void __launch_bounds__(192, 1)
         int acc = 0;
         uint32_t aph = 0;
         for (int t = blockIdx.x; t < g.tiles; t += gridDim.x) {
-            if (!tc::mbar_wait(bar_afull + 8 * acc, aph, abort)) break;
+            if (!mbar_wait_warp(bar_afull + 8 * acc, aph, abort)) break;
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
             int b, x0, y0, nt;
             tile_origin(g, t, b, x0, y0, nt);
@@ -294,7 +297,9 @@ __global__ void __launch_bounds__(192, 1)
                 float f[16];
 #pragma unroll
                 for (int i = 0; i < 16; ++i) f[i] = __uint_as_float(v[i]);
-                epi.store(m, nt * BN + j0, f, state, epi_const, epi.prefetch(m, nt * BN + j0), true);
+                uint32_t p[8];
+                epi.compute(m, nt * BN + j0, f, state, epi_const, epi.prefetch(m, nt * BN + j0), true, p);
+                if (epi.writes()) epi.write(m, nt * BN + j0, p);
             }
             epi.finish(m, state, epi_const, epi.prefetch_pixel(m));
             asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
@@ -325,7 +330,7 @@ __global__ void __launch_bounds__(192, 1)
 // one box row (10 pixels) apart, and the swizzle is a function of the shared-memory
 // address alone, so a group may start anywhere in a swizzle atom. 180 box rows feed
 // the nine taps; the TMA unit writes box rows at 2.7 cycles each, and a box a horizontal
-// offset makes 480 of them, one a tap 1152. (64 -> 64 channels, batch 64, 128 x 128: 76 us,
+// offset makes 480 of them, one a tap 1152. (64 -> 64 channels, batch 64, 128 x 128: 76 us against
 // 86 with a box a horizontal offset.) All weights of the layer (9 C x BN) are loaded into shared memory
 // once per CTA, so the K loop moves no weight rows at all. Pixels of a tile outside the
 // image are computed and not stored.
@@ -342,11 +347,54 @@ struct HaloCfg {
     static constexpr int A_BYTES = HROWS * CK * 2;
     static constexpr int STAGE = (A_BYTES + 1023) / 1024 * 1024;
     static constexpr int BBLK = BN * CK * 2;   // one (tap, channel block) of weights
+    static constexpr int OB = BN % 64 == 0 ? 64 : 32;  // channels of an output box
     static constexpr int ACC_COLS = BN <= 32 ? 32 : BN <= 64 ? 64 : 128;
     static constexpr int NACC = 4;             // accumulators
     static constexpr int TMEM_COLS = NACC * ACC_COLS;
     static constexpr int SMEM_BUDGET = 196608;
 };
+
+// Outputs of these kernels leave through shared memory: every epilogue warp packs OB
+// channels of its image rows into a buffer of its own (in the swizzled layout of a
+// TMA box, so that the lanes' 16-byte stores do not meet) and stores it as one box.
+// From registers a lane's 32 bytes a pixel are two stores of 16 bytes, each a partial
+// sector among 32 lines (32 -> 32 channels with the pooling, batch 64, 256 x 256: 133 us
+// against 153; 64 -> 64 at 128 x 128 67 against 76; 96 columns of data gradient, batch 32,
+// 85 against 133).
+// Pixels outside the image are clipped by the box.
+constexpr int kOutBytes = 4096;  // a warp's buffer
+
+template <int OB>
+__device__ __forceinline__ void out_put(uint32_t buf, int row, int c, const uint32_t (&p)[8]) {
+    const int key = OB == 64 ? row & 7 : (row >> 1) & 3, j = c >> 3;
+    const uint32_t a = buf + (uint32_t)(row * OB * 2);
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(a + (uint32_t)((j ^ key) << 4)), "r"(p[0]), "r"(p[1]),
+                 "r"(p[2]), "r"(p[3])
+                 : "memory");
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(a + (uint32_t)(((j + 1) ^ key) << 4)), "r"(p[4]),
+                 "r"(p[5]), "r"(p[6]), "r"(p[7])
+                 : "memory");
+}
+// the warp's buffer may be written again
+__device__ __forceinline__ void out_reuse(int lane) {
+    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
+    __syncwarp();
+}
+__device__ __forceinline__ void out_store(uint32_t buf, const CUtensorMap *map, int c, int x, int y, int b, int lane) {
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    __syncwarp();
+    if (lane == 0) {
+        asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3, %4}], [%5];\n" ::"l"(
+                         (uint64_t)map),
+                     "r"(c), "r"(x), "r"(y), "r"(b), "r"(buf)
+                     : "memory");
+        asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
+    }
+}
+__device__ __forceinline__ void out_drain(int lane) {
+    if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory");
+    __syncwarp();
+}
 
 // Descriptor of a tile's pixels in a box: image rows HPITCH pixels apart.
 template <int CK>
@@ -361,7 +409,8 @@ __device__ __forceinline__ uint64_t sdesc_box(uint32_t saddr) {
 
 template <int BN, int CK, class EPI>
 __global__ void __launch_bounds__(kHaloThreads, 1)
-    k_conv_halo(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, const ConvGeo g,
+    k_conv_halo(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
+                const __grid_constant__ CUtensorMap mapO, const __grid_constant__ CUtensorMap mapO2, const ConvGeo g,
                 const EPI epi, int S, int *err) {
     using Cf = HaloCfg<BN, CK>;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -370,7 +419,8 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
     const int nblk = 9 * g.nchunk;                       // resident weight blocks
     const uint32_t wres = base;                          // nblk x BBLK
     const uint32_t stages = wres + nblk * Cf::BBLK;      // S x STAGE
-    const uint32_t bar_w = stages + S * Cf::STAGE;
+    const uint32_t obuf = stages + S * Cf::STAGE;        // the epilogue warps' output buffers
+    const uint32_t bar_w = obuf + 8 * kOutBytes;
     const uint32_t bar_full = bar_w + 8;
     const uint32_t bar_empty = bar_full + 8 * S;
     const uint32_t bar_afull = bar_empty + 8 * S;
@@ -512,6 +562,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
         epi.prepare(epi_const, threadIdx.x - 64, 256);
         asm volatile("bar.sync 1, 256;\n" ::: "memory");  // the epilogue warps only
         const int q = warp & 3, group = (warp - 2) >> 2;
+        const uint32_t buf = obuf + (uint32_t)(warp - 2) * kOutBytes;
         int acc = group;
         uint32_t aph = 0;
         for (int t = first_tile + group * tile_step; t < end_tile; t += 2 * tile_step) {
@@ -525,7 +576,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
 #pragma unroll
             for (int j = 0; j < BN / 16; ++j) pre[j] = epi.prefetch(m, nt * BN + 16 * j);
             const typename EPI::PrePix pp = epi.prefetch_pixel(m);
-            if (!tc::mbar_wait(bar_afull + 8 * acc, aph, abort)) break;
+            if (!mbar_wait_warp(bar_afull + 8 * acc, aph, abort)) break;
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
             const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * Cf::ACC_COLS);
             float state = 0.0f;
@@ -536,7 +587,16 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
                 float f[16];
 #pragma unroll
                 for (int i = 0; i < 16; ++i) f[i] = __uint_as_float(v[i]);
-                epi.store(m, nt * BN + 16 * j, f, state, epi_const, pre[j], valid);
+                const int n = nt * BN + 16 * j;
+                uint32_t p[8];
+                epi.compute(m, n, f, state, epi_const, pre[j], valid, p);
+                if (epi.writes()) {
+                    constexpr int OB = Cf::OB;
+                    if (16 * j % OB == 0) out_reuse(lane);
+                    out_put<OB>(buf, lane, 16 * j % OB, p);
+                    if (16 * (j + 1) % OB == 0)
+                        out_store(buf, epi.second(n) ? &mapO2 : &mapO, epi.column(n + 16 - OB), x0, y0 + 4 * q, b, lane);
+                }
             }
             asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
             __syncwarp();
@@ -548,6 +608,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
                 aph ^= 1u;
             }
         }
+        out_drain(lane);
     }
     __syncthreads();
     if (threadIdx.x == 0 && *abort) atomicExch(err, 1);
@@ -572,8 +633,8 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
 // next to the odd one: 32 columns. 24 products a 32 channels and 256 pixels
 // instead of 36. The pixels of either parity are a box of their own (of the tensor as
 // W / 2 columns of 2 C channels).
-// Measured (forward, batch 64, 256 x 256): 32 -> 32 channels 153 us with the pooling (169),
-// 96 -> 32 224 (317), 32 -> 32 with the head 91 (137).
+// Measured (forward, batch 64, 256 x 256): 32 -> 32 channels 133 us with the pooling (169),
+// 96 -> 32 222 (317), 32 -> 32 with the head 91 (137).
 // ---------------------------------------------------------------------------
 
 struct PairCfg {
@@ -587,7 +648,8 @@ struct PairCfg {
 
 template <class EPI>
 __global__ void __launch_bounds__(kHaloThreads, 1)
-    k_conv_pair(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, const ConvGeo g,
+    k_conv_pair(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
+                const __grid_constant__ CUtensorMap mapO, const __grid_constant__ CUtensorMap mapO2, const ConvGeo g,
                 const EPI epi, int S, int *err) {
     using Cf = PairCfg;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -596,7 +658,8 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
     const int nblk = 9 * g.nchunk;                       // resident weight blocks
     const uint32_t wres = base;                          // nblk x BBLK
     const uint32_t stages = wres + nblk * Cf::BBLK;      // S x STAGE
-    const uint32_t bar_w = stages + S * Cf::STAGE;
+    const uint32_t obuf = stages + S * Cf::STAGE;        // the epilogue warps' output buffers
+    const uint32_t bar_w = obuf + 8 * kOutBytes;
     const uint32_t bar_full = bar_w + 8;
     const uint32_t bar_empty = bar_full + 8 * S;
     const uint32_t bar_afull = bar_empty + 8 * S;
@@ -746,6 +809,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
         epi.prepare(epi_const, threadIdx.x - 64, 256);
         asm volatile("bar.sync 1, 256;\n" ::: "memory");  // the epilogue warps only
         const int q = warp & 3, group = (warp - 2) >> 2;
+        const uint32_t buf = obuf + (uint32_t)(warp - 2) * kOutBytes;
         int acc = group;
         uint32_t aph = 0;
         for (int t = first_tile + group * tile_step; t < end_tile; t += 2 * tile_step) {
@@ -763,7 +827,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
                 for (int j = 0; j < 2; ++j) pre[h][j] = epi.prefetch(m + h, 16 * j);
                 pp[h] = epi.prefetch_pixel(m + h);
             }
-            if (!tc::mbar_wait(bar_afull + 8 * acc, aph, abort)) break;
+            if (!mbar_wait_warp(bar_afull + 8 * acc, aph, abort)) break;
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
             const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * Cf::ACC_COLS);
             float state[2] = {0.0f, 0.0f};
@@ -777,7 +841,14 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
 #pragma unroll
                     for (int i = 0; i < 16; ++i) f[h][i] = __uint_as_float(v[i]);
                 }
-                epi.store_pair(m, 16 * j, f, state, epi_const, pre[0][j], pre[1][j], valid);
+                uint32_t p[2][8];
+                epi.compute_pair(m, 16 * j, f, state, epi_const, pre[0][j], pre[1][j], valid, p);
+                if (epi.writes()) {
+                    if (j == 0) out_reuse(lane);
+                    out_put<32>(buf, 2 * lane, 16 * j, p[0]);
+                    out_put<32>(buf, 2 * lane + 1, 16 * j, p[1]);
+                    if (j == 1) out_store(buf, &mapO, 0, 2 * x0, y0 + 4 * q, b, lane);
+                }
             }
             asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
             __syncwarp();
@@ -792,6 +863,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
                 aph ^= 1u;
             }
         }
+        out_drain(lane);
     }
     __syncthreads();
     if (threadIdx.x == 0 && *abort) atomicExch(err, 1);
@@ -814,7 +886,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
 // the next are loaded: per tile and 64 channels 23 KB + 9 BN / G * 128 bytes instead of
 // 9 (16 KB + BN * 128). Roles as in k_conv_halo, with rings of boxes (A; a
 // group's boxes stay until its last taps) and of weights (W).
-// Measured (forward, batch 64, 256 x 256): 192 -> 64 channels 189 us (377; 202 with a box a
+// Measured (forward, batch 64, 256 x 256): 192 -> 64 channels 191 us (377; 202 with a box a
 // horizontal offset),
 // 384 -> 128 143 (204).
 // ---------------------------------------------------------------------------
@@ -825,15 +897,16 @@ struct GroupCfg {
     static constexpr int A_BYTES = HROWS * 128;     // one box
     static constexpr int A_SLOT = (A_BYTES + 1023) / 1024 * 1024;
     static constexpr int W_BYTES = 3 * BN * 128;    // the weights of three taps
-    static constexpr int AS = BN == 64 ? 6 : 5, WS = BN == 64 ? 3 : 2;  // ring slots
+    static constexpr int AS = BN == 64 ? 5 : 4, WS = BN == 64 ? 3 : 2;  // ring slots
     static constexpr int NACC = 512 / BN, GMAX = NACC / 2;  // accumulators; tiles a group at most
     static_assert(GMAX <= AS, "the boxes of a group");
-    static constexpr int SMEM = 1024 + AS * A_SLOT + WS * W_BYTES + 512;
+    static constexpr int SMEM = 1024 + AS * A_SLOT + WS * W_BYTES + 8 * kOutBytes + 512;
 };
 
 template <int BN, class EPI>
 __global__ void __launch_bounds__(kHaloThreads, 1)
-    k_conv_group(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, const ConvGeo g,
+    k_conv_group(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
+                const __grid_constant__ CUtensorMap mapO, const __grid_constant__ CUtensorMap mapO2, const ConvGeo g,
                  const EPI epi, int G, int *err) {
     using Cf = GroupCfg<BN>;
     constexpr int AS = Cf::AS, WS = Cf::WS, NACC = Cf::NACC;
@@ -841,7 +914,8 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     const uint32_t wbase = base + AS * Cf::A_SLOT;
-    const uint32_t bar_full = wbase + WS * Cf::W_BYTES;
+    const uint32_t obuf = wbase + WS * Cf::W_BYTES;  // the epilogue warps' output buffers
+    const uint32_t bar_full = obuf + 8 * kOutBytes;
     const uint32_t bar_empty = bar_full + 8 * AS;
     const uint32_t bar_wfull = bar_empty + 8 * AS;
     const uint32_t bar_wempty = bar_wfull + 8 * WS;
@@ -1026,6 +1100,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
         epi.prepare(epi_const, threadIdx.x - 64, 256);
         asm volatile("bar.sync 1, 256;\n" ::: "memory");  // the epilogue warps only
         const int q = warp & 3, half = (warp - 2) >> 2;
+        const uint32_t buf = obuf + (uint32_t)(warp - 2) * kOutBytes;
         int acc = 0;
         uint32_t aph = 0;
         int turn = 0;
@@ -1041,7 +1116,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
                     const int y = y0 + r / HBW, x = x0 + r % HBW;
                     const bool valid = x < g.W && y < g.H;
                     const int m = valid ? (b * g.H + y) * g.W + x : 0;
-                    if (!tc::mbar_wait(bar_afull + 8 * acc, aph, abort)) {
+                    if (!mbar_wait_warp(bar_afull + 8 * acc, aph, abort)) {
                         ok = false;
                         break;
                     }
@@ -1056,7 +1131,13 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
                         float f[16];
 #pragma unroll
                         for (int c = 0; c < 16; ++c) f[c] = __uint_as_float(v[c]);
-                        epi.store(m, nt * BN + 16 * j, f, state, epi_const, pre, valid);
+                        const int n = nt * BN + 16 * j;
+                        uint32_t p[8];
+                        epi.compute(m, n, f, state, epi_const, pre, valid, p);
+                        if (16 * j % 64 == 0) out_reuse(lane);
+                        out_put<64>(buf, lane, 16 * j % 64, p);
+                        if (16 * (j + 1) % 64 == 0)
+                            out_store(buf, epi.second(n) ? &mapO2 : &mapO, epi.column(n - 48), x0, y0 + 4 * q, b, lane);
                     }
                     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
                     __syncwarp();
@@ -1069,6 +1150,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
                 }
             }
         }
+        out_drain(lane);
     }
     __syncthreads();
     if (threadIdx.x == 0 && *abort) atomicExch(err, 1);
