@@ -28,14 +28,7 @@ __device__ __forceinline__ void pack16(const float (&w)[16], uint32_t (&p)[8]) {
 #pragma unroll
     for (int q = 0; q < 8; ++q) p[q] = pack2(w[2 * q], w[2 * q + 1]);
 }
-__device__ __forceinline__ void store16(__nv_bfloat16 *dst, const uint32_t (&p)[8]) {
-    uint4 *d4 = (uint4 *)dst;
-    d4[0] = make_uint4(p[0], p[1], p[2], p[3]);
-    d4[1] = make_uint4(p[4], p[5], p[6], p[7]);
-}
-
-// out[m][n..n+15] = relu?(v + bias) as bf16; pixel m's channels at out + m * N;
-// nb bias values (the output channels).
+// relu?(v + bias) as bf16; nb bias values (the output channels).
 // pool: also the 2x2 averages of the bf16 outputs (sums in the order of k_pool); a
 // warp has to hold 8 x 4 pixels then (k_conv_halo, k_conv_group). It saves the
 // kernel that read the output again: 120 us for the three poolings at 64 images of
@@ -44,10 +37,9 @@ __device__ __forceinline__ void store16(__nv_bfloat16 *dst, const uint32_t (&p)[
 // writing.
 struct FwdEpi {
     const float *bias;
-    __nv_bfloat16 *out;
-    int N, relu, nb;
-    __nv_bfloat16 *pool = nullptr;
-    int W = 1;
+    int relu, nb;
+    __nv_bfloat16 *pool;
+    int W;
     static constexpr int SMEM_FLOATS = 256;
     __device__ __forceinline__ void prepare(float *sm, int i, int n) const {
         for (int k = i; k < nb; k += n) sm[k] = bias[k];
@@ -59,9 +51,6 @@ struct FwdEpi {
     __device__ __forceinline__ bool writes() const { return true; }
     __device__ __forceinline__ bool second(int) const { return false; }
     __device__ __forceinline__ int column(int n) const { return n; }
-    __device__ __forceinline__ void write(int m, int n, const uint32_t (&p)[8]) const {
-        store16(out + (long long)m * N + n, p);
-    }
     __device__ __forceinline__ void pack(int n, const float (&v)[16], const float *sm, uint32_t (&p)[8]) const {
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
@@ -133,15 +122,15 @@ struct FwdEpi {
 };
 
 // The last convolution (32 channels, ReLU) with the 1x1 head and the input
-// skip: d[m][:] = bf16(relu(v + bias)) as FwdEpi (not stored when out is
-// null: inference needs only y), and
+// skip: d[m][:] = bf16(relu(v + bias)) as FwdEpi (stored for the
+// backward pass only: inference needs y alone), and
 // y[m] = f[m] (mask[m] != 0) + hb + sum_c hw[c] d[m][c] (FP32, c in order).
 struct HeadEpi {
     const float *bias;
-    __nv_bfloat16 *out;
     const float *hw, *hb, *f;
     const uint8_t *mask;
     float *y;
+    bool keep;  // d is wanted
     static constexpr int SMEM_FLOATS = 65;  // bias[32], hw[32], hb
     __device__ __forceinline__ void prepare(float *sm, int i, int n) const {
         for (int k = i; k < 65; k += n) sm[k] = k < 32 ? bias[k] : k < 64 ? hw[k - 32] : hb[0];
@@ -153,12 +142,9 @@ struct HeadEpi {
     };
     __device__ __forceinline__ Pre prefetch(int, int) const { return {}; }
     __device__ __forceinline__ PrePix prefetch_pixel(int m) const { return {f[m], mask[m]}; }
-    __device__ __forceinline__ bool writes() const { return out != nullptr; }
+    __device__ __forceinline__ bool writes() const { return keep; }
     __device__ __forceinline__ bool second(int) const { return false; }
     __device__ __forceinline__ int column(int n) const { return n; }
-    __device__ __forceinline__ void write(int m, int n, const uint32_t (&p)[8]) const {
-        store16(out + (long long)m * 32 + n, p);
-    }
     __device__ __forceinline__ void compute(int, int n, const float (&v)[16], float &st, const float *sm, Pre, bool,
                                             uint32_t (&p)[8]) const {
         float w[16];
@@ -182,12 +168,11 @@ struct HeadEpi {
     }
 };
 
-// Data gradient: columns < split go to din (times (act > 0) when act is
-// given), the others to din2; N columns in all.
+// Data gradient: columns < split go to the first tensor (times (act > 0) when act
+// is given), the others to the second.
 struct DgradEpi {
     const __nv_bfloat16 *act;
-    __nv_bfloat16 *din, *din2;
-    int split, N;
+    int split;
     static constexpr int SMEM_FLOATS = 1;
     __device__ __forceinline__ void prepare(float *, int, int) const {}
     struct Pre {
@@ -207,9 +192,6 @@ struct DgradEpi {
     __device__ __forceinline__ bool writes() const { return true; }
     __device__ __forceinline__ bool second(int n) const { return n >= split; }
     __device__ __forceinline__ int column(int n) const { return n < split ? n : n - split; }
-    __device__ __forceinline__ void write(int m, int n, const uint32_t (&p)[8]) const {
-        store16(n < split ? din + (long long)m * split + n : din2 + (long long)m * (N - split) + (n - split), p);
-    }
     __device__ __forceinline__ void compute(int, int n, const float (&v)[16], float &, const float *, const Pre &a, bool,
                                             uint32_t (&p)[8]) const {
         float w[16];
@@ -261,75 +243,6 @@ int *fault_ptr() {
     return (int *)p;
 }
 
-// Tile shape: bw x bh = 128 pixels of one image.
-bool tile_shape(int H, int W, int &bw, int &bh) {
-    bw = W >= 128 ? 128 : W;
-    if (bw < 1 || W % bw || 128 % bw) return false;
-    bh = 128 / bw;
-    return H % bh == 0;
-}
-
-template <int BN, int CK, class EPI>
-cudaError_t launch(const __nv_bfloat16 *A, int B, int H, int W, int C, const __nv_bfloat16 *wmat, int N, int flip,
-                   const EPI &epi, cudaStream_t s) {
-    using Cf = tma::Cfg<BN, CK>;
-    int bw, bh;
-    if (!tile_shape(H, W, bw, bh) || C % CK || N % BN) return cudaErrorNotSupported;
-    auto enc = encoder();
-    const int nsm = sm_count();
-    int *err = fault_ptr();
-    if (!enc || nsm <= 0 || !err) return cudaErrorNotSupported;
-    CUtensorMap ma, mb;
-    {
-        const cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B};
-        const cuuint64_t strides[3] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2, (cuuint64_t)H * W * C * 2};
-        const cuuint32_t box[4] = {(cuuint32_t)CK, (cuuint32_t)bw, (cuuint32_t)bh, 1};
-        const cuuint32_t es[4] = {1, 1, 1, 1};
-        if (enc(&ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void *)A, dims, strides, box, es,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CK == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
-                CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return cudaErrorInvalidValue;
-    }
-    {
-        const cuuint64_t dims[2] = {(cuuint64_t)9 * C, (cuuint64_t)N};
-        const cuuint64_t strides[1] = {(cuuint64_t)9 * C * 2};
-        const cuuint32_t box[2] = {(cuuint32_t)CK, (cuuint32_t)BN};
-        const cuuint32_t es[2] = {1, 1};
-        if (enc(&mb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void *)wmat, dims, strides, box, es,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CK == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
-                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return cudaErrorInvalidValue;
-    }
-    tma::ConvGeo g;
-    g.B = B;
-    g.H = H;
-    g.W = W;
-    g.C = C;
-    g.bw = bw;
-    g.bh = bh;
-    g.tiles_x = W / bw;
-    g.tiles_y = H / bh;
-    g.mtiles = B * g.tiles_x * g.tiles_y;
-    g.ntiles = N / BN;
-    g.tiles = g.mtiles * g.ntiles;
-    g.nchunk = C / CK;
-    g.KB = 9 * g.nchunk;
-    g.flip = flip;
-    auto *fn = &tma::k_conv_tma<BN, CK, EPI>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, Cf::SMEM);
-    if (e != cudaSuccess) return e;
-    const int grid = g.tiles < nsm ? g.tiles : nsm;
-    fn<<<grid, 192, Cf::SMEM, s>>>(ma, mb, g, epi, err);
-    return cudaGetLastError();
-}
-
-// Whether the kernels with 8 x 16 tiles take an image: at most half of the tiles'
-// pixels outside it.
-bool box_shape(int H, int W) {
-    const long long px = (long long)((W + tma::HBW - 1) / tma::HBW * tma::HBW) * ((H + tma::HBH - 1) / tma::HBH * tma::HBH);
-    return px <= 2LL * W * H;
-}
-
 // The tensors a kernel's output boxes go to (second: the columns from the first's
 // last on; no tensor: p null), and their maps: 8 or 16 pixels of 4 image rows, ob channels.
 struct OutTensor {
@@ -358,12 +271,15 @@ bool out_maps(PFN_cuTensorMapEncodeTiled_v12000 enc, const OutTensors &o, int B,
     return true;
 }
 
+// Images whose narrow layers are summed blocks first (conv_tma.cuh, SumOrder).
+bool whole_tiles(int H, int W) { return W % 16 == 0 && H % 8 == 0; }
+
 // Narrow layers: 8 x 16 tiles, halo boxes, weights resident in shared memory.
 template <int BN, int CK, class EPI>
 cudaError_t launch_halo(const __nv_bfloat16 *A, int B, int H, int W, int C, const __nv_bfloat16 *wmat, int N, int flip,
                         const EPI &epi, const OutTensors &o, cudaStream_t s) {
     using Cf = tma::HaloCfg<BN, CK>;
-    if (!box_shape(H, W) || C % CK || N % BN) return cudaErrorNotSupported;
+    if (C % CK || N % BN) return cudaErrorNotSupported;
     const int nblk = 9 * (C / CK);
     const int wbytes = nblk * Cf::BBLK;
     int S = (Cf::SMEM_BUDGET - wbytes) / Cf::STAGE;
@@ -408,8 +324,10 @@ cudaError_t launch_halo(const __nv_bfloat16 *A, int B, int H, int W, int C, cons
     g.ntiles = N / BN;
     g.tiles = g.mtiles * g.ntiles;
     g.nchunk = C / CK;
-    g.KB = 3 * g.nchunk;
+    g.KB = g.nchunk;
     g.flip = flip;
+    g.order = whole_tiles(H, W) ? tma::ORDER_BLOCKS : tma::ORDER_TAPS;
+    if (g.order == tma::ORDER_TAPS && S < g.nchunk) return cudaErrorNotSupported;
     const int smem = 1024 + wbytes + S * Cf::STAGE + 8 * tma::kOutBytes + 256;
     auto *fn = &tma::k_conv_halo<BN, CK, EPI>;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -427,7 +345,7 @@ template <class EPI>
 cudaError_t launch_pair(const __nv_bfloat16 *A, int B, int H, int W, int C, const __nv_bfloat16 *wmat, int flip,
                         const EPI &epi, const OutTensors &o, cudaStream_t s) {
     using Cf = tma::PairCfg;
-    if (W % 2 || !box_shape(H, W / 2) || C % 32) return cudaErrorNotSupported;
+    if (W % 2 || C % 32) return cudaErrorNotSupported;
     const int nblk = 9 * (C / 32);
     const int wbytes = nblk * Cf::BBLK;
     int S = (Cf::SMEM_BUDGET - wbytes) / Cf::STAGE;
@@ -452,6 +370,9 @@ cudaError_t launch_pair(const __nv_bfloat16 *A, int B, int H, int W, int C, cons
     g.nchunk = C / 32;
     g.KB = g.nchunk;
     g.flip = flip;
+    g.order = !whole_tiles(H, W) ? tma::ORDER_TAPS : C % 64 ? tma::ORDER_BLOCKS : tma::ORDER_OFFSETS;
+    if (g.order == tma::ORDER_OFFSETS && C > 64) return cudaErrorNotSupported;  // blocks of 64 in between
+    if (g.order != tma::ORDER_BLOCKS && S < g.nchunk) return cudaErrorNotSupported;
     CUtensorMap ma, mb, mo[2] = {};
     if (!out_maps(enc, o, B, H, W, 32, 2 * tma::HBW, mo)) return cudaErrorNotSupported;
     {
@@ -488,13 +409,13 @@ template <int BN, class EPI>
 cudaError_t launch_group(const __nv_bfloat16 *A, int B, int H, int W, int C, const __nv_bfloat16 *wmat, int N, int flip,
                          const EPI &epi, const OutTensors &o, cudaStream_t s) {
     using Cf = tma::GroupCfg<BN>;
-    if (!box_shape(H, W) || C % 64 || N % BN) return cudaErrorNotSupported;
+    if (C % 64 || N % BN) return cudaErrorNotSupported;
     auto enc = encoder();
     const int nsm = sm_count();
     int *err = fault_ptr();
     if (!enc || nsm <= 0 || !err) return cudaErrorNotSupported;
     CUtensorMap ma, mb, mo[2] = {};
-    if (!out_maps(enc, o, B, H, W, 64, tma::HBW, mo)) return cudaErrorNotSupported;
+    if (!out_maps(enc, o, B, H, W, Cf::OB, tma::HBW, mo)) return cudaErrorNotSupported;
     {
         const cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B};
         const cuuint64_t strides[3] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2, (cuuint64_t)H * W * C * 2};
@@ -528,17 +449,26 @@ cudaError_t launch_group(const __nv_bfloat16 *A, int B, int H, int W, int C, con
     g.ntiles = N / BN;
     g.tiles = g.mtiles * g.ntiles;
     g.nchunk = C / 64;
-    g.KB = 3 * g.nchunk;
+    g.KB = 9 * g.nchunk;
     g.flip = flip;
+    g.order = tma::ORDER_TAPS;
+    if (g.nchunk > Cf::AMAX) return cudaErrorNotSupported;  // a tile's boxes stay for all taps
     // as many tiles a group as leave every SM one
     int G = g.tiles / nsm;
     if (G > Cf::GMAX) G = Cf::GMAX;
+    if (G > Cf::AMAX / g.nchunk) G = Cf::AMAX / g.nchunk;
     if (G < 1) G = 1;
+    // boxes of a group and up to three (one of four or more) of the next, the rest for weights
+    const int boxes = G * g.nchunk, more = g.nchunk >= 4 ? 1 : boxes < 3 ? boxes : 3;
+    const int AS = boxes + more < Cf::AMAX ? boxes + more : Cf::AMAX;
+    int WS = (Cf::SMEM_BUDGET - AS * Cf::A_SLOT) / Cf::W_BYTES;
+    if (WS > Cf::WMAX) WS = Cf::WMAX;
+    const int smem = Cf::SMEM_REST + AS * Cf::A_SLOT + WS * Cf::W_BYTES;
     const int groups = (g.mtiles + G - 1) / G * g.ntiles;
     auto *fn = &tma::k_conv_group<BN, EPI>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, Cf::SMEM);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    fn<<<groups < nsm ? groups : nsm, tma::kHaloThreads, Cf::SMEM, s>>>(ma, mb, mo[0], mo[1], g, epi, G, err);
+    fn<<<groups < nsm ? groups : nsm, tma::kHaloThreads, smem, s>>>(ma, mb, mo[0], mo[1], g, epi, G, AS, WS, err);
     return cudaGetLastError();
 }
 
@@ -603,12 +533,12 @@ cudaError_t launch_wgrad(const __nv_bfloat16 *x, int B, int H, int W, int C, con
 namespace se2n {
 namespace nn {
 
-cudaError_t conv_wgrad_tma(const __nv_bfloat16 *x, int B, int H, int W, int C, const __nv_bfloat16 *gz, int Cout,
-                           float *dw, cudaStream_t s) {
+cudaError_t conv_wgrad(const __nv_bfloat16 *x, int B, int H, int W, int C, const __nv_bfloat16 *gz, int Cout, float *dw,
+                       cudaStream_t s) {
     return launch_wgrad(x, B, H, W, C, gz, Cout, dw, s);
 }
 
-cudaError_t tma_fault(int *host_flag, bool reset) {
+cudaError_t tc_fault(int *host_flag, bool reset) {
     cudaError_t e = cudaMemcpyFromSymbol(host_flag, g_tma_fault, sizeof(int));
     if (e == cudaSuccess && reset && *host_flag) {
         const int zero = 0;
@@ -617,85 +547,41 @@ cudaError_t tma_fault(int *host_flag, bool reset) {
     return e;
 }
 
-cudaError_t conv_forward_tma(const __nv_bfloat16 *in, int B, int H, int W, int Cin, const __nv_bfloat16 *w,
-                             const float *bias, int Cout, int relu, __nv_bfloat16 *out, int ldo, const HeadArgs *head,
-                             cudaStream_t s, __nv_bfloat16 *pool, bool *pooled) {
-    const bool ck64 = Cin % 64 == 0;
-    if (head) {
-        if (Cout != 32 || !relu || ldo != 32) return cudaErrorNotSupported;
-        const OutTensors o{{{out, 32, 32}, {nullptr, 0, 0}}};
-        const HeadEpi epi{bias, out, head->hw, head->hb, head->f, head->mask, head->y};
-        const cudaError_t e = launch_pair(in, B, H, W, Cin, w, 0, epi, o, s);
-        if (e != cudaErrorNotSupported) return e;
-        return ck64 ? launch<32, 64>(in, B, H, W, Cin, w, Cout, 0, epi, s)
-                    : launch<32, 32>(in, B, H, W, Cin, w, Cout, 0, epi, s);
-    }
-    // the kernels with 8 x 16 tiles write the averages too
+cudaError_t conv_forward(const __nv_bfloat16 *in, int B, int H, int W, int Cin, const __nv_bfloat16 *w,
+                         const float *bias, int Cout, int relu, __nv_bfloat16 *out, int ldo, __nv_bfloat16 *pool,
+                         cudaStream_t s) {
     const OutTensors o{{{out, Cout, ldo}, {nullptr, 0, 0}}};
-    FwdEpi fepi{bias, out, ldo, relu, Cout};
-    fepi.pool = pool;
-    fepi.W = W;
-    cudaError_t e = cudaErrorNotSupported;
-    if (Cout == 32)
-        e = launch_pair(in, B, H, W, Cin, w, 0, fepi, o, s);
-    else if (Cout == 64)
-        e = ck64 ? launch_halo<64, 64>(in, B, H, W, Cin, w, Cout, 0, fepi, o, s)
-                 : launch_halo<64, 32>(in, B, H, W, Cin, w, Cout, 0, fepi, o, s);
-    if (e == cudaErrorNotSupported && ck64 && Cout % 64 == 0)
-        e = launch_wide(in, B, H, W, Cin, w, Cout, 0, fepi, o, s);
-    if (e != cudaErrorNotSupported) {
-        if (pooled) *pooled = pool != nullptr;
-        return e;
+    const FwdEpi epi{bias, relu, Cout, pool, W};
+    if (Cout == 32) return launch_pair(in, B, H, W, Cin, w, 0, epi, o, s);
+    if (Cout == 64) {
+        const cudaError_t e = Cin % 64 == 0 ? launch_halo<64, 64>(in, B, H, W, Cin, w, Cout, 0, epi, o, s)
+                                            : launch_halo<64, 32>(in, B, H, W, Cin, w, Cout, 0, epi, o, s);
+        if (e != cudaErrorNotSupported) return e;  // more weights than shared memory holds
     }
-    const FwdEpi epi{bias, out, ldo, relu, Cout};
-    switch (Cout) {
-        case 32: return ck64 ? launch<32, 64>(in, B, H, W, Cin, w, Cout, 0, epi, s)
-                             : launch<32, 32>(in, B, H, W, Cin, w, Cout, 0, epi, s);
-        case 64: return ck64 ? launch<64, 64>(in, B, H, W, Cin, w, Cout, 0, epi, s)
-                             : launch<64, 32>(in, B, H, W, Cin, w, Cout, 0, epi, s);
-        case 128: return ck64 ? launch<128, 64>(in, B, H, W, Cin, w, Cout, 0, epi, s) : cudaErrorNotSupported;
-        case 256: return ck64 ? launch<256, 64>(in, B, H, W, Cin, w, Cout, 0, epi, s) : cudaErrorNotSupported;
-        default: return cudaErrorNotSupported;
-    }
+    return launch_wide(in, B, H, W, Cin, w, Cout, 0, epi, o, s);
 }
 
-cudaError_t conv_dgrad_tma(const __nv_bfloat16 *gz, int B, int H, int W, int Cout, const __nv_bfloat16 *wt, int Cin,
-                           const __nv_bfloat16 *act, __nv_bfloat16 *din, __nv_bfloat16 *din2, int split,
-                           cudaStream_t s) {
+cudaError_t conv_forward_head(const __nv_bfloat16 *in, int B, int H, int W, int Cin, const __nv_bfloat16 *w,
+                              const float *bias, __nv_bfloat16 *out, const HeadArgs &head, cudaStream_t s) {
+    const OutTensors o{{{out, 32, 32}, {nullptr, 0, 0}}};
+    const HeadEpi epi{bias, head.hw, head.hb, head.f, head.mask, head.y, out != nullptr};
+    return launch_pair(in, B, H, W, Cin, w, 0, epi, o, s);
+}
+
+cudaError_t conv_dgrad(const __nv_bfloat16 *gz, int B, int H, int W, int Cout, const __nv_bfloat16 *wt, int Cin,
+                       const __nv_bfloat16 *act, __nv_bfloat16 *din, __nv_bfloat16 *din2, int split, cudaStream_t s) {
     if (split % 16) return cudaErrorNotSupported;
-    const bool ck64 = Cout % 64 == 0;
-    const DgradEpi epi{act, din, din2, split, Cin};
+    const DgradEpi epi{act, split};
     const OutTensors o{{{din, split, split}, {split < Cin ? din2 : nullptr, Cin - split, Cin - split}}};
     // A = gz (Cout channels, taps mirrored), B = wt [Cin][9 Cout]
-    if (Cin == 32 || Cin == 64 || Cin == 96) {
-        cudaError_t e = cudaErrorNotSupported;
-        if (Cin == 32)
-            e = launch_pair(gz, B, H, W, Cout, wt, 1, epi, o, s);
-        else if (Cin == 64)
-            e = ck64 ? launch_halo<64, 64>(gz, B, H, W, Cout, wt, Cin, 1, epi, o, s)
-                     : launch_halo<64, 32>(gz, B, H, W, Cout, wt, Cin, 1, epi, o, s);
-        else if (!ck64)
-            e = launch_halo<96, 32>(gz, B, H, W, Cout, wt, Cin, 1, epi, o, s);
+    if (Cin == 32) return launch_pair(gz, B, H, W, Cout, wt, 1, epi, o, s);
+    if (Cin == 96) return launch_halo<96, 32>(gz, B, H, W, Cout, wt, Cin, 1, epi, o, s);
+    if (Cin == 64) {
+        const cudaError_t e = Cout % 64 == 0 ? launch_halo<64, 64>(gz, B, H, W, Cout, wt, Cin, 1, epi, o, s)
+                                             : launch_halo<64, 32>(gz, B, H, W, Cout, wt, Cin, 1, epi, o, s);
         if (e != cudaErrorNotSupported) return e;
     }
-    if (!ck64) {
-        if (Cin == 32) return launch<32, 32>(gz, B, H, W, Cout, wt, Cin, 1, epi, s);
-        if (Cin == 96) return launch<96, 32>(gz, B, H, W, Cout, wt, Cin, 1, epi, s);
-        return cudaErrorNotSupported;
-    }
-    if (Cin % 64 == 0) {
-        const cudaError_t e = launch_wide(gz, B, H, W, Cout, wt, Cin, 1, epi, o, s);
-        if (e != cudaErrorNotSupported) return e;
-    }
-    switch (Cin) {
-        case 32: return launch<32, 64>(gz, B, H, W, Cout, wt, Cin, 1, epi, s);
-        case 64: return launch<64, 64>(gz, B, H, W, Cout, wt, Cin, 1, epi, s);
-        case 128: return launch<128, 64>(gz, B, H, W, Cout, wt, Cin, 1, epi, s);
-        case 192:
-        case 384: return launch<192, 64>(gz, B, H, W, Cout, wt, Cin, 1, epi, s);
-        case 256: return launch<256, 64>(gz, B, H, W, Cout, wt, Cin, 1, epi, s);
-        default: return cudaErrorNotSupported;
-    }
+    return launch_wide(gz, B, H, W, Cout, wt, Cin, 1, epi, o, s);
 }
 
 }  // namespace nn

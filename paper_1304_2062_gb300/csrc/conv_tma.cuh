@@ -5,25 +5,21 @@
 //   k = tap * C + c,  A(m, tap * C + c) = In[pixel m shifted by tap][c],
 //   B = a K-major [N][9 C] weight matrix.
 //
-// Tiles of D are 128 pixels (a bw x bh rectangle of one image, bw * bh = 128)
-// by BN channels. The K loop runs over (tap, CK-channel chunk) blocks; for
-// each block one TMA box load brings the tile's 128 pixels shifted by the
-// tap (the tensor map's out-of-bounds zero fill is the convolution's
-// padding) and one brings the matching BN x CK weights, both in the
-// swizzled K-major layout the tensor core reads (CK = 64: 128-byte swizzle;
-// CK = 32: 64-byte swizzle).
+// Tiles of D are 128 pixels (8 x 16 of one image; pairs of pixels with 32 output
+// channels) by BN channels. TMA boxes bring the pixels around a tile, CK channels at a
+// time, and BN x CK weights a tap, in the swizzled K-major layout the tensor core reads
+// (CK = 64: 128-byte swizzle; CK = 32: 64-byte swizzle); the tensor map's out-of-bounds
+// zero fill is the convolution's padding.
 //
-// Roles (192 threads, one CTA per SM, tiles strided over CTAs):
-//   warp 0, one thread   TMA producer: fills a ring of STAGES stages, each
-//                        guarded by a "full" (transaction bytes) and an
-//                        "empty" (tensor core done) mbarrier;
-//   warp 1               allocates 2 x BN tensor-memory columns; one elected
-//                        lane issues tcgen05.mma (M = 128, N = BN, K = 16) into
-//                        one of two accumulators and commits to "empty" per
-//                        stage and to "acc full" per tile;
-//   warps 2-5            epilogue: tcgen05.ld of the accumulator rows their
-//                        lane quarter may access, then the functor EPI, then
-//                        "acc empty", so the next tile's MMAs overlap it.
+// Roles (one CTA per SM, tiles strided over CTAs):
+//   warp 0, one thread   TMA producer: fills a ring of stages, each guarded by a "full"
+//                        (transaction bytes) and an "empty" (tensor core done) mbarrier;
+//   warp 1               allocates tensor memory and issues tcgen05.mma (M = 128, K = 16)
+//                        into one of several accumulators, committing to "empty" per stage
+//                        and to "acc full" per tile;
+//   warps 2-9            epilogue, two groups of four: tcgen05.ld of the accumulator rows
+//                        their lane quarter may access, the functor EPI, "acc empty" (so the
+//                        next tiles' MMAs overlap it), and a TMA store.
 //
 // Every wait is bounded (about 2 s at the full clock). One that runs out sets *err and the
 // shared abort flag; the CTA then stops, lets what it issued complete
@@ -41,6 +37,19 @@ namespace se2n {
 namespace nn {
 namespace tma {
 
+// The order in which an output's products of 16 channels are added. It is part of the
+// result: another one moves a few stored BF16 values across a rounding boundary, and
+// that spreads (a different order in one layer changes the network's output by 2e-3). With
+// up to 64 (32 for 96 of them) channels a block and 32 or 64 outputs, images of whole 16 x 8
+// tiles have always been summed blocks first, then horizontal and vertical offsets of the
+// source; everything else taps first, then channels (taps of the weights: the source
+// offsets run backwards where they are mirrored).
+enum SumOrder {
+    ORDER_BLOCKS = 0,  // (32- or 64-channel block of the kernel, sx, sy)
+    ORDER_OFFSETS = 1, // (sx, sy, block): a 64-channel block in blocks of 32
+    ORDER_TAPS = 2     // (tap, block)
+};
+
 // Geometry of one convolution launch (passed by value).
 struct ConvGeo {
     int B, H, W, C;      // A tensor: B images of H x W pixels, C channels
@@ -49,32 +58,17 @@ struct ConvGeo {
     int nchunk;          // C / CK
     int KB;              // 9 * nchunk
     int flip;            // 1: taps mirrored (data gradient)
+    int order;           // of the sums: SumOrder
 };
 
-template <int BN, int CK>
-struct Cfg {
-    static_assert(CK == 32 || CK == 64, "channel chunk of 32 (64-byte swizzle) or 64 (128-byte swizzle)");
-    static_assert(BN % 16 == 0 && BN >= 16 && BN <= 256, "tcgen05 M=128 needs N in [16, 256], N % 16 == 0");
-    static constexpr int A_BYTES = 128 * CK * 2;
-    static constexpr int B_BYTES = BN * CK * 2;
-    static constexpr int STAGE = A_BYTES + B_BYTES;
-    static constexpr int STAGES = (196608 / STAGE) > 12 ? 12 : (196608 / STAGE);
-    // two accumulators, each at a power-of-two column offset
-    static constexpr int ACC_COLS = BN <= 16 ? 16 : BN <= 32 ? 32 : BN <= 64 ? 64 : BN <= 128 ? 128 : 256;
-    static constexpr int TMEM_COLS = 2 * ACC_COLS < 32 ? 32 : 2 * ACC_COLS;
-    static constexpr int SMEM = 1024 + STAGES * STAGE + 256;
-    static constexpr uint32_t SBO = 8 * CK * 2;              // 8-row atom
-    static constexpr uint64_t LAYOUT = CK == 64 ? 2 : 4;     // SWIZZLE_128B / SWIZZLE_64B
-};
-
-template <int BN, int CK>
+// K-major matrix descriptor of dense rows of CK channels (8-row atoms).
+template <int CK>
 __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
-    using C = Cfg<BN, CK>;
     uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
     d |= (uint64_t)(16u >> 4) << 16;
-    d |= (uint64_t)(C::SBO >> 4) << 32;
+    d |= (uint64_t)((uint32_t)(8 * CK * 2) >> 4) << 32;
     d |= (uint64_t)1 << 46;
-    d |= C::LAYOUT << 61;
+    d |= (uint64_t)(CK == 64 ? 2 : 4) << 61;
     return d;
 }
 
@@ -111,6 +105,32 @@ __device__ __forceinline__ void mma_f16_elect(uint32_t tmem_d, uint64_t adesc, u
         " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
 }
+// NK products of 16 channels each, both operands 32 bytes further on every time. One
+// election and one block of instructions: what the issuing warp spends on a product
+// (some ten instructions with an election each, 50 cycles) is as much as the product takes
+// with 32 or 64 columns.
+template <int NK>
+__device__ __forceinline__ void mma_chain_elect(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                                uint32_t accumulate) {
+    static_assert(NK == 2 || NK == 4, "32 or 64 channels");
+    if constexpr (NK == 2)
+        asm volatile(
+            "{\n .reg .pred p, q, t;\n .reg .b64 a, b;\n setp.ne.b32 p, %4, 0;\n setp.eq.b32 t, 0, 0;\n"
+            " elect.sync _|q, 0xffffffff;\n add.s64 a, %1, 2;\n add.s64 b, %2, 2;\n"
+            " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
+            " @q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, t;\n}\n" ::"r"(tmem_d),
+            "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
+    else
+        asm volatile(
+            "{\n .reg .pred p, q, t;\n .reg .b64 a, b, c, d, e, f;\n setp.ne.b32 p, %4, 0;\n setp.eq.b32 t, 0, 0;\n"
+            " elect.sync _|q, 0xffffffff;\n add.s64 a, %1, 2;\n add.s64 b, %2, 2;\n add.s64 c, %1, 4;\n"
+            " add.s64 d, %2, 4;\n add.s64 e, %1, 6;\n add.s64 f, %2, 6;\n"
+            " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
+            " @q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, t;\n"
+            " @q tcgen05.mma.cta_group::1.kind::f16 [%0], c, d, %3, t;\n"
+            " @q tcgen05.mma.cta_group::1.kind::f16 [%0], e, f, %3, t;\n}\n" ::"r"(tmem_d),
+            "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
+}
 __device__ __forceinline__ void mma_commit_elect(uint32_t bar) {
     asm volatile(
         "{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n"
@@ -143,184 +163,8 @@ __device__ __forceinline__ void tile_origin(const ConvGeo &g, int t, int &b, int
 //                                      for lanes without one
 //   compute_pair(m, n, v[2][16], float (&state)[2], sm, pre, pre1, valid, p[2][8])  the same of
 //                                      pixels m and m + 1 (k_conv_pair)
-//   write(m, n, p[8])                 stores them (k_conv_tma; the other kernels write boxes)
 //   writes(), second(n), column(n)    whether they are wanted, in which tensor column n goes and where
 //   finish(m, float state, sm, pre)   after the last column group of pixel m
-template <int BN, int CK, class EPI>
-__global__ void __launch_bounds__(192, 1)
-    k_conv_tma(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, const ConvGeo g,
-               const EPI epi, int *err) {
-    using Cf = Cfg<BN, CK>;
-    constexpr int S = Cf::STAGES;
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    const uint32_t raw = smem_u32(smem_raw);
-    const uint32_t base = (raw + 1023u) & ~1023u;
-    const uint32_t bar_full = base + S * Cf::STAGE;
-    const uint32_t bar_empty = bar_full + 8 * S;
-    const uint32_t bar_afull = bar_empty + 8 * S;   // 2
-    const uint32_t bar_aempty = bar_afull + 16;     // 2
-    const uint32_t tmem_slot = bar_aempty + 16;
-    volatile int *abort = (volatile int *)(smem_raw + (tmem_slot + 4 - raw));
-    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
-
-    if (threadIdx.x == 0) {
-        *abort = *(volatile int *)err;
-        for (int s = 0; s < S; ++s) {
-            tc::mbar_init(bar_full + 8 * s, 1);
-            tc::mbar_init(bar_empty + 8 * s, 1);
-        }
-        for (int a = 0; a < 2; ++a) {
-            tc::mbar_init(bar_afull + 8 * a, 1);
-            tc::mbar_init(bar_aempty + 8 * a, 4);
-        }
-        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-        asm volatile("prefetch.tensormap [%0];\n" ::"l"((uint64_t)&mapA) : "memory");
-        asm volatile("prefetch.tensormap [%0];\n" ::"l"((uint64_t)&mapB) : "memory");
-    }
-    __syncthreads();
-    if (*abort) return;
-    if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(tmem_slot),
-                     "r"((uint32_t)Cf::TMEM_COLS));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::);
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    uint32_t tmem_base;
-    asm volatile("ld.shared.u32 %0, [%1];\n" : "=r"(tmem_base) : "r"(tmem_slot));
-    tmem_base = __shfl_sync(0xffffffffu, tmem_base, 0);
-
-    if (warp == 0) {
-        if (lane == 0) {
-            // ---------------- TMA producer ----------------
-            int s = 0;
-            uint32_t ph = 0;
-            bool ok = true;
-            for (int t = blockIdx.x; t < g.tiles && ok; t += gridDim.x) {
-                int b, x0, y0, nt;
-                tile_origin(g, t, b, x0, y0, nt);
-                for (int kb = 0; kb < g.KB; ++kb) {
-                    const int tap = kb / g.nchunk, ch = kb - tap * g.nchunk;
-                    int dy = tap / 3 - 1, dx = tap % 3 - 1;
-                    if (g.flip) {
-                        dy = -dy;
-                        dx = -dx;
-                    }
-                    if (!tc::mbar_wait(bar_empty + 8 * s, ph ^ 1u, abort)) {
-                        ok = false;
-                        break;
-                    }
-                    const uint32_t sa = base + s * Cf::STAGE, sb = sa + Cf::A_BYTES;
-                    arrive_expect_tx(bar_full + 8 * s, Cf::STAGE);
-                    tma_load_4d(sa, &mapA, ch * CK, x0 + dx, y0 + dy, b, bar_full + 8 * s);
-                    tma_load_2d(sb, &mapB, tap * g.C + ch * CK, nt * BN, bar_full + 8 * s);
-                    if (++s == S) {
-                        s = 0;
-                        ph ^= 1u;
-                    }
-                }
-            }
-            if (!ok) {
-                // loads already issued finish on their own within microseconds
-                const long long t0 = clock64();
-                while (clock64() - t0 < 200000LL) {
-                }
-            }
-        }
-    } else if (warp == 1) {
-        {  // the whole warp
-            // ---------------- MMA issuer ----------------
-            constexpr uint32_t IDESC = tc::idesc_bf16_f32<BN>();
-            const uint64_t base_desc = sdesc<BN, CK>(base);
-            int s = 0, acc = 0;
-            uint32_t ph = 0, aph = 0;
-            bool ok = true;
-            uint32_t last_bar = 0, last_par = 0;
-            for (int t = blockIdx.x; t < g.tiles && ok; t += gridDim.x) {
-                if (!mbar_wait_warp(bar_aempty + 8 * acc, aph ^ 1u, abort)) {
-                    ok = false;
-                    break;
-                }
-                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                const uint32_t d = tmem_base + (uint32_t)(acc * Cf::ACC_COLS);
-                for (int kb = 0; kb < g.KB; ++kb) {
-                    if (!mbar_wait_warp(bar_full + 8 * s, ph, abort)) {
-                        ok = false;
-                        break;
-                    }
-                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                    const uint32_t sa = base + s * Cf::STAGE, sb = sa + Cf::A_BYTES;
-                    const uint64_t da = base_desc + ((sa - base) >> 4), db = base_desc + ((sb - base) >> 4);
-#pragma unroll
-                    for (int kk = 0; kk < CK / 16; ++kk)
-                        mma_f16_elect(d, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), IDESC, (kb > 0 || kk > 0) ? 1u : 0u);
-                    mma_commit_elect(bar_empty + 8 * s);
-                    last_bar = bar_empty + 8 * s;
-                    last_par = ph;
-                    if (++s == S) {
-                        s = 0;
-                        ph ^= 1u;
-                    }
-                }
-                if (!ok) break;
-                mma_commit_elect(bar_afull + 8 * acc);
-                if (++acc == 2) {
-                    acc = 0;
-                    aph ^= 1u;
-                }
-            }
-            if (!ok && last_bar) tc::mbar_wait(last_bar, last_par, nullptr);  // tensor core idle before release
-        }
-    } else {
-        // ---------------- epilogue (warps 2..5) ----------------
-        __shared__ float epi_const[EPI::SMEM_FLOATS];
-        epi.prepare(epi_const, threadIdx.x - 64, 128);
-        asm volatile("bar.sync 1, 128;\n" ::: "memory");  // the four epilogue warps only
-        const int q = warp & 3;  // lane quarter this warp may read
-        int acc = 0;
-        uint32_t aph = 0;
-        for (int t = blockIdx.x; t < g.tiles; t += gridDim.x) {
-            if (!mbar_wait_warp(bar_afull + 8 * acc, aph, abort)) break;
-            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-            int b, x0, y0, nt;
-            tile_origin(g, t, b, x0, y0, nt);
-            const int r = q * 32 + lane;
-            const int y = y0 + r / g.bw, x = x0 + r % g.bw;
-            const int m = (b * g.H + y) * g.W + x;
-            const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * Cf::ACC_COLS);
-            float state = 0.0f;
-#pragma unroll 1
-            for (int j0 = 0; j0 < BN; j0 += 16) {
-                uint32_t v[16];
-                tc::tmem_ld16(taddr + (uint32_t)j0, v);
-                float f[16];
-#pragma unroll
-                for (int i = 0; i < 16; ++i) f[i] = __uint_as_float(v[i]);
-                uint32_t p[8];
-                epi.compute(m, nt * BN + j0, f, state, epi_const, epi.prefetch(m, nt * BN + j0), true, p);
-                if (epi.writes()) epi.write(m, nt * BN + j0, p);
-            }
-            epi.finish(m, state, epi_const, epi.prefetch_pixel(m));
-            asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-            __syncwarp();
-            if (lane == 0) arrive(bar_aempty + 8 * acc);
-            if (++acc == 2) {
-                acc = 0;
-                aph ^= 1u;
-            }
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0 && *abort) atomicExch(err, 1);
-    if (warp == 1) {
-        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_base),
-                     "r"((uint32_t)Cf::TMEM_COLS));
-    }
-}
-
-
 // ---------------------------------------------------------------------------
 // Narrow layers (64 or 96 output channels): halo boxes and resident weights.
 //
@@ -501,7 +345,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
         {  // the whole warp
             // ---------------- MMA issuer ----------------
             constexpr uint32_t IDESC = tc::idesc_bf16_f32<BN>();
-            const uint64_t a_desc0 = sdesc_box<CK>(stages), w_desc0 = sdesc<BN, CK>(wres);
+            const uint64_t a_desc0 = sdesc_box<CK>(stages), w_desc0 = sdesc<CK>(wres);
             const int wstep = (g.nchunk * Cf::BBLK) >> 4;  // weights of the next tap, in 16-byte units
             int s = 0, acc = 0;
             uint32_t ph = 0, aph = 0;
@@ -514,37 +358,53 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 const uint32_t d = tmem_base + (uint32_t)(acc * Cf::ACC_COLS);
+                // weights of source offset t = 3 syi + sxi: tap t, or 8 - t when mirrored
+                const uint64_t dw0 = w_desc0 + (g.flip ? (uint64_t)(8 * wstep) : 0);
+                const uint64_t step = (uint64_t)(int64_t)(g.flip ? -wstep : wstep);
                 for (int ch = 0; ch < g.nchunk; ++ch) {
-                    if (!mbar_wait_warp(bar_full + 8 * s, ph, abort)) {
+                    const int sl = s + ch < S ? s + ch : s + ch - S;
+                    if (!mbar_wait_warp(bar_full + 8 * sl, s + ch < S ? ph : ph ^ 1u, abort)) {
                         ok = false;
                         break;
                     }
+                    if (g.order != ORDER_BLOCKS) continue;  // all blocks first
                     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                    const uint64_t da = a_desc0 + (uint64_t)((uint32_t)(s * Cf::STAGE) >> 4);
-                    uint64_t dw = w_desc0 + (uint64_t)((uint32_t)(ch * Cf::BBLK) >> 4);
-                    // source offset (sy, sx) = (syi - 1, sxi - 1) of tap syi * 3 + sxi (mirrored: 8 - that)
-                    if (g.flip) dw += (uint64_t)(8 * wstep);
-                    const uint64_t step = (uint64_t)(int64_t)(g.flip ? -wstep : wstep);
+                    const uint64_t da = a_desc0 + (uint64_t)((uint32_t)(sl * Cf::STAGE) >> 4);
+                    const uint64_t dw = dw0 + (uint64_t)((uint32_t)(ch * Cf::BBLK) >> 4);
 #pragma unroll
-                    for (int syi = 0; syi < 3; ++syi)
+                    for (int sxi = 0; sxi < 3; ++sxi)
 #pragma unroll
-                        for (int sxi = 0; sxi < 3; ++sxi) {
-#pragma unroll
-                            for (int kk = 0; kk < CK / 16; ++kk)
-                                mma_f16_elect(d, da + (uint64_t)((syi * HPITCH + sxi) * CK * 2 / 16 + kk * 2),
-                                            dw + (uint64_t)(kk * 2), IDESC,
-                                            syi + sxi + kk > 0 || ch > 0 ? 1u : 0u);
-                            dw += step;
-                        }
-                    mma_commit_elect(bar_empty + 8 * s);
-                    last_bar = bar_empty + 8 * s;
-                    last_par = ph;
-                    if (++s == S) {
-                        s = 0;
-                        ph ^= 1u;
-                    }
+                        for (int syi = 0; syi < 3; ++syi)
+                            mma_chain_elect<CK / 16>(d, da + (uint64_t)((syi * HPITCH + sxi) * CK * 2 / 16),
+                                                     dw + (uint64_t)(syi * 3 + sxi) * step, IDESC,
+                                                     syi + sxi > 0 || ch > 0 ? 1u : 0u);
+                    mma_commit_elect(bar_empty + 8 * sl);
+                    last_bar = bar_empty + 8 * sl;
+                    last_par = s + ch < S ? ph : ph ^ 1u;
                 }
                 if (!ok) break;
+                if (g.order != ORDER_BLOCKS) {
+                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                    for (int tap = 0; tap < 9; ++tap) {
+                        const int t = g.flip ? 8 - tap : tap;
+                        for (int ch = 0; ch < g.nchunk; ++ch) {
+                            const int sl = s + ch < S ? s + ch : s + ch - S;
+                            const uint64_t da = a_desc0 + (uint64_t)((uint32_t)(sl * Cf::STAGE + (t / 3 * HPITCH + t % 3) * CK * 2) >> 4);
+                            const uint64_t dw = w_desc0 + (uint64_t)((uint32_t)((tap * g.nchunk + ch) * Cf::BBLK) >> 4);
+                            mma_chain_elect<CK / 16>(d, da, dw, IDESC, tap + ch > 0 ? 1u : 0u);
+                            if (tap == 8) {
+                                mma_commit_elect(bar_empty + 8 * sl);
+                                last_bar = bar_empty + 8 * sl;
+                                last_par = s + ch < S ? ph : ph ^ 1u;
+                            }
+                        }
+                    }
+                }
+                s += g.nchunk;
+                if (s >= S) {
+                    s -= S;
+                    ph ^= 1u;
+                }
                 mma_commit_elect(bar_afull + 8 * acc);
                 if (++acc == Cf::NACC) {
                     acc = 0;
@@ -633,8 +493,8 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
 // next to the odd one: 32 columns. 24 products a 32 channels and 256 pixels
 // instead of 36. The pixels of either parity are a box of their own (of the tensor as
 // W / 2 columns of 2 C channels).
-// Measured (forward, batch 64, 256 x 256): 32 -> 32 channels 133 us with the pooling (169),
-// 96 -> 32 222 (317), 32 -> 32 with the head 91 (137).
+// Measured (forward, batch 64, 256 x 256): 32 -> 32 channels 130 us with the pooling (169),
+// 96 -> 32 236 (317), 32 -> 32 with the head 98 (137).
 // ---------------------------------------------------------------------------
 
 struct PairCfg {
@@ -740,7 +600,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
         {  // the whole warp
             // ---------------- MMA issuer ----------------
             constexpr uint32_t IDESC2 = tc::idesc_bf16_f32<64>(), IDESC1 = tc::idesc_bf16_f32<32>();
-            const uint64_t a_desc0 = sdesc_box<32>(stages), w_desc0 = sdesc<32, 32>(wres);
+            const uint64_t a_desc0 = sdesc_box<32>(stages), w_desc0 = sdesc<32>(wres);
             const uint64_t wrow = (uint64_t)(uint32_t)((3 * g.nchunk * Cf::BBLK) >> 4);  // the next vertical offset
             int s = 0, acc = 0;
             uint32_t ph = 0, aph = 0;
@@ -753,45 +613,74 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 const uint32_t d = tmem_base + (uint32_t)(acc * Cf::ACC_COLS);
+                // The products of 32 channels with one row of taps, X = 0 .. 3: the odd pixel of the
+                // pair before (source offset -1 of the even output), the even pixel (0 of the even, -1
+                // of the odd output), the odd one (1 and 0), the even pixel of the next (1 of the odd
+                // output). Either output meets its offsets in ascending order as X ascends, in
+                // descending order as it descends. first: the first of this X, whose outputs met
+                // there for the first time are set, not added to.
+                const bool desc = g.order == ORDER_TAPS && g.flip;
+                auto products = [&](int X, int syi, uint64_t da, uint64_t dw, bool first) {
+                    constexpr uint32_t W1 = Cf::BBLK / 16, ODD = Cf::A_SLOT / 16, PX = 64 / 16;
+                    const uint64_t a = da + (uint64_t)(syi * HPITCH * PX), w = dw + (uint64_t)(uint32_t)syi * wrow;
+                    if (X == 0) {
+                        mma_chain_elect<2>(d, a + ODD, w + 2 * W1, IDESC1, first && !desc ? 0u : 1u);
+                    } else if (X == 3) {
+                        mma_chain_elect<2>(d + 32u, a + 2 * PX, w, IDESC1, first && desc ? 0u : 1u);
+                    } else {
+                        const uint64_t ax = a + PX + (X == 2 ? ODD : 0u), wx = w + (X == 1 ? W1 : 0u);
+                        if (first && (X == 1) != desc) {
+                            mma_chain_elect<2>(d, ax, wx, IDESC1, desc ? 0u : 1u);
+                            mma_chain_elect<2>(d + 32u, ax, wx + W1, IDESC1, desc ? 1u : 0u);
+                        } else {
+                            mma_chain_elect<2>(d, ax, wx, IDESC2, 1u);
+                        }
+                    }
+                };
                 for (int ch = 0; ch < g.nchunk; ++ch) {
-                    if (!mbar_wait_warp(bar_full + 8 * s, ph, abort)) {
+                    const int sl = s + ch < S ? s + ch : s + ch - S;
+                    if (!mbar_wait_warp(bar_full + 8 * sl, s + ch < S ? ph : ph ^ 1u, abort)) {
                         ok = false;
                         break;
                     }
+                    if (g.order != ORDER_BLOCKS) continue;  // all blocks first
                     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                    const uint64_t da = a_desc0 + (uint64_t)((uint32_t)(s * Cf::STAGE) >> 4);
-                    uint64_t dw = w_desc0 + (uint64_t)((uint32_t)(3 * ch * Cf::BBLK) >> 4);
+                    const uint64_t da = a_desc0 + (uint64_t)((uint32_t)(sl * Cf::STAGE) >> 4);
+                    const uint64_t dw = w_desc0 + (uint64_t)((uint32_t)(3 * ch * Cf::BBLK) >> 4);
 #pragma unroll
-                    for (int syi = 0; syi < 3; ++syi) {
-                        // even pixel: 0 away from an even output, -1 from an odd one; odd pixel: 1 and 0; the
-                        // odd pixel of the pair before: -1 from the even output; the even one of the next: 1
-                        // from the odd output
-                        constexpr uint32_t W1 = Cf::BBLK / 16, ODD = Cf::A_SLOT / 16, PX = 64 / 16;
-                        const uint64_t dr = da + (uint64_t)(syi * HPITCH * PX);
+                    for (int X = 0; X < 4; ++X)
 #pragma unroll
-                        for (int kk = 0; kk < 2; ++kk)
-                            mma_f16_elect(d, dr + (uint64_t)(PX + kk * 2), dw + (uint64_t)(W1 + kk * 2), IDESC2,
-                                          syi + kk > 0 || ch > 0 ? 1u : 0u);
-#pragma unroll
-                        for (int kk = 0; kk < 2; ++kk)
-                            mma_f16_elect(d, dr + (uint64_t)(ODD + PX + kk * 2), dw + (uint64_t)(kk * 2), IDESC2, 1u);
-#pragma unroll
-                        for (int kk = 0; kk < 2; ++kk)
-                            mma_f16_elect(d, dr + (uint64_t)(ODD + kk * 2), dw + (uint64_t)(2 * W1 + kk * 2), IDESC1, 1u);
-#pragma unroll
-                        for (int kk = 0; kk < 2; ++kk)
-                            mma_f16_elect(d + 32u, dr + (uint64_t)(2 * PX + kk * 2), dw + (uint64_t)(kk * 2), IDESC1, 1u);
-                        dw += wrow;
-                    }
-                    mma_commit_elect(bar_empty + 8 * s);
-                    last_bar = bar_empty + 8 * s;
-                    last_par = ph;
-                    if (++s == S) {
-                        s = 0;
-                        ph ^= 1u;
-                    }
+                        for (int syi = 0; syi < 3; ++syi) products(X, syi, da, dw, ch == 0 && syi == 0);
+                    mma_commit_elect(bar_empty + 8 * sl);
+                    last_bar = bar_empty + 8 * sl;
+                    last_par = s + ch < S ? ph : ph ^ 1u;
                 }
                 if (!ok) break;
+                if (g.order != ORDER_BLOCKS) {
+                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+#pragma unroll 1
+                    for (int i = 0; i < 12; ++i) {
+                        const int X = g.order == ORDER_OFFSETS ? i / 3 : desc ? 3 - (i & 3) : i & 3;
+                        const int syi = g.order == ORDER_OFFSETS ? i % 3 : desc ? 2 - (i >> 2) : i >> 2;
+                        const bool first = g.order == ORDER_OFFSETS ? syi == 0 : i < 4;
+                        for (int ch = 0; ch < g.nchunk; ++ch) {
+                            const int sl = s + ch < S ? s + ch : s + ch - S;
+                            products(X, syi, a_desc0 + (uint64_t)((uint32_t)(sl * Cf::STAGE) >> 4),
+                                     w_desc0 + (uint64_t)((uint32_t)(3 * ch * Cf::BBLK) >> 4), first && ch == 0);
+                        }
+                    }
+                    for (int ch = 0; ch < g.nchunk; ++ch) {
+                        const int sl = s + ch < S ? s + ch : s + ch - S;
+                        mma_commit_elect(bar_empty + 8 * sl);
+                        last_bar = bar_empty + 8 * sl;
+                        last_par = s + ch < S ? ph : ph ^ 1u;
+                    }
+                }
+                s += g.nchunk;
+                if (s >= S) {
+                    s -= S;
+                    ph ^= 1u;
+                }
                 mma_commit_elect(bar_afull + 8 * acc);
                 if (++acc == Cf::NACC) {
                     acc = 0;
@@ -879,16 +768,18 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
 // Wide layers (64 channels a chunk, weights too large to stay in shared
 // memory): halo boxes and groups of tiles that share each weight.
 //
-// k_conv_tma reads 128 pixels and BN weight rows of 128 bytes for every four MMAs
-// and is bound by what L2 delivers (14 TB/s, tensor pipe 23 .. 38 % active). Here a box of
-// 10 x 18 pixels serves all nine taps (180 rows instead of 1152), and each three taps'
-// weights serve the G tiles of a group, each with an accumulator of its own, before
-// the next are loaded: per tile and 64 channels 23 KB + 9 BN / G * 128 bytes instead of
-// 9 (16 KB + BN * 128). Roles as in k_conv_halo, with rings of boxes (A; a
-// group's boxes stay until its last taps) and of weights (W).
-// Measured (forward, batch 64, 256 x 256): 192 -> 64 channels 191 us (377; 202 with a box a
-// horizontal offset),
-// 384 -> 128 143 (204).
+// With 128 pixels and BN weight rows loaded for every tap and 64 channels (four MMAs) the
+// layers are bound by what L2 delivers (14 TB/s, tensor pipe 23 .. 38 % active). Here the boxes
+// of 10 x 18 pixels of a tile, one a chunk, stay for all nine taps (180 rows a chunk instead
+// of 1152), and each tap's weights serve the G tiles of a group, each with an
+// accumulator of its own: per tile and chunk 23 KB + 9 BN / G * 128 bytes instead of
+// 9 (16 KB + BN * 128). G is as large as the accumulators, four boxes a group and
+// enough groups for every SM allow. Roles as in k_conv_halo, with rings of boxes (in the
+// order of the first tap, released in that order with the last) and of weights. The rings
+// share what there is of shared memory. (Two or three chunks of weights a slot, or one
+// tile a group and twice the boxes, are no faster: 192 -> 64 281 and 403 us.)
+// Measured (forward, batch 64, 256 x 256): 192 -> 64 channels 292 us (381 with a box a
+// tap), all layers of 128 and 256 outputs 487 (495).
 // ---------------------------------------------------------------------------
 
 template <int BN>
@@ -896,26 +787,27 @@ struct GroupCfg {
     static_assert(BN == 64 || BN == 128, "accumulators of 64 or 128 columns");
     static constexpr int A_BYTES = HROWS * 128;     // one box
     static constexpr int A_SLOT = (A_BYTES + 1023) / 1024 * 1024;
-    static constexpr int W_BYTES = 3 * BN * 128;    // the weights of three taps
-    static constexpr int AS = BN == 64 ? 5 : 4, WS = BN == 64 ? 3 : 2;  // ring slots
+    static constexpr int W_BYTES = BN * 128;        // the weights of a tap and chunk
     static constexpr int NACC = 512 / BN, GMAX = NACC / 2;  // accumulators; tiles a group at most
-    static_assert(GMAX <= AS, "the boxes of a group");
-    static constexpr int SMEM = 1024 + AS * A_SLOT + WS * W_BYTES + 8 * kOutBytes + 512;
+    static constexpr int AMAX = 6, WMAX = 8;        // ring slots at most
+    static constexpr int OB = 32, OUT_BYTES = 2048; // channels of an output box, a warp's buffer
+    static constexpr int SMEM_BUDGET = 212992;      // both rings
+    static constexpr int SMEM_REST = 1024 + 8 * OUT_BYTES + 512;
 };
 
 template <int BN, class EPI>
 __global__ void __launch_bounds__(kHaloThreads, 1)
     k_conv_group(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                 const __grid_constant__ CUtensorMap mapO, const __grid_constant__ CUtensorMap mapO2, const ConvGeo g,
-                 const EPI epi, int G, int *err) {
+                 const EPI epi, int G, int AS, int WS, int *err) {
     using Cf = GroupCfg<BN>;
-    constexpr int AS = Cf::AS, WS = Cf::WS, NACC = Cf::NACC;
+    constexpr int NACC = Cf::NACC;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     const uint32_t wbase = base + AS * Cf::A_SLOT;
     const uint32_t obuf = wbase + WS * Cf::W_BYTES;  // the epilogue warps' output buffers
-    const uint32_t bar_full = obuf + 8 * kOutBytes;
+    const uint32_t bar_full = obuf + 8 * Cf::OUT_BYTES;
     const uint32_t bar_empty = bar_full + 8 * AS;
     const uint32_t bar_wfull = bar_empty + 8 * AS;
     const uint32_t bar_wempty = bar_wfull + 8 * WS;
@@ -974,38 +866,34 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
             for (int u = blockIdx.x; u < groups && ok; u += gridDim.x) {
                 int t0, n;
                 group_tiles(u, t0, n);
-                for (int kb = 0; kb < g.KB && ok; ++kb) {  // KB = 3 nchunk: chunk, then vertical offset
-                    const int ch = kb / 3, syi = kb - 3 * ch;
-                    if (!tc::mbar_wait(bar_wempty + 8 * ws, wph ^ 1u, abort)) {
-                        ok = false;
-                        break;
-                    }
-                    arrive_expect_tx(bar_wfull + 8 * ws, Cf::W_BYTES);
-#pragma unroll
-                    for (int sxi = 0; sxi < 3; ++sxi) {
-                        const int tap = g.flip ? 8 - (syi * 3 + sxi) : syi * 3 + sxi;
-                        tma_load_2d(wbase + ws * Cf::W_BYTES + sxi * (BN * 128), &mapB, tap * g.C + ch * 64,
-                                    (t0 / g.mtiles) * BN, bar_wfull + 8 * ws);
-                    }
-                    if (++ws == WS) {
-                        ws = 0;
-                        wph ^= 1u;
-                    }
-                    for (int i = 0; i < n && syi == 0; ++i) {
-                        int b, x0, y0, nt;
-                        tile_origin(g, t0 + i, b, x0, y0, nt);
-                        if (!tc::mbar_wait(bar_empty + 8 * s, ph ^ 1u, abort)) {
+                for (int tap = 0; tap < 9 && ok; ++tap)
+                    for (int ch = 0; ch < g.nchunk && ok; ++ch) {
+                        if (!tc::mbar_wait(bar_wempty + 8 * ws, wph ^ 1u, abort)) {
                             ok = false;
                             break;
                         }
-                        arrive_expect_tx(bar_full + 8 * s, Cf::A_BYTES);
-                        tma_load_4d(base + s * Cf::A_SLOT, &mapA, ch * 64, x0 - 1, y0 - 1, b, bar_full + 8 * s);
-                        if (++s == AS) {
-                            s = 0;
-                            ph ^= 1u;
+                        arrive_expect_tx(bar_wfull + 8 * ws, Cf::W_BYTES);
+                        tma_load_2d(wbase + ws * Cf::W_BYTES, &mapB, tap * g.C + ch * 64, (t0 / g.mtiles) * BN,
+                                    bar_wfull + 8 * ws);
+                        if (++ws == WS) {
+                            ws = 0;
+                            wph ^= 1u;
+                        }
+                        for (int i = 0; i < n && tap == 0; ++i) {
+                            int b, x0, y0, nt;
+                            tile_origin(g, t0 + i, b, x0, y0, nt);
+                            if (!tc::mbar_wait(bar_empty + 8 * s, ph ^ 1u, abort)) {
+                                ok = false;
+                                break;
+                            }
+                            arrive_expect_tx(bar_full + 8 * s, Cf::A_BYTES);
+                            tma_load_4d(base + s * Cf::A_SLOT, &mapA, ch * 64, x0 - 1, y0 - 1, b, bar_full + 8 * s);
+                            if (++s == AS) {
+                                s = 0;
+                                ph ^= 1u;
+                            }
                         }
                     }
-                }
             }
             if (!ok) {
                 // loads already issued finish on their own within microseconds
@@ -1018,7 +906,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
         {  // the whole warp
             // ---------------- MMA issuer ----------------
             constexpr uint32_t IDESC = tc::idesc_bf16_f32<BN>();
-            const uint64_t a_desc0 = sdesc_box<64>(base), w_desc0 = sdesc<BN, 64>(wbase);
+            const uint64_t a_desc0 = sdesc_box<64>(base), w_desc0 = sdesc<64>(wbase);
             int s = 0, ws = 0, acc0 = 0;  // acc0: the group's first accumulator
             uint32_t ph = 0, wph = 0, aph = 0;
             bool ok = true;
@@ -1036,50 +924,53 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
                 }
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                for (int kb = 0; kb < g.KB && ok; ++kb) {
-                    if (!mbar_wait_warp(bar_wfull + 8 * ws, wph, abort)) {
-                        ok = false;
-                        break;
-                    }
-                    const uint64_t dw = w_desc0 + (uint64_t)((uint32_t)(ws * Cf::W_BYTES) >> 4);
-                    const int syi = kb % 3;
-                    // the chunk's boxes are slots s .. s + n - 1 (mod AS), waited for with its first
-                    // taps and released with its last
-                    for (int i = 0; i < n; ++i) {
-                        const int acc = acc0 + i < NACC ? acc0 + i : acc0 + i - NACC;
-                        const int sl = s + i < AS ? s + i : s + i - AS;
-                        const uint32_t slp = s + i < AS ? ph : ph ^ 1u;
-                        if (syi == 0 && !mbar_wait_warp(bar_full + 8 * sl, slp, abort)) {
+                for (int tap = 0; tap < 9 && ok; ++tap) {
+                    const int t = g.flip ? 8 - tap : tap;  // source offset 3 (sy + 1) + sx + 1
+                    const uint64_t off = a_desc0 + (uint64_t)(uint32_t)((t / 3 * HPITCH + t % 3) * 8);
+                    // the boxes of (chunk, tile) are slots s + ch n + i (mod AS), waited for with
+                    // the first tap and released with the last
+                    int sl = s;
+                    uint32_t slp = ph;
+                    for (int ch = 0; ch < g.nchunk; ++ch) {
+                        if (!mbar_wait_warp(bar_wfull + 8 * ws, wph, abort)) {
                             ok = false;
                             break;
                         }
                         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                        const uint32_t d = tmem_base + (uint32_t)(acc * BN);
-                        const uint64_t da = a_desc0 + (uint64_t)((uint32_t)(sl * Cf::A_SLOT + syi * HPITCH * 128) >> 4);
-#pragma unroll
-                        for (int sxi = 0; sxi < 3; ++sxi)
-#pragma unroll
-                            for (int kk = 0; kk < 4; ++kk)
-                                mma_f16_elect(d, da + (uint64_t)(sxi * 128 / 16 + kk * 2),
-                                              dw + (uint64_t)(sxi * BN * 128 / 16 + kk * 2), IDESC,
-                                              sxi + kk > 0 || kb > 0 ? 1u : 0u);
-                        if (syi == 2) mma_commit_elect(bar_empty + 8 * sl);
-                    }
-                    if (!ok) break;
-                    if (syi == 2) {
-                        s += n;
-                        if (s >= AS) {
-                            s -= AS;
-                            ph ^= 1u;
+                        const uint64_t dw = w_desc0 + (uint64_t)((uint32_t)ws * (Cf::W_BYTES / 16));
+                        int acc = acc0;
+                        for (int i = 0; i < n; ++i) {
+                            if (tap == 0) {
+                                if (!mbar_wait_warp(bar_full + 8 * sl, slp, abort)) {
+                                    ok = false;
+                                    break;
+                                }
+                                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                            }
+                            mma_chain_elect<4>(tmem_base + (uint32_t)(acc * BN),
+                                               off + (uint64_t)((uint32_t)sl * (Cf::A_SLOT / 16)), dw, IDESC,
+                                               tap + ch > 0 ? 1u : 0u);
+                            if (tap == 8) mma_commit_elect(bar_empty + 8 * sl);
+                            if (++acc == NACC) acc = 0;
+                            if (++sl == AS) {
+                                sl = 0;
+                                slp ^= 1u;
+                            }
                         }
-                    }
-                    mma_commit_elect(bar_wempty + 8 * ws);
-                    if (++ws == WS) {
-                        ws = 0;
-                        wph ^= 1u;
+                        if (!ok) break;
+                        mma_commit_elect(bar_wempty + 8 * ws);
+                        if (++ws == WS) {
+                            ws = 0;
+                            wph ^= 1u;
+                        }
                     }
                 }
                 if (!ok) break;
+                s += n * g.nchunk;
+                if (s >= AS) {
+                    s -= AS;
+                    ph ^= 1u;
+                }
                 for (int i = 0; i < n; ++i) {
                     mma_commit_elect(bar_afull + 8 * acc0);
                     if (++acc0 == NACC) {
@@ -1100,7 +991,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
         epi.prepare(epi_const, threadIdx.x - 64, 256);
         asm volatile("bar.sync 1, 256;\n" ::: "memory");  // the epilogue warps only
         const int q = warp & 3, half = (warp - 2) >> 2;
-        const uint32_t buf = obuf + (uint32_t)(warp - 2) * kOutBytes;
+        const uint32_t buf = obuf + (uint32_t)(warp - 2) * Cf::OUT_BYTES;
         int acc = 0;
         uint32_t aph = 0;
         int turn = 0;
@@ -1134,10 +1025,11 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
                         const int n = nt * BN + 16 * j;
                         uint32_t p[8];
                         epi.compute(m, n, f, state, epi_const, pre, valid, p);
-                        if (16 * j % 64 == 0) out_reuse(lane);
-                        out_put<64>(buf, lane, 16 * j % 64, p);
-                        if (16 * (j + 1) % 64 == 0)
-                            out_store(buf, epi.second(n) ? &mapO2 : &mapO, epi.column(n - 48), x0, y0 + 4 * q, b, lane);
+                        if (16 * j % Cf::OB == 0) out_reuse(lane);
+                        out_put<Cf::OB>(buf, lane, 16 * j % Cf::OB, p);
+                        if (16 * (j + 1) % Cf::OB == 0)
+                            out_store(buf, epi.second(n) ? &mapO2 : &mapO, epi.column(n + 16 - Cf::OB), x0, y0 + 4 * q, b,
+                                      lane);
                     }
                     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
                     __syncwarp();

@@ -101,7 +101,6 @@ se2n_status forward(se2n_unet *u, const float *f, const uint8_t *mask, int n, bo
     const int H = u->H, W = u->W;
     auto Wt = [&](int l) { return u->pb + u->w_off[l]; };
     auto Bi = [&](int l) { return u->p + u->b_off[l]; };
-    bool pooled = false;  // the last convolution has written its output's 2x2 averages as well
     for (int l = 0; l < 4; ++l) {
         const int Hl = H >> l, Wl = W >> l;
         const LayerSpec &A = kLayers[2 * l], &Bb = kLayers[2 * l + 1];
@@ -109,15 +108,12 @@ se2n_status forward(se2n_unet *u, const float *f, const uint8_t *mask, int n, bo
             // the first layer reads the image and mask directly (2 meaningful input channels)
             TRYC(conv0_direct(f, mask, Wt(0), Bi(0), u->a[0], n, H, W, s));
         } else {
-            if (!pooled)
-                TRYC(pool(u->e[l - 1], u->e_ld[l - 1], u->pl[l], n, H >> (l - 1), W >> (l - 1), kLayers[2 * l - 1].cout,
-                          s));
-            TRYC(conv_forward(u->pl[l], nullptr, 0, n, Hl, Wl, A.cin, Wt(2 * l), Bi(2 * l), A.cout, 1, u->a[l], A.cout,
-                              s));
+            TRYC(conv_forward(u->pl[l], n, Hl, Wl, A.cin, Wt(2 * l), Bi(2 * l), A.cout, 1, u->a[l], A.cout, nullptr, s));
         }
-        // e[l] (l < 3) is written straight into the skip channels of decoder level l's input
-        TRYC(conv_forward(u->a[l], nullptr, 0, n, Hl, Wl, Bb.cin, Wt(2 * l + 1), Bi(2 * l + 1), Bb.cout, 1, u->e[l],
-                          u->e_ld[l], s, l < 3 ? u->pl[l + 1] : nullptr, &pooled));
+        // e[l] (l < 3) is written straight into the skip channels of decoder level l's input, and
+        // its 2x2 averages with it
+        TRYC(conv_forward(u->a[l], n, Hl, Wl, Bb.cin, Wt(2 * l + 1), Bi(2 * l + 1), Bb.cout, 1, u->e[l], u->e_ld[l],
+                          l < 3 ? u->pl[l + 1] : nullptr, s));
     }
     // decoder levels 2, 1, 0 (layer indices 8..13)
     const __nv_bfloat16 *below = u->e[3];
@@ -129,19 +125,15 @@ se2n_status forward(se2n_unet *u, const float *f, const uint8_t *mask, int n, bo
         // the input [up(below), e[level]] is one NHWC tensor (read with TMA boxes):
         // e[level] is already in it, the upsampled half is written here
         TRYC(upsample_into(below, A.lo_ch, u->cat[k], A.cin, n, Hl, Wl, s));
-        TRYC(conv_forward(u->cat[k], nullptr, 0, n, Hl, Wl, A.cin, Wt(la), Bi(la), A.cout, 1, u->c[k], A.cout, s));
+        TRYC(conv_forward(u->cat[k], n, Hl, Wl, A.cin, Wt(la), Bi(la), A.cout, 1, u->c[k], A.cout, nullptr, s));
         if (k == 2) {
-            // last convolution with the head and the input skip fused, when the tile shape allows
+            // the last convolution, with the head and the input skip
             const HeadArgs h{u->p + u->hw_off, u->p + u->hb_off, f, mask, u->out};
-            const cudaError_t e = conv_forward_tma(u->c[k], n, Hl, Wl, Bb.cin, Wt(lb), Bi(lb), Bb.cout, 1,
-                                                   keep ? u->d[k] : nullptr, Bb.cout, &h, s);
-            if (e == cudaSuccess) break;
-            if (e != cudaErrorNotSupported) return cuda_st(e);
+            TRYC(conv_forward_head(u->c[k], n, Hl, Wl, Bb.cin, Wt(lb), Bi(lb), keep ? u->d[k] : nullptr, h, s));
+        } else {
+            TRYC(conv_forward(u->c[k], n, Hl, Wl, Bb.cin, Wt(lb), Bi(lb), Bb.cout, 1, u->d[k], Bb.cout, nullptr, s));
+            below = u->d[k];
         }
-        TRYC(conv_forward(u->c[k], nullptr, 0, n, Hl, Wl, Bb.cin, Wt(lb), Bi(lb), Bb.cout, 1, u->d[k], Bb.cout, s));
-        below = u->d[k];
-        if (k == 2)
-            TRYC(head(u->d[2], u->p + u->hw_off, u->p + u->hb_off, f, mask, u->out, (long long)n * H * W, 32, s));
     }
     return SE2N_OK;
 }
@@ -167,11 +159,11 @@ se2n_status backward(se2n_unet *u, const float *f, const uint8_t *mask, int n) {
         const int Hl = H >> level, Wl = W >> level;
         const long long P = (long long)n * Hl * Wl;
         // second conv: c[k] -> d[k]
-        TRYC(conv_wgrad_tma(u->c[k], n, Hl, Wl, Bb.cin, u->gd[k], Bb.cout, dW(lb), s));
+        TRYC(conv_wgrad(u->c[k], n, Hl, Wl, Bb.cin, u->gd[k], Bb.cout, dW(lb), s));
         TRYC(colsum(u->gd[k], P, Bb.cout, dB(lb), s));
         TRYC(conv_backward_data(u->gd[k], n, Hl, Wl, Bb.cout, Wt(lb), Bb.cin, u->c[k], u->gc[k], nullptr, Bb.cin, u->wt, s));
         // first conv: [up(below), e[level]] -> c[k]
-        TRYC(conv_wgrad_tma(u->cat[k], n, Hl, Wl, A.cin, u->gc[k], A.cout, dW(la), s));
+        TRYC(conv_wgrad(u->cat[k], n, Hl, Wl, A.cin, u->gc[k], A.cout, dW(la), s));
         TRYC(colsum(u->gc[k], P, A.cout, dB(la), s));
         TRYC(conv_backward_data(u->gc[k], n, Hl, Wl, A.cout, Wt(la), A.cin, nullptr, u->gup[k], u->gskip[k],
                                 A.lo_ch, u->wt, s));
@@ -193,11 +185,11 @@ se2n_status backward(se2n_unet *u, const float *f, const uint8_t *mask, int n) {
                                         Bb.cout, s));
         }
         const __nv_bfloat16 *in = (l == 0) ? u->x0 : u->pl[l];
-        TRYC(conv_wgrad_tma(u->a[l], n, Hl, Wl, Bb.cin, u->ge[l], Bb.cout, dW(2 * l + 1), s));
+        TRYC(conv_wgrad(u->a[l], n, Hl, Wl, Bb.cin, u->ge[l], Bb.cout, dW(2 * l + 1), s));
         TRYC(colsum(u->ge[l], P, Bb.cout, dB(2 * l + 1), s));
         TRYC(conv_backward_data(u->ge[l], n, Hl, Wl, Bb.cout, Wt(2 * l + 1), Bb.cin, u->a[l], u->ga[l], nullptr,
                                 Bb.cin, u->wt, s));
-        TRYC(conv_wgrad_tma(in, n, Hl, Wl, A.cin, u->ga[l], A.cout, dW(2 * l), s));
+        TRYC(conv_wgrad(in, n, Hl, Wl, A.cin, u->ga[l], A.cout, dW(2 * l), s));
         TRYC(colsum(u->ga[l], P, A.cout, dB(2 * l), s));
         if (l > 0) {
             TRYC(conv_backward_data(u->ga[l], n, Hl, Wl, A.cout, Wt(2 * l), A.cin, nullptr, u->gp[l], nullptr, A.cin, u->wt, s));
