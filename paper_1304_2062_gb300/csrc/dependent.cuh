@@ -6,6 +6,11 @@
 // are harmless: the kernel as a whole is not complete before its waiting blocks.
 // After a library kernel, which never lets its successor start, such a launch
 // is an ordinary one.
+// A kernel launched so may start while what it is going to read is still being
+// written: none of that is read-only data for its lifetime, and it must not be read
+// through the non-coherent path (__ldg, const __restrict__ pointers), which may hold what
+// an earlier kernel read there. Such loads are __ldcg. (With __ldg in the row pass one
+// in some two hundred inpaints issued back to back had a stale row.)
 #pragma once
 
 #include <cuda_runtime.h>

@@ -40,7 +40,6 @@ __global__ void __launch_bounds__(256) k_colsum(const __nv_bfloat16 *g, long lon
     const int cg = threadIdx.x % groups, rr = threadIdx.x / groups;
     float s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     if (rr < rows) {
-#pragma unroll 4
         for (long long p = (long long)blockIdx.x * rows + rr; p < P; p += (long long)gridDim.x * rows) {
             const uint4 v = *(const uint4 *)(g + p * C + cg * 8);
             const __nv_bfloat16 *h = (const __nv_bfloat16 *)&v;

@@ -31,8 +31,8 @@ __global__ void k_orient_prep(const float2 *__restrict__ f, const uchar2 *__rest
     if (blockIdx.x == 0 && threadIdx.x == 0) *gmax = 0;  // for k_grad_max
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < npairs;
          i += (long long)gridDim.x * blockDim.x) {
-        const float2 v = f[i];
-        const uchar2 m = mask[i];
+        const float2 v = __ldcg(f + i);
+        const uchar2 m = __ldcg(mask + i);
         spec[i] = make_float4(m.x ? v.x : 0.0f, 0.0f, m.y ? v.y : 0.0f, 0.0f);
     }
 }
@@ -57,7 +57,7 @@ __global__ void k_grad_spec(const float2 *__restrict__ F, float2 *__restrict__ g
         const float g = expf(c * (fx * fx + fy * fy));
         const float dx = (2 * ls == -W) ? 0.0f : two_pi * fx * g;
         const float dy = (2 * ks == -H) ? 0.0f : two_pi * fy * g;
-        const float2 v = F[i];
+        const float2 v = __ldcg(F + i);
         gx[i] = make_float2(-v.y * dx, v.x * dx);  // i * dx * F
         gy[i] = make_float2(-v.y * dy, v.x * dy);
     }
@@ -72,7 +72,7 @@ __global__ void k_grad_max(const float2 *__restrict__ gx, const float2 *__restri
     float m = 0.0f;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < HW;
          i += (long long)gridDim.x * blockDim.x) {
-        const float x = gx[i].x, y = gy[i].x;
+        const float x = __ldcg(gx + i).x, y = __ldcg(gy + i).x;
         m = fmaxf(m, fmaf(x, x, y * y));
     }
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -95,10 +95,10 @@ __global__ void k_bins(const float2 *__restrict__ gx, const float2 *__restrict__
     dependent_launch();
     dependent_wait();
     const float pi = 3.14159265358979323846f;
-    const float thresh = flat_tol2 * __uint_as_float(*gmax);
+    const float thresh = flat_tol2 * __uint_as_float(__ldcg(gmax));
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < HW;
          i += (long long)gridDim.x * blockDim.x) {
-        const float x = gx[i].x, y = gy[i].x;
+        const float x = __ldcg(gx + i).x, y = __ldcg(gy + i).x;
         const float m2 = fmaf(x, x, y * y);
         uint8_t b = SE2N_BIN_FLAT;
         if (!(m2 <= thresh)) {
@@ -226,9 +226,9 @@ __global__ void k_lift_r(const float2 *__restrict__ f, const uchar2 *__restrict_
     dependent_wait();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < npairs;
          i += (long long)gridDim.x * blockDim.x) {
-        const float2 v = f[i];
-        const uchar2 m = mask[i];
-        const uchar2 b = bins[i];
+        const float2 v = __ldcg(f + i);
+        const uchar2 m = __ldcg(mask + i);
+        const uchar2 b = __ldcg(bins + i);
         const float a0 = m.x ? v.x : 0.0f, a1 = m.y ? v.y : 0.0f;
         float2 *out = (float2 *)(vol + real_off(i, W, Wp));
         for (int r = 0; r < N; ++r) {
@@ -254,9 +254,9 @@ __global__ void k_mix_r(float *__restrict__ vol, const float2 *__restrict__ f, c
             ht0 = fmaxf(ht0, v.x * scale);
             ht1 = fmaxf(ht1, v.y * scale);
         }
-        const float2 fv = f[i];
-        const uchar2 m = mask[i];
-        const uchar2 b = bins[i];
+        const float2 fv = __ldcg(f + i);
+        const uchar2 m = __ldcg(mask + i);
+        const uchar2 b = __ldcg(bins + i);
         const float a0 = m.x ? fv.x : 0.0f, a1 = m.y ? fv.y : 0.0f;
         const float h00 = (b.x == SE2N_BIN_FLAT) ? a0 : fmaxf(a0, 0.0f);
         const float h01 = (b.y == SE2N_BIN_FLAT) ? a1 : fmaxf(a1, 0.0f);
@@ -284,7 +284,7 @@ __global__ void k_project_r(const float *__restrict__ vol, long long npairs, int
             a0 = -INFINITY;
             a1 = -INFINITY;
             for (int r = 0; r < N; ++r) {
-                const float2 v = col[(long long)r * ps];
+                const float2 v = __ldcg(col + (long long)r * ps);
                 a0 = fmaxf(a0, v.x * scale);
                 a1 = fmaxf(a1, v.y * scale);
             }
@@ -292,7 +292,7 @@ __global__ void k_project_r(const float *__restrict__ vol, long long npairs, int
             a0 = 0.0f;
             a1 = 0.0f;
             for (int r = 0; r < N; ++r) {
-                const float2 v = col[(long long)r * ps];
+                const float2 v = __ldcg(col + (long long)r * ps);
                 a0 += v.x * scale;
                 a1 += v.y * scale;
             }
@@ -300,8 +300,8 @@ __global__ void k_project_r(const float *__restrict__ vol, long long npairs, int
             a1 /= (float)N;
         }
         if (mask) {
-            const uchar2 m = mask[i];
-            const float2 fv = f[i];
+            const uchar2 m = __ldcg(mask + i);
+            const float2 fv = __ldcg(f + i);
             if (m.x) a0 = fv.x;
             if (m.y) a1 = fv.y;
         }

@@ -64,9 +64,9 @@ __global__ void __launch_bounds__(row_threads<W>()) k_row(const __grid_constant_
     // 1. the row
     if (a.in_mode == SE2N_ROW_IN_LIFT) {
         for (int m = tid; m < WH; m += T) {
-            const float2 fv = reinterpret_cast<const float2 *>(a.f + row)[m];
-            const uchar2 mk = reinterpret_cast<const uchar2 *>(a.mask + row)[m];
-            const uchar2 bn = reinterpret_cast<const uchar2 *>(a.bins + row)[m];
+            const float2 fv = __ldcg(reinterpret_cast<const float2 *>(a.f + row) + m);
+            const uchar2 mk = __ldcg(reinterpret_cast<const uchar2 *>(a.mask + row) + m);
+            const uchar2 bn = __ldcg(reinterpret_cast<const uchar2 *>(a.bins + row) + m);
             const float a0 = mk.x ? fv.x : 0.0f, a1 = mk.y ? fv.y : 0.0f;
             float2 *Zm = Z + xoff<WH>(m);
 #pragma unroll 8
@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(row_threads<W>()) k_row(const __grid_constant_
     } else if (a.in_mode == SE2N_ROW_IN_REAL) {
         for (int e = tid; e < N * WH; e += T) {
             const int n = e / WH, m = e - n * WH;
-            Z[xsm<WH>(e)] = reinterpret_cast<const float2 *>(a.real_in + (n * H + y) * (W + 2))[m];
+            Z[xsm<WH>(e)] = __ldcg(reinterpret_cast<const float2 *>(a.real_in + (n * H + y) * (W + 2)) + m);
         }
     } else {
         // pairs (l, W/2 - l), l = 0 .. W/4: thread tid takes angle tid mod N
@@ -94,8 +94,10 @@ __global__ void __launch_bounds__(row_threads<W>()) k_row(const __grid_constant_
         for (int i = 0; i < IT; ++i) {
             const int l = l0 + i * TL;
             if (LP % TL == 0 || l < LP) {
-                xl[i] = __ldg(a.spec_in + ((long long)l * H + y) * N + n);
-                xb[i] = __ldg(a.spec_in + ((long long)(WH - l) * H + y) * N + n);
+                // from L2: the column pass may still be writing when this kernel starts
+                // (dependent.cuh), so nothing of it is read-only data
+                xl[i] = __ldcg(a.spec_in + ((long long)l * H + y) * N + n);
+                xb[i] = __ldcg(a.spec_in + ((long long)(WH - l) * H + y) * N + n);
             }
         }
         __syncthreads();  // twiddles
@@ -130,9 +132,9 @@ __global__ void __launch_bounds__(row_threads<W>()) k_row(const __grid_constant_
                 ht0 = fmaxf(ht0, v.x * a.scale);
                 ht1 = fmaxf(ht1, v.y * a.scale);
             }
-            const float2 fv = reinterpret_cast<const float2 *>(a.f + row)[m];
-            const uchar2 mk = reinterpret_cast<const uchar2 *>(a.mask + row)[m];
-            const uchar2 bn = reinterpret_cast<const uchar2 *>(a.bins + row)[m];
+            const float2 fv = __ldcg(reinterpret_cast<const float2 *>(a.f + row) + m);
+            const uchar2 mk = __ldcg(reinterpret_cast<const uchar2 *>(a.mask + row) + m);
+            const uchar2 bn = __ldcg(reinterpret_cast<const uchar2 *>(a.bins + row) + m);
             const float a0 = mk.x ? fv.x : 0.0f, a1 = mk.y ? fv.y : 0.0f;
             const float h00 = (bn.x == SE2N_BIN_FLAT) ? a0 : fmaxf(a0, 0.0f);
             const float h01 = (bn.y == SE2N_BIN_FLAT) ? a1 : fmaxf(a1, 0.0f);
@@ -181,8 +183,8 @@ __global__ void __launch_bounds__(row_threads<W>()) k_row(const __grid_constant_
                 a1 /= (float)NE;
             }
             if (a.reinject) {
-                const float2 fv = reinterpret_cast<const float2 *>((a.rf ? a.rf : a.f) + row)[m];
-                const uchar2 mk = reinterpret_cast<const uchar2 *>((a.rmask ? a.rmask : a.mask) + row)[m];
+                const float2 fv = __ldcg(reinterpret_cast<const float2 *>((a.rf ? a.rf : a.f) + row) + m);
+                const uchar2 mk = __ldcg(reinterpret_cast<const uchar2 *>((a.rmask ? a.rmask : a.mask) + row) + m);
                 if (mk.x) a0 = fv.x;
                 if (mk.y) a1 = fv.y;
             }
