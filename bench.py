@@ -5,24 +5,25 @@ piecewise-smooth image, 80 % random mask plus 4-px bars every 32 px,
 beta = 0.25, 10 restoration intervals of 500 Crank-Nicolson steps, T = 2 per
 interval): orientation, lift, the 2-D DFT, 10 x diffusion, 9 x (inverse
 DFT, static restoration, forward DFT), inverse DFT, projection, all through
-se2n_inpaint with the inputs resident in HBM. By default each interval's
-500 steps are applied as one precomputed S-step propagator per class of
-frequencies, built inside every timed inpaint, and each interval runs as
-one column pass (DFT along y, propagators, inverse DFT) and one row pass
-(real DFTs along x around the restoration) (--diffusion propagator);
---diffusion steps runs the fused step-by-step kernel between cuFFT
+se2n_inpaint with the inputs resident in HBM. By default
+(--diffusion propagator) each interval's 500 steps are applied as one
+linear map per frequency, the polynomial of its operator that equals the
+steps' product to FP32 resolution, and each interval runs as one column
+pass (DFT along y, the polynomial, inverse DFT) and one row pass (real DFTs
+along x around the restoration); --diffusion steps runs the fused
+step-by-step kernel (asked for by its split-diagonal form) between cuFFT
 transforms instead, and the default line reports that path too.
 
 Metric: Mathieu updates per second over the whole inpaint time (value),
 counting the frequencies the path integrates: the lifted volume is real, so
 the H x (W/2 + 1) frequencies of the Hermitian half carry the whole
 spectrum, and updates = 512 * 257 * 32 * 500 * 10 per inpaint (on the
-propagator path these are equivalent updates: each interval's 500 steps
-are applied as one precomputed map). The count over all M^2 frequencies
+default path these are equivalent updates: each interval's 500 steps
+are applied as one map). The count over all M^2 frequencies
 that the method's own formulation integrates is reported beside it
 (m2_updates_per_s). Plus ms per inpaint (the first figure of the line), the FP32 error against the FP64 oracle, the roofline of the
 dominant kernel (the column pass against the measured copy rate, with the
-row pass and the propagator build beside it; or the step kernel, FP32 ALU
+row pass beside it; or the step kernel, FP32 ALU
 bound, whose flops are those of the frequencies it integrates, the
 Hermitian half 512 x 257 of the spectrum), the end-to-end number from host
 buffers (se2n_inpaint_host) and the oracle's CPU rate.
@@ -54,6 +55,13 @@ import synth  # noqa: E402
 METRIC = "Mathieu updates/s (M²·N·steps); ms per 512² N=32 inpaint, err vs FP64"
 UNIT = "updates/s"
 FLOPS_PER_UPDATE = 22          # per complex angle per CN step: 2 x (1 add + 5 FMA)
+# the step kernel's split-diagonal form, which the benchmark asks for: one more FMA a component
+FLOPS_PER_UPDATE_SPLIT = FLOPS_PER_UPDATE + 4
+# coefficients of the interval polynomial in the eight ranges of wx^2 + wy^2 (quarters
+# of [0, 2]), as the library makes them for beta = 0.25: T = 2 in 500 steps (increment form) and
+# T = 50 in 1000 (Reinsch's form)
+POLY_512 = (9, 10, 10, 11, 11, 12, 12, 13)
+POLY_2048 = (33, 36, 39, 42, 44, 46, 48, 50)
 GOLDEN = os.path.join(ROOT, "tests", "golden", "curves_noise_512_N32.npz")
 L2_FLUSH_BYTES = 256 << 20
 SM_COUNT, FP32_LANES_PER_SM = 152, 128
@@ -182,7 +190,8 @@ class ClockSampler:
 
 KERNEL_SOURCES = {"diffuse": ("diffuse_impl.cuh", "diffuse_x2.cuh", "diffuse.cu"),
                   "prop_build": ("propagator.cu", "prop_classes.cuh", "diffuse_x2.cuh", "diffuse_impl.cuh"),
-                  "col_prop": ("colprop.cu", "bulk_copy.cuh", "rowdft.cuh", "smem_fft.cuh", "prop_classes.cuh", "diffuse_x2.cuh"),
+                  "col_prop": ("colprop.cu", "poly.cuh", "bulk_copy.cuh", "rowdft.cuh", "smem_fft.cuh", "prop_classes.cuh",
+                               "diffuse_x2.cuh"),
                   "row_pass": ("rowfft.cu", "smem_fft.cuh", "restore.cuh"),
                   "prop_build_wide": ("propagator.cu", "prop_classes.cuh", "diffuse_x2.cuh", "diffuse_impl.cuh"),
                   "prop_apply_tiled": ("propagator.cu", "prop_classes.cuh", "diffuse_x2.cuh", "diffuse_impl.cuh")}
@@ -220,34 +229,15 @@ def stored_traffic(kind="diffuse"):
     return rec.get("dram_bytes_per_launch") if rec else None
 
 
-def propagator_gemm_flops(classes, N, S):
-    """FP32 flops of building the S-step propagators and the products a class:
-    every op of the library's powering program but its copies is one
-    N x N x N product (2 N^3 flops); the O(N^2) solves of the first step are
-    not counted."""
-    from paper_1304_2062_gb300 import se2n
-    ops, _ = se2n.se2n_prop_chain(S)
-    products = sum(o != se2n.PROP_COPY for o in ops)
-    return classes * products * 2 * N ** 3, products
-
-
-def propagator_classes(H, W, half=True):
-    """Classes of frequencies that share one propagator: row slots s in
-    [0, H/4] (rows s, H/2 - s, and H/2 + s, H - s reversed) times column
-    pairs l and (W/2 - l) (Hermitian half: l <= W/2)."""
-    row_slots = H // 4 + 1
-    cols = W // 4 + 1 if half else W // 4 + 1 + (3 * W) // 4 - W // 2
-    return row_slots * cols
-
-
-def propagator_build_items(H, W, half=True):
-    """Classes the build computes: on square planes (Hermitian half) a class
-    and its transpose share one build, so n (n + 1) / 2 of the n x n slot
-    pairs; otherwise every class."""
-    if half and H == W:
-        n = W // 4 + 1
-        return n * (n + 1) // 2
-    return propagator_classes(H, W, half)
+def poly_flops(H, W, N, coeffs, reinsch):
+    """FP32 flops of the interval polynomial over the Hermitian half: an angle takes
+    3 (m - 1) + 6 packed instructions in the increment form, 5 (m - 1) + 2 in
+    Reinsch's, of up to 4 flops each (FMAs of a real and an imaginary part: all are
+    counted as such); m is the frequency's, by wx^2 + wy^2 with w = sin 2 pi k / n."""
+    wy = np.sin(2 * np.pi * np.arange(H) / H)[:, None]
+    wx = np.sin(2 * np.pi * np.arange(W // 2 + 1) / W)[None, :]
+    m = np.asarray(coeffs)[np.minimum(7, ((wx ** 2 + wy ** 2) * 4).astype(int))]
+    return int(4 * N * ((5 * (m - 1) + 2) if reinsch else (3 * (m - 1) + 6)).sum())
 
 
 def max_over_ranks(value, dist=None, device="cpu"):
@@ -291,7 +281,7 @@ def run_ours(args, rank, world, local_rank):
     plan = se2n.se2n_plan_create(w.H, w.W, w.N, 0, stream)
     dynamic = args.workload == "dr"
     prop = args.diffusion == "propagator"
-    flags = se2n.SE2N_DIFFUSE_PROPAGATOR if prop else 0
+    flags = se2n.SE2N_DIFFUSE_PROPAGATOR if prop else se2n.SE2N_DIFFUSE_SPLIT_DIAG
     prm = se2n.se2n_params_default(N=w.N, beta=w.beta, T=w.T, steps=w.steps, rounds=w.rounds, eps=w.eps,
                                    sigma_smooth=w.sigma, dynamic=int(dynamic), diffuse_flags=flags)
     f_d = torch.tensor(f32, device=dev)
@@ -348,47 +338,33 @@ def run_ours(args, rank, world, local_rank):
     # the path integrates the Hermitian half of the spectrum: H x (W/2 + 1) frequencies
     updates_per_launch = w.H * (w.W // 2 + 1) * w.N * w.steps
     if prop:
-        # every interval is one column pass (DFT along y, propagators, inverse
+        # every interval is one column pass (DFT along y, the polynomial, inverse
         # DFT along y) and one row pass (inverse real DFT along x, restoration,
-        # forward real DFT along x); the propagators are built once. The
-        # column passes take the largest share of the inpaint.
+        # forward real DFT along x). The column passes take the largest share of
+        # the inpaint.
         c_ms, c_calls = prof["diffuse"]
         c_s = c_ms / c_calls / 1e3
         r_ms, r_calls = prof["fft"]
         r_s = r_ms / r_calls / 1e3
-        b_ms, b_calls = prof["propagator"]
-        b_s = b_ms / b_calls / 1e3
-        classes = propagator_classes(w.H, w.W)
         wc = w.W // 2 + 1
         spec_bytes = 8 * wc * w.H * w.N
-        # the method's bytes: the half spectrum in and out, and every class's
-        # propagator once as its N (N + 1) / 2 distinct entries (the kernel
-        # reads the stored rows, 4 N^2 bytes a class: stored_bytes_per_launch)
-        col_bytes = 2 * spec_bytes + 4 * (w.N * (w.N + 1) // 2) * classes
-        col_stored_bytes = 2 * spec_bytes + 4 * w.N * w.N * classes
+        col_bytes = 2 * spec_bytes
         row_bytes = 2 * spec_bytes + 6 * w.H * w.W
-        col_flops = 2 * wc * w.N * 5 * w.H * int(math.log2(w.H)) + 4 * w.N * w.N * w.H * wc
-        items = propagator_build_items(w.H, w.W)
-        flops, products = propagator_gemm_flops(items, w.N, w.steps)
-        # the symmetric build (N = 16, 32) computes the 10 upper-triangle 8 x 8
-        # tiles of the 16 of every product and mirrors them
-        exec_flops = flops * 10 // 16 if w.N in (16, 32) else flops
+        col_flops = 2 * wc * w.N * 5 * w.H * int(math.log2(w.H)) + poly_flops(w.H, w.W, w.N, POLY_512, False)
         hbm = _peaks().get("hbm_gbs")
         hbm_basis = "MEASURED_PEAKS.json hbm_gbs (copy, burst)"
         roofline = {"bound": "hbm", "achieved": round(col_bytes / c_s / 1e9, 1), "peak": hbm, "unit": "GB/s",
                     "frac": round(col_bytes / c_s / 1e9 / hbm, 4) if hbm else None,
                     "traffic": args.traffic if args.traffic is not None else stored_traffic("col_prop"),
-                    "kernel": f"k_col_tma<{w.N},{w.H}> (column pass: DFT along y, x <- x + D_S x, inverse DFT; "
-                              "whole columns in shared memory, bulk copies in and out, one persistent block an SM)",
+                    "kernel": f"k_col_tma<{w.N},{w.H}> (column pass: DFT along y, the interval's polynomial, inverse "
+                              "DFT; whole columns in shared memory, bulk copies in and out, one persistent block an SM)",
                     "bytes_per_launch": col_bytes,
                     "bytes_basis": "one read and one write of the row-transformed half spectrum (8 (W/2+1) H N "
-                                   "bytes each) + every class's symmetric propagator once, as its N (N + 1) / 2 "
-                                   "distinct entries (4 N (N + 1) / 2 bytes a class)",
-                    "stored_bytes_per_launch": col_stored_bytes,
-                    "stored_basis": "the propagators as the kernel reads them, full rows (4 N^2 bytes a class)",
+                                   "bytes each)",
                     "avg_launch_ms": round(c_s * 1e3, 4), "peak_basis": hbm_basis,
                     "flops_per_launch": col_flops,
-                    "flops_basis": "2 (W/2+1) N complex DFTs of length H at 5 H log2 H + 4 N^2 a frequency",
+                    "flops_basis": "2 (W/2+1) N complex DFTs of length H at 5 H log2 H + the polynomial, 3 (m - 1) + 6 "
+                                   "packed instructions an angle at 4 flops",
                     "frac_of_fp32_peak": round(col_flops / c_s / 1e12 / peak, 4),
                     "row_pass": {"kernel": f"k_row<{w.N},{w.W}> (inverse real DFT along x, restoration, forward "
                                            "real DFT; one block a row)", "bound": "hbm",
@@ -397,31 +373,16 @@ def run_ours(args, rank, world, local_rank):
                                  "achieved_gbs": round(row_bytes / r_s / 1e9, 1), "peak_gbs": hbm,
                                  "frac": round(row_bytes / r_s / 1e9 / hbm, 4) if hbm else None,
                                  "traffic": stored_traffic("row_pass")},
-                    "build": {"kernel": f"k_prop_build_sym<{w.N}> ({items} of the {classes} classes computed, each "
-                                        "also stored permuted for its transpose; FP32 symmetric products; on a side "
-                                        "stream, overlapping the orientation and the first row pass)",
-                              "bound": "alu",
-                              "avg_launch_ms": round(b_s * 1e3, 4),
-                              "flops_basis": "executed flops: classes built x products x 2 N^3 x 10/16 (the symmetric "
-                              "kernel computes the 10 upper-triangle 8x8 tiles of 16 and mirrors them), "
-                              f"S = {w.steps}: {products} products (se2n_prop_chain's program; binary powering "
-                              f"takes {w.steps.bit_length() - 1 + bin(w.steps).count('1') - 1})",
-                              "flops_per_launch": exec_flops,
-                              "full_product_flops_per_launch": flops,
-                              "achieved_tflops": round(exec_flops / b_s / 1e12, 3), "peak_tflops": round(peak, 3),
-                              "frac": round(exec_flops / b_s / 1e12 / peak, 4), "peak_basis": peak_basis,
-                              "frac_full_product_equivalent": round(flops / b_s / 1e12 / peak, 4),
-                              "traffic": stored_traffic("prop_build")},
                     "frequencies_integrated": "Hermitian half, H x (W/2 + 1)"}
     else:
         d_ms, d_calls = prof["diffuse"]
         d_avg_s = d_ms / d_calls / 1e3
-        achieved = FLOPS_PER_UPDATE * updates_per_launch / d_avg_s / 1e12
+        achieved = FLOPS_PER_UPDATE_SPLIT * updates_per_launch / d_avg_s / 1e12
         roofline = {"bound": "alu", "achieved": round(achieved, 3), "peak": round(peak, 3), "unit": "TFLOP/s",
                     "frac": round(achieved / peak, 4),
                     "traffic": args.traffic if args.traffic is not None else stored_traffic(),
-                    "kernel": "k_diffuse_x2<32,2,false> (packed FP32 pairs, truncated corner correction)",
-                    "flops_per_update": FLOPS_PER_UPDATE, "updates_per_launch": updates_per_launch,
+                    "kernel": "k_diffuse_x2<32,2,true> (packed FP32 pairs, truncated corner correction)",
+                    "flops_per_update": FLOPS_PER_UPDATE_SPLIT, "updates_per_launch": updates_per_launch,
                     "avg_launch_ms": round(d_avg_s * 1e3, 4), "peak_basis": peak_basis,
                     "diffuse_updates_per_s": updates_per_launch / d_avg_s,
                     "hbm_gbs_of_diffuse": round(16 * w.H * (w.W // 2 + 1) * w.N / d_avg_s / 1e9, 1),
@@ -430,7 +391,8 @@ def run_ours(args, rank, world, local_rank):
               for k, v in prof.items() if k != "kernels"}
     launches = int(prof["kernels"])
 
-    cfg = _config(w, {"diffusion": "S-step propagators built every inpaint (SE2N_DIFFUSE_PROPAGATOR)" if prop
+    cfg = _config(w, {"diffusion": "each interval's steps as one map, a polynomial of the operator "
+                                   "(SE2N_DIFFUSE_PROPAGATOR, nothing kept between inpaints)" if prop
                       else "step by step, the fused Crank-Nicolson kernel"}, dynamic=dynamic)
     result = {"metric": METRIC, "ms_per_inpaint": round(ms_per_step, 4), "value": value, "unit": UNIT,
               "m2_updates_per_s": world * w.updates() * args.steps / (total_ms / 1e3),
@@ -443,8 +405,8 @@ def run_ours(args, rank, world, local_rank):
                               "steps run without them (they add about 0.1 ms an inpaint)"}
     if prop:
         # the other two ways to run the same inpaint, on the same plan and inputs:
-        # propagators kept from the previous call (serving one beta dt and S),
-        # and the step-by-step kernel with its own roofline
+        # without dropping what the plan keeps between calls (the polynomial's
+        # coefficients), and the step-by-step kernel with its own roofline
         with torch.cuda.stream(stream):
             def timed3(fn):
                 evs = []
@@ -465,7 +427,8 @@ def run_ours(args, rank, world, local_rank):
             kprof = se2n.se2n_plan_profile_read(plan, reset=True)
             se2n.se2n_plan_profile(plan, False)
             prm_s = se2n.se2n_params_default(N=w.N, beta=w.beta, T=w.T, steps=w.steps, rounds=w.rounds, eps=w.eps,
-                                             sigma_smooth=w.sigma, dynamic=int(dynamic))
+                                             sigma_smooth=w.sigma, dynamic=int(dynamic),
+                                             diffuse_flags=se2n.SE2N_DIFFUSE_SPLIT_DIAG)
             se2n.se2n_inpaint(plan, f_d, m_d, None, prm_s, vol, out)
             torch.cuda.synchronize(dev)
             se2n.se2n_plan_profile(plan, True)
@@ -473,10 +436,9 @@ def run_ours(args, rank, world, local_rank):
             sprof = se2n.se2n_plan_profile_read(plan, reset=True)
             se2n.se2n_plan_profile(plan, False)
         sd_s = sprof["diffuse"][0] / sprof["diffuse"][1] / 1e3
-        s_ach = FLOPS_PER_UPDATE * updates_per_launch / sd_s / 1e12
+        s_ach = FLOPS_PER_UPDATE_SPLIT * updates_per_launch / sd_s / 1e12
         result["propagators_kept"] = {"ms_per_step": round(kept, 4), "value": world * upd / (kept / 1e3)}
-        # the row and column passes timed where nothing runs beside them (in the
-        # timed inpaints the build overlaps the orientation and the first row pass)
+        # the row and column passes as timed in those
         c_s = kprof["diffuse"][0] / kprof["diffuse"][1] / 1e3
         r_s = kprof["fft"][0] / kprof["fft"][1] / 1e3
         hbm = roofline["peak"]
@@ -484,18 +446,18 @@ def run_ours(args, rank, world, local_rank):
         roofline.update({"achieved": round(col_bytes / c_s / 1e9, 1), "avg_launch_ms": round(c_s * 1e3, 4),
                          "frac": round(col_bytes / c_s / 1e9 / hbm, 4) if hbm else None,
                          "frac_of_fp32_peak": round(roofline["flops_per_launch"] / c_s / 1e12 / peak, 4),
-                         "timed_on": "the inpaints that reuse the propagators (CUDA events around each launch)"})
+                         "timed_on": "the inpaints of propagators_kept (CUDA events around each launch)"})
         roofline["row_pass"].update({"avg_launch_ms": round(r_s * 1e3, 4),
                                      "achieved_gbs": round(row_bytes / r_s / 1e9, 1),
                                      "frac": round(row_bytes / r_s / 1e9 / hbm, 4) if hbm else None,
-                                     "timed_on": "the inpaints that reuse the propagators; the average over all "
+                                     "timed_on": "the inpaints of propagators_kept; the average over all "
                                                  "row passes of an inpaint (lift and projection included)"})
         result["step_by_step"] = {
             "ms_per_step": round(stepwise, 4), "value": world * upd / (stepwise / 1e3),
-            "roofline": {"bound": "alu", "kernel": "k_diffuse_x2<32,2,false>", "avg_launch_ms": round(sd_s * 1e3, 4),
+            "roofline": {"bound": "alu", "kernel": "k_diffuse_x2<32,2,true>", "avg_launch_ms": round(sd_s * 1e3, 4),
                          "achieved": round(s_ach, 3), "peak": round(peak, 3), "unit": "TFLOP/s",
                          "frac": round(s_ach / peak, 4), "traffic": stored_traffic(),
-                         "flops_per_update": FLOPS_PER_UPDATE, "updates_per_launch": updates_per_launch}}
+                         "flops_per_update": FLOPS_PER_UPDATE_SPLIT, "updates_per_launch": updates_per_launch}}
     if dynamic:
         # with propagators the image value h and its argmax angle come from a
         # row pass (counted with the row passes); the growth kernel reads h,
@@ -674,7 +636,7 @@ def run_2048(args, rank, world, local_rank):
     f32 = w.f.astype(np.float32)
     plan = se2n.se2n_plan_create(w.H, w.W, w.N, 0, stream)
     prop = args.diffusion == "propagator"
-    flags = se2n.SE2N_DIFFUSE_PROPAGATOR if prop else 0
+    flags = se2n.SE2N_DIFFUSE_PROPAGATOR if prop else se2n.SE2N_DIFFUSE_SPLIT_DIAG
 
     def params(wk, fl):
         return se2n.se2n_params_default(N=wk.N, beta=wk.beta, T=wk.T, steps=wk.steps, rounds=wk.rounds, eps=wk.eps,
@@ -722,53 +684,20 @@ def run_2048(args, rank, world, local_rank):
     d_ms, d_calls = prof["diffuse"]
     d_s = d_ms / d_calls / 1e3
     if prop:
-        b_ms, b_calls = prof["propagator"]
-        b_s = b_ms / b_calls / 1e3
-        items = propagator_build_items(w.H, w.W)
-        flops, products = propagator_gemm_flops(items, w.N, w.steps)
-        # the symmetric build computes the 36 upper-triangle 8 x 8 tiles of the
-        # 64 of every N = 64 product and mirrors them
-        exec_flops = flops * 36 // 64
-        # DRAM traffic from a one-launch capture of a smaller square plane of
-        # the same workload, scaled to this launch by the classes built (the
-        # build) and by the method's bytes (the apply)
-        rec_b, rec_a = stored_record("prop_build_wide"), stored_record("prop_apply_tiled")
-        b_traffic = round(rec_b["dram_bytes_per_launch"] * items / rec_b["classes_built"]) if rec_b else None
-        roofline = {"bound": "alu",
-                    "kernel": f"k_prop_build_symw<{w.N}> ({items} classes computed, row slot <= column slot; a "
-                              "transposed class applies its transpose's rows; FP32 symmetric products)",
-                    "achieved": round(exec_flops / b_s / 1e12, 3), "peak": round(peak, 3), "unit": "TFLOP/s",
-                    "frac": round(exec_flops / b_s / 1e12 / peak, 4), "traffic": b_traffic,
-                    "traffic_basis": (f"ncu on {rec_b['workload']} ({rec_b['dram_bytes_per_launch']} bytes, "
-                                      f"{rec_b['classes_built']} classes) x classes built") if rec_b else None,
-                    "avg_launch_ms": round(b_s * 1e3, 4), "flops_per_launch": exec_flops,
-                    "flops_basis": f"executed flops: classes x {products} products x 2 N^3 x 36/64 (the upper-triangle "
-                                   "8x8 tiles)",
-                    "full_product_flops_per_launch": flops,
-                    "frac_full_product_equivalent": round(flops / b_s / 1e12 / peak, 4),
+        flops = poly_flops(w.H, w.W, w.N, POLY_2048, True)
+        a_bytes = 2 * 8 * w.N * w.H * (w.W // 2 + 1)
+        roofline = {"bound": "alu", "kernel": f"k_poly<{w.N},true> (the interval as a polynomial of its operator, "
+                                              "Reinsch's form)",
+                    "achieved": round(flops / d_s / 1e12, 3), "peak": round(peak, 3), "unit": "TFLOP/s",
+                    "frac": round(flops / d_s / 1e12 / peak, 4), "traffic": None,
+                    "avg_launch_ms": round(d_s * 1e3, 4), "flops_per_launch": flops,
+                    "flops_basis": "5 (m - 1) + 2 packed instructions an angle at 4 flops",
                     "peak_basis": "152 SMs x 128 FP32 lanes x 2 flop/FMA x 2070 MHz (derived, not measured)",
-                    "apply_avg_launch_ms": round(d_s * 1e3, 4)}
-        # the separate apply on the Hermitian half, tile by tile: the half
-        # spectrum in and out, and every built class's N x N rows once (a
-        # transposed class reads its transpose's rows, from L2 when the
-        # super-tile order works)
-        wc = w.W // 2 + 1
-        a_bytes = 2 * 8 * w.N * w.H * wc + 4 * w.N * w.N * items
-        hbm = _peaks().get("hbm_gbs")
-        roofline["apply"] = {"kernel": f"k_prop_apply_tiled<{w.N}>", "bound": "hbm", "avg_launch_ms": round(d_s * 1e3, 4),
-                             "bytes_per_launch": a_bytes,
-                             "traffic": round(rec_a["dram_bytes_per_launch"] * a_bytes / rec_a["method_bytes"])
-                             if rec_a else None,
-                             "traffic_basis": (f"ncu on {rec_a['workload']} ({rec_a['dram_bytes_per_launch']} bytes for "
-                                               f"{rec_a['method_bytes']} method's bytes) x method's bytes")
-                             if rec_a else None,
-                             "bytes_basis": "8 N H (W/2 + 1) bytes in and out + 4 N^2 bytes a built class",
-                             "achieved": round(a_bytes / d_s / 1e9, 1), "peak": hbm, "unit": "GB/s",
-                             "frac": round(a_bytes / d_s / 1e9 / hbm, 4) if hbm else None,
-                             "peak_basis": "MEASURED_PEAKS.json hbm_gbs (copy, burst)"}
+                    "bytes_per_launch": a_bytes, "bytes_basis": "8 N H (W/2 + 1) bytes in and out",
+                    "hbm_gbs": round(a_bytes / d_s / 1e9, 1)}
     else:
-        achieved = FLOPS_PER_UPDATE * upd / d_s / 1e12
-        roofline = {"bound": "alu", "kernel": f"k_diffuse_x2<{w.N},4,...> (packed FP32 pairs)",
+        achieved = FLOPS_PER_UPDATE_SPLIT * upd / d_s / 1e12
+        roofline = {"bound": "alu", "kernel": f"k_diffuse_x2<{w.N},4,true> (packed FP32 pairs)",
                     "achieved": round(achieved, 3), "peak": round(peak, 3), "unit": "TFLOP/s",
                     "frac": round(achieved / peak, 4), "traffic": None, "flops_per_update": FLOPS_PER_UPDATE,
                     "updates_per_launch": upd, "avg_launch_ms": round(d_s * 1e3, 4),
@@ -778,7 +707,7 @@ def run_2048(args, rank, world, local_rank):
               if k != "kernels" and v[1] > 0}
 
     # the other diffusion on the same inpaint, for comparison
-    other = params(w, 0 if prop else se2n.SE2N_DIFFUSE_PROPAGATOR)
+    other = params(w, se2n.SE2N_DIFFUSE_SPLIT_DIAG if prop else se2n.SE2N_DIFFUSE_PROPAGATOR)
     other_ms = timed(other, 2, 1)
     # the stiff run: split diagonal (beta T > 8), FP32 and FP64 corrections
     stiff = {}
@@ -792,7 +721,7 @@ def run_2048(args, rank, world, local_rank):
               "config": {"workload": f"{w.name}: {w.H}x{w.W} lines plus textured patches, N=64, 85% "
                                      "random mask, beta=0.25, T=50, one interval of 1000 CN steps",
                          "updates_per_step": upd, "m2_updates_per_step": w.updates(),
-                         "diffusion": "S-step propagators (separate apply)" if prop else
+                         "diffusion": "the interval as a polynomial of its operator (SE2N_DIFFUSE_PROPAGATOR)" if prop else
                                       "step by step, the fused Crank-Nicolson kernel",
                          "l2": "flushed between timed steps (256 MiB write); the 2 GiB volume exceeds L2",
                          "parallelism": "replicas"},
@@ -990,11 +919,8 @@ def run_batch(args, rank, world, local_rank):
     h2d = sum(hf.nbytes + hm.nbytes for hf, hm in host_in)
     d2h = sum(ho.nbytes for ho in host_out)
     # the persistent launch integrates the Hermitian half of the spectra of the
-    # images it keeps (all of them step by step; with propagators, the shapes
-    # the batch left to it), one interval
+    # images it keeps, one interval
     half_updates = info["step_updates"]
-    achieved = FLOPS_PER_UPDATE * half_updates / (ms_diff / 1e3) / 1e12
-    peak = SM_COUNT * FP32_LANES_PER_SM * 2 * 2070e6 / 1e12
     batch.close()
     if dist:
         dist.destroy_process_group()
@@ -1008,22 +934,22 @@ def run_batch(args, rank, world, local_rank):
                        "updates_basis": "H x (W/2 + 1) frequencies (the Hermitian half) x N x steps, summed over "
                                         "the images; m2_updates_per_step counts all H x W",
                        "m2_updates_per_step": info["updates_per_run"] * world,
-                       "diffusion": ("S-step propagators for the shapes where they are estimated cheaper "
+                       "diffusion": ("each interval as one map (the polynomial) for the shapes where it is estimated cheaper "
                                      f"({info['prop_images']} images; {info['fused_images']} of them, the "
                                      "shapes the row and column passes cover (N = 16, 30, 32), whole inpaints on "
-                                     "them, the others with the separate apply), the persistent step kernel for "
+                                     "them, the others with the separate apply), the persistent kernel for "
                                      "the rest")
-                       if prop else "the persistent step-by-step kernel for every image",
+                       if prop else "the persistent kernel for every image (the polynomial where it takes "
+                                    "the place of the steps)",
                        "l2": "flushed between timed steps (256 MiB write)", "parallelism": "replicas"},
             "per_image_launches": {"ms_per_step": ms_per_image, "value": total_updates / (ms_per_image / 1e3),
                                    "speedup_of_batched": ms_per_image / ms},
-            "roofline": ({"bound": "alu", "achieved": round(achieved, 3), "peak": round(peak, 3), "unit": "TFLOP/s",
-                          "frac": round(achieved / peak, 4), "traffic": None, "kernel": "k_diffuse_batch",
-                          "avg_launch_ms": round(ms_diff, 3)} if half_updates > 0 else
-                         {"bound": None, "kernel": None,
-                          "note": "every image is integrated by propagators (the persistent step kernel has no "
-                                  "work): the rooflines of the build, the row and column passes and the separate "
-                                  "apply are those of the 512 and 2048 workloads"}),
+            "roofline": {"bound": None, "kernel": "k_poly_batch" if half_updates > 0 else None,
+                         "avg_launch_ms": round(ms_diff, 3),
+                         "equivalent_updates_per_s": half_updates / (ms_diff / 1e3) if half_updates > 0 else None,
+                         "note": "the intervals are polynomials: the rooflines of the row and column passes and of "
+                                 "the polynomial kernel are those of the 512 and 2048 workloads; the persistent "
+                                 "launch integrates the shapes left to it"},
             "e2e": {"value": total_updates / (ms_e2e / 1e3), "unit": UNIT, "ms_per_step": ms_e2e,
                     "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                     "api": "se2n_batch_run on device inputs refreshed from pinned host buffers"},

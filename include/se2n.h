@@ -82,7 +82,9 @@ typedef enum se2n_status {
  * 50 for 75), whose coefficients the host makes when beta, T or steps change;
  * where more than 64 coefficients would be needed, and in the column pass (below)
  * with N = 16 or where applying kept matrices is faster (T (2 + 4 beta) / 2 above
- * about 3), as a matrix:
+ * about 3), and on the Hermitian half of other sizes where it is faster (above some 30
+ * to 60) from the second call for the same beta, T and steps on (not in a stream
+ * capture, and not without room for them), as a matrix:
  * for every class of frequencies that share it (rows s, H/2 - s as they are
  * and rows H/2 + s, H - s with the angles reversed, times columns l and
  * (W/2 - l) mod W) (B-^{-1} B+)^S - I is built once in FP32 by the powering

@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(col_threads<H>(), H >= 768 ? 1 : 2) k_col_prop
 #pragma unroll 4
     for (int q = 0; q < C::NP; ++q) {
         const int f = tid + q * T, k = 2 * f / N, n = 2 * f % N;
-        const float4 x0 = g[f], x1 = g[HALF4 + f];
+        const float4 x0 = __ldcg(g + f), x1 = __ldcg(g + HALF4 + f);
         const float2 w = tws[k];
         put2<N, L>(X, k, n, make_float2(x0.x + x1.x, x0.y + x1.y), make_float2(x0.z + x1.z, x0.w + x1.w));
         const float2 d0 = twiddle<-1>(make_float2(x0.x - x1.x, x0.y - x1.y), w);

@@ -29,7 +29,7 @@ __device__ __forceinline__ void pack16(const float (&w)[16], uint32_t (&p)[8]) {
     for (int q = 0; q < 8; ++q) p[q] = pack2(w[2 * q], w[2 * q + 1]);
 }
 // relu?(v + bias) as bf16; nb bias values (the output channels).
-// pool: also the 2x2 averages of the bf16 outputs (sums in the order of k_pool); a
+// pool: also the 2x2 averages of the bf16 outputs (a + b + c + d of the rows in turn, FP32); a
 // warp has to hold 8 x 4 pixels then (k_conv_halo, k_conv_group). It saves the
 // kernel that read the output again: 120 us for the three poolings at 64 images of
 // 256 x 256, for about 40 of a longer epilogue. The upsampling in the same way (four

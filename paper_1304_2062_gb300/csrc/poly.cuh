@@ -192,7 +192,7 @@ __device__ __forceinline__ void poly_group(const PolyTable &t, const float *sc, 
     f32x2 x[K];
 #pragma unroll
     for (int j = 0; j < K; ++j) {
-        const float2 v = col[j * HW];
+        const float2 v = __ldcg(col + j * HW);
         x[j] = pk2(v.x, v.y);
     }
     const int k = (int)(fc / Wc);

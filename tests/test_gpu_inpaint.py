@@ -289,3 +289,80 @@ def test_inpaint_rejects_bad_parameters():
     with pytest.raises(se2n.Se2nError):
         se2n.se2n_inpaint(plan, np.ones((16, 16), np.float32), m, None, prm, vol, out)   # host image
     plan.close()
+
+
+@pytest.mark.parametrize("N,H,W,T,steps,flags", [
+    # every column length, with the polynomial in place of the steps and of the matrices
+    (32, 64, 64, 2.0, 20, 0), (16, 128, 64, 2.0, 20, 0), (30, 256, 64, 2.0, 20, 8), (32, 384, 64, 2.0, 20, 8),
+    (32, 512, 64, 2.0, 20, 0), (30, 768, 64, 2.0, 20, 0), (16, 1024, 64, 2.0, 20, 0), (32, 1024, 64, 2.0, 20, 8),
+    # on either side of the cost up to which it replaces matrices (48: T = 2.7), and of
+    # the steps it replaces (5 a step and 36)
+    (32, 64, 128, 2.6, 20, 8), (32, 64, 128, 3.0, 20, 8), (30, 128, 64, 2.6, 20, 8), (30, 128, 64, 3.0, 20, 8),
+    (32, 64, 64, 0.5, 1, 0), (16, 64, 64, 1.0, 2, 0), (32, 64, 64, 2.0, 4, 0),
+    # Reinsch's form: no column pass without a flag, matrices with it
+    (32, 64, 64, 13.0, 40, 0), (32, 64, 64, 13.0, 40, 8), (16, 64, 64, 13.0, 40, 0)])
+def test_column_pass_polynomial_matches_oracle(N, H, W, T, steps, flags):
+    """One interval on the row and column passes, over the rule that picks
+    polynomial, matrices or steps, against the oracle (single-result bound)."""
+    w = synth.workload_512(H=H, W=W, steps=steps, rounds=1)
+    _compare(w, oracle.Params(N=N, beta=0.25, T=T, steps=steps, rounds=1), flags=flags)
+
+
+@pytest.mark.parametrize("N,H,W,T", [(64, 20, 36, 25.0), (64, 20, 36, 45.0), (32, 36, 20, 55.0), (16, 30, 34, 55.0)])
+def test_repeated_calls_with_propagators_match_oracle(N, H, W, T):
+    """At large T a plan applies the polynomial in the first call and the
+    matrices it keeps in later ones; another interval or dropping them begins
+    again with the polynomial. Every call within the single-result bound."""
+    steps = int(4 * T)
+    w = synth.workload_512(H=H, W=W, steps=steps, rounds=1)
+    f32 = w.f.astype(np.float32)
+    f64 = f32.astype(np.float64)
+    bins = oracle.orient(f64, w.mask, N)["bins"]
+    plan = se2n.se2n_plan_create(H, W, N)
+    fd, md, bd = t_f32(f32), t_u8(w.mask), t_u8(bins)
+    vol = torch.empty((N, H, W), dtype=torch.complex64, device="cuda")
+    out = torch.empty((H, W), dtype=torch.float32, device="cuda")
+    for t in (T, T, T, T / 2, T, None, T):
+        if t is None:
+            se2n.se2n_plan_drop_propagators(plan, 1)
+            continue
+        p = oracle.Params(N=N, beta=0.25, T=t, steps=steps, rounds=1)
+        se2n.se2n_inpaint(plan, fd, md, bd, _params(p, se2n.SE2N_DIFFUSE_PROPAGATOR), vol, out)
+        ref = oracle.inpaint(f64, w.mask, p, bins=bins)["out"]
+        assert np.abs(host(out) - ref).max() / np.abs(f64).max() <= MAX_REL
+        assert rel_l2(host(out), ref) <= REL_L2
+    plan.close()
+
+
+@pytest.mark.parametrize("N,H,W,flags", [(32, 512, 512, se2n.SE2N_DIFFUSE_PROPAGATOR), (32, 256, 256, 0),
+                                         (16, 128, 128, 0), (24, 120, 144, 0)])
+def test_back_to_back_inpaints_repeat_their_bits(N, H, W, flags):
+    """Inpaints of two plans issued in turn without waiting: every kernel may
+    start while the one before still runs, and none may read what an earlier
+    one left in a cache. All results equal the first, to the bit."""
+    runs = []
+    for seed in range(2):
+        w = synth.workload_512(H=H, W=W, steps=20, rounds=4)
+        f = np.roll(w.f.astype(np.float32), 5 * seed, axis=0)
+        p = oracle.Params(N=N, beta=0.25, T=8.0, steps=20, rounds=4)
+        plan = se2n.se2n_plan_create(H, W, N)
+        vol = torch.empty((N, H, W), dtype=torch.complex64, device="cuda")
+        runs.append((plan, t_f32(f), t_u8(w.mask), _params(p, flags), vol))
+
+    def one(r):
+        plan, f, m, prm, vol = r
+        out = torch.empty((H, W), dtype=torch.float32, device="cuda")
+        se2n.se2n_inpaint(plan, f, m, None, prm, vol, out)
+        return out
+
+    first = []
+    for r in runs:
+        first.append(one(r).clone())
+        torch.cuda.synchronize()
+    outs = [[one(r) for r in runs] for _ in range(60)]
+    torch.cuda.synchronize()
+    for pair in outs:
+        for got, want in zip(pair, first):
+            assert torch.equal(got, want)
+    for r in runs:
+        r[0].close()
