@@ -324,7 +324,6 @@ cudaError_t launch_halo(const __nv_bfloat16 *A, int B, int H, int W, int C, cons
     g.ntiles = N / BN;
     g.tiles = g.mtiles * g.ntiles;
     g.nchunk = C / CK;
-    g.KB = g.nchunk;
     g.flip = flip;
     g.order = whole_tiles(H, W) ? tma::ORDER_BLOCKS : tma::ORDER_TAPS;
     if (g.order == tma::ORDER_TAPS && S < g.nchunk) return cudaErrorNotSupported;
@@ -368,7 +367,6 @@ cudaError_t launch_pair(const __nv_bfloat16 *A, int B, int H, int W, int C, cons
     g.ntiles = 1;
     g.tiles = g.mtiles;
     g.nchunk = C / 32;
-    g.KB = g.nchunk;
     g.flip = flip;
     g.order = !whole_tiles(H, W) ? tma::ORDER_TAPS : C % 64 ? tma::ORDER_BLOCKS : tma::ORDER_OFFSETS;
     if (g.order == tma::ORDER_OFFSETS && C > 64) return cudaErrorNotSupported;  // blocks of 64 in between
@@ -449,7 +447,6 @@ cudaError_t launch_group(const __nv_bfloat16 *A, int B, int H, int W, int C, con
     g.ntiles = N / BN;
     g.tiles = g.mtiles * g.ntiles;
     g.nchunk = C / 64;
-    g.KB = 9 * g.nchunk;
     g.flip = flip;
     g.order = tma::ORDER_TAPS;
     if (g.nchunk > Cf::AMAX) return cudaErrorNotSupported;  // a tile's boxes stay for all taps
@@ -503,9 +500,16 @@ cudaError_t launch_wgrad(const __nv_bfloat16 *x, int B, int H, int W, int C, con
     const int cv = F * C, nv = F * Cout;
     g.cgroups = cv / 64;
     g.ngroups = nv / 64;
-    // one unit a CTA and one CTA an SM: as many pixel ranges as fill the device once
+    // the lengths of the sums (conv_tma.cuh), and CTAs that fill the device once
     const int groups = g.cgroups * g.ngroups;
-    g.ksplit = nsm / groups;
+    const int mtiles = (9 * C + 127) / 128;
+    int ranges = F == 8 ? nsm : (2 * nsm + mtiles - 1) / mtiles;
+    if (F == 2) ranges = (ranges + 1) / 2;
+    g.parts = F == 8 ? 1 : (2 * nsm + groups * ranges) / (2 * groups * ranges);  // nsm / (groups ranges), rounded
+    if (g.parts > 3) g.parts = 3;
+    if (g.parts < 1) g.parts = 1;
+    g.ksplit = nsm / (groups * g.parts);
+    if (g.ksplit > ranges) g.ksplit = ranges;
     if (g.ksplit > g.kblocks) g.ksplit = g.kblocks;
     if (g.ksplit < 1) g.ksplit = 1;
     auto map = [&](CUtensorMap *m, const __nv_bfloat16 *p, int ch, int cols, int rows) {
@@ -524,7 +528,7 @@ cudaError_t launch_wgrad(const __nv_bfloat16 *x, int B, int H, int W, int C, con
     auto *fn = bkx == 32 ? &tma::k_wgrad_tma<32> : &tma::k_wgrad_tma<16>;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    fn<<<groups * g.ksplit, 192, smem, s>>>(mx, mg, g, dw, err);
+    fn<<<groups * g.ksplit * g.parts, 192, smem, s>>>(mx, mg, g, dw, err);
     return cudaGetLastError();
 }
 

@@ -56,7 +56,6 @@ struct ConvGeo {
     int bw, bh;          // tile shape in pixels (bw * bh == 128)
     int tiles_x, tiles_y, mtiles, ntiles, tiles;
     int nchunk;          // C / CK
-    int KB;              // 9 * nchunk
     int flip;            // 1: taps mirrored (data gradient)
     int order;           // of the sums: SumOrder
 };
@@ -1078,11 +1077,16 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
 //    dx = F s + px - pg; s = -1, 0, 1 give every combination that is a tap, the
 //    others are left out by the epilogue (or not loaded, where a group of 64
 //    channels holds no such pixels). 1 / F of the box rows.
-// A unit of work is (64 channels of In, 64 of gz, a range of pixel blocks); every
-// CTA takes one, accumulates it in tensor memory (up to 5 tiles of 64
-// columns) and adds it to dW with FP32 atomics at the end.
-// Measured (batch 32, 256 x 256): 32 -> 32 channels 71 us (1008 with a box a tap and
-// operand), 96 -> 32 193, all 14 layers 886 us (4832; 1071 with a box a column offset).
+// A unit of work is (64 channels of In, 64 of gz, a range of pixel blocks),
+// accumulated in tensor memory (up to 5 tiles of 64 columns) and added to dW with FP32
+// atomics at the end. The tensor core's sums truncate, so a sum loses bits in
+// proportion to its length, and the number of ranges is part of the result (4e-5 of a
+// gradient of 32 images when the ranges are a third as long): it stays at the two units an SM
+// of tiles of 128 (tap, channel) rows that the kernel once had, half as many where a
+// pixel pair makes two sums of each. Where that leaves SMs idle up to three
+// CTAs share a unit's tiles.
+// Measured (batch 32, 256 x 256): all 14 layers 1525 us (4832 with a box a tap and
+// operand; 888 with as many ranges as SMs).
 // ---------------------------------------------------------------------------
 
 constexpr int kWgR = 8;                    // image rows of a pixel block
@@ -1100,6 +1104,7 @@ struct WgradGeo {
     int xblocks, yblocks, kblocks;
     int cgroups, ngroups;  // 64-channel groups of In and gz as read
     int ksplit;         // pixel ranges a (channel group, channel group)
+    int parts;          // CTAs that share a unit's tiles
 };
 
 // MN-major matrix descriptor, 128-byte swizzle: leading byte offset = stride
@@ -1141,7 +1146,8 @@ __global__ void __launch_bounds__(192, 1)
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
     // the unit: channel groups cg (of In) and ng (of gz), pixel blocks [kb0, kb1)
-    const int ks = blockIdx.x % g.ksplit, gr = blockIdx.x / g.ksplit;
+    const int part = blockIdx.x % g.parts, unit = blockIdx.x / g.parts;
+    const int ks = unit % g.ksplit, gr = unit / g.ksplit;
     const int c0 = (gr % g.cgroups) * 64, n0 = (gr / g.cgroups) * 64;
     const int per = (g.kblocks + g.ksplit - 1) / g.ksplit;
     const int kb0 = ks * per, kb1 = min(g.kblocks, kb0 + per);
@@ -1166,7 +1172,8 @@ __global__ void __launch_bounds__(192, 1)
         asm volatile("prefetch.tensormap [%0];\n" ::"l"((uint64_t)&mapG) : "memory");
     }
     __syncthreads();
-    if (*abort || kb0 >= kb1) return;
+    const int ns = s1 - s0 + 1, nt = ns + (ns + 1) / 2;  // tiles of the unit; this CTA's: part, part + parts, ..
+    if (*abort || kb0 >= kb1 || part >= nt) return;
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(tmem_slot),
                      "r"((uint32_t)TMEM_COLS));
@@ -1230,7 +1237,6 @@ __global__ void __launch_bounds__(192, 1)
             constexpr uint32_t IDESC = idesc_bf16_mn<64>();
             const uint64_t x_desc0 = sdesc_mn(base, ROW), x_desc1 = sdesc_mn(base, 128u);
             const uint64_t g_desc0 = sdesc_mn(gbase, GROW);
-            const int ns = s1 - s0 + 1;
             int xs = 0, gs = 0;
             uint32_t xph = 0, gph = 0;
             bool ok = true;
@@ -1260,12 +1266,10 @@ __global__ void __launch_bounds__(192, 1)
                     for (int kk = 0; kk < BKX / 16; ++kk) {
                         const uint64_t off = (j * ROW + kk * 2048u) / 16, goff = (j * GROW + kk * 2048u) / 16;
                         const uint32_t add = j + kk > 0 || kb > kb0 ? 1u : 0u;
-                        for (int t = 0; t < ns; ++t)
-                            mma_f16_elect(tmem_base + (uint32_t)(t * 64), d0 + off + (uint64_t)(t * 8), dg + goff, IDESC,
-                                          add);
-                        for (int t = 0; t < ns; t += 2)
-                            mma_f16_elect(tmem_base + (uint32_t)(ns * 64 + t * 32), d1 + off + (uint64_t)(t * 8),
-                                          dg + goff, IDESC, add);
+                        for (int t = part; t < nt; t += g.parts)
+                            mma_f16_elect(tmem_base + (uint32_t)(t * 64),
+                                          (t < ns ? d0 + (uint64_t)(t * 8) : d1 + (uint64_t)((t - ns) * 16)) + off, dg + goff,
+                                          IDESC, add);
                     }
                 }
                 mma_commit_elect(bar_xempty + 8 * xs);
@@ -1294,27 +1298,26 @@ __global__ void __launch_bounds__(192, 1)
             const int i = (q & 1) * 32 + lane;   // channel of In in the group
             const int e = c0 + i;
             const int px = g.F > 1 ? e / g.C : 0, ci = e - px * g.C;
-            const int ns = s1 - s0 + 1;
-            for (int t = 0; t < ns + (ns + 1) / 2; ++t) {
-                    // tiles (dy -1 | 0) of each s, then (s | s + 1) of dy 1
-                    const int s = t < ns ? s0 + t : s0 + 2 * (t - ns) + (q >> 1);
-                    const int dy = t < ns ? (q >> 1) - 1 : 1;
-                    if (s > s1) continue;  // no tap (warp-uniform)
-                    const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(t * 64);
+            for (int t = part; t < nt; t += g.parts) {
+                // tiles (dy -1 | 0) of each s, then (s | s + 1) of dy 1
+                const int s = t < ns ? s0 + t : s0 + 2 * (t - ns) + (q >> 1);
+                const int dy = t < ns ? (q >> 1) - 1 : 1;
+                if (s > s1) continue;  // no tap (warp-uniform)
+                const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(t * 64);
 #pragma unroll 1
-                    for (int j0 = 0; j0 < 64; j0 += 16) {
-                        uint32_t v[16];
-                        tc::tmem_ld16(taddr + (uint32_t)j0, v);
-                        const int f = n0 + j0;  // 16 channels of one pixel: Cout is a multiple of 32
-                        const int pg = g.F > 1 ? f / g.Cout : 0, co = f - pg * g.Cout;
-                        const int dx = g.F * s + px - pg;
-                        if (dx >= -1 && dx <= 1) {
-                            float *p = dw + ((long long)co * 9 + (dy + 1) * 3 + (dx + 1)) * g.C + ci;
+                for (int j0 = 0; j0 < 64; j0 += 16) {
+                    uint32_t v[16];
+                    tc::tmem_ld16(taddr + (uint32_t)j0, v);
+                    const int f = n0 + j0;  // 16 channels of one pixel: Cout is a multiple of 32
+                    const int pg = g.F > 1 ? f / g.Cout : 0, co = f - pg * g.Cout;
+                    const int dx = g.F * s + px - pg;
+                    if (dx >= -1 && dx <= 1) {
+                        float *p = dw + ((long long)co * 9 + (dy + 1) * 3 + (dx + 1)) * g.C + ci;
 #pragma unroll
-                            for (int c = 0; c < 16; ++c) atomicAdd(p + (long long)c * 9 * g.C, __uint_as_float(v[c]));
-                        }
+                        for (int c = 0; c < 16; ++c) atomicAdd(p + (long long)c * 9 * g.C, __uint_as_float(v[c]));
                     }
                 }
+            }
             asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
         }
     }

@@ -18,14 +18,17 @@ using namespace se2n::nn;
 namespace {
 
 // Weights rearranged for the data gradient, K-major in the output channel:
-// wt[ci][tap * Cout + co] = w[co][tap * Cin + ci].
-__global__ void k_transpose_dgrad(const __nv_bfloat16 *w, __nv_bfloat16 *wt, int Cout, int Cin) {
-    const long long total = (long long)Cout * 9 * Cin;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-        const int co = (int)(i % Cout);
-        const long long t = i / Cout;
-        const int tap = (int)(t % 9), ci = (int)(t / 9);
-        wt[i] = w[((long long)co * 9 + tap) * Cin + ci];
+// wt[ci][tap * Cout + co] = w[co][tap * Cin + ci], layer blockIdx.y at the same offset in
+// both. One launch for all layers: a launch of a few microseconds each took 51 us of a
+// backward pass.
+__global__ void k_transpose_dgrad(const __nv_bfloat16 *w0, __nv_bfloat16 *wt0, const __grid_constant__ ConvLayers d) {
+    const int Cout = d.cout[blockIdx.y], Cin = d.cin[blockIdx.y];
+    const __nv_bfloat16 *w = w0 + d.off[blockIdx.y];
+    __nv_bfloat16 *wt = wt0 + d.off[blockIdx.y];
+    const int total = Cout * 9 * Cin;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+        const int co = i % Cout, t = i / Cout, tap = t % 9, ci = t / 9;
+        wt[i] = w[(co * 9 + tap) * Cin + ci];
     }
 }
 
@@ -391,13 +394,9 @@ int grid_for(long long n) {
 namespace se2n {
 namespace nn {
 
-cudaError_t conv_backward_data(const __nv_bfloat16 *gz, int B, int H, int W, int Cout, const __nv_bfloat16 *w, int Cin,
-                               const __nv_bfloat16 *act, __nv_bfloat16 *din, __nv_bfloat16 *din2, int split,
-                               __nv_bfloat16 *wt_scratch, cudaStream_t s) {
-    const long long nw = (long long)Cout * 9 * Cin;
-    k_transpose_dgrad<<<grid_for(nw), 256, 0, s>>>(w, wt_scratch, Cout, Cin);
-    const cudaError_t e = cudaGetLastError();
-    return e != cudaSuccess ? e : conv_dgrad(gz, B, H, W, Cout, wt_scratch, Cin, act, din, din2, split, s);
+cudaError_t dgrad_weights(const __nv_bfloat16 *w, __nv_bfloat16 *wt, const ConvLayers &d, cudaStream_t s) {
+    k_transpose_dgrad<<<dim3(48, d.n), 256, 0, s>>>(w, wt, d);
+    return cudaGetLastError();
 }
 
 cudaError_t colsum(const __nv_bfloat16 *g, long long P, int C, float *db, cudaStream_t s) {

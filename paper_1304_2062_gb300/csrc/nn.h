@@ -25,13 +25,17 @@ struct HeadArgs {
 };
 cudaError_t conv_forward_head(const __nv_bfloat16 *in, int B, int H, int W, int Cin, const __nv_bfloat16 *w,
                               const float *bias, __nv_bfloat16 *out, const HeadArgs &head, cudaStream_t s);
+// The weights of n layers rearranged for conv_dgrad, wt [Cin][9 Cout] at each
+// layer's offset.
+struct ConvLayers {
+    int n;
+    int cout[16], cin[16];
+    long long off[16];
+};
+cudaError_t dgrad_weights(const __nv_bfloat16 *w, __nv_bfloat16 *wt, const ConvLayers &d, cudaStream_t s);
 // Gradient w.r.t. the input from the pre-activation gradient gz [P][Cout];
 // channels < split go to din (multiplied by act > 0 when act != null),
-// channels >= split to din2. wt_scratch (Cout*9*Cin elements) receives the
-// rearranged weights [Cin][9 Cout], which conv_dgrad reads.
-cudaError_t conv_backward_data(const __nv_bfloat16 *gz, int B, int H, int W, int Cout, const __nv_bfloat16 *w, int Cin,
-                               const __nv_bfloat16 *act, __nv_bfloat16 *din, __nv_bfloat16 *din2, int split,
-                               __nv_bfloat16 *wt_scratch, cudaStream_t s);
+// channels >= split to din2.
 cudaError_t conv_dgrad(const __nv_bfloat16 *gz, int B, int H, int W, int Cout, const __nv_bfloat16 *wt, int Cin,
                        const __nv_bfloat16 *act, __nv_bfloat16 *din, __nv_bfloat16 *din2, int split, cudaStream_t s);
 // Weight gradient: dw [Cout][9 C] += sum over pixels of x[p shifted by tap][ci]

@@ -45,10 +45,12 @@ struct RowCfg {
     static constexpr int SMEM = (XF + W + FftTw<WH>::SIZE) * 8;
 };
 
+// Two blocks an SM for W = 512 (70 KB of shared memory each): at most 128 registers. (With
+// 146 for N = 30, one block, a row pass took 43 us instead of 28.)
 // NE < N: an NE-angle system at the slots of slot_of_angle (prop_classes.cuh);
 // the empty slots take no part in the maxima, means and argmaxima and stay zero
 template <int N, int W, int NE = N>
-__global__ void __launch_bounds__(row_threads<W>()) k_row(const __grid_constant__ RowArgs a) {
+__global__ void __launch_bounds__(row_threads<W>(), W == 512 ? 2 : 1) k_row(const __grid_constant__ RowArgs a) {
     constexpr int WH = W / 2, T = row_threads<W>();
     extern __shared__ __align__(16) float2 rsm[];
     float2 *Z = rsm;                       // [N][W/2]: z_m of every angle

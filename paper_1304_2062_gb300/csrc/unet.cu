@@ -58,7 +58,7 @@ struct se2n_unet {
     __nv_bfloat16 *cat[3];  // decoder inputs [up(below), skip]; e[0..2] live inside them
     int e_ld[4];            // channels per pixel of the tensor e[l] lives in
     float *out = nullptr, *target = nullptr, *loss = nullptr, *resid = nullptr;
-    __nv_bfloat16 *wt = nullptr;  // one layer's weights rearranged for the data gradient
+    __nv_bfloat16 *wt = nullptr;  // the weights rearranged for the data gradients, at the offsets of pb
 };
 
 namespace {
@@ -142,9 +142,18 @@ se2n_status backward(se2n_unet *u, const float *f, const uint8_t *mask, int n) {
     using namespace se2n::nn;
     cudaStream_t s = u->stream;
     const int H = u->H, W = u->W;
-    auto Wt = [&](int l) { return u->pb + u->w_off[l]; };
+    auto Wd = [&](int l) { return u->wt + u->w_off[l]; };
     auto dW = [&](int l) { return u->g + u->w_off[l]; };
     auto dB = [&](int l) { return u->g + u->b_off[l]; };
+    // the weights as the data gradients read them (the first layer has none)
+    ConvLayers layers;
+    layers.n = 13;
+    for (int l = 1; l < 14; ++l) {
+        layers.cout[l - 1] = kLayers[l].cout;
+        layers.cin[l - 1] = kLayers[l].cin;
+        layers.off[l - 1] = (long long)u->w_off[l];
+    }
+    TRYC(dgrad_weights(u->pb, u->wt, layers, s));
     // the first layer's input as the weight gradient reads it (8 channels: f m, m, zeros)
     TRYC(pack_input(f, mask, u->x0, (long long)n * H * W, s));
     TRYC(cudaMemsetAsync(u->g, 0, sizeof(float) * u->n_params, s));
@@ -161,12 +170,11 @@ se2n_status backward(se2n_unet *u, const float *f, const uint8_t *mask, int n) {
         // second conv: c[k] -> d[k]
         TRYC(conv_wgrad(u->c[k], n, Hl, Wl, Bb.cin, u->gd[k], Bb.cout, dW(lb), s));
         TRYC(colsum(u->gd[k], P, Bb.cout, dB(lb), s));
-        TRYC(conv_backward_data(u->gd[k], n, Hl, Wl, Bb.cout, Wt(lb), Bb.cin, u->c[k], u->gc[k], nullptr, Bb.cin, u->wt, s));
+        TRYC(conv_dgrad(u->gd[k], n, Hl, Wl, Bb.cout, Wd(lb), Bb.cin, u->c[k], u->gc[k], nullptr, Bb.cin, s));
         // first conv: [up(below), e[level]] -> c[k]
         TRYC(conv_wgrad(u->cat[k], n, Hl, Wl, A.cin, u->gc[k], A.cout, dW(la), s));
         TRYC(colsum(u->gc[k], P, A.cout, dB(la), s));
-        TRYC(conv_backward_data(u->gc[k], n, Hl, Wl, A.cout, Wt(la), A.cin, nullptr, u->gup[k], u->gskip[k],
-                                A.lo_ch, u->wt, s));
+        TRYC(conv_dgrad(u->gc[k], n, Hl, Wl, A.cout, Wd(la), A.cin, nullptr, u->gup[k], u->gskip[k], A.lo_ch, s));
         // gradient into the tensor below (half resolution), through the upsampling
         if (k > 0) {
             TRYC(up_backward_mask(u->gup[k], u->d[k - 1], u->gd[k - 1], n, Hl / 2, Wl / 2, A.lo_ch, s));
@@ -187,12 +195,11 @@ se2n_status backward(se2n_unet *u, const float *f, const uint8_t *mask, int n) {
         const __nv_bfloat16 *in = (l == 0) ? u->x0 : u->pl[l];
         TRYC(conv_wgrad(u->a[l], n, Hl, Wl, Bb.cin, u->ge[l], Bb.cout, dW(2 * l + 1), s));
         TRYC(colsum(u->ge[l], P, Bb.cout, dB(2 * l + 1), s));
-        TRYC(conv_backward_data(u->ge[l], n, Hl, Wl, Bb.cout, Wt(2 * l + 1), Bb.cin, u->a[l], u->ga[l], nullptr,
-                                Bb.cin, u->wt, s));
+        TRYC(conv_dgrad(u->ge[l], n, Hl, Wl, Bb.cout, Wd(2 * l + 1), Bb.cin, u->a[l], u->ga[l], nullptr, Bb.cin, s));
         TRYC(conv_wgrad(in, n, Hl, Wl, A.cin, u->ga[l], A.cout, dW(2 * l), s));
         TRYC(colsum(u->ga[l], P, A.cout, dB(2 * l), s));
         if (l > 0) {
-            TRYC(conv_backward_data(u->ga[l], n, Hl, Wl, A.cout, Wt(2 * l), A.cin, nullptr, u->gp[l], nullptr, A.cin, u->wt, s));
+            TRYC(conv_dgrad(u->ga[l], n, Hl, Wl, A.cout, Wd(2 * l), A.cin, nullptr, u->gp[l], nullptr, A.cin, s));
         }
     }
     return SE2N_OK;
@@ -283,12 +290,7 @@ se2n_status se2n_unet_create(se2n_unet **out, int batch, int H, int W, void *str
     if (e == cudaSuccess) e = cudaMalloc(&u->target, sizeof(float) * P0);
     if (e == cudaSuccess) e = cudaMalloc(&u->loss, 256);
     if (e == cudaSuccess) e = cudaMalloc(&u->resid, sizeof(float) * batch);
-    size_t wmax = 0;
-    for (int l = 0; l < 14; ++l) {
-        const size_t nw = (size_t)kLayers[l].cout * 9 * kLayers[l].cin;
-        if (nw > wmax) wmax = nw;
-    }
-    if (e == cudaSuccess) e = cudaMalloc(&u->wt, sizeof(__nv_bfloat16) * wmax);
+    if (e == cudaSuccess) e = cudaMalloc(&u->wt, sizeof(__nv_bfloat16) * np);
     if (e == cudaSuccess) e = cudaMemsetAsync(u->p, 0, sizeof(float) * np, u->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(u->m, 0, sizeof(float) * np, u->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(u->v, 0, sizeof(float) * np, u->stream);
