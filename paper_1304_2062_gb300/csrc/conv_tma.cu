@@ -500,15 +500,24 @@ cudaError_t launch_wgrad(const __nv_bfloat16 *x, int B, int H, int W, int C, con
     const int cv = F * C, nv = F * Cout;
     g.cgroups = cv / 64;
     g.ngroups = nv / 64;
-    // the lengths of the sums (conv_tma.cuh), and CTAs that fill the device once
-    const int groups = g.cgroups * g.ngroups;
+    // the lengths of the sums (conv_tma.cuh), and CTAs that fill the device once: as few
+    // tiles each (5, 3 or 2) as leave the ranges within a fifth of their number
     const int mtiles = (9 * C + 127) / 128;
     int ranges = F == 8 ? nsm : (2 * nsm + mtiles - 1) / mtiles;
     if (F == 2) ranges = (ranges + 1) / 2;
-    g.parts = F == 8 ? 1 : (2 * nsm + groups * ranges) / (2 * groups * ranges);  // nsm / (groups ranges), rounded
-    if (g.parts > 3) g.parts = 3;
-    if (g.parts < 1) g.parts = 1;
-    g.ksplit = nsm / (groups * g.parts);
+    for (int parts = F == 8 ? 1 : 3; parts >= 1; --parts) {
+        g.parts = parts;
+        g.tiles = (5 + parts - 1) / parts;
+        int ctas = 0;  // a range
+        for (int gr = 0; gr < g.cgroups * g.ngroups; ++gr) {
+            int s0, s1;
+            tma::wgrad_offsets(g, gr % g.cgroups * 64, gr / g.cgroups * 64, s0, s1);
+            ctas += (tma::wgrad_tiles(s0, s1) + g.tiles - 1) / g.tiles;
+        }
+        g.ksplit = nsm / ctas;
+        if (5 * g.ksplit >= 4 * ranges) break;
+    }
+    const int groups = g.cgroups * g.ngroups;
     if (g.ksplit > ranges) g.ksplit = ranges;
     if (g.ksplit > g.kblocks) g.ksplit = g.kblocks;
     if (g.ksplit < 1) g.ksplit = 1;

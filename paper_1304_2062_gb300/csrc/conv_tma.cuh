@@ -1083,9 +1083,9 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
 // proportion to its length, and the number of ranges is part of the result (4e-5 of a
 // gradient of 32 images when the ranges are a third as long): it stays at the two units an SM
 // of tiles of 128 (tap, channel) rows that the kernel once had, half as many where a
-// pixel pair makes two sums of each. Where that leaves SMs idle up to three
-// CTAs share a unit's tiles.
-// Measured (batch 32, 256 x 256): all 14 layers 1525 us (4832 with a box a tap and
+// pixel pair makes two sums of each, or up to a fifth fewer where that lets more CTAs
+// share a unit's tiles (up to three do; 5e-6).
+// Measured (batch 32, 256 x 256): all 14 layers 1462 us (4832 with a box a tap and
 // operand; 888 with as many ranges as SMs).
 // ---------------------------------------------------------------------------
 
@@ -1104,8 +1104,21 @@ struct WgradGeo {
     int xblocks, yblocks, kblocks;
     int cgroups, ngroups;  // 64-channel groups of In and gz as read
     int ksplit;         // pixel ranges a (channel group, channel group)
-    int parts;          // CTAs that share a unit's tiles
+    int tiles;          // of a unit a CTA takes at most
+    int parts;          // CTAs that share a unit's tiles, at most (the others return)
 };
+
+// Column offsets s0 .. s1 of a unit: -1 needs In's last pixel and gz's first one, 1 the
+// reverse (c0 / C is 0 and every group holds all there is when F = 1).
+__host__ __device__ __forceinline__ void wgrad_offsets(const WgradGeo &g, int c0, int n0, int &s0, int &s1) {
+    s0 = g.F == 1 || ((c0 + 63) / g.C >= g.F - 1 && n0 / g.Cout == 0) ? -1 : 0;
+    s1 = g.F == 1 || (c0 / g.C == 0 && (n0 + 63) / g.Cout >= g.F - 1) ? 1 : 0;
+}
+// Its tiles: (dy -1 | 0) of each offset, dy 1 of two offsets each.
+__host__ __device__ __forceinline__ int wgrad_tiles(int s0, int s1) {
+    const int ns = s1 - s0 + 1;
+    return ns + (ns + 1) / 2;
+}
 
 // MN-major matrix descriptor, 128-byte swizzle: leading byte offset = stride
 // between 64-row groups, stride byte offset = stride between 8-pixel groups.
@@ -1151,10 +1164,8 @@ __global__ void __launch_bounds__(192, 1)
     const int c0 = (gr % g.cgroups) * 64, n0 = (gr / g.cgroups) * 64;
     const int per = (g.kblocks + g.ksplit - 1) / g.ksplit;
     const int kb0 = ks * per, kb1 = min(g.kblocks, kb0 + per);
-    // column offsets s0 .. s1: -1 needs In's last pixel and gz's first one, 1 the
-    // reverse (c0 / C is 0 and every group holds all there is when F = 1)
-    const int s0 = (c0 + 63) / g.C >= g.F - 1 && n0 / g.Cout == 0 || g.F == 1 ? -1 : 0;
-    const int s1 = c0 / g.C == 0 && (n0 + 63) / g.Cout >= g.F - 1 || g.F == 1 ? 1 : 0;
+    int s0, s1;
+    wgrad_offsets(g, c0, n0, s0, s1);
 
     if (threadIdx.x == 0) {
         *abort = *(volatile int *)err;
@@ -1172,8 +1183,9 @@ __global__ void __launch_bounds__(192, 1)
         asm volatile("prefetch.tensormap [%0];\n" ::"l"((uint64_t)&mapG) : "memory");
     }
     __syncthreads();
-    const int ns = s1 - s0 + 1, nt = ns + (ns + 1) / 2;  // tiles of the unit; this CTA's: part, part + parts, ..
-    if (*abort || kb0 >= kb1 || part >= nt) return;
+    // the unit's tiles; this CTA's: part, part + parts, ..
+    const int ns = s1 - s0 + 1, nt = wgrad_tiles(s0, s1), parts = (nt + g.tiles - 1) / g.tiles;
+    if (*abort || kb0 >= kb1 || part >= parts) return;
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(tmem_slot),
                      "r"((uint32_t)TMEM_COLS));
@@ -1266,7 +1278,7 @@ __global__ void __launch_bounds__(192, 1)
                     for (int kk = 0; kk < BKX / 16; ++kk) {
                         const uint64_t off = (j * ROW + kk * 2048u) / 16, goff = (j * GROW + kk * 2048u) / 16;
                         const uint32_t add = j + kk > 0 || kb > kb0 ? 1u : 0u;
-                        for (int t = part; t < nt; t += g.parts)
+                        for (int t = part; t < nt; t += parts)
                             mma_f16_elect(tmem_base + (uint32_t)(t * 64),
                                           (t < ns ? d0 + (uint64_t)(t * 8) : d1 + (uint64_t)((t - ns) * 16)) + off, dg + goff,
                                           IDESC, add);
@@ -1298,7 +1310,7 @@ __global__ void __launch_bounds__(192, 1)
             const int i = (q & 1) * 32 + lane;   // channel of In in the group
             const int e = c0 + i;
             const int px = g.F > 1 ? e / g.C : 0, ci = e - px * g.C;
-            for (int t = part; t < nt; t += g.parts) {
+            for (int t = part; t < nt; t += parts) {
                 // tiles (dy -1 | 0) of each s, then (s | s + 1) of dy 1
                 const int s = t < ns ? s0 + t : s0 + 2 * (t - ns) + (q >> 1);
                 const int dy = t < ns ? (q >> 1) - 1 : 1;
