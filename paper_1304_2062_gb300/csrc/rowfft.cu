@@ -38,6 +38,16 @@ namespace {
 template <int W>
 __host__ __device__ constexpr int row_threads() { return W >= 768 ? 512 : 256; }
 
+// blocks an SM the registers are shaped for. Left to itself the compiler takes 146
+// registers for N = 30, W = 512, one block, and a row pass 43 us instead of 28; with
+// one block asked for everywhere, 148 for W = 384 instead of 80 (24 uneven images 2712
+// us instead of 2566).
+template <int N, int W>
+__host__ __device__ constexpr int row_blocks() {
+    return W >= 768 ? (N <= 16 ? 2 : 1) : W == 512 ? (N <= 16 ? 3 : 2) : W == 384 ? (N <= 16 ? 4 : 3) : W == 256 ? (N <= 16 ? 4 : 3)
+           : W == 128 ? 6 : 8;
+}
+
 template <int N, int W>
 struct RowCfg {
     static constexpr int WH = W / 2;
@@ -45,12 +55,10 @@ struct RowCfg {
     static constexpr int SMEM = (XF + W + FftTw<WH>::SIZE) * 8;
 };
 
-// Two blocks an SM for W = 512 (70 KB of shared memory each): at most 128 registers. (With
-// 146 for N = 30, one block, a row pass took 43 us instead of 28.)
 // NE < N: an NE-angle system at the slots of slot_of_angle (prop_classes.cuh);
 // the empty slots take no part in the maxima, means and argmaxima and stay zero
 template <int N, int W, int NE = N>
-__global__ void __launch_bounds__(row_threads<W>(), W == 512 ? 2 : 1) k_row(const __grid_constant__ RowArgs a) {
+__global__ void __launch_bounds__(row_threads<W>(), row_blocks<N, W>()) k_row(const __grid_constant__ RowArgs a) {
     constexpr int WH = W / 2, T = row_threads<W>();
     extern __shared__ __align__(16) float2 rsm[];
     float2 *Z = rsm;                       // [N][W/2]: z_m of every angle
