@@ -41,7 +41,7 @@ __host__ __device__ constexpr int row_threads() { return W >= 768 ? 512 : 256; }
 // blocks an SM the registers are shaped for. Left to itself the compiler takes 146
 // registers for N = 30, W = 512, one block, and a row pass 43 us instead of 28; with
 // one block asked for everywhere, 148 for W = 384 instead of 80 (24 uneven images 2712
-// us instead of 2566).
+// us instead of 2588).
 template <int N, int W>
 __host__ __device__ constexpr int row_blocks() {
     return W >= 768 ? (N <= 16 ? 2 : 1) : W == 512 ? (N <= 16 ? 3 : 2) : W == 384 ? (N <= 16 ? 4 : 3) : W == 256 ? (N <= 16 ? 4 : 3)
