@@ -84,7 +84,10 @@ typedef enum se2n_status {
  * with N = 16 or where applying kept matrices is faster (T (2 + 4 beta) / 2 above
  * about 3), and on the Hermitian half of other sizes where it is faster (above some 30
  * to 60) from the second call for the same beta, T and steps on (not in a stream
- * capture, and not without room for them), as a matrix:
+ * capture, and not without room for them), and in every interval of an inpaint
+ * with a restoration (rounds > 1 or final_mix; its threshold turns rounding into
+ * different values of a few pixels, so that those intervals keep one
+ * arithmetic), as a matrix:
  * for every class of frequencies that share it (rows s, H/2 - s as they are
  * and rows H/2 + s, H - s with the angles reversed, times columns l and
  * (W/2 - l) mod W) (B-^{-1} B+)^S - I is built once in FP32 by the powering
@@ -101,8 +104,8 @@ typedef enum se2n_status {
  * N = 32). The other flags do not apply.
  * In se2n_inpaint on the Hermitian half with N = 16, 30 or 32 and H, W each one
  * of 64, 128, 256, 384, 512, 768, 1024, this flag alone selects the row and column passes (as
- * does flags = 0 where the polynomial takes the place of the steps and has at
- * most 32 coefficients): the
+ * does flags = 0 for one interval without a restoration, where the polynomial
+ * takes the place of the steps and has at most 32 coefficients): the
  * volume stays row-transformed between intervals in the caller's volume
  * buffer, each interval is one kernel a column (DFT along y,
  * the interval's map, inverse DFT) and one kernel a row (real DFTs along x around
@@ -268,7 +271,8 @@ SE2N_API se2n_status se2n_inverse(se2n_plan *plan, void *vol);
  * With flags = 0 and dt (2 + 4 beta) <= 2, an interval whose polynomial (see
  * SE2N_DIFFUSE_PROPAGATOR) takes fewer operations than its steps is applied as
  * that polynomial, the same map of S steps to FP32 rounding; any flag keeps
- * the steps.
+ * the steps, and so does se2n_inpaint with a restoration (rounds > 1 or
+ * final_mix), whose decisions depend on that rounding.
  * When beta*dt <= ~0.067 (no FP64 flag), a packed fast path runs: the corner
  * correction vector decays by a factor <= 1e-9 within 6 angles of the tear,
  * so it is applied on those angles only (below FP32 resolution elsewhere);

@@ -291,16 +291,26 @@ bool kept_matrices(se2n_plan *plan, const PolyTable &t, double beta, double bdt,
     return cudaStreamIsCapturing(plan->stream, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone;
 }
 
+// Whether the restoration of Section 5 follows an interval of these inpaints. It
+// takes one of two formulas a pixel by comparing h(t) with a threshold (restore.cuh),
+// so a value within rounding of the threshold goes either way with the arithmetic of
+// the interval, and the intervals after it spread the difference (5e-4 of an image in
+// about one run in a hundred). Such intervals are integrated by the steps or the matrices
+// alone, whose rounding the decisions have always been made on; the polynomial serves
+// inpaints of one interval, which nothing but the projection follows.
+bool restores(const se2n_params *p) { return p->rounds > 1 || p->final_mix; }
+
 // The polynomial the column pass takes for one interval with these flags (0 or
 // SE2N_DIFFUSE_PROPAGATOR); null where it takes matrices, or with flags = 0
-// where there is no column pass. Asked for propagators, N = 30 and 32 take the
+// where there is no column pass. restored: as restores(). Asked for propagators, N = 30 and 32 take the
 // polynomial while it is no slower than applying matrices the plan has kept
 // from an earlier call (512 x 512, T = 2, 42 instructions an angle: 43.2 us a
 // column pass against 45.3; about 1 us more every 3 instructions), and N = 16
 // matrices, which are small (768 x 1024: 65 us against 68, 512 x 512: 21 against 23). A batch builds its
 // matrices again in every run and takes the polynomial wherever it applies (a
 // build is 60 .. 300 us).
-const PolyTable *col_poly(se2n_plan *plan, double beta, double T, int steps, int flags) {
+const PolyTable *col_poly(se2n_plan *plan, double beta, double T, int steps, int flags, bool restored) {
+    if (restored) return nullptr;
     if (flags != 0 && !plan->rebuilds && plan->N < 30) return nullptr;
     const PolyTable *t = poly_get(plan, beta, T, steps);
     if (!t || !se2n_col_has_poly(*t)) return nullptr;
@@ -310,14 +320,14 @@ const PolyTable *col_poly(se2n_plan *plan, double beta, double T, int steps, int
 
 // Row and column passes of the Hermitian half (rowfft.cu, colprop.cu): the
 // row-transformed volume [Wc][H][N] complex and the twiddle tables. Taken with
-// propagators, and with no flag where the interval's polynomial takes the
-// place of the steps.
+// propagators, and with no flag for one interval without a restoration, where
+// the interval's polynomial takes the place of the steps.
 bool col_path(se2n_plan *plan, const se2n_params *p) {
     if (p->full_spectrum || (p->diffuse_flags & ~SE2N_DIFFUSE_PROPAGATOR) || !(p->T > 0.0)) return false;
     const double Tr = p->T / p->rounds;
     if (!prop_admissible(p->beta, Tr / p->steps)) return false;
     if (!se2n_col_supported(plan->N, plan->H) || !se2n_row_supported(plan->N, plan->W)) return false;
-    return p->diffuse_flags != 0 || col_poly(plan, p->beta, Tr, p->steps, 0) != nullptr;
+    return p->diffuse_flags != 0 || col_poly(plan, p->beta, Tr, p->steps, 0, restores(p)) != nullptr;
 }
 
 // exp(-2 pi i m / n), m < n, from the exact fraction m / n
@@ -355,7 +365,8 @@ se2n_status col_ensure(se2n_plan *plan) {
 se2n_status col_start(se2n_plan *plan, const se2n_params *p) {
     SE2N_TRY(col_ensure(plan));
     const double Tr = p->T / p->rounds, bdt = p->beta * Tr / p->steps;
-    if (p->T > 0.0 && bdt >= 1e-30 && bdt <= 1e3 && !col_poly(plan, p->beta, Tr, p->steps, p->diffuse_flags))
+    if (p->T > 0.0 && bdt >= 1e-30 && bdt <= 1e3 &&
+        !col_poly(plan, p->beta, Tr, p->steps, p->diffuse_flags, restores(p)))
         SE2N_TRY(prop_ensure(plan, p->beta, bdt, p->steps, true, PROP_CHUNKS, true));
     return SE2N_OK;
 }
@@ -395,13 +406,13 @@ se2n_status row_pass(se2n_plan *plan, const RowArgs &r) {
     return cuda_status(plan, se2n_launch_row(plan->N, plan->W, r, plan->stream));
 }
 
-se2n_status col_diffuse(se2n_plan *plan, float2 *spec, double beta, double T, int steps, int flags) {
+se2n_status col_diffuse(se2n_plan *plan, float2 *spec, double beta, double T, int steps, int flags, bool restored) {
     if (!(beta > 0.0) || !(T >= 0.0) || steps < 1 || !isfinite(beta) || !isfinite(T)) return SE2N_EINVAL;
     if (T == 0.0) return SE2N_OK;
     const double bdt = beta * (T / steps);
     if (!(bdt >= 1e-30 && bdt <= 1e3)) return SE2N_ENUMERIC;
     ColArgs a;
-    if (const PolyTable *t = col_poly(plan, beta, T, steps, flags)) {
+    if (const PolyTable *t = col_poly(plan, beta, T, steps, flags, restored)) {
         if (flags & SE2N_DIFFUSE_PROPAGATOR) poly_count_build(plan);
         a.use_poly = 1;
         a.t = *t;
@@ -442,10 +453,10 @@ se2n_status poly_impl(se2n_plan *plan, float2 *vol, const PolyTable &t, bool hal
 }
 
 // half: vol holds the Hermitian half [N][H][W/2 + 1] of the spectrum.
-// rows >= 0: vol holds only spectrum rows k0 .. k0 + rows - 1 of every plane
-// ([N][rows][W], a row shard of the full spectrum).
+// restored: no polynomial (restores()). rows >= 0: vol holds only spectrum rows
+// k0 .. k0 + rows - 1 of every plane ([N][rows][W], a row shard of the full spectrum).
 se2n_status diffuse_impl(se2n_plan *plan, float2 *vol, double beta, double T, int steps, int flags, bool half = false,
-                         int k0 = 0, int rows = -1) {
+                         bool restored = false, int k0 = 0, int rows = -1) {
     if (!(beta > 0.0) || !(T >= 0.0) || steps < 1 || !isfinite(beta) || !isfinite(T)) return SE2N_EINVAL;
     if (flags & ~(SE2N_DIFFUSE_SM_FP64 | SE2N_DIFFUSE_SPLIT_DIAG | SE2N_DIFFUSE_FULL_CORRECTION |
                   SE2N_DIFFUSE_PROPAGATOR))
@@ -457,7 +468,7 @@ se2n_status diffuse_impl(se2n_plan *plan, float2 *vol, double beta, double T, in
     if (flags & SE2N_DIFFUSE_PROPAGATOR) {
         if (!se2n_prop_supported(plan->N) || rows >= 0) return SE2N_EUNSUPPORTED;
         if (prop_admissible(beta, dt)) {
-            const PolyTable *t = poly_get(plan, beta, T, steps);
+            const PolyTable *t = restored ? nullptr : poly_get(plan, beta, T, steps);
             if (!t) return propagate_impl(plan, vol, beta, bdt, steps, half);
             if (kept_matrices(plan, *t, beta, bdt, steps, half)) {
                 const se2n_status st = propagate_impl(plan, vol, beta, bdt, steps, half);
@@ -468,7 +479,7 @@ se2n_status diffuse_impl(se2n_plan *plan, float2 *vol, double beta, double T, in
         }
         flags &= ~SE2N_DIFFUSE_PROPAGATOR;  // stiff: the step kernel keeps the accuracy
     }
-    if (flags == 0) {
+    if (flags == 0 && !restored) {
         const PolyTable *t = poly_get(plan, beta, T, steps);
         if (t && poly_beats_steps(*t, steps)) return poly_impl(plan, vol, *t, half, k0, rows);
     }
@@ -705,6 +716,7 @@ se2n_status inpaint_impl(se2n_plan *plan, const float *f, const uint8_t *mask, c
         bins = plan->bins;
     }
     const double Tr = p->T / p->rounds;
+    const bool restored = restores(p);
     const float inv_hw = (float)(1.0 / (double)HW);
     const float eps = (float)p->eps, guard = (float)p->guard;
     DrState *dr = nullptr;
@@ -730,7 +742,7 @@ se2n_status inpaint_impl(se2n_plan *plan, const float *f, const uint8_t *mask, c
             RowArgs r = row_args(plan, vol, f, mask, bins, inv_hw, eps, guard);
             r.in_mode = SE2N_ROW_IN_LIFT;
             SE2N_TRY(row_pass(plan, r));
-            SE2N_TRY(col_diffuse(plan, vol, p->beta, Tr, p->steps, p->diffuse_flags));
+            SE2N_TRY(col_diffuse(plan, vol, p->beta, Tr, p->steps, p->diffuse_flags, restored));
             for (int i = 1; i <= p->rounds; ++i) {
                 const bool last = i == p->rounds;
                 const float *rf = f;
@@ -763,18 +775,18 @@ se2n_status inpaint_impl(se2n_plan *plan, const float *f, const uint8_t *mask, c
                 }
                 r.mix = 1;
                 SE2N_TRY(row_pass(plan, r));
-                SE2N_TRY(col_diffuse(plan, vol, p->beta, Tr, p->steps, p->diffuse_flags));
+                SE2N_TRY(col_diffuse(plan, vol, p->beta, Tr, p->steps, p->diffuse_flags, restored));
             }
         } else {
             SE2N_TRY(ensure_half(plan));
             SE2N_TRY(lift_half_impl(plan, f, mask, bins, vol));
             SE2N_TRY(fft_half(plan, vol, true));
-            SE2N_TRY(diffuse_impl(plan, vol, p->beta, Tr, p->steps, p->diffuse_flags, true));
+            SE2N_TRY(diffuse_impl(plan, vol, p->beta, Tr, p->steps, p->diffuse_flags, true, restored));
             for (int i = 1; i < p->rounds; ++i) {
                 SE2N_TRY(fft_half(plan, vol, false));
                 SE2N_TRY(restore_impl(plan, dr, vol, f, mask, bins, inv_hw, eps, guard, true));
                 SE2N_TRY(fft_half(plan, vol, true));
-                SE2N_TRY(diffuse_impl(plan, vol, p->beta, Tr, p->steps, p->diffuse_flags, true));
+                SE2N_TRY(diffuse_impl(plan, vol, p->beta, Tr, p->steps, p->diffuse_flags, true, restored));
             }
             SE2N_TRY(fft_half(plan, vol, false));
         }
@@ -788,13 +800,13 @@ se2n_status inpaint_impl(se2n_plan *plan, const float *f, const uint8_t *mask, c
     }
     SE2N_TRY(lift_impl(plan, f, mask, bins, vol));
     SE2N_TRY(fft(plan, plan->fft_vol, vol, CUFFT_FORWARD));
-    SE2N_TRY(diffuse_impl(plan, vol, p->beta, Tr, p->steps, p->diffuse_flags));
+    SE2N_TRY(diffuse_impl(plan, vol, p->beta, Tr, p->steps, p->diffuse_flags, false, restored));
     for (int i = 1; i < p->rounds; ++i) {
         // inverse DFT; its 1/(H W) is folded into the restoration kernel
         SE2N_TRY(fft(plan, plan->fft_vol, vol, CUFFT_INVERSE));
         SE2N_TRY(restore_impl(plan, dr, vol, f, mask, bins, inv_hw, eps, guard, false));
         SE2N_TRY(fft(plan, plan->fft_vol, vol, CUFFT_FORWARD));
-        SE2N_TRY(diffuse_impl(plan, vol, p->beta, Tr, p->steps, p->diffuse_flags));
+        SE2N_TRY(diffuse_impl(plan, vol, p->beta, Tr, p->steps, p->diffuse_flags, false, restored));
     }
     SE2N_TRY(fft(plan, plan->fft_vol, vol, CUFFT_INVERSE));
     float scale = inv_hw;
@@ -994,7 +1006,7 @@ se2n_status se2n_diffuse_rows(se2n_plan *plan, void *vol_rows, int k0, int rows,
                               int flags) {
     SE2N_TRY(check_plan(plan));
     if (!device_ptr(vol_rows, 16) || k0 < 0 || rows < 1 || k0 + rows > plan->H) return SE2N_EINVAL;
-    return diffuse_impl(plan, (float2 *)vol_rows, beta, T, steps, flags, false, k0, rows);
+    return diffuse_impl(plan, (float2 *)vol_rows, beta, T, steps, flags, false, false, k0, rows);
 }
 
 se2n_status se2n_dr_grow(se2n_plan *plan, const void *vol, const uint8_t *mask_in, uint8_t *mask_out, float *fref,
@@ -1274,12 +1286,13 @@ se2n_status batch_interval(se2n_batch *b, double Tr, bool half) {
     if (b->prop_images > 0)
         for (int i = 0; i < b->count; ++i)
             if (b->img_prop[i] && !b->img_fused[i])
-                SE2N_TRY(diffuse_impl(b->plan_of[i], b->vols[i], p.beta, Tr, p.steps, p.diffuse_flags, half));
+                SE2N_TRY(diffuse_impl(b->plan_of[i], b->vols[i], p.beta, Tr, p.steps, p.diffuse_flags, half,
+                                      restores(&p)));
     return SE2N_OK;
 }
 
-// With SE2N_DIFFUSE_PROPAGATOR, where the interval polynomial does not apply,
-// the images of one shape are integrated by
+// With SE2N_DIFFUSE_PROPAGATOR, where the interval polynomial does not apply
+// (or a restoration follows, restores()), the images of one shape are integrated by
 // that shape's propagators when building them once and applying them to every
 // image and interval is estimated to cost less than the step-by-step kernel on
 // those images. The estimate uses this library's measured rates on a GB300:
@@ -1649,7 +1662,7 @@ se2n_status create_batch(se2n_batch *b, const se2n_image_desc *imgs) {
     const double bdt = b->p.beta * Tr / b->p.steps;
     b->split = (b->p.diffuse_flags & SE2N_DIFFUSE_SPLIT_DIAG) || b->p.beta * Tr > 8.0;
     b->fast = !(b->p.diffuse_flags & SE2N_DIFFUSE_FULL_CORRECTION) && se2n_diffuse_truncation_ok(bdt);
-    b->poly_on = (b->p.diffuse_flags & ~SE2N_DIFFUSE_PROPAGATOR) == 0 && b->p.T > 0.0 &&
+    b->poly_on = (b->p.diffuse_flags & ~SE2N_DIFFUSE_PROPAGATOR) == 0 && b->p.T > 0.0 && !restores(&b->p) &&
                  se2n_poly_make(b->p.beta, Tr, b->p.steps, b->poly) && poly_beats_steps(b->poly, b->p.steps);
     if (cudaMemsetAsync(b->arena, 0, b->vol_bytes, b->stream) != cudaSuccess) return SE2N_ECUDA;
     // transforms of the Hermitian-half path are planned before the capture
@@ -1667,7 +1680,7 @@ se2n_status create_batch(se2n_batch *b, const se2n_image_desc *imgs) {
             // everything the whole inpaints allocate or create, before the capture
             SE2N_TRY(col_ensure(pl));
             SE2N_TRY(side_ensure(pl));
-            if (!col_poly(pl, b->p.beta, Tr, b->p.steps, b->p.diffuse_flags))
+            if (!col_poly(pl, b->p.beta, Tr, b->p.steps, b->p.diffuse_flags, restores(&b->p)))
                 SE2N_TRY(prop_reserve(pl, true, PROP_CHUNKS));
             if (b->p.dynamic) SE2N_TRY(dr_alloc(pl->dr, pl->HW));
         } else if (!b->poly_on) {

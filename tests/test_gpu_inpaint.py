@@ -366,3 +366,42 @@ def test_back_to_back_inpaints_repeat_their_bits(N, H, W, flags):
             assert torch.equal(got, want)
     for r in runs:
         r[0].close()
+
+
+@pytest.mark.parametrize("N,H,W,rounds,final_mix,dynamic,full", [
+    (32, 64, 64, 2, 0, 0, 0), (16, 128, 64, 1, 1, 0, 0), (30, 64, 64, 3, 0, 1, 0),   # sides of the passes
+    (24, 30, 26, 2, 0, 0, 0), (64, 22, 34, 1, 1, 0, 0), (8, 20, 20, 2, 1, 0, 1)])
+def test_restored_intervals_are_stepped(N, H, W, rounds, final_mix, dynamic, full):
+    """The restoration decides by a threshold, so the intervals it follows keep
+    the steps' rounding: where beta T > 8 (an interval) the steps take the split diagonal
+    with or without SE2N_DIFFUSE_SPLIT_DIAG, so both give the same bits."""
+    w = synth.workload_512(H=H, W=W, steps=300, rounds=rounds)
+    p = oracle.Params(N=N, beta=1.0, T=9.0 * rounds, steps=300, rounds=rounds, final_mix=final_mix)
+    got = []
+    for flags in (0, se2n.SE2N_DIFFUSE_SPLIT_DIAG):
+        prm = _params(p, flags, full)
+        prm.dynamic = dynamic
+        got.append(_gpu_inpaint(w.f.astype(np.float32), w.mask, None, prm))
+    np.testing.assert_array_equal(got[0], got[1])
+
+
+@pytest.mark.parametrize("rounds,final_mix,builds", [(2, 0, 1), (1, 1, 1), (1, 0, 0)])
+@pytest.mark.parametrize("N,H,W,kernels", [(32, 64, 64, 1), (30, 64, 128, 1), (32, 36, 20, 2), (64, 20, 36, 2)])
+def test_restored_intervals_with_propagators_take_matrices(N, H, W, kernels, rounds, final_mix, builds):
+    """The same with propagators: one launch builds the matrices, none is made
+    for a single interval without a restoration. Launches: the row or column
+    pass before, between and after (lift, mix and projection at other sides)."""
+    w = synth.workload_512(H=H, W=W, steps=60, rounds=rounds)
+    p = oracle.Params(N=N, beta=0.25, T=2.0 * rounds, steps=60, rounds=rounds, final_mix=final_mix)
+    f32 = w.f.astype(np.float32)
+    bins = oracle.orient(f32.astype(np.float64), w.mask, N)["bins"]
+    plan = se2n.se2n_plan_create(H, W, N)
+    se2n.se2n_plan_profile(plan, True)
+    vol = torch.empty((N, H, W), dtype=torch.complex64, device="cuda")
+    out = torch.empty((H, W), dtype=torch.float32, device="cuda")
+    se2n.se2n_inpaint(plan, t_f32(f32), t_u8(w.mask), t_u8(bins), _params(p, se2n.SE2N_DIFFUSE_PROPAGATOR), vol, out)
+    host(out)
+    prof = se2n.se2n_plan_profile_read(plan)
+    plan.close()
+    between = 2 * rounds + 1 if kernels == 1 else 2 * rounds + 1 + final_mix
+    assert prof["kernels"] == between + builds
