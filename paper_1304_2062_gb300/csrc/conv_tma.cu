@@ -480,47 +480,13 @@ cudaError_t launch_wide(const __nv_bfloat16 *A, int B, int H, int W, int C, cons
 // [Cout][9 C] FP32 (accumulated).
 cudaError_t launch_wgrad(const __nv_bfloat16 *x, int B, int H, int W, int C, const __nv_bfloat16 *gz, int Cout,
                          float *dw, cudaStream_t s) {
-    const int F = C % 64 == 0 && Cout % 64 == 0 ? 1 : C % 32 == 0 ? 2 : 8;
-    if ((F * C) % 64 || Cout % 32 || W % F) return cudaErrorNotSupported;
-    auto enc = encoder();
     const int nsm = sm_count();
-    int *err = fault_ptr();
-    if (!enc || nsm <= 0 || !err) return cudaErrorNotSupported;
     tma::WgradGeo g;
-    g.B = B;
-    g.H = H;
-    g.W = W / F;
-    g.C = C;
-    g.Cout = Cout;
-    g.F = F;
-    const int bkx = g.W > 16 ? 32 : 16;  // columns of a pixel block
-    g.xblocks = (g.W + bkx - 1) / bkx;
-    g.yblocks = (H + tma::kWgR - 1) / tma::kWgR;
-    g.kblocks = B * g.xblocks * g.yblocks;
-    const int cv = F * C, nv = F * Cout;
-    g.cgroups = cv / 64;
-    g.ngroups = nv / 64;
-    // the lengths of the sums (conv_tma.cuh), and CTAs that fill the device once: as few
-    // tiles each (5, 3 or 2) as leave the ranges within a fifth of their number
-    const int mtiles = (9 * C + 127) / 128;
-    int ranges = F == 8 ? nsm : (2 * nsm + mtiles - 1) / mtiles;
-    if (F == 2) ranges = (ranges + 1) / 2;
-    for (int parts = F == 8 ? 1 : 3; parts >= 1; --parts) {
-        g.parts = parts;
-        g.tiles = (5 + parts - 1) / parts;
-        int ctas = 0;  // a range
-        for (int gr = 0; gr < g.cgroups * g.ngroups; ++gr) {
-            int s0, s1;
-            tma::wgrad_offsets(g, gr % g.cgroups * 64, gr / g.cgroups * 64, s0, s1);
-            ctas += (tma::wgrad_tiles(s0, s1) + g.tiles - 1) / g.tiles;
-        }
-        g.ksplit = nsm / ctas;
-        if (5 * g.ksplit >= 4 * ranges) break;
-    }
-    const int groups = g.cgroups * g.ngroups;
-    if (g.ksplit > ranges) g.ksplit = ranges;
-    if (g.ksplit > g.kblocks) g.ksplit = g.kblocks;
-    if (g.ksplit < 1) g.ksplit = 1;
+    if (nsm <= 0 || !tma::wgrad_split(g, B, H, W, C, Cout, nsm)) return cudaErrorNotSupported;
+    auto enc = encoder();
+    int *err = fault_ptr();
+    if (!enc || !err) return cudaErrorNotSupported;
+    const int bkx = g.bkx, cv = g.F * C, nv = g.F * Cout;
     auto map = [&](CUtensorMap *m, const __nv_bfloat16 *p, int ch, int cols, int rows) {
         const cuuint64_t dims[4] = {(cuuint64_t)ch, (cuuint64_t)g.W, (cuuint64_t)H, (cuuint64_t)B};
         const cuuint64_t strides[3] = {(cuuint64_t)ch * 2, (cuuint64_t)g.W * ch * 2, (cuuint64_t)H * g.W * ch * 2};
@@ -532,12 +498,13 @@ cudaError_t launch_wgrad(const __nv_bfloat16 *x, int B, int H, int W, int C, con
     };
     CUtensorMap mx, mg;
     if (!map(&mx, x, cv, bkx + 2, tma::kWgR + 2) || !map(&mg, gz, nv, bkx, tma::kWgR)) return cudaErrorInvalidValue;
-    const int smem = 1024 + tma::kWgXSlots * (bkx == 32 ? tma::kWgXSlot<32> : tma::kWgXSlot<16>) +
+    int smem = 1024 + tma::kWgXSlots * (bkx == 32 ? tma::kWgXSlot<32> : tma::kWgXSlot<16>) +
                      tma::kWgGSlots * tma::kWgR * bkx * 128 + 256;
+    if (smem < 120 * 1024) smem = 120 * 1024;  // one CTA an SM: each takes all of tensor memory
     auto *fn = bkx == 32 ? &tma::k_wgrad_tma<32> : &tma::k_wgrad_tma<16>;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    fn<<<groups * g.ksplit * g.parts, 192, smem, s>>>(mx, mg, g, dw, err);
+    fn<<<g.cgroups * g.ngroups * g.ksplit * g.parts, 192, smem, s>>>(mx, mg, g, dw, err);
     return cudaGetLastError();
 }
 

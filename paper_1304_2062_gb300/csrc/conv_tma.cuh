@@ -32,6 +32,7 @@
 #include <stdint.h>
 
 #include "conv_tc.cuh"
+#include "wgrad_plan.h"
 
 namespace se2n {
 namespace nn {
@@ -1079,46 +1080,21 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
 //    channels holds no such pixels). 1 / F of the box rows.
 // A unit of work is (64 channels of In, 64 of gz, a range of pixel blocks),
 // accumulated in tensor memory (up to 5 tiles of 64 columns) and added to dW with FP32
-// atomics at the end. The tensor core's sums truncate, so a sum loses bits in
-// proportion to its length, and the number of ranges is part of the result (4e-5 of a
-// gradient of 32 images when the ranges are a third as long): it stays at the two units an SM
-// of tiles of 128 (tap, channel) rows that the kernel once had, half as many where a
-// pixel pair makes two sums of each, or up to a fifth fewer where that lets more CTAs
-// share a unit's tiles (up to three do; 5e-6).
+// atomics. The tensor core's sums truncate, so a sum loses bits in proportion to its
+// length, and the length is part of the result (4e-5 of a gradient of 32 images when it
+// is a third): wgrad_plan.h ends every sum where it ended when a unit was a tile of
+// 128 (tap, channel) rows, or earlier, however long the range of a CTA is. Up to three
+// CTAs share a unit's tiles.
 // Measured (batch 32, 256 x 256): all 14 layers 1462 us (4832 with a box a tap and
 // operand; 888 with as many ranges as SMs).
 // ---------------------------------------------------------------------------
 
-constexpr int kWgR = 8;                    // image rows of a pixel block
 constexpr int kWgXSlots = 3, kWgGSlots = 2;  // ring slots of In and of gz
 // a box of In, and its slot: the last operand's second group may end one pixel behind it
 template <int BKX>
 constexpr int kWgXBytes = (kWgR + 2) * (BKX + 2) * 128;
 template <int BKX>
 constexpr int kWgXSlot = (kWgXBytes<BKX> + 128 + 1023) / 1024 * 1024;
-
-struct WgradGeo {
-    int B, H, W;        // of the tensors as read (W columns of F pixels)
-    int C, Cout;        // channels of the layer
-    int F;              // pixels a column
-    int xblocks, yblocks, kblocks;
-    int cgroups, ngroups;  // 64-channel groups of In and gz as read
-    int ksplit;         // pixel ranges a (channel group, channel group)
-    int tiles;          // of a unit a CTA takes at most
-    int parts;          // CTAs that share a unit's tiles, at most (the others return)
-};
-
-// Column offsets s0 .. s1 of a unit: -1 needs In's last pixel and gz's first one, 1 the
-// reverse (c0 / C is 0 and every group holds all there is when F = 1).
-__host__ __device__ __forceinline__ void wgrad_offsets(const WgradGeo &g, int c0, int n0, int &s0, int &s1) {
-    s0 = g.F == 1 || ((c0 + 63) / g.C >= g.F - 1 && n0 / g.Cout == 0) ? -1 : 0;
-    s1 = g.F == 1 || (c0 / g.C == 0 && (n0 + 63) / g.Cout >= g.F - 1) ? 1 : 0;
-}
-// Its tiles: (dy -1 | 0) of each offset, dy 1 of two offsets each.
-__host__ __device__ __forceinline__ int wgrad_tiles(int s0, int s1) {
-    const int ns = s1 - s0 + 1;
-    return ns + (ns + 1) / 2;
-}
 
 // MN-major matrix descriptor, 128-byte swizzle: leading byte offset = stride
 // between 64-row groups, stride byte offset = stride between 8-pixel groups.
@@ -1154,7 +1130,8 @@ __global__ void __launch_bounds__(192, 1)
     const uint32_t bar_gfull = bar_xempty + 8 * XS;
     const uint32_t bar_gempty = bar_gfull + 8 * GS;
     const uint32_t bar_done = bar_gempty + 8 * GS;
-    const uint32_t tmem_slot = bar_done + 8;
+    const uint32_t bar_drained = bar_done + 8;
+    const uint32_t tmem_slot = bar_drained + 8;
     volatile int *abort = (volatile int *)(smem_raw + (tmem_slot + 4 - raw));
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
@@ -1162,8 +1139,7 @@ __global__ void __launch_bounds__(192, 1)
     const int part = blockIdx.x % g.parts, unit = blockIdx.x / g.parts;
     const int ks = unit % g.ksplit, gr = unit / g.ksplit;
     const int c0 = (gr % g.cgroups) * 64, n0 = (gr / g.cgroups) * 64;
-    const int per = (g.kblocks + g.ksplit - 1) / g.ksplit;
-    const int kb0 = ks * per, kb1 = min(g.kblocks, kb0 + per);
+    const int kb0 = ks * g.per, kb1 = min(g.kblocks, kb0 + g.per);
     int s0, s1;
     wgrad_offsets(g, c0, n0, s0, s1);
 
@@ -1178,6 +1154,7 @@ __global__ void __launch_bounds__(192, 1)
             tc::mbar_init(bar_gempty + 8 * s, 1);
         }
         tc::mbar_init(bar_done, 1);
+        tc::mbar_init(bar_drained, 4);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         asm volatile("prefetch.tensormap [%0];\n" ::"l"((uint64_t)&mapX) : "memory");
         asm volatile("prefetch.tensormap [%0];\n" ::"l"((uint64_t)&mapG) : "memory");
@@ -1252,8 +1229,17 @@ __global__ void __launch_bounds__(192, 1)
             int xs = 0, gs = 0;
             uint32_t xph = 0, gph = 0;
             bool ok = true;
-            uint32_t last_bar = 0, last_par = 0;
+            uint32_t last_bar = 0, last_par = 0, dph = 0;
+            int in = 0;  // blocks of the sum so far
             for (int kb = kb0; kb < kb1 && ok; ++kb) {
+                if (in == g.len) {  // the accumulators have been read
+                    if (!mbar_wait_warp(bar_drained, dph, abort)) {
+                        ok = false;
+                        break;
+                    }
+                    dph ^= 1u;
+                    in = 0;
+                }
                 int b, y0, x0;
                 block(kb, b, y0, x0);
                 const int rows = min(R, g.H - y0);
@@ -1277,7 +1263,7 @@ __global__ void __launch_bounds__(192, 1)
 #pragma unroll
                     for (int kk = 0; kk < BKX / 16; ++kk) {
                         const uint64_t off = (j * ROW + kk * 2048u) / 16, goff = (j * GROW + kk * 2048u) / 16;
-                        const uint32_t add = j + kk > 0 || kb > kb0 ? 1u : 0u;
+                        const uint32_t add = j + kk > 0 || in > 0 ? 1u : 0u;
                         for (int t = part; t < nt; t += parts)
                             mma_f16_elect(tmem_base + (uint32_t)(t * 64),
                                           (t < ns ? d0 + (uint64_t)(t * 8) : d1 + (uint64_t)((t - ns) * 16)) + off, dg + goff,
@@ -1296,16 +1282,17 @@ __global__ void __launch_bounds__(192, 1)
                     gs = 0;
                     gph ^= 1u;
                 }
+                if (++in == g.len || kb + 1 == kb1) mma_commit_elect(bar_done);
             }
-            if (ok)
-                mma_commit_elect(bar_done);
-            else if (last_bar)
+            if (!ok && last_bar)
                 tc::mbar_wait(last_bar, last_par, nullptr);  // tensor core idle before release
         }
     } else {
-        // ---------------- epilogue (warps 2..5): atomic adds into dW ----------------
+        // ---------------- epilogue (warps 2..5): atomic adds into dW, sum after sum ----------------
         const int q = warp & 3;
-        if (tc::mbar_wait(bar_done, 0, abort)) {
+        uint32_t ph = 0;
+        for (int kb = kb0; kb < kb1; kb += g.len, ph ^= 1u) {
+            if (!mbar_wait_warp(bar_done, ph, abort)) break;
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
             const int i = (q & 1) * 32 + lane;   // channel of In in the group
             const int e = c0 + i;
@@ -1331,6 +1318,8 @@ __global__ void __launch_bounds__(192, 1)
                 }
             }
             asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+            __syncwarp();
+            if (lane == 0) arrive(bar_drained);
         }
     }
     __syncthreads();
