@@ -82,9 +82,7 @@ typedef enum se2n_status {
  * 50 for 75), whose coefficients the host makes when beta, T or steps change;
  * where more than 64 coefficients would be needed, and in the column pass (below)
  * with N = 16 or where applying kept matrices is faster (T (2 + 4 beta) / 2 above
- * about 3), and on the Hermitian half of other sizes where it is faster (above some 30
- * to 60) from the second call for the same beta, T and steps on (not in a stream
- * capture, and not without room for them), and in every interval of an inpaint
+ * about 3), and in every interval of an inpaint
  * with a restoration (rounds > 1 or final_mix; its threshold turns rounding into
  * different values of a few pixels, so that those intervals keep one
  * arithmetic), as a matrix:

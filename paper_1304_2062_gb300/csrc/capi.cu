@@ -271,24 +271,6 @@ void poly_count_build(se2n_plan *plan) {
     if (plan->poly_built) return;
     StageTimer timer(plan, SE2N_STAGE_PROPAGATOR);
     plan->poly_built = true;
-    plan->poly_call = plan->calls;
-}
-
-// Whether one interval asked for with SE2N_DIFFUSE_PROPAGATOR takes matrices from
-// device memory although the polynomial applies: only where that is faster (on the
-// Hermitian half, whose frequencies share matrices, and from a cost of the polynomial
-// on: N = 64, 2048 x 2048, 247 instructions an angle: 1.24 ms against 1.88; N = 32,
-// 1000 x 1000, T = 8 / 50: an inpaint 527 / 642 us with the polynomial, 619 with matrices),
-// and only from the second call for the same beta, T and steps on, since a build (16
-// ms there) costs as much as some ten intervals. A call in a stream capture builds none.
-bool kept_matrices(se2n_plan *plan, const PolyTable &t, double beta, double bdt, int steps, bool half) {
-    if (plan->rebuilds || !half || !t.reinsch || se2n_poly_cost(t) <= (plan->N > 32 ? 160 : 210)) return false;
-    if (plan->prop_valid && plan->prop_beta == beta && plan->prop_bdt == bdt && plan->prop_steps == steps &&
-        plan->prop_half == half && plan->prop_fmt == se2n_prop_apply_fmt(plan->N, half))
-        return true;
-    if (!plan->poly_built || plan->poly_call == plan->calls) return false;
-    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    return cudaStreamIsCapturing(plan->stream, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone;
 }
 
 // Whether the restoration of Section 5 follows an interval of these inpaints. It
@@ -468,12 +450,12 @@ se2n_status diffuse_impl(se2n_plan *plan, float2 *vol, double beta, double T, in
     if (flags & SE2N_DIFFUSE_PROPAGATOR) {
         if (!se2n_prop_supported(plan->N) || rows >= 0) return SE2N_EUNSUPPORTED;
         if (prop_admissible(beta, dt)) {
+            // The polynomial wherever there is one, in the first call and in later ones: a call's
+            // bits depend on its arguments alone. (Applying matrices kept from an earlier call
+            // is faster at large T on the Hermitian half, N = 64, 2048 x 2048, T = 50: an inpaint 3.56 ms
+            // against 4.18, but building them costs 16 ms; at T = 8, N = 32, 1000 x 1000, 619 us against 527.)
             const PolyTable *t = restored ? nullptr : poly_get(plan, beta, T, steps);
             if (!t) return propagate_impl(plan, vol, beta, bdt, steps, half);
-            if (kept_matrices(plan, *t, beta, bdt, steps, half)) {
-                const se2n_status st = propagate_impl(plan, vol, beta, bdt, steps, half);
-                if (st != SE2N_ENOMEM) return st;  // no room for them: the polynomial again
-            }
             poly_count_build(plan);
             return poly_impl(plan, vol, *t, half, k0, rows);
         }
@@ -708,7 +690,6 @@ se2n_status inpaint_impl(se2n_plan *plan, const float *f, const uint8_t *mask, c
     const long long HW = plan->HW;
     const int N = plan->N;
     const uint8_t *bins = bins_in;
-    plan->calls += 1;
     const bool col = allow_col && col_path(plan, p);
     if (col) SE2N_TRY(col_start(plan, p));
     if (!bins) {

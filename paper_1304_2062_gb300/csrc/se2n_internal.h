@@ -61,7 +61,6 @@ struct se2n_plan {
     // poly_built while it stands for the propagators asked for by
     // SE2N_DIFFUSE_PROPAGATOR
     bool poly_made, poly_ok, poly_built;
-    unsigned calls, poly_call;  // public calls so far; the one that set poly_built
     bool rebuilds;         // a batch's plan: matrices would be built again in every run
     double poly_beta, poly_T;
     int poly_steps;

@@ -405,3 +405,27 @@ def test_restored_intervals_with_propagators_take_matrices(N, H, W, kernels, rou
     plan.close()
     between = 2 * rounds + 1 if kernels == 1 else 2 * rounds + 1 + final_mix
     assert prof["kernels"] == between + builds
+
+
+@pytest.mark.parametrize("N,H,W,T", [(64, 20, 36, 25.0), (64, 136, 72, 45.0), (32, 36, 20, 55.0), (16, 30, 34, 2.0),
+                                     (32, 64, 64, 5.0), (16, 64, 64, 2.0)])
+def test_a_call_with_propagators_does_not_depend_on_earlier_ones(N, H, W, T):
+    """The first inpaint of a plan, the following ones, one after another interval
+    and one after dropping what the plan keeps: the same bits."""
+    w = synth.workload_512(H=H, W=W, steps=int(8 * T), rounds=1)
+    plan = se2n.se2n_plan_create(H, W, N)
+    fd, md = t_f32(w.f.astype(np.float32)), t_u8(w.mask)
+    vol = torch.empty((N, H, W), dtype=torch.complex64, device="cuda")
+    got = []
+    for t in (T, T, T, T / 2, T, None, T):
+        if t is None:
+            se2n.se2n_plan_drop_propagators(plan, 1)
+            continue
+        out = torch.empty((H, W), dtype=torch.float32, device="cuda")
+        p = oracle.Params(N=N, beta=0.25, T=t, steps=int(8 * T), rounds=1)
+        se2n.se2n_inpaint(plan, fd, md, None, _params(p, se2n.SE2N_DIFFUSE_PROPAGATOR), vol, out)
+        if t == T:
+            got.append(host(out))
+    plan.close()
+    for g in got[1:]:
+        np.testing.assert_array_equal(g, got[0])
