@@ -269,8 +269,9 @@ SE2N_API se2n_status se2n_inverse(se2n_plan *plan, void *vol);
  * With flags = 0 and dt (2 + 4 beta) <= 2, an interval whose polynomial (see
  * SE2N_DIFFUSE_PROPAGATOR) takes fewer operations than its steps is applied as
  * that polynomial, the same map of S steps to FP32 rounding; any flag keeps
- * the steps, and so does se2n_inpaint with a restoration (rounds > 1 or
- * final_mix), whose decisions depend on that rounding.
+ * the steps, and so do a tuned plan (se2n_plan_tune_diffuse) and se2n_inpaint
+ * with a restoration (rounds > 1 or final_mix), whose decisions depend on
+ * that rounding.
  * When beta*dt <= ~0.067 (no FP64 flag), a packed fast path runs: the corner
  * correction vector decays by a factor <= 1e-9 within 6 angles of the tear,
  * so it is applied on those angles only (below FP32 resolution elsewhere);
@@ -363,10 +364,12 @@ SE2N_API se2n_status se2n_plan_drop_propagators(se2n_plan *plan, int free_memory
  * threads a block and one frequency group a thread for the packed kernels
  * below N = 48, one resident 384-thread block an SM for them from N = 48 on,
  * and 256-thread resident blocks for the others. SE2N_EUNSUPPORTED if no
- * kernel exists for (N, P). */
+ * kernel exists for (N, P). A plan tuned so integrates by its step kernel
+ * wherever no flag is given, never by the polynomial; P = 0 with
+ * block_threads = 0 makes it an ordinary plan again. */
 SE2N_API se2n_status se2n_plan_tune_diffuse(se2n_plan *plan, int threads_per_freq, int block_threads, int blocks);
 
-/* Resource use of the current diffusion kernel choice: registers per thread,
+/* Resource use of the step kernel that the plan would launch: registers per thread,
  * resident blocks per SM and threads per frequency. Any output may be NULL. */
 SE2N_API se2n_status se2n_plan_diffuse_info(se2n_plan *plan, int *regs_per_thread, int *blocks_per_sm,
                                    int *threads_per_freq);

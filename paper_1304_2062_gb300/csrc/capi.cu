@@ -265,6 +265,13 @@ const PolyTable *poly_get(se2n_plan *plan, double beta, double T, int steps) {
 // 1024 x 1024, T = 2: 136 us against 120 us + 15 us a step).
 bool poly_beats_steps(const PolyTable &t, int steps) { return se2n_poly_cost(t) < 5.0 * steps + 36.0; }
 
+// The polynomial of an interval asked for with no flag; null where the steps are taken,
+// as always in a plan whose step kernel the caller has tuned.
+const PolyTable *steps_poly(se2n_plan *plan, double beta, double T, int steps) {
+    const PolyTable *t = plan->tuned ? nullptr : poly_get(plan, beta, T, steps);
+    return t && poly_beats_steps(*t, steps) ? t : nullptr;
+}
+
 // The polynomial stands for the propagators: one build a change of beta, T or
 // steps, as for the matrices (it is made on the host, the stage times nothing).
 void poly_count_build(se2n_plan *plan) {
@@ -294,10 +301,9 @@ bool restores(const se2n_params *p) { return p->rounds > 1 || p->final_mix; }
 const PolyTable *col_poly(se2n_plan *plan, double beta, double T, int steps, int flags, bool restored) {
     if (restored) return nullptr;
     if (flags != 0 && !plan->rebuilds && plan->N < 30) return nullptr;
-    const PolyTable *t = poly_get(plan, beta, T, steps);
+    const PolyTable *t = flags == 0 ? steps_poly(plan, beta, T, steps) : poly_get(plan, beta, T, steps);
     if (!t || !se2n_col_has_poly(*t)) return nullptr;
-    if (flags == 0) return poly_beats_steps(*t, steps) ? t : nullptr;
-    return plan->rebuilds || se2n_poly_cost(*t) <= 48 ? t : nullptr;
+    return flags == 0 || plan->rebuilds || se2n_poly_cost(*t) <= 48 ? t : nullptr;
 }
 
 // Row and column passes of the Hermitian half (rowfft.cu, colprop.cu): the
@@ -462,8 +468,8 @@ se2n_status diffuse_impl(se2n_plan *plan, float2 *vol, double beta, double T, in
         flags &= ~SE2N_DIFFUSE_PROPAGATOR;  // stiff: the step kernel keeps the accuracy
     }
     if (flags == 0 && !restored) {
-        const PolyTable *t = poly_get(plan, beta, T, steps);
-        if (t && poly_beats_steps(*t, steps)) return poly_impl(plan, vol, *t, half, k0, rows);
+        const PolyTable *t = steps_poly(plan, beta, T, steps);
+        if (t) return poly_impl(plan, vol, *t, half, k0, rows);
     }
     const bool fp64 = (flags & SE2N_DIFFUSE_SM_FP64) != 0;
     // The fused diagonal 2 + a^2/beta perturbs decay rates by ~1.2e-7 beta per
@@ -1102,6 +1108,7 @@ se2n_status se2n_plan_tune_diffuse(se2n_plan *plan, int threads_per_freq, int bl
     plan->diffuse_P = P;
     plan->diffuse_block = block;
     plan->diffuse_blocks = blocks;
+    plan->tuned = threads_per_freq != 0 || block_threads != 0;
     return SE2N_OK;
 }
 

@@ -79,6 +79,7 @@ struct se2n_plan {
     int diffuse_P;         // threads per frequency
     int diffuse_block;     // threads per block; 0 = the default shape for N
     int diffuse_blocks;    // 0 = fill the device
+    bool tuned;            // by the caller: the step kernel it tuned is the one that runs
     int num_sms;
     int last_cuda_error;
     // stage timing (se2n_plan_profile): event pairs per stage, reused

@@ -143,6 +143,10 @@ class GpuBackend:
         self.dev = device or torch.device("cuda", torch.cuda.current_device())
         self.plane_plans = {p: se2n.se2n_plan_create(H, W, N // P, angle_conv, stream) for p in ranks}
         self.full_plan = se2n.se2n_plan_create(H, W, N, angle_conv, stream)
+        # a tuned plan steps: the restoration between intervals decides by a
+        # threshold, so its outcome depends on the rounding of the interval
+        se2n.se2n_plan_tune_diffuse(self.full_plan,
+                                    se2n.se2n_plan_diffuse_info(self.full_plan)["threads_per_freq"])
 
     def close(self):
         for pl in self.plane_plans.values():

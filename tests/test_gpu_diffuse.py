@@ -264,3 +264,44 @@ def test_interval_polynomial_matches_oracle(N, H, W, beta, T, S, flags, conv):
     err = rel_l2(got, ref)
     print(f"N={N} {H}x{W} beta={beta} T={T} S={S} flags={flags} conv={conv}: rel-L2 {err:.2e}")
     assert err <= REL_L2
+
+
+@pytest.mark.parametrize("N,P", VARIANTS)
+def test_a_tuned_plan_steps(N, P):
+    """A caller that tunes the step kernel gets it, with no flag too: past
+    beta T = 8 the steps take the split diagonal by themselves, so the bits are those of
+    SE2N_DIFFUSE_SPLIT_DIAG. The fast kernel (beta dt = 0.03) and the general one (0.1)."""
+    vol = synth.random_volume(N, 12, 14, seed=N + P, dtype=np.complex64)
+    for beta, T, S in ((1.0, 9.0, 300), (2.0, 5.0, 100)):
+        got = _run(vol, N, beta, T, S, tune=(P, 128, 0))
+        want = _run(vol, N, beta, T, S, flags=se2n.SE2N_DIFFUSE_SPLIT_DIAG, tune=(P, 128, 0))
+        np.testing.assert_array_equal(got, want)
+        assert rel_l2(got, oracle.diffuse(vol.astype(np.complex128), beta, T, S)) <= REL_L2
+
+
+def test_tuning_back_to_the_default_is_an_untuned_plan():
+    vol = synth.random_volume(32, 12, 14, seed=3, dtype=np.complex64)
+    plain = _run(vol, 32, 1.0, 9.0, 300)
+    np.testing.assert_array_equal(_run(vol, 32, 1.0, 9.0, 300, tune=(0, 0, 0)), plain)
+    assert (_run(vol, 32, 1.0, 9.0, 300, tune=(2, 0, 0)) != plain).any()
+
+
+@pytest.mark.parametrize("N,beta,T,S", [(32, 0.25, 2.0, 40), (16, 0.05, 7.5, 200), (64, 0.25, 2.0, 20)])
+def test_split_diagonal_matches_oracle(N, beta, T, S):
+    """SE2N_DIFFUSE_SPLIT_DIAG where it is not taken by itself, packed and general kernels."""
+    vol = synth.random_volume(N, 18, 26, seed=N + S, dtype=np.complex64)
+    ref = oracle.diffuse(vol.astype(np.complex128), beta, T, S)
+    for more in (0, se2n.SE2N_DIFFUSE_FULL_CORRECTION):
+        assert rel_l2(_run(vol, N, beta, T, S, flags=se2n.SE2N_DIFFUSE_SPLIT_DIAG | more), ref) <= REL_L2
+
+
+def test_full_size_2048_N64_1000_steps_on_the_step_kernel_sampled():
+    """The main run of the largest workload by its steps (split diagonal)."""
+    N, H, W = 64, 2048, 2048
+    vol_h = synth.random_volume(N, H, W, seed=45, dtype=np.complex64)
+    freqs = _sampled(H, W, 100, 3)
+    full = np.zeros((N, H * W), np.complex128)
+    full[:, freqs] = vol_h.reshape(N, -1)[:, freqs]
+    got = _run(vol_h, N, 0.25, 50.0, 1000, tune=(4, 0, 0)).reshape(N, -1)[:, freqs]
+    ref = oracle.diffuse(full.reshape(N, H, W), 0.25, 50.0, 1000, freqs=freqs).reshape(N, -1)[:, freqs]
+    assert rel_l2(got, ref) <= REL_L2

@@ -101,3 +101,19 @@ def test_sharded_inpaint_on_one_gpu_matches_the_whole_path_and_the_oracle(P):
     assert rel_l2(got[0], whole) <= 1e-6
     assert rel_l2(got[0], ref) <= REL_L2
     assert np.abs(got[0] - ref).max() <= MAX_REL * np.abs(f64).max()
+
+
+def test_sharded_intervals_are_stepped():
+    """The row shards of the sharded method take the steps, as the whole method
+    with a restoration does: past beta T = 8 (the split diagonal) the bits of
+    SE2N_DIFFUSE_SPLIT_DIAG on the same rows."""
+    N, H, W = 32, 32, 20
+    vol = synth.random_volume(N, H, W, seed=9).astype(np.complex64)
+    backend = shard.GpuBackend(H, W, N, 2, [0, 1])
+    got = host(backend.diffuse_rows(1, t_c64(np.ascontiguousarray(vol[:, 16:])), 16, 1.0, 9.0, 300))
+    backend.close()
+    plan = se2n.se2n_plan_create(H, W, N)
+    want = t_c64(np.ascontiguousarray(vol[:, 16:]))
+    se2n.se2n_diffuse_rows(plan, want, 16, 1.0, 9.0, 300, se2n.SE2N_DIFFUSE_SPLIT_DIAG)
+    plan.close()
+    np.testing.assert_array_equal(got, host(want))
