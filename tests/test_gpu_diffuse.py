@@ -305,3 +305,19 @@ def test_full_size_2048_N64_1000_steps_on_the_step_kernel_sampled():
     got = _run(vol_h, N, 0.25, 50.0, 1000, tune=(4, 0, 0)).reshape(N, -1)[:, freqs]
     ref = oracle.diffuse(full.reshape(N, H, W), 0.25, 50.0, 1000, freqs=freqs).reshape(N, -1)[:, freqs]
     assert rel_l2(got, ref) <= REL_L2
+
+
+@pytest.mark.parametrize("N", [4, 16, 30, 32, 64])
+@pytest.mark.parametrize("T", [5.0, 13.0, 50.0])
+def test_constant_modes_are_exact_at_every_interval(N, T):
+    """Constant angular vectors where both sines are 0 (frequency 0 and the
+    Nyquist ones) come back bit for bit from both forms of the polynomial."""
+    rng = np.random.default_rng(N)
+    vol = synth.random_volume(N, 8, 10, seed=N, dtype=np.complex64)
+    at = [(0, 0), (4, 0), (0, 5), (4, 5)]
+    for k, l in at:
+        vol[:, k, l] = np.complex64(1000.0 * complex(*rng.standard_normal(2)))
+    got = _run(vol, N, 0.25, T, int(20 * T))
+    for k, l in at:
+        np.testing.assert_array_equal(got[:, k, l], vol[:, k, l])
+    assert rel_l2(got, oracle.diffuse(vol.astype(np.complex128), 0.25, T, int(20 * T))) <= REL_L2
