@@ -1087,7 +1087,7 @@ se2n_status se2n_inpaint_host(se2n_plan *plan, const float *f_host, const uint8_
 se2n_status se2n_plan_drop_propagators(se2n_plan *plan, int free_memory) {
     SE2N_TRY(check_plan(plan));
     plan->prop_valid = false;
-    plan->poly_built = false;
+    plan->poly_built = plan->poly_made = false;
     if (free_memory && plan->prop_D) {
         prop_join(plan);  // a build still running on the side stream
         SE2N_TRY(cuda_status(plan, cudaStreamSynchronize(plan->stream)));

@@ -16,7 +16,7 @@ struct PolyTable {
 };
 
 // Fill t for S steps of dt = T / S. False where the polynomial form does not
-// apply: a Crank-Nicolson factor may be negative (dt (2 + 4 beta) > 2, where
+// apply: beta below 1e-12, a Crank-Nicolson factor may be negative (dt (2 + 4 beta) > 2, where
 // f oscillates up to -1 and is no longer smooth), or more than kPolyMax
 // coefficients would be needed.
 bool se2n_poly_make(double beta, double T, int steps, PolyTable &t);
