@@ -177,3 +177,31 @@ def test_batch_with_propagators(full):
         ref = oracle.inpaint(f64, m, oracle.Params(N=N, beta=0.25, T=T, steps=S, rounds=R), bins=bb)["out"]
         assert rel_l2(a, ref) <= REL_L2
         assert np.abs(a - ref).max() <= MAX_REL * np.abs(f64).max()
+
+
+@pytest.mark.parametrize("full", [0, 1])
+@pytest.mark.parametrize("T,flags", [(2.0, 0), (25.0, 0), (2.0, se2n.SE2N_DIFFUSE_PROPAGATOR),
+                                     (25.0, se2n.SE2N_DIFFUSE_PROPAGATOR)])
+def test_one_interval_batches_take_the_polynomial(T, flags, full):
+    """A batch of one interval applies the interval polynomial in its
+    persistent launch (both forms), or per shape: bitwise the per-image path,
+    and the oracle's result."""
+    inputs = _inputs(SHAPES + [(64, 64, 32), (128, 64, 64)], seed=31)
+    S = int(20 * T)
+    bins = [oracle.orient(f.astype(np.float32).astype(np.float64), m, N)["bins"] for f, m, N in inputs]
+    prm = se2n.se2n_params_default(beta=0.25, T=T, steps=S, rounds=1, eps=0.5, diffuse_flags=flags,
+                                   full_spectrum=full)
+    b, outs = _batch(inputs, prm, bins=bins)
+    se2n.se2n_batch_run(b)
+    got = [host(o).copy() for o in outs]
+    for o in outs:
+        o.zero_()
+    se2n.se2n_batch_run_per_image(b)
+    per = [host(o).copy() for o in outs]
+    b.close()
+    for (f, m, N), bb, g, d in zip(inputs, bins, got, per):
+        np.testing.assert_array_equal(g, d)
+        f64 = f.astype(np.float32).astype(np.float64)
+        ref = oracle.inpaint(f64, m, oracle.Params(N=N, beta=0.25, T=T, steps=S, rounds=1), bins=bb)["out"]
+        assert rel_l2(g, ref) <= REL_L2
+        assert np.abs(g - ref).max() <= MAX_REL * np.abs(f64).max()

@@ -213,3 +213,41 @@ def test_edges_of_the_convolution_tiles(B, H, W):
     network summed in FP32 differs from the FP64-summed one by up to 0.046
     (gradients) and 1.1e-3 (output) on these inputs."""
     test_forward_and_gradients_match_oracle(B, H, W)
+
+
+@pytest.mark.parametrize("B,H,W", [(32, 256, 256), (64, 72, 136), (128, 8, 24)])
+def test_copies_of_an_image_repeat_its_output_and_gradients(B, H, W):
+    """Enough copies of one image that every CTA takes several tiles, in turn
+    by both epilogue groups, in rings that wrap, in full and partial groups of
+    tiles, and several pixel ranges and sums a weight gradient. A pixel's
+    arithmetic does not depend on its CTA, so every copy has the single image's
+    output, to the bit. B is a power of two, so the loss's gradient at a pixel is the
+    single image's over B exactly in bf16, and the parameters' gradients are sums of B equal
+    parts over B: the same to the rounding of their FP32 sums (below 4e-9 a term of the
+    longest sum on the tensor cores, 2e-4 for 47616 terms; one tile or pixel range
+    missed or counted twice moves a tensor by 1 % and more)."""
+    p32 = ou.he_params(13).astype(np.float32)
+    f, mask, target = _inputs(1, H, W, 6)
+    outs, grads = [], []
+    for n in (1, B):
+        u = se2n.se2n_unet_create(n, H, W)
+        se2n.se2n_unet_set_params(u, p32)
+        fd, md, td = (t(np.repeat(a, n, 0)) for t, a in ((t_f32, f), (t_u8, mask), (t_f32, target)))
+        out = torch.zeros((n, H, W), dtype=torch.float32, device="cuda")
+        se2n.se2n_unet_forward(u, fd, md, n, out)
+        loss = torch.zeros(1, dtype=torch.float32, device="cuda")
+        se2n.se2n_unet_backward(u, fd, md, td, n, loss)
+        g = np.zeros(se2n.se2n_unet_param_count(u), np.float32)
+        se2n.se2n_unet_get_grads(u, g)
+        u.close()
+        outs.append(out)
+        grads.append(g)
+    assert torch.equal(outs[1], outs[0].expand_as(outs[1]))
+    offs, hw, hb, _ = ou.layout()
+    parts = [("head", slice(hw, hb + 1))]
+    for i, ((w, b), (cin, cout, _)) in enumerate(zip(offs, ou.LAYERS)):
+        parts += [(f"dW {i}", slice(w, w + cout * 9 * cin)), (f"db {i}", slice(b, b + cout))]
+    for name, s in parts:
+        e = _rel(grads[1][s], grads[0][s])
+        print(f"{name}: {e:.2e}")
+        assert e <= 2e-4, name
