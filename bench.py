@@ -5,25 +5,24 @@ piecewise-smooth image, 80 % random mask plus 4-px bars every 32 px,
 beta = 0.25, 10 restoration intervals of 500 Crank-Nicolson steps, T = 2 per
 interval): orientation, lift, the 2-D DFT, 10 x diffusion, 9 x (inverse
 DFT, static restoration, forward DFT), inverse DFT, projection, all through
-se2n_inpaint with the inputs resident in HBM. By default
-(--diffusion propagator) each interval's 500 steps are applied as one
-linear map per frequency, the polynomial of its operator that equals the
-steps' product to FP32 resolution, and each interval runs as one column
-pass (DFT along y, the polynomial, inverse DFT) and one row pass (real DFTs
-along x around the restoration); --diffusion steps runs the fused
-step-by-step kernel (asked for by its split-diagonal form) between cuFFT
+se2n_inpaint with the inputs resident in HBM. By default each interval's
+500 steps are applied as one precomputed S-step propagator per class of
+frequencies, built inside every timed inpaint, and each interval runs as
+one column pass (DFT along y, propagators, inverse DFT) and one row pass
+(real DFTs along x around the restoration) (--diffusion propagator);
+--diffusion steps runs the fused step-by-step kernel between cuFFT
 transforms instead, and the default line reports that path too.
 
 Metric: Mathieu updates per second over the whole inpaint time (value),
 counting the frequencies the path integrates: the lifted volume is real, so
 the H x (W/2 + 1) frequencies of the Hermitian half carry the whole
 spectrum, and updates = 512 * 257 * 32 * 500 * 10 per inpaint (on the
-default path these are equivalent updates: each interval's 500 steps
-are applied as one map). The count over all M^2 frequencies
+propagator path these are equivalent updates: each interval's 500 steps
+are applied as one precomputed map). The count over all M^2 frequencies
 that the method's own formulation integrates is reported beside it
 (m2_updates_per_s). Plus ms per inpaint (the first figure of the line), the FP32 error against the FP64 oracle, the roofline of the
 dominant kernel (the column pass against the measured copy rate, with the
-row pass beside it; or the step kernel, FP32 ALU
+row pass and the propagator build beside it; or the step kernel, FP32 ALU
 bound, whose flops are those of the frequencies it integrates, the
 Hermitian half 512 x 257 of the spectrum), the end-to-end number from host
 buffers (se2n_inpaint_host) and the oracle's CPU rate.
@@ -55,12 +54,10 @@ import synth  # noqa: E402
 METRIC = "Mathieu updates/s (M²·N·steps); ms per 512² N=32 inpaint, err vs FP64"
 UNIT = "updates/s"
 FLOPS_PER_UPDATE = 22          # per complex angle per CN step: 2 x (1 add + 5 FMA)
-# the step kernel's split-diagonal form, which the benchmark asks for: one more FMA a component
+# the step kernel's split-diagonal form (beta T > 8): one more FMA a component
 FLOPS_PER_UPDATE_SPLIT = FLOPS_PER_UPDATE + 4
 # coefficients of the interval polynomial in the eight ranges of wx^2 + wy^2 (quarters
-# of [0, 2]), as the library makes them for beta = 0.25: T = 2 in 500 steps (increment form) and
-# T = 50 in 1000 (Reinsch's form)
-POLY_512 = (9, 10, 10, 11, 11, 12, 12, 13)
+# of [0, 2]), as the library makes them for beta = 0.25, T = 50 in 1000 steps (Reinsch's form)
 POLY_2048 = (33, 36, 39, 42, 44, 46, 48, 50)
 GOLDEN = os.path.join(ROOT, "tests", "golden", "curves_noise_512_N32.npz")
 L2_FLUSH_BYTES = 256 << 20
@@ -240,6 +237,36 @@ def poly_flops(H, W, N, coeffs, reinsch):
     return int(4 * N * ((5 * (m - 1) + 2) if reinsch else (3 * (m - 1) + 6)).sum())
 
 
+def propagator_gemm_flops(classes, N, S):
+    """FP32 flops of building the S-step propagators and the products a class:
+    every op of the library's powering program but its copies is one
+    N x N x N product (2 N^3 flops); the O(N^2) solves of the first step are
+    not counted."""
+    from paper_1304_2062_gb300 import se2n
+    ops, _ = se2n.se2n_prop_chain(S)
+    products = sum(o != se2n.PROP_COPY for o in ops)
+    return classes * products * 2 * N ** 3, products
+
+
+def propagator_classes(H, W, half=True):
+    """Classes of frequencies that share one propagator: row slots s in
+    [0, H/4] (rows s, H/2 - s, and H/2 + s, H - s reversed) times column
+    pairs l and (W/2 - l) (Hermitian half: l <= W/2)."""
+    row_slots = H // 4 + 1
+    cols = W // 4 + 1 if half else W // 4 + 1 + (3 * W) // 4 - W // 2
+    return row_slots * cols
+
+
+def propagator_build_items(H, W, half=True):
+    """Classes the build computes: on square planes (Hermitian half) a class
+    and its transpose share one build, so n (n + 1) / 2 of the n x n slot
+    pairs; otherwise every class."""
+    if half and H == W:
+        n = W // 4 + 1
+        return n * (n + 1) // 2
+    return propagator_classes(H, W, half)
+
+
 def max_over_ranks(value, dist=None, device="cpu"):
     """The largest value over all ranks (the job's time is its slowest rank's)."""
     if dist is None or not dist.is_initialized() or dist.get_world_size() == 1:
@@ -281,7 +308,7 @@ def run_ours(args, rank, world, local_rank):
     plan = se2n.se2n_plan_create(w.H, w.W, w.N, 0, stream)
     dynamic = args.workload == "dr"
     prop = args.diffusion == "propagator"
-    flags = se2n.SE2N_DIFFUSE_PROPAGATOR if prop else se2n.SE2N_DIFFUSE_SPLIT_DIAG
+    flags = se2n.SE2N_DIFFUSE_PROPAGATOR if prop else 0
     prm = se2n.se2n_params_default(N=w.N, beta=w.beta, T=w.T, steps=w.steps, rounds=w.rounds, eps=w.eps,
                                    sigma_smooth=w.sigma, dynamic=int(dynamic), diffuse_flags=flags)
     f_d = torch.tensor(f32, device=dev)
@@ -338,33 +365,47 @@ def run_ours(args, rank, world, local_rank):
     # the path integrates the Hermitian half of the spectrum: H x (W/2 + 1) frequencies
     updates_per_launch = w.H * (w.W // 2 + 1) * w.N * w.steps
     if prop:
-        # every interval is one column pass (DFT along y, the polynomial, inverse
+        # every interval is one column pass (DFT along y, propagators, inverse
         # DFT along y) and one row pass (inverse real DFT along x, restoration,
-        # forward real DFT along x). The column passes take the largest share of
-        # the inpaint.
+        # forward real DFT along x); the propagators are built once. The
+        # column passes take the largest share of the inpaint.
         c_ms, c_calls = prof["diffuse"]
         c_s = c_ms / c_calls / 1e3
         r_ms, r_calls = prof["fft"]
         r_s = r_ms / r_calls / 1e3
+        b_ms, b_calls = prof["propagator"]
+        b_s = b_ms / b_calls / 1e3
+        classes = propagator_classes(w.H, w.W)
         wc = w.W // 2 + 1
         spec_bytes = 8 * wc * w.H * w.N
-        col_bytes = 2 * spec_bytes
+        # the method's bytes: the half spectrum in and out, and every class's
+        # propagator once as its N (N + 1) / 2 distinct entries (the kernel
+        # reads the stored rows, 4 N^2 bytes a class: stored_bytes_per_launch)
+        col_bytes = 2 * spec_bytes + 4 * (w.N * (w.N + 1) // 2) * classes
+        col_stored_bytes = 2 * spec_bytes + 4 * w.N * w.N * classes
         row_bytes = 2 * spec_bytes + 6 * w.H * w.W
-        col_flops = 2 * wc * w.N * 5 * w.H * int(math.log2(w.H)) + poly_flops(w.H, w.W, w.N, POLY_512, False)
+        col_flops = 2 * wc * w.N * 5 * w.H * int(math.log2(w.H)) + 4 * w.N * w.N * w.H * wc
+        items = propagator_build_items(w.H, w.W)
+        flops, products = propagator_gemm_flops(items, w.N, w.steps)
+        # the symmetric build (N = 16, 32) computes the 10 upper-triangle 8 x 8
+        # tiles of the 16 of every product and mirrors them
+        exec_flops = flops * 10 // 16 if w.N in (16, 32) else flops
         hbm = _peaks().get("hbm_gbs")
         hbm_basis = "MEASURED_PEAKS.json hbm_gbs (copy, burst)"
         roofline = {"bound": "hbm", "achieved": round(col_bytes / c_s / 1e9, 1), "peak": hbm, "unit": "GB/s",
                     "frac": round(col_bytes / c_s / 1e9 / hbm, 4) if hbm else None,
                     "traffic": args.traffic if args.traffic is not None else stored_traffic("col_prop"),
-                    "kernel": f"k_col_tma<{w.N},{w.H}> (column pass: DFT along y, the interval's polynomial, inverse "
-                              "DFT; whole columns in shared memory, bulk copies in and out, one persistent block an SM)",
+                    "kernel": f"k_col_tma<{w.N},{w.H}> (column pass: DFT along y, x <- x + D_S x, inverse DFT; "
+                              "whole columns in shared memory, bulk copies in and out, one persistent block an SM)",
                     "bytes_per_launch": col_bytes,
                     "bytes_basis": "one read and one write of the row-transformed half spectrum (8 (W/2+1) H N "
-                                   "bytes each)",
+                                   "bytes each) + every class's symmetric propagator once, as its N (N + 1) / 2 "
+                                   "distinct entries (4 N (N + 1) / 2 bytes a class)",
+                    "stored_bytes_per_launch": col_stored_bytes,
+                    "stored_basis": "the propagators as the kernel reads them, full rows (4 N^2 bytes a class)",
                     "avg_launch_ms": round(c_s * 1e3, 4), "peak_basis": hbm_basis,
                     "flops_per_launch": col_flops,
-                    "flops_basis": "2 (W/2+1) N complex DFTs of length H at 5 H log2 H + the polynomial, 3 (m - 1) + 6 "
-                                   "packed instructions an angle at 4 flops",
+                    "flops_basis": "2 (W/2+1) N complex DFTs of length H at 5 H log2 H + 4 N^2 a frequency",
                     "frac_of_fp32_peak": round(col_flops / c_s / 1e12 / peak, 4),
                     "row_pass": {"kernel": f"k_row<{w.N},{w.W}> (inverse real DFT along x, restoration, forward "
                                            "real DFT; one block a row)", "bound": "hbm",
@@ -373,16 +414,31 @@ def run_ours(args, rank, world, local_rank):
                                  "achieved_gbs": round(row_bytes / r_s / 1e9, 1), "peak_gbs": hbm,
                                  "frac": round(row_bytes / r_s / 1e9 / hbm, 4) if hbm else None,
                                  "traffic": stored_traffic("row_pass")},
+                    "build": {"kernel": f"k_prop_build_sym<{w.N}> ({items} of the {classes} classes computed, each "
+                                        "also stored permuted for its transpose; FP32 symmetric products; on a side "
+                                        "stream, overlapping the orientation and the first row pass)",
+                              "bound": "alu",
+                              "avg_launch_ms": round(b_s * 1e3, 4),
+                              "flops_basis": "executed flops: classes built x products x 2 N^3 x 10/16 (the symmetric "
+                              "kernel computes the 10 upper-triangle 8x8 tiles of 16 and mirrors them), "
+                              f"S = {w.steps}: {products} products (se2n_prop_chain's program; binary powering "
+                              f"takes {w.steps.bit_length() - 1 + bin(w.steps).count('1') - 1})",
+                              "flops_per_launch": exec_flops,
+                              "full_product_flops_per_launch": flops,
+                              "achieved_tflops": round(exec_flops / b_s / 1e12, 3), "peak_tflops": round(peak, 3),
+                              "frac": round(exec_flops / b_s / 1e12 / peak, 4), "peak_basis": peak_basis,
+                              "frac_full_product_equivalent": round(flops / b_s / 1e12 / peak, 4),
+                              "traffic": stored_traffic("prop_build")},
                     "frequencies_integrated": "Hermitian half, H x (W/2 + 1)"}
     else:
         d_ms, d_calls = prof["diffuse"]
         d_avg_s = d_ms / d_calls / 1e3
-        achieved = FLOPS_PER_UPDATE_SPLIT * updates_per_launch / d_avg_s / 1e12
+        achieved = FLOPS_PER_UPDATE * updates_per_launch / d_avg_s / 1e12
         roofline = {"bound": "alu", "achieved": round(achieved, 3), "peak": round(peak, 3), "unit": "TFLOP/s",
                     "frac": round(achieved / peak, 4),
                     "traffic": args.traffic if args.traffic is not None else stored_traffic(),
-                    "kernel": "k_diffuse_x2<32,2,true> (packed FP32 pairs, truncated corner correction)",
-                    "flops_per_update": FLOPS_PER_UPDATE_SPLIT, "updates_per_launch": updates_per_launch,
+                    "kernel": "k_diffuse_x2<32,2,false> (packed FP32 pairs, truncated corner correction)",
+                    "flops_per_update": FLOPS_PER_UPDATE, "updates_per_launch": updates_per_launch,
                     "avg_launch_ms": round(d_avg_s * 1e3, 4), "peak_basis": peak_basis,
                     "diffuse_updates_per_s": updates_per_launch / d_avg_s,
                     "hbm_gbs_of_diffuse": round(16 * w.H * (w.W // 2 + 1) * w.N / d_avg_s / 1e9, 1),
@@ -391,8 +447,7 @@ def run_ours(args, rank, world, local_rank):
               for k, v in prof.items() if k != "kernels"}
     launches = int(prof["kernels"])
 
-    cfg = _config(w, {"diffusion": "each interval's steps as one map, a polynomial of the operator "
-                                   "(SE2N_DIFFUSE_PROPAGATOR, nothing kept between inpaints)" if prop
+    cfg = _config(w, {"diffusion": "S-step propagators built every inpaint (SE2N_DIFFUSE_PROPAGATOR)" if prop
                       else "step by step, the fused Crank-Nicolson kernel"}, dynamic=dynamic)
     result = {"metric": METRIC, "ms_per_inpaint": round(ms_per_step, 4), "value": value, "unit": UNIT,
               "m2_updates_per_s": world * w.updates() * args.steps / (total_ms / 1e3),
@@ -405,8 +460,8 @@ def run_ours(args, rank, world, local_rank):
                               "steps run without them (they add about 0.1 ms an inpaint)"}
     if prop:
         # the other two ways to run the same inpaint, on the same plan and inputs:
-        # without dropping what the plan keeps between calls (the polynomial's
-        # coefficients), and the step-by-step kernel with its own roofline
+        # propagators kept from the previous call (serving one beta dt and S),
+        # and the step-by-step kernel with its own roofline
         with torch.cuda.stream(stream):
             def timed3(fn):
                 evs = []
@@ -427,8 +482,7 @@ def run_ours(args, rank, world, local_rank):
             kprof = se2n.se2n_plan_profile_read(plan, reset=True)
             se2n.se2n_plan_profile(plan, False)
             prm_s = se2n.se2n_params_default(N=w.N, beta=w.beta, T=w.T, steps=w.steps, rounds=w.rounds, eps=w.eps,
-                                             sigma_smooth=w.sigma, dynamic=int(dynamic),
-                                             diffuse_flags=se2n.SE2N_DIFFUSE_SPLIT_DIAG)
+                                             sigma_smooth=w.sigma, dynamic=int(dynamic))
             se2n.se2n_inpaint(plan, f_d, m_d, None, prm_s, vol, out)
             torch.cuda.synchronize(dev)
             se2n.se2n_plan_profile(plan, True)
@@ -436,9 +490,10 @@ def run_ours(args, rank, world, local_rank):
             sprof = se2n.se2n_plan_profile_read(plan, reset=True)
             se2n.se2n_plan_profile(plan, False)
         sd_s = sprof["diffuse"][0] / sprof["diffuse"][1] / 1e3
-        s_ach = FLOPS_PER_UPDATE_SPLIT * updates_per_launch / sd_s / 1e12
+        s_ach = FLOPS_PER_UPDATE * updates_per_launch / sd_s / 1e12
         result["propagators_kept"] = {"ms_per_step": round(kept, 4), "value": world * upd / (kept / 1e3)}
-        # the row and column passes as timed in those
+        # the row and column passes timed where nothing runs beside them (in the
+        # timed inpaints the build overlaps the orientation and the first row pass)
         c_s = kprof["diffuse"][0] / kprof["diffuse"][1] / 1e3
         r_s = kprof["fft"][0] / kprof["fft"][1] / 1e3
         hbm = roofline["peak"]
@@ -446,18 +501,18 @@ def run_ours(args, rank, world, local_rank):
         roofline.update({"achieved": round(col_bytes / c_s / 1e9, 1), "avg_launch_ms": round(c_s * 1e3, 4),
                          "frac": round(col_bytes / c_s / 1e9 / hbm, 4) if hbm else None,
                          "frac_of_fp32_peak": round(roofline["flops_per_launch"] / c_s / 1e12 / peak, 4),
-                         "timed_on": "the inpaints of propagators_kept (CUDA events around each launch)"})
+                         "timed_on": "the inpaints that reuse the propagators (CUDA events around each launch)"})
         roofline["row_pass"].update({"avg_launch_ms": round(r_s * 1e3, 4),
                                      "achieved_gbs": round(row_bytes / r_s / 1e9, 1),
                                      "frac": round(row_bytes / r_s / 1e9 / hbm, 4) if hbm else None,
-                                     "timed_on": "the inpaints of propagators_kept; the average over all "
+                                     "timed_on": "the inpaints that reuse the propagators; the average over all "
                                                  "row passes of an inpaint (lift and projection included)"})
         result["step_by_step"] = {
             "ms_per_step": round(stepwise, 4), "value": world * upd / (stepwise / 1e3),
-            "roofline": {"bound": "alu", "kernel": "k_diffuse_x2<32,2,true>", "avg_launch_ms": round(sd_s * 1e3, 4),
+            "roofline": {"bound": "alu", "kernel": "k_diffuse_x2<32,2,false>", "avg_launch_ms": round(sd_s * 1e3, 4),
                          "achieved": round(s_ach, 3), "peak": round(peak, 3), "unit": "TFLOP/s",
                          "frac": round(s_ach / peak, 4), "traffic": stored_traffic(),
-                         "flops_per_update": FLOPS_PER_UPDATE_SPLIT, "updates_per_launch": updates_per_launch}}
+                         "flops_per_update": FLOPS_PER_UPDATE, "updates_per_launch": updates_per_launch}}
     if dynamic:
         # with propagators the image value h and its argmax angle come from a
         # row pass (counted with the row passes); the growth kernel reads h,
@@ -937,8 +992,8 @@ def run_batch(args, rank, world, local_rank):
                        "diffusion": ("each interval as one map (the polynomial) for the shapes where it is estimated cheaper "
                                      f"({info['prop_images']} images; {info['fused_images']} of them, the "
                                      "shapes the row and column passes cover (N = 16, 30, 32), whole inpaints on "
-                                     "them, the others with the separate apply), the persistent kernel for "
-                                     "the rest")
+                                     "them, the others with a polynomial launch of their own), the persistent "
+                                     "kernel for the rest")
                        if prop else "the persistent kernel for every image (the polynomial where it takes "
                                     "the place of the steps)",
                        "l2": "flushed between timed steps (256 MiB write)", "parallelism": "replicas"},

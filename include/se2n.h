@@ -71,26 +71,28 @@ typedef enum se2n_status {
 /* se2n_diffuse flags. */
 #define SE2N_DIFFUSE_SM_FP64 1     /* Sherman-Morrison correction scalars in FP64 */
 #define SE2N_DIFFUSE_SPLIT_DIAG 2  /* keep a_r^2/beta apart from the angular second difference
-                                      (always on when beta * T > 8, see se2n_diffuse) */
+                                      (the step kernel takes it by itself when beta * T > 8, see se2n_diffuse) */
 #define SE2N_DIFFUSE_FULL_CORRECTION 4  /* apply the corner correction on every angle (no truncation) */
 /* Integrate by the S-step propagator: the S steps of an interval are one
  * linear map (B-^{-1} B+)^S a frequency (Section 4: the integration over an
  * interval is one linear map), the same result as S Crank-Nicolson steps up to
- * rounding. The map is applied as a polynomial of the operator, the truncated Chebyshev series of ((1 + dt x / 2) / (1 - dt x / 2))^S
- * on the operator's spectrum (cut off below FP32 resolution: about 12
- * multiplications by the three-point operator for T (2 + 4 beta) / 2 = 3, about
- * 50 for 75), whose coefficients the host makes when beta, T or steps change;
- * where more than 64 coefficients would be needed, and in the column pass (below)
- * with N = 16 or where applying kept matrices is faster (T (2 + 4 beta) / 2 above
- * about 3), and in every interval of an inpaint
- * with a restoration (rounds > 1 or final_mix; its threshold turns rounding into
- * different values of a few pixels, so that those intervals keep one
- * arithmetic), as a matrix:
- * for every class of frequencies that share it (rows s, H/2 - s as they are
- * and rows H/2 + s, H - s with the angles reversed, times columns l and
- * (W/2 - l) mod W) (B-^{-1} B+)^S - I is built once in FP32 by the powering
- * program of se2n_prop_chain, in increment form, and applied as one N x N
- * product per frequency. The plan keeps the matrices
+ * rounding, in one of two forms; which one follows from the call's arguments.
+ * A polynomial of the operator: the truncated Chebyshev series of
+ * ((1 + dt x / 2) / (1 - dt x / 2))^S on the operator's spectrum (cut off below
+ * FP32 resolution: about 12 multiplications by the three-point operator for
+ * T (2 + 4 beta) / 2 = 3, about 50 for 75), whose coefficients the host makes
+ * when beta, T or steps change (13 to 75 us).
+ * A matrix: where more than 64 coefficients would be needed; in the column
+ * pass (below) with N = 16 or where applying kept matrices is faster
+ * (T (2 + 4 beta) / 2 above about 3; a batch builds them in every run and takes
+ * the polynomial there too); and in every interval of an inpaint with a restoration
+ * (rounds > 1 or final_mix): it decides by a threshold, which turns rounding
+ * into different values of a few pixels, so those intervals keep the arithmetic
+ * they have always had. For every class of frequencies that share it (rows s,
+ * H/2 - s as they are and rows H/2 + s, H - s with the angles reversed, times
+ * columns l and (W/2 - l) mod W) (B-^{-1} B+)^S - I is built once in FP32 by the
+ * powering program of se2n_prop_chain, in increment form, and applied as one
+ * N x N product per frequency. The plan keeps the matrices
  * (symmetric; by cyclic diagonals, 4 N (N/2 + 1) bytes a class, or as rows,
  * 4 N^2 bytes a class, for the column pass below and for N = 64 on the
  * Hermitian half, where they are applied 16 classes of one row slot at a
@@ -101,18 +103,18 @@ typedef enum se2n_status {
  * 32 x 32 matrices whose last two rows and columns are zero (the bytes of
  * N = 32). The other flags do not apply.
  * In se2n_inpaint on the Hermitian half with N = 16, 30 or 32 and H, W each one
- * of 64, 128, 256, 384, 512, 768, 1024, this flag alone selects the row and column passes (as
- * does flags = 0 for one interval without a restoration, where the polynomial
- * takes the place of the steps and has at most 32 coefficients): the
- * volume stays row-transformed between intervals in the caller's volume
- * buffer, each interval is one kernel a column (DFT along y,
- * the interval's map, inverse DFT) and one kernel a row (real DFTs along x around
- * the restoration), and no cuFFT call is made between intervals. The first
- * such call allocates two tables of 8 H and 8 W bytes and, where matrices are
- * built, a second stream of the plan, on which each
- * build runs beside the orientation and the lift (ordered after the work
- * already on the plan's stream, joined before the first column pass);
- * call once before capturing se2n_inpaint into a graph.
+ * of 64, 128, 256, 384, 512, 768, 1024, this flag alone selects the row and
+ * column passes (as does flags = 0 for one interval without a restoration,
+ * where the polynomial takes the place of the steps and has at most 32
+ * coefficients): the volume stays row-transformed between intervals in the
+ * caller's volume buffer, each interval is one kernel a column (DFT along y,
+ * the interval's map, inverse DFT) and one kernel a row (real DFTs along x
+ * around the restoration), and no cuFFT call is made between intervals. The
+ * first such call allocates two tables of 8 H and 8 W bytes and, where matrices
+ * are built, a second stream of the plan, on which each build runs beside the
+ * orientation and the lift (ordered after the work already on the plan's
+ * stream, joined before the first column pass); call once before capturing
+ * se2n_inpaint into a graph.
  * Accuracy guard: the FP32 powering in increment form cancels digits when
  * a Crank-Nicolson factor (1 - dt lambda/2) / (1 + dt lambda/2) of the
  * system approaches -1 (stiff modes at large beta dt). The flag is therefore
@@ -265,13 +267,14 @@ SE2N_API se2n_status se2n_inverse(se2n_plan *plan, void *vol);
  * side as (psi_{r-1} + psi_{r+1} - 2 psi_r) - (a_r^2/beta) psi_r instead of
  * with the fused coefficient 2 + a_r^2/beta, whose FP32 rounding perturbs
  * decay rates by ~1.2e-7 beta per unit time; it costs one FMA more per angle
- * and is selected automatically when beta * T > 8.
+ * and is selected automatically when beta * T > 8, where the interval is stepped.
  * With flags = 0 and dt (2 + 4 beta) <= 2, an interval whose polynomial (see
  * SE2N_DIFFUSE_PROPAGATOR) takes fewer operations than its steps is applied as
  * that polynomial, the same map of S steps to FP32 rounding; any flag keeps
  * the steps, and so do a tuned plan (se2n_plan_tune_diffuse) and se2n_inpaint
  * with a restoration (rounds > 1 or final_mix), whose decisions depend on
- * that rounding.
+ * that rounding. The polynomial's own error stays below 1.2e-6 of the volume
+ * at any beta T (its angular second difference and a_r^2/beta are fused).
  * When beta*dt <= ~0.067 (no FP64 flag), a packed fast path runs: the corner
  * correction vector decays by a factor <= 1e-9 within 6 angles of the tear,
  * so it is applied on those angles only (below FP32 resolution elsewhere);
@@ -412,8 +415,8 @@ SE2N_API se2n_status se2n_plan_profile_read(se2n_plan *plan, se2n_profile *out, 
  * method (orientation, lift, DFT, diffusion, restoration, inverse DFT,
  * projection) for every image, captured on the batch's stream. Each warp of
  * the persistent kernel claims (image, frequency-tile) items from an atomic
- * counter, integrated as se2n_diffuse would (the interval polynomial or the
- * steps); the tile size, block size and threads per frequency are taken
+ * counter, integrated as se2n_inpaint would (the steps, or the interval polynomial
+ * where nothing is restored); the tile size, block size and threads per frequency are taken
  * from the built-in table or, with SE2N_BATCH_AUTOTUNE, chosen by timing
  * the candidates on this batch. se2n_batch_run replays the graph.
  * ------------------------------------------------------------------------- */
@@ -435,14 +438,15 @@ typedef struct se2n_batch_info {
     int items;              /* work items of the persistent kernel */
     int tile_passes;        /* warp passes (32/P frequencies each) per item */
     int block, blocks;      /* launch shape of the persistent kernel */
-    int p16, p32, p64;      /* threads per frequency for N = 16, 32, 64 */
-    int fast, split;        /* packed fast path; split diagonal */
+    int p16, p32, p64;      /* threads per frequency for N = 16, 32, 64, where the intervals are stepped */
+    int fast, split;        /* packed fast path; split diagonal, where the intervals are stepped */
     int candidates;         /* launch shapes timed by the autotuner (0 if not run) */
     double best_ms, worst_ms;        /* their fastest and slowest diffusion time */
     double updates_per_run;          /* sum of H W N steps rounds over the images */
     double volume_bytes;             /* device bytes of the lifted volumes */
-    int prop_images;                 /* images integrated by their shape's propagators */
-    double step_updates;             /* frequencies x N x steps of one interval the persistent kernel integrates */
+    int prop_images;                 /* images integrated by their shape's propagators (in either form) */
+    double step_updates;             /* frequencies x N x steps of one interval the persistent kernel integrates,
+                                        by steps or by the polynomial that stands for them */
     int fused_images;                /* of prop_images, those whose whole inpaint runs on the row and column passes */
 } se2n_batch_info;
 
@@ -553,7 +557,8 @@ SE2N_API se2n_status se2n_surrogate_inpaint(se2n_unet *u, se2n_plan *plan, const
  * cudaFree may cause.
  *
  * It integrates the same per-frequency Crank-Nicolson systems as
- * se2n_diffuse, with the same per-frequency kernel code, for up to
+ * se2n_diffuse, step by step (with the per-frequency code that se2n_diffuse has
+ * for its steps; never by the interval polynomial), for up to
  * SE2N_NOALLOC_MAX_VOLUMES transformed volumes (N = 16, 32 or 64, H and W
  * even) in one persistent launch, in place. The caller passes the volumes;
  * the only other memory used is a fixed array of SE2N_NOALLOC_SCRATCH_BYTES

@@ -59,8 +59,8 @@ __global__ void __launch_bounds__(FAST ? kDiffuseMaxBlock : 256, 1) k_diffuse_ba
     }
 }
 
-// The interval polynomial on the same items (poly_group), so that a batched
-// result is again bitwise the image's own.
+// The interval polynomial on the same items (poly_group): bitwise what k_poly does with
+// the same plane.
 template <int N, bool REINSCH>
 __device__ __forceinline__ void poly_item(const PolyTable &t, const float *sc, const float *tables,
                                           const BatchImage &im, const BatchItem &item, int lane) {

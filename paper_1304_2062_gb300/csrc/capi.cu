@@ -1300,7 +1300,7 @@ void choose_propagators(se2n_batch *b) {
     if (!prop_admissible(p.beta, p.T / p.rounds / p.steps)) return;
     const bool half = !p.full_spectrum;
     if (b->poly_on) {
-        // The interval polynomial runs the same arithmetic either way. Shapes
+        // One interval without a restoration: the polynomial either way. Shapes
         // on the row and column passes, and planes with enough angles to give
         // a launch of their own work for the whole device, run apart from the
         // others (which the graph can then do side by side); the small ones

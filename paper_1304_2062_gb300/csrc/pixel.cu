@@ -415,7 +415,8 @@ __global__ void k_scale(float4 *__restrict__ v, long long n4, float s) {
 cudaError_t se2n_launch_orient_prep(const float *f, const uint8_t *mask, float2 *spec, long long HW,
                                     unsigned int *gmax, cudaStream_t s) {
     const long long n = HW / 2;
-    return launch_dependent(k_orient_prep, grid_for(n), kBlock, 0, s, (const float2 *)f, (const uchar2 *)mask, (float4 *)spec, n, gmax);
+    return launch_dependent(k_orient_prep, grid_for(n), kBlock, 0, s, (const float2 *)f, (const uchar2 *)mask,
+                            (float4 *)spec, n, gmax);
 }
 
 cudaError_t se2n_launch_grad_spec(float2 *spec, int H, int W, float sigma, cudaStream_t s) {
@@ -472,21 +473,24 @@ cudaError_t se2n_launch_lift_r(const float *f, const uint8_t *mask, const uint8_
                                int N, cudaStream_t s) {
     const long long n = (long long)H * W / 2;
     const int Wp = W + 2;
-    return launch_dependent(k_lift_r, grid_for(n), kBlock, 0, s, (const float2 *)f, (const uchar2 *)mask, (const uchar2 *)bins, vol, n, W, Wp, (long long)H * Wp, N);
+    return launch_dependent(k_lift_r, grid_for(n), kBlock, 0, s, (const float2 *)f, (const uchar2 *)mask,
+                            (const uchar2 *)bins, vol, n, W, Wp, (long long)H * Wp, N);
 }
 
 cudaError_t se2n_launch_mix_r(float *vol, const float *f, const uint8_t *mask, const uint8_t *bins, int H, int W,
                               int N, float scale, float eps, float guard, cudaStream_t s) {
     const long long n = (long long)H * W / 2;
     const int Wp = W + 2;
-    return launch_dependent(k_mix_r, grid_for(n), kBlock, 0, s, vol, (const float2 *)f, (const uchar2 *)mask, (const uchar2 *)bins, n, W, Wp, (long long)H * Wp, N, scale, eps, guard);
+    return launch_dependent(k_mix_r, grid_for(n), kBlock, 0, s, vol, (const float2 *)f, (const uchar2 *)mask,
+                            (const uchar2 *)bins, n, W, Wp, (long long)H * Wp, N, scale, eps, guard);
 }
 
 cudaError_t se2n_launch_project_r(const float *vol, int H, int W, int N, float scale, int proj, const float *f,
                                   const uint8_t *mask, float *out, cudaStream_t s) {
     const long long n = (long long)H * W / 2;
     const int Wp = W + 2;
-    return launch_dependent(k_project_r, grid_for(n), kBlock, 0, s, vol, n, W, Wp, (long long)H * Wp, N, scale, proj, (const float2 *)f, (const uchar2 *)mask, (float2 *)out);
+    return launch_dependent(k_project_r, grid_for(n), kBlock, 0, s, vol, n, W, Wp, (long long)H * Wp, N, scale, proj,
+                            (const float2 *)f, (const uchar2 *)mask, (float2 *)out);
 }
 
 cudaError_t se2n_launch_dr_max(const float2 *vol, long long HW, int N, float scale, float *h, uint8_t *amax,
