@@ -1085,7 +1085,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1)
 // is a third): wgrad_plan.h ends every sum where it ended when a unit was a tile of
 // 128 (tap, channel) rows, or earlier, however long the range of a CTA is. Up to three
 // CTAs share a unit's tiles.
-// Measured (batch 32, 256 x 256): all 14 layers 1462 us (4832 with a box a tap and
+// Measured (batch 32, 256 x 256): all 14 layers 1540 us (4832 with a box a tap and
 // operand; 888 with as many ranges as SMs).
 // ---------------------------------------------------------------------------
 
